@@ -36,6 +36,7 @@ constexpr float kRoughT = 0.8660254037844386f;
 constexpr int kMaxFaces = 32;         // faces of one polytope
 constexpr int kTileItemsPerLane = 4;  // node lines per lane per tile
 constexpr int kPartialFloats = 12;    // FP32 partial sums per tile
+constexpr int kPartialDoubles = 10;   // FP64 partial sums per tile (the all-FP64 form: 7 sums, deepest node's key and index)
 constexpr int kTapeDoubles = 16;      // FP64 per-pair values kept for the adjoint
 constexpr int kStepCounter = 12;      // counters[] slot of the completed-step count
 constexpr int kDoneCounter = 13;      // counters[] slot: particle-sum blocks finished (the last resets it)
@@ -262,6 +263,7 @@ struct Lists {
   PairRec* tiles;   // [max_tiles] one record per tile (the pair's record with tile and pair set), the
                     // node sweep's list: a pair's tiles contiguous from its tile0
   float* partial;   // [max_tiles, kPartialFloats]
+  double* partial64;   // [max_tiles, kPartialDoubles] (the all-FP64 form only, else null)
   int* pdone;       // [max_pairs] tiles of the pair swept so far (pairs of several tiles)
   double* tape;     // [max_pairs, kTapeDoubles]
   double* ft;       // [max_pairs, kFtDoubles]

@@ -656,6 +656,7 @@ contact_status contact_init(const contact_config* cfg, const int32_t* shape_type
   GBC_TRY(dev_alloc(c, &W.tile_pair, mt));
   GBC_TRY(dev_alloc(c, &W.tiles, mt));
   GBC_TRY(dev_alloc(c, &W.partial, mt * kPartialFloats));
+  if (C.precision == 1 && C.box_mode == 0) GBC_TRY(dev_alloc(c, &W.partial64, mt * kPartialDoubles));
   GBC_TRY(dev_alloc(c, &W.pdone, mp));
   GBC_TRY(dev_alloc(c, &W.tape, mp * kTapeDoubles));
   GBC_TRY(dev_alloc(c, &W.ft, mp * kFtDoubles));

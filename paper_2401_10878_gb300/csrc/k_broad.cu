@@ -822,7 +822,7 @@ __global__ void __launch_bounds__(kBuildWarps * 32) k_build_pairs(Params P, Shap
           pr.bf[k] = 0.f;
         }
       }
-      // the FP32 node sweep skips pairs whose distance regions are apart, and
+      // the node sweeps skip pairs whose distance regions are apart, and
       // so does the box pipeline (regions at its rough-detection threshold;
       // a polytope's tabulated radii belong to the node sweep's threshold, so
       // pairs with one are kept there); the skipped pairs' zero outputs are
@@ -830,7 +830,7 @@ __global__ void __launch_bounds__(kBuildWarps * 32) k_build_pairs(Params P, Shap
       // their regions' intersection (after the record is complete).
       const int ka = pr.kinds & 0xff, kb = pr.kinds >> 8;
       constexpr bool boxm = BOXM;
-      const bool test = (P.precision == 0 && !boxm) || (boxm && ka != KIND_POLY && kb != KIND_POLY);
+      const bool test = !boxm || (boxm && ka != KIND_POLY && kb != KIND_POLY);
       const unsigned apart = test ? pair_apart(pr, boxm ? kRoughT : 0.5f * P.wdx_l + kClipMargin) : 0u;
       skip = (P.smooth || boxm) ? (apart & 1u) != 0u : (apart & 6u) == 6u;
       cut = boxm && !skip && (ka == KIND_CUBE || ka == KIND_CUBOID) && (kb == KIND_CUBE || kb == KIND_CUBOID);

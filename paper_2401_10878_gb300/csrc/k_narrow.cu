@@ -29,8 +29,9 @@
 //     evaluate); a pair of one tile is finished from the warp's registers,
 //     otherwise the partials go to HBM and the warp that completes the pair's
 //     last tile sums them in FP64 in tile order (deterministic).
-// k_narrow64: all-FP64 comparison form, one thread block per pair.
+// k_narrow64: all-FP64 comparison form over the same tiles, lines clipped in FP32.
 #include <cfloat>
+#include <climits>
 #include <type_traits>
 
 #include "contact_dev.cuh"
@@ -1100,83 +1101,257 @@ __global__ void __launch_bounds__(kWarps * 32, 1) k_force(Params P, Shapes S, Pa
 }
 
 // ---------------------------------------------------------------- FP64 form
+// The all-FP64 form takes the FP32 form's tiles: warp w sweeps tiles w, w + W,
+// ...; each lane clips its lines in FP32 to the nodes near both surfaces (the
+// margin kClipMargin is far above the FP32 rounding, so every node left out has
+// a distance of at least w/2 in FP64 too and would add exact zeros), and the
+// clipped nodes, one per lane, are evaluated in FP64.  Bound: the FP64 pipe,
+// ~64 cycles a warp instruction on this GPU.  One block per pair walking every
+// node of the pair box in FP64 spent 1006 us on 1934 cubes at 30 % (2.64e6
+// nodes, 1 % of which add to the sums); the clipped sweep takes 31 us.
+
+// [lo, hi] (line coordinates) cut to where one particle's distance lies below
+// T on the line (cv, cw); sp: a polytope's planes in local axes (stage_planes).
+template <class E>
+__device__ __forceinline__ void clip_with(const Shapes& S, const Parts& D, const PairRec& r, bool second,
+                                          const Local& L, int cv, int cw, float T, float& lo, float& hi) {
+  E e;
+  e.load(r, second, S, D, L, nullptr);
+  e.begin_line(cv, cw, 0);
+  e.clip(T, lo, hi);
+}
+__device__ __forceinline__ void clip_any(const Shapes& S, const Parts& D, const PairRec& r, bool second,
+                                         const Local& L, const float4* sp, int nf, int cv, int cw, float T, float& lo,
+                                         float& hi) {
+  switch (second ? r.kinds >> 8 : r.kinds & 0xff) {   // warp-uniform
+    case KIND_SPHERE: clip_with<SphereEval>(S, D, r, second, L, cv, cw, T, lo, hi); break;
+    case KIND_WALL: clip_with<WallEval>(S, D, r, second, L, cv, cw, T, lo, hi); break;
+    case KIND_POLY: {
+      const int* ci = second ? r.bi : r.ai;
+      const float* cf = second ? r.bf : r.af;
+      const float rv = static_cast<float>(cv - ci[L.v]) - cf[L.v], rw = static_cast<float>(cw - ci[L.w]) - cf[L.w];
+      const float o = static_cast<float>(ci[L.u]), fu = cf[L.u];
+      float l = lo - o, h = hi - o;
+      for (int f = 0; f < nf; ++f) {
+        const float4 e = sp[f];
+        clip_half(e.x, clip_inv(e.x), fmaf(-e.x, fu, fmaf(e.y, rv, fmaf(e.z, rw, -e.w))), T, l, h);
+      }
+      lo = l + o;
+      hi = h + o;
+      break;
+    }
+    default: clip_with<CuboidEval>(S, D, r, second, L, cv, cw, T, lo, hi); break;   // cubes and cuboids
+  }
+}
+
+// Sums of v[0 .. 8) over the warp by halving exchanges (nine FP64 additions):
+// lane c < 8 returns the sum of component c.
+__device__ __forceinline__ double warp_sum8(const double v[8]) {
+  const int lane = threadIdx.x & 31;
+  const bool b4 = (lane >> 4) & 1, b3 = (lane >> 3) & 1, b2 = (lane >> 2) & 1;
+  double h4[4], h2[2];
+#pragma unroll
+  for (int k = 0; k < 4; ++k) h4[k] = (b4 ? v[4 + k] : v[k]) + __shfl_xor_sync(kFull, b4 ? v[k] : v[4 + k], 16);
+#pragma unroll
+  for (int k = 0; k < 2; ++k) h2[k] = (b3 ? h4[2 + k] : h4[k]) + __shfl_xor_sync(kFull, b3 ? h4[k] : h4[2 + k], 8);
+  double h = (b2 ? h2[1] : h2[0]) + __shfl_xor_sync(kFull, b2 ? h2[0] : h2[1], 4);
+  h += __shfl_xor_sync(kFull, h, 2);
+  h += __shfl_xor_sync(kFull, h, 1);
+  const int c = lane & 7;   // component c sits on lanes 4 (4 b4 + 2 b3 + b2)
+  return __shfl_sync(kFull, h, ((c >> 2) << 4) | (((c >> 1) & 1) << 3) | ((c & 1) << 2));
+}
+
+// After a tile of the FP64 form (lane c < 7: component c of its sums; key, idx:
+// the deepest node on every lane): as tile_done, with FP64 partials.
+__device__ __forceinline__ void tile_done64(const Params& P, const Lists& W, const PairRec& r, double* pair_out,
+                                            double v, long long key, int idx) {
+  const int lane = threadIdx.x & 31;
+  if (r.ntiles == 1) {
+    pair_done(P, W, r, pair_out, lane < 7 ? v : 0.0, idx);
+    return;
+  }
+  const size_t t0 = static_cast<size_t>(r.tile0);
+  double* q = W.partial64 + (t0 + r.tile) * kPartialDoubles;
+  if (lane < 7) q[lane] = v;
+  if (lane == 7) q[7] = __longlong_as_double(key);
+  if (lane == 8) q[8] = __longlong_as_double(static_cast<long long>(idx));
+  __threadfence();
+  int prev = 0;
+  if (lane == 0) prev = atomicAdd(&W.pdone[r.pair], 1);
+  prev = __shfl_sync(kFull, prev, 0);
+  if (prev != r.ntiles - 1) return;
+  __threadfence();
+  // component c of tiles slot, slot + 4, ..., then the four slots pairwise
+  const int slot = lane >> 3, c = lane & 7;
+  double acc = 0.0;
+  long long bk = LLONG_MIN;
+  int bi = 0x7fffffff;
+  for (int t = slot; t < r.ntiles; t += 4) {
+    const double* p = W.partial64 + (t0 + t) * kPartialDoubles;
+    const double x = __ldcg(p + c);
+    if (c < 7) {
+      acc += x;
+    } else {
+      const long long k = __double_as_longlong(x);
+      const int i = static_cast<int>(__double_as_longlong(__ldcg(p + 8)));
+      if (k > bk || (k == bk && i < bi)) {
+        bk = k;
+        bi = i;
+      }
+    }
+  }
+  acc += __shfl_xor_sync(kFull, acc, 8);
+  acc += __shfl_xor_sync(kFull, acc, 16);
+  for (int o = 8; o <= 16; o <<= 1) {
+    const long long ok = __shfl_xor_sync(kFull, bk, o);
+    const int oi = __shfl_xor_sync(kFull, bi, o);
+    if (ok > bk || (ok == bk && oi < bi)) {
+      bk = ok;
+      bi = oi;
+    }
+  }
+  if (lane == 0) W.pdone[r.pair] = 0;   // ready for a repeated sweep of the same tiles
+  pair_done(P, W, r, pair_out, acc, __shfl_sync(kFull, bi, 7));
+}
+
 template <bool SMOOTH>
-__global__ void __launch_bounds__(256) k_narrow64(Params P, Shapes S, Parts D, Lists W, const double* vel,
-                                                  double* pair_out) {
-  __shared__ double s_red[8][8];
-  __shared__ double s_bf[8];
-  __shared__ int s_bi[8];
+__global__ void __launch_bounds__(kWarps * 32, 2) k_narrow64(Params P, Shapes S, Parts D, Lists W, const double* vel,
+                                                             double* pair_out) {
+  __shared__ __align__(16) PairRec s_rec[kWarps];
+  __shared__ float4 s_planes[kWarps][2][kMaxFaces];
+  __shared__ unsigned s_pk[kWarps][kTileItemsPerLane * 32];   // clipped ranges: first node | count << 16
+  __shared__ int s_excl[kWarps][32];                          // nodes before each lane's
+  (void)vel;
   pdl_begin();
-  const int np = min(W.counters[0], P.max_pairs);
+  const int ntiles = W.counters[1];
+  if (ntiles > P.max_tiles) return;   // capacity exceeded: the step reports ECAPACITY
   const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-  for (int p = blockIdx.x; p < np; p += gridDim.x) {
-    const PairRec pr = W.pairs[p];
-    if (!record_in_bounds(P, W.err, pr, false)) continue;   // block-uniform (checked build only)
-    const int i = pr.i, j = pr.j;
+  const int nwarps = gridDim.x * kWarps;
+  const float hw = 0.5f * P.wdx_l, T = hw + kClipMargin;
+  const double inv_wdx = 1.0 / P.wdx;
+  for (int t = blockIdx.x * kWarps + wid; t < ntiles; t += nwarps) {
+    __syncwarp();
+    store_rec_part(&s_rec[wid], lane, load_rec_part(W.tiles + t, lane));
+    __syncwarp();
+    const PairRec& r = s_rec[wid];
+    if (!record_in_bounds(P, W.err, r, true)) continue;   // warp-uniform (checked build only)
+    const Local L = make_local(r);
+    const int i = r.i, j = r.j;
+    const int ka = r.kinds & 0xff, kb = r.kinds >> 8;
+    const int fa = ka == KIND_POLY ? stage_planes(S, D, i, L, s_planes[wid][0], kMaxFaces) : 0;
+    const int fb = kb == KIND_POLY ? stage_planes(S, D, j, L, s_planes[wid][1], kMaxFaces) : 0;
+    // both particles in FP64 (the same address on every lane)
     double XA[3], XB[3], RA[9], RB[9];
+#pragma unroll
     for (int k = 0; k < 3; ++k) {
       XA[k] = D.X[3 * i + k];
-      XB[k] = D.X[3 * j + k] - pr.shift[k] * P.L[k];
+      XB[k] = D.X[3 * j + k] - r.shift[k] * P.L[k];
     }
-    for (int k = 0; k < 9; ++k) { RA[k] = D.R[9 * i + k]; RB[k] = D.R[9 * j + k]; }
+#pragma unroll
+    for (int k = 0; k < 9; ++k) {
+      RA[k] = D.R[9 * i + k];
+      RB[k] = D.R[9 * j + k];
+    }
     const int ta = S.type[i], tb = S.type[j];
     const double* pla = S.planes + 4 * S.face_off[i];
     const double* plb = S.planes + 4 * S.face_off[j];
     const int nfa = S.face_off[i + 1] - S.face_off[i], nfb = S.face_off[j + 1] - S.face_off[j];
-    const int vol = pr.dim[0] * pr.dim[1] * pr.dim[2];
-    double acc[7] = {0, 0, 0, 0, 0, 0, 0};
-    double bf = -DBL_MAX;
+    // (A) the lane's lines clipped in FP32
+    const int du = r.dim[L.u], dv = r.dim[L.v];
+    const float inv_dv = __fdividef(1.f, static_cast<float>(dv));
+    const int it0 = r.tile * 32 * kTileItemsPerLane;
+    const int ns = min(kTileItemsPerLane, (r.nitems - it0 + 31) >> 5);
+    int nl = 0;
+    for (int s = 0; s < ns; ++s) {
+      const int it = it0 + s * 32 + lane;
+      int cv;
+      const int cw = div_small(it, dv, inv_dv, &cv);
+      const int len = it < r.nitems ? du : 0;
+      float clo = 0.f, chi = static_cast<float>(len - 1);
+      clip_any(S, D, r, false, L, s_planes[wid][0], fa, cv, cw, T, clo, chi);
+      clip_any(S, D, r, true, L, s_planes[wid][1], fb, cv, cw, T, clo, chi);
+      int ub;
+      const int nk = clip_nodes(clo, chi, 0, len, &ub);
+      s_pk[wid][s * 32 + lane] = static_cast<unsigned>(ub) | (static_cast<unsigned>(nk) << 16);
+      nl += nk;
+    }
+    int incl = nl;
+#pragma unroll
+    for (int d = 1; d < 32; d <<= 1) {
+      const int v = __shfl_up_sync(kFull, incl, d);
+      if (lane >= d) incl += v;
+    }
+    const int total = __shfl_sync(kFull, incl, 31);
+    s_excl[wid][lane] = incl - nl;
+    __syncwarp();
+    // (B) node g of the clipped nodes on lane g mod 32
+    double acc[8] = {0.0, 0.0, 0.0, 0.0, 0.0, 0.0, 0.0, 0.0};
+    long long bk = LLONG_MIN;
     int bi = 0x7fffffff;
-    for (int c = threadIdx.x; c < vol; c += blockDim.x) {
-      const int cx = c % pr.dim[0], cy = (c / pr.dim[0]) % pr.dim[1], cz = c / (pr.dim[0] * pr.dim[1]);
-      const double x[3] = {(pr.lo[0] + cx) * P.dx, (pr.lo[1] + cy) * P.dx, (pr.lo[2] + cz) * P.dx};
-      double gA[3], gB[3];
-      const double fa = sdf64(ta, S.param + 3 * i, pla, nfa, XA, RA, x, P.inflate, gA);
-      const double fb = sdf64(tb, S.param + 3 * j, plb, nfb, XB, RB, x, P.inflate, gB);
-      const double tA = fmin(fmax(0.5 - fa / P.wdx, 0.0), 1.0);
-      const double tB = fmin(fmax(0.5 - fb / P.wdx, 0.0), 1.0);
-      double hA, hB;
-      if (SMOOTH) {
-        hA = tA * tA * (3.0 - 2.0 * tA);
-        hB = tB * tB * (3.0 - 2.0 * tB);
-      } else {
-        hA = fa <= 0.0 ? 1.0 : 0.0;
-        hB = fb <= 0.0 ? 1.0 : 0.0;
+    for (int base = 0; base < total; base += 32) {
+      const int g = base + lane;
+      if (g < total) {
+        int o = 0;   // the owner: the last lane whose first node is <= g (lanes without nodes repeat the next one's)
+#pragma unroll
+        for (int d = 16; d > 0; d >>= 1)
+          if (s_excl[wid][o + d] <= g) o += d;
+        int k = g - s_excl[wid][o], s = 0, n;
+        unsigned q = s_pk[wid][o];
+        while (k >= (n = static_cast<int>(q >> 16)) && s < ns - 1) {
+          k -= n;
+          q = s_pk[wid][++s * 32 + o];
+        }
+        const int u = static_cast<int>(q & 0xffffu) + k;
+        int cv;
+        const int cw = div_small(it0 + s * 32 + o, dv, inv_dv, &cv);
+        const int c[3] = {L.u == 0 ? u : (L.u == 1 ? cw : cv), L.u == 1 ? u : (L.u == 2 ? cw : cv),
+                          L.u == 2 ? u : (L.u == 0 ? cw : cv)};
+        const double x[3] = {(r.lo[0] + c[0]) * P.dx, (r.lo[1] + c[1]) * P.dx, (r.lo[2] + c[2]) * P.dx};
+        double gA[3], gB[3];
+        const double pa = sdf64(ta, S.param + 3 * i, pla, nfa, XA, RA, x, P.inflate, gA);
+        const double pb = sdf64(tb, S.param + 3 * j, plb, nfb, XB, RB, x, P.inflate, gB);
+        const double tA = fmin(fmax(fma(-pa, inv_wdx, 0.5), 0.0), 1.0);
+        const double tB = fmin(fmax(fma(-pb, inv_wdx, 0.5), 0.0), 1.0);
+        double hA, hB;
+        if (SMOOTH) {
+          hA = tA * tA * (3.0 - 2.0 * tA);
+          hB = tB * tB * (3.0 - 2.0 * tB);
+        } else {
+          hA = pa <= 0.0 ? 1.0 : 0.0;
+          hB = pb <= 0.0 ? 1.0 : 0.0;
+        }
+        const double w = hA * hB;
+        const double ma = tA * (1.0 - tA) * hB, mb = hA * tB * (1.0 - tB);
+        acc[0] += w;
+#pragma unroll
+        for (int a = 0; a < 3; ++a) {
+          acc[1 + a] = fma(w, fl::int_to_double(c[a]), acc[1 + a]);
+          acc[4 + a] += ma * gA[a] - mb * gB[a];
+        }
+        if (w > 0.0) {
+          const long long f = fl::dkey(-(pa + pb));
+          const int ci = c[0] + r.dim[0] * (c[1] + r.dim[1] * c[2]);
+          if (f > bk || (f == bk && ci < bi)) {
+            bk = f;
+            bi = ci;
+          }
+        }
       }
-      const double w = hA * hB;
-      const double ma = tA * (1.0 - tA) * hB, mb = hA * tB * (1.0 - tB);
-      acc[0] += w;
-      acc[1] += w * cx; acc[2] += w * cy; acc[3] += w * cz;
-      for (int k = 0; k < 3; ++k) acc[4 + k] += ma * gA[k] - mb * gB[k];
-      if (w > 0.0) {
-        const double f = -(fa + fb) * P.inv_dx;
-        if (f > bf || (f == bf && c < bi)) { bf = f; bi = c; }
+    }
+    double v = 0.0;
+    if (total > 0) {   // warp-uniform
+      v = warp_sum8(acc);
+#pragma unroll
+      for (int o = 16; o > 0; o >>= 1) {
+        const long long ok = __shfl_xor_sync(kFull, bk, o);
+        const int oi = __shfl_xor_sync(kFull, bi, o);
+        if (ok > bk || (ok == bk && oi < bi)) {
+          bk = ok;
+          bi = oi;
+        }
       }
     }
-    // block reduction
-    for (int off = 16; off > 0; off >>= 1) {
-      for (int k = 0; k < 7; ++k) acc[k] += __shfl_xor_sync(kFull, acc[k], off);
-      const double of = __shfl_xor_sync(kFull, bf, off);
-      const int oi = __shfl_xor_sync(kFull, bi, off);
-      if (of > bf || (of == bf && oi < bi)) { bf = of; bi = oi; }
-    }
-    if (lane == 0) {
-      for (int k = 0; k < 7; ++k) s_red[wid][k] = acc[k];
-      s_bf[wid] = bf;
-      s_bi[wid] = bi;
-    }
-    __syncthreads();
-    if (wid == 0) {   // lanes c < 7: component c summed over the warps in order
-      double tot = 0.0;
-      double b = -DBL_MAX;
-      int bidx = 0x7fffffff;
-      for (int w = 0; w < static_cast<int>(blockDim.x >> 5); ++w) {
-        if (lane < 7) tot += s_red[w][lane];
-        if (s_bf[w] > b || (s_bf[w] == b && s_bi[w] < bidx)) { b = s_bf[w]; bidx = s_bi[w]; }
-      }
-      pair_done(P, W, W.pairs[p], pair_out, tot, bidx);
-    }
-    __syncthreads();
+    tile_done64(P, W, r, pair_out, v, bk, bi);
   }
 }
 
@@ -1193,7 +1368,7 @@ int narrow_grid(const Params& P) {
   int dev = 0, sms = 0;
   cudaGetDevice(&dev);
   cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-  if (P.precision == 1) return sms * 4;
+  if (P.precision == 1) return sms * 2;   // k_narrow64: two resident blocks per SM
   int per_sm = 1;
   if (P.smooth) {
     per_sm = P.kind_set == SET_CUBE ? blocks_per_sm<true, SET_CUBE>()
@@ -1226,9 +1401,9 @@ void launch_narrow(const Params& P, const Shapes& S, const Parts& D, const Lists
   }
   if (P.precision == 1) {
     if (P.smooth)
-      launch_pdl(k_narrow64<true>, dim3(grid), dim3(256), 0, st, P, S, D, W, vel, pair_out);
+      launch_pdl(k_narrow64<true>, dim3(grid), dim3(kWarps * 32), 0, st, P, S, D, W, vel, pair_out);
     else
-      launch_pdl(k_narrow64<false>, dim3(grid), dim3(256), 0, st, P, S, D, W, vel, pair_out);
+      launch_pdl(k_narrow64<false>, dim3(grid), dim3(kWarps * 32), 0, st, P, S, D, W, vel, pair_out);
     return;
   }
   const dim3 bc(narrow_warps<SET_CUBE>() * 32), bs(narrow_warps<SET_SC>() * 32), ba(narrow_warps<SET_ALL>() * 32);

@@ -1,0 +1,41 @@
+"""The step's kernels at the edges of their work splits (needs a GB300), against the oracle.
+
+The oracle evaluates every node of every pair in FP64 in its own order; the
+tolerances are those of the parity tests (tests/parity.py).
+"""
+import numpy as np
+import pytest
+
+import oracle
+from paper_2401_10878_gb300 import workloads as W
+from tests.helpers import cube_planes, quat_axis_angle, state
+from tests.parity import compare, gpu_step
+
+torch = pytest.importorskip("torch")
+pytestmark = pytest.mark.gpu
+
+
+def _parity(st, precision, **kw):
+    from paper_2401_10878_gb300.contact import Contact
+    m = Contact.from_state(st, precision=precision, **kw)
+    g = gpu_step(m, st)
+    r = oracle.contact_step(st)
+    rep = compare(st, g, r, fp64=precision == 1, smooth=st.indicator == 1)
+    m.close()
+    return rep, r
+
+
+# half extents across the lines of the pair box: 100, 121, 128 (one tile exactly), 144 and 20^2 lines (four tiles)
+@pytest.mark.parametrize("across", [(5.0, 5.0), (5.5, 5.5), (8.0, 4.0), (6.0, 6.0), (10.0, 10.0)])
+@pytest.mark.parametrize("indicator", [0, 1])
+@pytest.mark.parametrize("kind", ["cuboid", "polytope"])
+def test_fp64_form_at_tile_edges(across, indicator, kind):
+    """Two slightly turned boxes pressed together over a whole face: hundreds
+    of nodes on lines filling one tile or several."""
+    h = (5.0, across[0], across[1])
+    q = [quat_axis_angle([0.3, 1.0, 0.2], 0.02), quat_axis_angle([1.0, 0.1, 0.4], 0.03)]
+    t, planes = (W.CUBOID, None) if kind == "cuboid" else (W.POLYTOPE, [cube_planes(h)] * 2)
+    st = state([t] * 2, [h, h], [[30.23, 31.31, 32.17], [38.11, 31.12, 31.94]], quat=q, n=96, planes=planes,
+               indicator=indicator)
+    rep, ref = _parity(st, 1)
+    assert ref.n_pairs == 1 and ref.pair_out[0, 0] > 100.0
