@@ -4,8 +4,8 @@
 //   shape tables (read-only): type/kind per particle, FP64 body parameters,
 //     body planes, offset-shape vertices (for the AABB), E and nu;
 //   per-step particle records: FP64 pose copy (the adjoint's tape), FP64
-//     rotation, node ranges, bins, FP32 geometry for the node sweep
-//     (R^T rows, effective sizes, world-frame polytope planes);
+//     rotation, one 128-byte line of node range, bin and FP32 geometry for the
+//     pair kernels (PartRec), world-frame polytope planes;
 //   pair list: PairRec per candidate pair, tile -> pair map, FP32 tile
 //     partials, FP64 per-pair sums and results.
 #pragma once
@@ -105,7 +105,9 @@ struct Params {
   double damp_K;         // history: c = damp_K / u0 at a contact's first step (u0 > 0)
   double mu_s_star, mu_k, inv_u_k;   // friction law
   int nbin[3];           // bins per axis
-  int bin_cap;           // particles one bin can hold (bin_items row length)
+  int bin_cap;           // particles one bin can hold
+  int bin_stride;        // entries of a bin's rows (bin_cap rounded up to a multiple of four: 16-byte loads)
+  int wide;              // 1: a node range may span more than kMaxLen nodes (BinRec's lengths do not hold it)
   double binw[3];        // bin width (physical)
   float inv_binw_f[3];   // FP32 reciprocal of the bin width
   int max_pairs, max_nbr, max_tiles;
@@ -133,19 +135,43 @@ struct Shapes {
   const int* poly_ids;     // [npoly] the polytope particles (the pose kernel's polytope warps)
 };
 
+// What the pair kernels read of one particle, as one 128-byte line (seven
+// 16-byte loads).  Read as separate arrays it was 27 scattered 4-byte loads a
+// pair side in the pair builder and nine a candidate in the broad phase.
+struct __align__(128) PartRec {
+  int lo[3];       // node range of the offset shape, lower ...
+  int kind;        // sweep kind | nominal lane-ops of one signed-distance test << 8
+  int hi[3];       // ... and upper corner
+  int bin;         // cell-list bin
+  int kX[3];       // nearest node of X / dx
+  float sz0;       // size_l: lattice units incl. inflate (Shapes::size_l)
+  float fX[3];     // X / dx - kX, in [-1/2, 1/2] (FP64 difference, rounded once)
+  float sz1;
+  float rt[9];     // FP32 R^T (row k = body axis k in world)
+  float sz2;
+  int pad[6];
+};
+static_assert(sizeof(PartRec) == 128, "one particle record per 128-byte line");
+constexpr int kPartRecParts = 7;   // 16-byte pieces in use
+
+// A cell-list entry: all that the broad phase's test needs of a candidate, so
+// that it takes one 16-byte load.  Lower corner of the node range and its
+// nodes per axis (ten bits each); a range without nodes has lo[0] = kNoNodes.
+struct __align__(16) BinRec {
+  int lo[3];
+  unsigned len;
+};
+constexpr int kMaxLen = 1023;
+constexpr int kNoNodes = -0x40000000;
+
 // Per-step particle records; rows N .. N + nwall - 1 are the walls (set once:
-// X = 0, R = I, Rt row 0 = the wall normal m, kX = fX = 0).
+// X = 0, R = I, rec's rt row 0 = the wall normal m, kX = fX = 0).
 struct Parts {
   double* X;       // [N,3] copy of the positions of the step
   double* qhat;    // [N,4] the step's quaternion as given (normalised by the adjoint)
   double* R;       // [N,9] FP64 rotation, row-major, body -> world
-  int* lohi;       // [N,6]
-  int* bin;        // [N]
-  float* Rt;       // [N,9] FP32 R^T (row k = body axis k in world)
+  PartRec* rec;    // [N] node range, bin and FP32 sweep geometry
   float4* wplane;  // [F] FP32 world normal, offset (lattice units, incl. inflate)
-  float* Xf;       // [N,3] FP32 positions (periodic image choice only)
-  int* kX;         // [N,3] nearest node of X / dx
-  float* fX;       // [N,3] X / dx - kX, in [-1/2, 1/2] (FP64 difference, rounded once)
   const double* rest6;   // [6] zeros: the velocity of a wall
 };
 
@@ -243,7 +269,8 @@ static_assert(sizeof(OvlRec) == 128, "one overlap record per 128-byte line");
 
 struct Lists {
   int* bin_count;   // [nbins]
-  int* bin_items;   // [nbins, bin_cap] particles of each bin, in arrival order
+  int* bin_items;   // [nbins, bin_stride] particles of each bin, in arrival order
+  BinRec* bin_rec;  // [nbins, bin_stride] their node ranges
   int* up_count;    // [N] partners j > p
   int* up_list;     // [N, max_nbr]
   int* dn_count;    // [N] partners i < p
@@ -323,6 +350,42 @@ __device__ inline void rotation_rn(const double q[4], double* qh, double* qn, do
   R[6] = dmul(2.0, dsub(dmul(x, z), dmul(w, y)));
   R[7] = dmul(2.0, dadd(dmul(y, z), dmul(w, x)));
   R[8] = dsub(1.0, dmul(2.0, dadd(dmul(x, x), dmul(y, y))));
+}
+
+// Order-preserving integer key of an FP64 value (comparisons without FP64 instructions).
+__device__ __forceinline__ long long order_key(double x) {
+  const long long b = __double_as_longlong(x);
+  return b ^ ((b >> 63) & 0x7fffffffffffffffLL);
+}
+
+// floor(v) as an int clamped to +-1e9 with integer operations (finite v): the
+// conversions, roundings and comparisons of FP64 values run on the FP64 pipe.
+__device__ __forceinline__ int floor_node(double v) {
+  const long long b = __double_as_longlong(v);
+  const int e = static_cast<int>((b >> 52) & 0x7ff) - 1023;
+  if (e < 0) return (b < 0 && (b << 1) != 0) ? -1 : 0;   // |v| < 1
+  if (e >= 30) return b < 0 ? -1000000000 : 1000000000;
+  const unsigned long long m = (static_cast<unsigned long long>(b) & 0xfffffffffffffULL) | 0x10000000000000ULL;
+  const int ip = static_cast<int>(m >> (52 - e));
+  const bool frac = (m << (12 + e)) != 0ULL;
+  const int f = b < 0 ? -ip - (frac ? 1 : 0) : ip;
+  return min(max(f, -1000000000), 1000000000);
+}
+__device__ __forceinline__ int ceil_node(double v) {
+  return -floor_node(__longlong_as_double(__double_as_longlong(v) ^ static_cast<long long>(0x8000000000000000ULL)));
+}
+
+// FP64 -> FP32, round to nearest even, with integer operations where the
+// result is a normal number or the argument zero.
+__device__ __forceinline__ float narrow(double v) {
+  const unsigned long long b = static_cast<unsigned long long>(__double_as_longlong(v));
+  const unsigned long long a = b & 0x7fffffffffffffffULL;
+  const unsigned sgn = static_cast<unsigned>(b >> 32) & 0x80000000u;
+  const unsigned e = static_cast<unsigned>(a >> 52);
+  if (a == 0ULL) return __uint_as_float(sgn);
+  if (e - 897u >= 253u) return static_cast<float>(v);   // subnormal or near overflow: the conversion instruction
+  const unsigned long long r = a + 0xfffffffULL + ((a >> 29) & 1ULL);
+  return __uint_as_float(sgn | (static_cast<unsigned>(r >> 29) - (896u << 23)));
 }
 
 // FP64 signed distance (physical units, reduced by inflate) at world point x
@@ -415,6 +478,9 @@ void launch_broad(const Params& P, const Parts& D, const Lists& W, cudaStream_t 
 void launch_plan(const Params& P, const Shapes& S, const Parts& D, const Lists& W, int32_t* pair_ij, int32_t* n_pairs,
                  double* pair_out, cudaStream_t st);
 constexpr int kRowGroup = 256;   // particles per group sum of the pair-row offsets
+// the row length of bin_cap entries, and whether BinRec's lengths suffice for particles of circumradius rmax
+inline int bin_row(int bin_cap) { return (bin_cap + 3) & ~3; }
+inline int wide_ranges(double rmax, double dx) { return 2.0 * rmax / dx + 3.0 >= kMaxLen ? 1 : 0; }
 int bin_capacity(int n, const double binw[3], double rin_min, long long nbins, long long max_entries);
 void launch_narrow(const Params& P, const Shapes& S, const Parts& D, const Lists& W, const double* vel,
                    double* pair_out, int grid, cudaStream_t st);

@@ -70,11 +70,7 @@ __device__ __forceinline__ double nr_rsqrt(double a) {
 }
 
 // max of two doubles by their order-preserving integer keys (no FP64 instruction)
-__device__ __forceinline__ long long dkey(double x) {
-  const long long b = __double_as_longlong(x);
-  return b ^ ((b >> 63) & 0x7fffffffffffffffLL);
-}
-__device__ __forceinline__ double dmax(double a, double b) { return dkey(a) >= dkey(b) ? a : b; }
+__device__ __forceinline__ double dmax(double a, double b) { return order_key(a) >= order_key(b) ? a : b; }
 
 // Exact int -> FP64 conversion with integer operations (|v| < 2^31).
 __device__ __forceinline__ double int_to_double(int v) {

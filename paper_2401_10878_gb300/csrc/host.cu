@@ -492,6 +492,8 @@ contact_status contact_init(const contact_config* cfg, const int32_t* shape_type
     P.inv_binw_f[k] = static_cast<float>(nb / L[k]);
   }
   P.bin_cap = bin_capacity(n, P.binw, rin_min, static_cast<long long>(P.nbin[0]) * P.nbin[1] * P.nbin[2], 1LL << 26);
+  P.bin_stride = bin_row(P.bin_cap);
+  P.wide = wide_ranges(rmax, C.dx);
   P.dx = C.dx;
   P.inv_dx = 1.0 / C.dx;
   {
@@ -591,39 +593,29 @@ contact_status contact_init(const contact_config* cfg, const int32_t* shape_type
   GBC_TRY(dev_alloc(c, &D.X, 3 * static_cast<size_t>(nrows)));
   GBC_TRY(dev_alloc(c, &D.qhat, 4 * static_cast<size_t>(n)));
   GBC_TRY(dev_alloc(c, &D.R, 9 * static_cast<size_t>(nrows)));
-  GBC_TRY(dev_alloc(c, &D.lohi, 6 * static_cast<size_t>(nrows)));
-  GBC_TRY(dev_alloc(c, &D.bin, static_cast<size_t>(n)));
-  GBC_TRY(dev_alloc(c, &D.Rt, 9 * static_cast<size_t>(nrows)));
+  GBC_TRY(dev_alloc(c, &D.rec, static_cast<size_t>(nrows)));
   GBC_TRY(dev_alloc(c, &D.wplane, static_cast<size_t>(std::max(nplanes, 1))));
-  GBC_TRY(dev_alloc(c, &D.Xf, 3 * static_cast<size_t>(nrows)));
-  GBC_TRY(dev_alloc(c, &D.kX, 3 * static_cast<size_t>(nrows)));
-  GBC_TRY(dev_alloc(c, &D.fX, 3 * static_cast<size_t>(nrows)));
   {
     double* rest = nullptr;
     GBC_TRY(dev_alloc(c, &rest, 8));
     GBC_TRY(cudaMemset(rest, 0, 8 * sizeof(double)));
     D.rest6 = rest;
   }
-  if (nw > 0) {   // wall rows: at the origin, identity rotation, Rt row 0 = m, world plane
+  if (nw > 0) {   // wall rows: at the origin, identity rotation, rec's rt row 0 = m, world plane
     std::vector<double> X0(3 * static_cast<size_t>(nw), 0.0), R0(9 * static_cast<size_t>(nw), 0.0);
-    std::vector<float> Rt0(9 * static_cast<size_t>(nw), 0.f), f0(3 * static_cast<size_t>(nw), 0.f);
-    std::vector<int> k0(3 * static_cast<size_t>(nw), 0), lohi0(6 * static_cast<size_t>(nw), 0);
+    std::vector<PartRec> rec0(nw, PartRec{});
     std::vector<float4> wp(nw);
     for (int w = 0; w < nw; ++w) {
       R0[9 * w] = R0[9 * w + 4] = R0[9 * w + 8] = 1.0;
-      for (int k = 0; k < 3; ++k) Rt0[9 * w + k] = static_cast<float>(C.walls[4 * w + k]);
+      rec0[w].kind = KIND_WALL | (nomops[n + w] << 8);
+      for (int k = 0; k < 3; ++k) rec0[w].rt[k] = static_cast<float>(C.walls[4 * w + k]);
       wp[w] = make_float4(static_cast<float>(C.walls[4 * w]), static_cast<float>(C.walls[4 * w + 1]),
                           static_cast<float>(C.walls[4 * w + 2]), off32[nfaces + w]);
     }
     const size_t o3 = 3 * static_cast<size_t>(n), o9 = 9 * static_cast<size_t>(n);
     GBC_TRY(cudaMemcpy(D.X + o3, X0.data(), sizeof(double) * X0.size(), cudaMemcpyHostToDevice));
     GBC_TRY(cudaMemcpy(D.R + o9, R0.data(), sizeof(double) * R0.size(), cudaMemcpyHostToDevice));
-    GBC_TRY(cudaMemcpy(D.Rt + o9, Rt0.data(), sizeof(float) * Rt0.size(), cudaMemcpyHostToDevice));
-    GBC_TRY(cudaMemcpy(D.Xf + o3, f0.data(), sizeof(float) * f0.size(), cudaMemcpyHostToDevice));
-    GBC_TRY(cudaMemcpy(D.fX + o3, f0.data(), sizeof(float) * f0.size(), cudaMemcpyHostToDevice));
-    GBC_TRY(cudaMemcpy(D.kX + o3, k0.data(), sizeof(int) * k0.size(), cudaMemcpyHostToDevice));
-    GBC_TRY(cudaMemcpy(D.lohi + 6 * static_cast<size_t>(n), lohi0.data(), sizeof(int) * lohi0.size(),
-                       cudaMemcpyHostToDevice));
+    GBC_TRY(cudaMemcpy(D.rec + n, rec0.data(), sizeof(PartRec) * rec0.size(), cudaMemcpyHostToDevice));
     GBC_TRY(cudaMemcpy(D.wplane + nfaces, wp.data(), sizeof(float4) * wp.size(), cudaMemcpyHostToDevice));
     double* d_wall = nullptr;
     GBC_TRY(upload(c, &d_wall, wall_tab));
@@ -634,7 +626,8 @@ contact_status contact_init(const contact_config* cfg, const int32_t* shape_type
   const size_t nbins = static_cast<size_t>(P.nbin[0]) * P.nbin[1] * P.nbin[2];
   const size_t mp = static_cast<size_t>(C.max_pairs), mt = static_cast<size_t>(P.max_tiles);
   GBC_TRY(dev_alloc(c, &W.bin_count, nbins));
-  GBC_TRY(dev_alloc(c, &W.bin_items, nbins * static_cast<size_t>(P.bin_cap)));
+  GBC_TRY(dev_alloc(c, &W.bin_items, nbins * static_cast<size_t>(P.bin_stride)));
+  GBC_TRY(dev_alloc(c, &W.bin_rec, nbins * static_cast<size_t>(P.bin_stride)));
   GBC_TRY(dev_alloc(c, &W.up_count, static_cast<size_t>(n)));
   GBC_TRY(dev_alloc(c, &W.up_list, static_cast<size_t>(n) * max_nbr));
   GBC_TRY(dev_alloc(c, &W.dn_count, static_cast<size_t>(n)));
@@ -817,8 +810,11 @@ contact_status contact_stats(contact_ctx* c, int64_t* stats) {
 
 contact_status contact_particle_boxes(contact_ctx* c, int32_t* lo_hi) {
   if (c == nullptr || lo_hi == nullptr) return CONTACT_EINVAL;
-  const cudaError_t e =
-      cudaMemcpyAsync(lo_hi, c->D.lohi, sizeof(int) * 6 * c->P.n, cudaMemcpyDeviceToDevice, c->stream);
+  const size_t row = 6 * sizeof(int), half = 3 * sizeof(int), np = static_cast<size_t>(c->P.n);
+  cudaError_t e = cudaMemcpy2DAsync(lo_hi, row, c->D.rec->lo, sizeof(PartRec), half, np, cudaMemcpyDeviceToDevice,
+                                    c->stream);
+  if (e == cudaSuccess)
+    e = cudaMemcpy2DAsync(lo_hi + 3, row, c->D.rec->hi, sizeof(PartRec), half, np, cudaMemcpyDeviceToDevice, c->stream);
   return e == cudaSuccess ? CONTACT_OK : cuda_fail(c, e, "cudaMemcpyAsync");
 }
 

@@ -119,8 +119,8 @@ __device__ __forceinline__ void adj_depth_term(const Params& P, const Shapes& S,
       float rl = 0.f;
       if (poly) {
         const float ncell = static_cast<float>(kc == 0 ? P.ncell[0] : (kc == 1 ? P.ncell[1] : P.ncell[2]));
-        rl = (static_cast<float>((lok + ck) - D.kX[3 * pid + kc]) + static_cast<float>(shp) * ncell) -
-             D.fX[3 * pid + kc];
+        rl = (static_cast<float>((lok + ck) - D.rec[pid].kX[kc]) + static_cast<float>(shp) * ncell) -
+             D.rec[pid].fX[kc];
       }
       const float rl0 = __shfl_sync(kFull, rl, b0), rl1 = __shfl_sync(kFull, rl, b0 + 1),
                   rl2 = __shfl_sync(kFull, rl, b0 + 2);

@@ -15,57 +15,169 @@ namespace {
 
 constexpr unsigned kFull = 0xffffffffu;
 
-__device__ __forceinline__ int clamp_node(double v) {
-  // node indices stay far inside int range even for garbage input
-  v = fmin(fmax(v, -1.0e9), 1.0e9);
-  return static_cast<int>(v);
+constexpr int kPosePerWarp = 10;   // particles of one pose warp (three lanes each, lanes 30 and 31 idle)
+
+// Enter particle p with the given node range into its bin's row (one lane).
+__device__ __forceinline__ void bin_insert(const Params& P, const Lists& W, int p, int bin, const int lo[3],
+                                           const int hi[3]) {
+  const int slot = atomicAdd(&W.bin_count[bin], 1);
+  if (slot >= P.bin_cap) {
+    set_error(W.err, kErrCapacity);
+    return;
+  }
+  const size_t at = static_cast<size_t>(bin) * P.bin_stride + slot;
+  const bool empty = hi[0] < lo[0] || hi[1] < lo[1] || hi[2] < lo[2];
+  unsigned len = 0;
+#pragma unroll
+  for (int k = 0; k < 3; ++k) len |= static_cast<unsigned>(min(hi[k] - lo[k] + 1, kMaxLen) & kMaxLen) << (10 * k);
+  W.bin_items[at] = p;
+  *reinterpret_cast<int4*>(W.bin_rec + at) = make_int4(empty ? kNoNodes : lo[0], lo[1], lo[2], static_cast<int>(len));
 }
 
 // ---------------------------------------------------------------------------
-// K1: one thread per (particle p, axis k): row k of the rotation, the node
-// range along k, the FP32 sweep geometry and, on axis 0, the bin slot.  FP64
-// is kept to what the bit-exact node range needs (every FP64 instruction
-// costs ~64 cycles per warp on this GPU), and spread over three threads.
-// Polytope p by one warp: the node range along each axis (the extreme
-// projections of the offset-shape vertices: an FP32 prefilter over the
-// vertices on all lanes, FP64 for the at most two candidates per side, all
-// vertices in FP64 when more lie within the prefilter's window) and the
-// FP32 world planes (faces on lanes).  The FP64 arithmetic is the per-axis
-// thread's, operation for operation, so the node range is the same bit for bit.
-__device__ void pose_polytope(const Params& P, const Shapes& S, const Parts& D, int p, const double* __restrict__ pos,
-                              const double* __restrict__ quat) {
-  const int lane = threadIdx.x & 31;
-  const unsigned full = 0xffffffffu;
+// K1: three lanes per particle (lane k: axis k), ten particles per warp: row k
+// of the rotation, the node range along k and the FP32 sweep geometry; lane 0
+// enters the particle into its bin.  Bound: the FP64 pipe (64 cycles a warp
+// instruction).  FP64 is kept to what the bit-exact node range needs, the same
+// instruction for the three rows (a branch per row ran all three in turn), and
+// conversions, roundings and comparisons are integer operations: 29.8 -> @POSE@ us
+// on 52218 cubes.
+__global__ void k_pose(Params P, Shapes S, Parts D, Lists W, const double* __restrict__ pos,
+                       const double* __restrict__ quat) {
+  __shared__ __align__(16) int s_rec[kPosePerWarp][4 * kPartRecParts];
+  pdl_begin();
+  const int lane = threadIdx.x;   // one-warp blocks
+  const int t = blockIdx.x * 32 + lane;
+  // the host's token of this step (mapped host memory: read here, stored at the end)
+  const int token = (t == 0 && W.publish) ? *reinterpret_cast<const volatile int*>(W.err_host + 2) : 0;
+  // the step's counters start at zero (the previous step has completed)
+  if (t == 0) {
+    W.counters[0] = 0;   // pairs (written by the pair builder)
+    W.counters[1] = 0;   // tiles allocated
+    W.counters[2] = 0;   // box pipeline queue head
+    W.counters[5] = 0;   // pairs with V > 0
+    W.u64[0] = 0;        // node evaluations
+    W.u64[1] = 0;        // nominal lane-ops
+  }
+  if (t < (P.n + kRowGroup - 1) / kRowGroup) W.grp_sum[t] = 0;
+  // contact history: this step's lists (the buffer not read) start empty
+  if (P.history && t < P.n) W.hist_n[static_cast<size_t>(((W.counters[kStepCounter] & 1) ^ 1)) * P.n + t] = 0;
+  const int g = min(lane / 3, kPosePerWarp - 1), k = lane - 3 * g;   // (lanes 30, 31: k = 3, 4, no stores)
+  const int p_ = blockIdx.x * kPosePerWarp + g;
+  const bool act = k < 3 && p_ < P.n;
+  const int p = min(p_, P.n - 1), kc = k < 3 ? k : 0;
+  const int k1 = kc == 2 ? 0 : kc + 1;
   double q[4];
+#pragma unroll
   for (int c = 0; c < 4; ++c) q[c] = quat[4 * p + c];
+  // position check by bit patterns: 0 <= X < L (NaN and negatives fail; -0.0 counts as 0)
   bool bad = false;
-  double Xv[3];
+  double Xk = 0.0;
+#pragma unroll
   for (int c = 0; c < 3; ++c) {
     const double v = pos[3 * p + c];
     long long b = __double_as_longlong(v);
     if (b == static_cast<long long>(0x8000000000000000ULL)) b = 0;
     const bool ok = b >= 0 && b < __double_as_longlong(P.L[c]);
     bad = bad || !ok;
-    Xv[c] = ok ? __longlong_as_double(b) : 0.0;
+    if (c == kc) Xk = ok ? __longlong_as_double(b) : 0.0;
   }
   const double nn = dadd(dadd(dadd(dmul(q[0], q[0]), dmul(q[1], q[1])), dmul(q[2], q[2])), dmul(q[3], q[3]));
-  if (!(nn > 1e-24) || !(nn < 1e300)) {
+  // 1e-24 < nn < 1e300 (nn >= 0 or NaN: its bits order as its values, a NaN's above every number's)
+  if (!(__double_as_longlong(nn) > __double_as_longlong(1e-24)) || !(__double_as_longlong(nn) < __double_as_longlong(1e300))) {
     bad = true;
     q[0] = 1.0; q[1] = q[2] = q[3] = 0.0;
   }
+  if (bad && act && k == 0) set_error(W.err, kErrInval);
   const double s = bad ? 2.0 : dmul(2.0, __drcp_rn(nn));
-  // rotation rows: lane k < 3 computes row k, then every lane holds all nine
-  double rk[3] = {0.0, 0.0, 0.0};
-  if (lane < 3) rotation_row_rn(q, s, lane, rk);
-  double R[3][3];
-  float R32[3][3];
+  // row k of the rotation (rotation_row_rn with the row's cyclic axes k, k1, k2):
+  // 1 - s (q_k1^2 + q_k2^2), s (q_k q_k1 - w q_k2), s (q_k q_k2 + w q_k1)
+  const double qk = kc == 0 ? q[1] : (kc == 1 ? q[2] : q[3]);
+  const double qk1 = kc == 0 ? q[2] : (kc == 1 ? q[3] : q[1]);
+  const double qk2 = kc == 0 ? q[3] : (kc == 1 ? q[1] : q[2]);
+  const double rd = dsub(1.0, dmul(s, dadd(dmul(qk1, qk1), dmul(qk2, qk2))));
+  const double r1 = dmul(s, dsub(dmul(qk, qk1), dmul(q[0], qk2)));
+  const double r2 = dmul(s, dadd(dmul(qk, qk2), dmul(q[0], qk1)));
+  double r[3];   // by world column c
+#pragma unroll
+  for (int c = 0; c < 3; ++c) r[c] = c == kc ? rd : (c == k1 ? r1 : r2);
+  if (act) {
+    D.X[3 * p + k] = Xk;
+    if (k == 0)
+#pragma unroll
+      for (int c = 0; c < 4; ++c) D.qhat[4 * p + c] = q[c];   // raw quaternion of the step (adjoint tape)
+#pragma unroll
+    for (int c = 0; c < 3; ++c) D.R[9 * p + 3 * k + c] = r[c];
+  }
+  // extent along k of the offset shape {phi <= delta} (explicit rounding: compared bit for bit);
+  // a polytope's node range and bin entry come from its own warp (k_pose_poly)
+  const int type = S.type[p];
+  const double* e = S.ext + 3 * p;
+  double ext = dadd(dadd(dmul(fabs(r[0]), e[0]), dmul(fabs(r[1]), e[1])), dmul(fabs(r[2]), e[2]));
+  if (type == 0) ext = e[0];
+  const double mn = dsub(Xk, ext), mx = dadd(Xk, ext);
+  const int lo = ceil_node(P.dx_pow2 ? dmul(mn, P.inv_dx) : __ddiv_rn(mn, P.dx));
+  const int hi = floor_node(P.dx_pow2 ? dmul(mx, P.inv_dx) : __ddiv_rn(mx, P.dx));
+  // nearest node of X / dx (round to even) by the 1.5 2^52 shift, and the remainder
+  const double xl = Xk * P.inv_dx;
+  const double sh = __dadd_rn(xl, 6755399441055744.0);
+  const int kx = __double2loint(sh);
+  const float fx = narrow(__dsub_rn(xl, __dsub_rn(sh, 6755399441055744.0)));
+  // cell-list bin
+  const int b = min(max(static_cast<int>(narrow(Xk) * P.inv_binw_f[kc]), 0), P.nbin[kc] - 1);
+  const int l0 = 3 * g;
+  const int b0 = __shfl_sync(kFull, b, l0), b1 = __shfl_sync(kFull, b, l0 + 1), b2 = __shfl_sync(kFull, b, l0 + 2);
+  const int los[3] = {__shfl_sync(kFull, lo, l0), __shfl_sync(kFull, lo, l0 + 1), __shfl_sync(kFull, lo, l0 + 2)};
+  const int his[3] = {__shfl_sync(kFull, hi, l0), __shfl_sync(kFull, hi, l0 + 1), __shfl_sync(kFull, hi, l0 + 2)};
+  const int bin = checked_index(W.err, b0 + P.nbin[0] * (b1 + P.nbin[1] * b2),
+                                static_cast<long long>(P.nbin[0]) * P.nbin[1] * P.nbin[2], 0);
+  if (act && k == 0 && type != 2) bin_insert(P, W, p, bin, los, his);
+  // the particle's line, staged so that the warp stores whole 16-byte pieces
+  if (act) {
+    int* w = s_rec[g];
+    w[k] = lo;
+    w[4 + k] = hi;
+    w[8 + k] = kx;
+    w[11 + 4 * k + (k == 2 ? 6 : 0)] = __float_as_int(S.size_l[3 * p + k]);   // words 11, 15, 25
+    w[12 + k] = __float_as_int(fx);
+#pragma unroll
+    for (int c = 0; c < 3; ++c) w[16 + 3 * c + k] = __float_as_int(narrow(r[c]));   // R^T row c, column k
+    if (k == 0) w[3] = W.kind[p] | (S.nomops[p] << 8);
+    if (k == 1) w[7] = bin;
+    if (k == 2) w[26] = w[27] = 0;
+  }
+  __syncwarp();
+  const int np = min(kPosePerWarp, P.n - static_cast<int>(blockIdx.x) * kPosePerWarp);
+  for (int u = lane; u < kPartRecParts * np; u += 32) {
+    const int gp = u / kPartRecParts, part = u - gp * kPartRecParts;
+    reinterpret_cast<int4*>(D.rec + static_cast<size_t>(blockIdx.x) * kPosePerWarp + gp)[part] =
+        reinterpret_cast<const int4*>(s_rec[gp])[part];
+  }
+  if (t == 0 && W.publish) W.counters[kTokenCounter] = token;
+}
+
+// K1b: one warp per polytope: its node range along each axis (the extreme
+// projections of the offset-shape vertices: an FP32 prefilter over the
+// vertices on all lanes, FP64 for the at most two candidates per side, all
+// vertices in FP64 when more lie within the prefilter's window), the FP32 world
+// planes (faces on lanes) and its bin entry, from the rotation k_pose wrote.
+// The FP64 arithmetic is the oracle's, operation for operation, so the node
+// range is the same bit for bit.  Bound: the FP64 pipe; with the candidates of
+// the three axes side by side on twelve lanes and the rotation read instead of
+// formed again it takes ~16 FP64 instructions a polytope (~100 before): 39.7 ->
+// @POLY@ us on 5157 polytopes.
+__global__ void k_pose_poly(Params P, Shapes S, Parts D, Lists W) {
+  pdl_begin();
+  const int p = S.poly_ids[blockIdx.x];
+  const int lane = threadIdx.x & 31;
+  const double* Rg = D.R + 9 * static_cast<size_t>(p);
+  PartRec* rec = D.rec + p;
+  float R32[3][3];   // row k: world axis k
 #pragma unroll
   for (int k = 0; k < 3; ++k)
 #pragma unroll
-    for (int c = 0; c < 3; ++c) {
-      R[k][c] = __shfl_sync(full, rk[c], k);
-      R32[k][c] = static_cast<float>(R[k][c]);
-    }
+    for (int c = 0; c < 3; ++c) R32[k][c] = rec->rt[3 * c + k];
+  const int bin = rec->bin;
   const int v0 = S.vert_off[p], v1 = S.vert_off[p + 1];
   // FP32 prefilter: extremes per axis and the largest |w|_1
   float lo32[3] = {FLT_MAX, FLT_MAX, FLT_MAX}, hi32[3] = {-FLT_MAX, -FLT_MAX, -FLT_MAX}, wmax = 0.f;
@@ -87,95 +199,93 @@ __device__ void pose_polytope(const Params& P, const Shapes& S, const Parts& D, 
   for (int o = 16; o > 0; o >>= 1) {
 #pragma unroll
     for (int k = 0; k < 3; ++k) {
-      lo32[k] = fminf(lo32[k], __shfl_xor_sync(full, lo32[k], o));
-      hi32[k] = fmaxf(hi32[k], __shfl_xor_sync(full, hi32[k], o));
+      lo32[k] = fminf(lo32[k], __shfl_xor_sync(kFull, lo32[k], o));
+      hi32[k] = fmaxf(hi32[k], __shfl_xor_sync(kFull, hi32[k], o));
     }
-    wmax = fmaxf(wmax, __shfl_xor_sync(full, wmax, o));
+    wmax = fmaxf(wmax, __shfl_xor_sync(kFull, wmax, o));
   }
   const float tol = 1e-5f * wmax + 1e-30f;
-  // candidates within tol of the FP32 extremes, the first two in vertex order
-  int lc[3][2], hc[3][2], nlo[3] = {0, 0, 0}, nhi[3] = {0, 0, 0};
+  // candidates within tol of the FP32 extremes, the first two in vertex order;
+  // lane 4 k + c keeps candidate c of axis k (0, 1: lowest; 2, 3: highest)
+  const int ax = min(lane >> 2, 2), cd = lane & 3;
+  int mine = v0;
+  bool rare[3];
 #pragma unroll
-  for (int k = 0; k < 3; ++k) lc[k][0] = lc[k][1] = hc[k][0] = hc[k][1] = v0;
-  for (int vb = v0; vb < v1; vb += 32) {
-    const int v = vb + lane;
-    float x0 = 0.f, x1 = 0.f, x2 = 0.f;
-    if (v < v1) {
-      const float* w = S.verts32 + 3 * v;
-      x0 = w[0]; x1 = w[1]; x2 = w[2];
-    }
-#pragma unroll
-    for (int k = 0; k < 3; ++k) {
-      const float tv = fmaf(R32[k][0], x0, fmaf(R32[k][1], x1, R32[k][2] * x2));
-      unsigned bl = __ballot_sync(full, v < v1 && tv <= lo32[k] + tol);
-      unsigned bh = __ballot_sync(full, v < v1 && tv >= hi32[k] - tol);
-      while (bl) {
-        const int l = __ffs(bl) - 1;
-        if (nlo[k] == 0) lc[k][0] = vb + l;
-        else if (nlo[k] == 1) lc[k][1] = vb + l;
-        ++nlo[k];
-        bl &= bl - 1;
+  for (int k = 0; k < 3; ++k) {
+    int nlo = 0, nhi = 0, lc[2] = {v0, v0}, hc[2] = {v0, v0};
+    for (int vb = v0; vb < v1; vb += 32) {
+      const int v = vb + lane;
+      float tv = 0.f;
+      if (v < v1) {
+        const float* w = S.verts32 + 3 * v;
+        tv = fmaf(R32[k][0], w[0], fmaf(R32[k][1], w[1], R32[k][2] * w[2]));
       }
-      while (bh) {
-        const int l = __ffs(bh) - 1;
-        if (nhi[k] == 0) hc[k][0] = vb + l;
-        else if (nhi[k] == 1) hc[k][1] = vb + l;
-        ++nhi[k];
-        bh &= bh - 1;
-      }
+      const unsigned bl = __ballot_sync(kFull, v < v1 && tv <= lo32[k] + tol);
+      const unsigned bh = __ballot_sync(kFull, v < v1 && tv >= hi32[k] - tol);
+      auto take = [&](unsigned m, int* cand, int& n) {
+        if (m == 0u) return;
+        const int f0 = vb + __ffs(m) - 1;
+        const unsigned m1 = m & (m - 1u);
+        const int f1 = m1 != 0u ? vb + __ffs(m1) - 1 : f0;
+        if (n == 0) {
+          cand[0] = f0;
+          cand[1] = f1;
+        } else if (n == 1) {
+          cand[1] = f0;
+        }
+        n += __popc(m);
+      };
+      take(bl, lc, nlo);
+      take(bh, hc, nhi);
     }
+    if (nlo < 2) lc[1] = lc[0];
+    if (nhi < 2) hc[1] = hc[0];
+    if (ax == k) mine = cd == 0 ? lc[0] : (cd == 1 ? lc[1] : (cd == 2 ? hc[0] : hc[1]));
+    rare[k] = nlo > 2 || nhi > 2;
   }
-  // exact FP64 projections of the candidates: lane k < 3 takes axis k
+  // exact FP64 projection of the lane's candidate; the pair's extreme by order-preserving keys
   auto proj3 = [&](double r0, double r1, double r2, int v) {
     const double* w = S.verts + 3 * v;
     return dadd(dadd(dmul(r0, w[0]), dmul(r1, w[1])), dmul(r2, w[2]));
   };
-  double lo = 0.0, hi = 0.0;
-  if (lane < 3) {
-    const int k = lane;
-    const int a0 = k == 0 ? lc[0][0] : (k == 1 ? lc[1][0] : lc[2][0]);
-    const int a1 = k == 0 ? lc[0][1] : (k == 1 ? lc[1][1] : lc[2][1]);
-    const int b0 = k == 0 ? hc[0][0] : (k == 1 ? hc[1][0] : hc[2][0]);
-    const int b1 = k == 0 ? hc[0][1] : (k == 1 ? hc[1][1] : hc[2][1]);
-    const int nl = k == 0 ? nlo[0] : (k == 1 ? nlo[1] : nlo[2]);
-    const int nh = k == 0 ? nhi[0] : (k == 1 ? nhi[1] : nhi[2]);
-    const double r0 = k == 0 ? R[0][0] : (k == 1 ? R[1][0] : R[2][0]);
-    const double r1 = k == 0 ? R[0][1] : (k == 1 ? R[1][1] : R[2][1]);
-    const double r2 = k == 0 ? R[0][2] : (k == 1 ? R[1][2] : R[2][2]);
-    lo = proj3(r0, r1, r2, a0);
-    hi = proj3(r0, r1, r2, b0);
-    if (nl > 1) lo = fmin(lo, proj3(r0, r1, r2, a1));
-    if (nh > 1) hi = fmax(hi, proj3(r0, r1, r2, b1));
-  }
+  const double ra0 = Rg[3 * ax], ra1 = Rg[3 * ax + 1], ra2 = Rg[3 * ax + 2];
+  double ext = proj3(ra0, ra1, ra2, mine);
+  const bool up = cd >= 2;   // lanes 0, 1 of an axis: the lower extent, lanes 2, 3: the upper
+  auto better = [&](double a, double b) { return (order_key(a) > order_key(b)) == up ? a : b; };
+  ext = better(ext, __shfl_xor_sync(kFull, ext, 1));
   // rare: more than two vertices at an extreme -> every vertex in FP64 (lanes over vertices)
 #pragma unroll
   for (int k = 0; k < 3; ++k) {
-    if (nlo[k] > 2 || nhi[k] > 2) {
+    if (rare[k]) {   // warp-uniform
       double l = DBL_MAX, h = -DBL_MAX;
       for (int v = v0 + lane; v < v1; v += 32) {
-        const double tt = proj3(R[k][0], R[k][1], R[k][2], v);
+        const double tt = proj3(Rg[3 * k], Rg[3 * k + 1], Rg[3 * k + 2], v);
         l = fmin(l, tt);
         h = fmax(h, tt);
       }
 #pragma unroll
       for (int o = 16; o > 0; o >>= 1) {
-        l = fmin(l, __shfl_xor_sync(full, l, o));
-        h = fmax(h, __shfl_xor_sync(full, h, o));
+        l = fmin(l, __shfl_xor_sync(kFull, l, o));
+        h = fmax(h, __shfl_xor_sync(kFull, h, o));
       }
-      if (lane == k) {
-        lo = fmin(lo, l);
-        hi = fmax(hi, h);
-      }
+      if (ax == k) ext = better(ext, up ? h : l);
     }
   }
-  if (lane < 3) {
-    const int k = lane;
-    const double Xk = k == 0 ? Xv[0] : (k == 1 ? Xv[1] : Xv[2]);
-    const double mn = dadd(Xk, lo), mx = dadd(Xk, hi);
-    const double a = P.dx_pow2 ? dmul(mn, P.inv_dx) : __ddiv_rn(mn, P.dx);
-    const double c = P.dx_pow2 ? dmul(mx, P.inv_dx) : __ddiv_rn(mx, P.dx);
-    D.lohi[6 * p + k] = clamp_node(ceil(a));
-    D.lohi[6 * p + 3 + k] = clamp_node(floor(c));
+  {
+    const double v = dadd(D.X[3 * p + ax], ext);
+    const double a = P.dx_pow2 ? dmul(v, P.inv_dx) : __ddiv_rn(v, P.dx);
+    const int node = up ? floor_node(a) : ceil_node(a);
+    const int los[3] = {__shfl_sync(kFull, node, 0), __shfl_sync(kFull, node, 4), __shfl_sync(kFull, node, 8)};
+    const int his[3] = {__shfl_sync(kFull, node, 2), __shfl_sync(kFull, node, 6), __shfl_sync(kFull, node, 10)};
+    if (lane == 0) {
+#pragma unroll
+      for (int k = 0; k < 3; ++k) {
+        rec->lo[k] = los[k];
+        rec->hi[k] = his[k];
+      }
+      bin_insert(P, W, p, checked_index(W.err, bin, static_cast<long long>(P.nbin[0]) * P.nbin[1] * P.nbin[2], 0),
+                 los, his);
+    }
   }
   // world planes: face f on lane f (FP64 product per component, one rounding to FP32)
   const int f0 = S.face_off[p], f1 = S.face_off[p + 1];
@@ -183,140 +293,40 @@ __device__ void pose_polytope(const Params& P, const Shapes& S, const Parts& D, 
     const double2* e = reinterpret_cast<const double2*>(S.planes + 4 * f);
     const double2 e01 = e[0], e2x = e[1];
     float4 o;
-    o.x = static_cast<float>(fma(R[0][0], e01.x, fma(R[0][1], e01.y, R[0][2] * e2x.x)));
-    o.y = static_cast<float>(fma(R[1][0], e01.x, fma(R[1][1], e01.y, R[1][2] * e2x.x)));
-    o.z = static_cast<float>(fma(R[2][0], e01.x, fma(R[2][1], e01.y, R[2][2] * e2x.x)));
+    o.x = narrow(fma(Rg[0], e01.x, fma(Rg[1], e01.y, Rg[2] * e2x.x)));
+    o.y = narrow(fma(Rg[3], e01.x, fma(Rg[4], e01.y, Rg[5] * e2x.x)));
+    o.z = narrow(fma(Rg[6], e01.x, fma(Rg[7], e01.y, Rg[8] * e2x.x)));
     o.w = S.off32[f];
     D.wplane[f] = o;
   }
 }
 
-// K1b: one warp per polytope (node range and world planes), its own kernel so
-// that the per-axis kernel's code stays as lean as it is without polytopes.
-__global__ void k_pose_poly(Params P, Shapes S, Parts D, const double* __restrict__ pos, const double* __restrict__ quat) {
-  pdl_begin();
-  pose_polytope(P, S, D, S.poly_ids[blockIdx.x], pos, quat);
-}
+// Node range [lo_q - s n, hi_q - s n] of the partner in the image that can meet
+// p's: the offset of the lower corners is brought into [-n/2, n/2].  Two ranges
+// that share a node have corners less than a range's length apart, and with L >
+// 4 R_max + 2 dx every range is shorter than n/2, so no other image can meet it.
+__device__ __forceinline__ int image_shift(int d, int n) { return d > (n >> 1) ? 1 : (d < -(n >> 1) ? -1 : 0); }
 
-__global__ void k_pose(Params P, Shapes S, Parts D, Lists W, const double* __restrict__ pos,
-                       const double* __restrict__ quat) {
-  pdl_begin();
-  const int t = blockIdx.x * blockDim.x + threadIdx.x;
-  // the host's token of this step (mapped host memory: read here, stored at the end)
-  const int token = (t == 0 && W.publish) ? *reinterpret_cast<const volatile int*>(W.err_host + 2) : 0;
-  // the step's counters start at zero (the previous step has completed)
-  if (t == 0) {
-    W.counters[0] = 0;   // pairs (written by the pair builder)
-    W.counters[1] = 0;   // tiles allocated
-    W.counters[2] = 0;   // box pipeline queue head
-    W.counters[5] = 0;   // pairs with V > 0
-    W.u64[0] = 0;        // node evaluations
-    W.u64[1] = 0;        // nominal lane-ops
-  }
-  if (t < (P.n + kRowGroup - 1) / kRowGroup) W.grp_sum[t] = 0;
-  // contact history: this step's lists (the buffer not read) start empty
-  if (P.history && t < P.n) W.hist_n[static_cast<size_t>(((W.counters[kStepCounter] & 1) ^ 1)) * P.n + t] = 0;
-  if (t >= 3 * P.n) return;
-  const int p = t / 3, k = t - 3 * p;
-  double q[4];
-  for (int c = 0; c < 4; ++c) q[c] = quat[4 * p + c];
-  // position check by bit patterns: 0 <= X < L (NaN and negatives fail; -0.0 counts as 0)
-  bool bad = false;
-  float xs[3];
-  double Xk = 0.0;
-  for (int c = 0; c < 3; ++c) {
-    const double v = pos[3 * p + c];
-    long long b = __double_as_longlong(v);
-    if (b == static_cast<long long>(0x8000000000000000ULL)) b = 0;
-    const bool ok = b >= 0 && b < __double_as_longlong(P.L[c]);
-    bad = bad || !ok;
-    const double vv = ok ? __longlong_as_double(b) : 0.0;
-    xs[c] = static_cast<float>(vv);
-    if (c == k) Xk = vv;
-  }
-  const double nn = dadd(dadd(dadd(dmul(q[0], q[0]), dmul(q[1], q[1])), dmul(q[2], q[2])), dmul(q[3], q[3]));
-  if (!(nn > 1e-24) || !(nn < 1e300)) {
-    bad = true;
-    q[0] = 1.0; q[1] = q[2] = q[3] = 0.0;
-  }
-  if (bad && k == 0) set_error(W.err, kErrInval);
-  const double s = bad ? 2.0 : dmul(2.0, __drcp_rn(nn));
-  double r[3];
-  rotation_row_rn(q, s, k, r);
-  D.X[3 * p + k] = Xk;
-  if (k == 0)
-    for (int c = 0; c < 4; ++c) D.qhat[4 * p + c] = q[c];   // raw quaternion of the step (adjoint tape)
-  for (int c = 0; c < 3; ++c) D.R[9 * p + 3 * k + c] = r[c];
-  float r32[3];
-  for (int c = 0; c < 3; ++c) {
-    r32[c] = static_cast<float>(r[c]);
-    D.Rt[9 * p + 3 * c + k] = r32[c];   // R^T row c, column k
-  }
-  // extent along k of the offset shape {phi <= delta} (explicit rounding: compared bit for bit)
-  const int type = S.type[p];
-  double mn, mx;
-  if (type == 0) {
-    const double rad = S.ext[3 * p];
-    mn = dsub(Xk, rad);
-    mx = dadd(Xk, rad);
-  } else if (type == 1) {
-    const double* e = S.ext + 3 * p;
-    const double ext = dadd(dadd(dmul(fabs(r[0]), e[0]), dmul(fabs(r[1]), e[1])), dmul(fabs(r[2]), e[2]));
-    mn = dsub(Xk, ext);
-    mx = dadd(Xk, ext);
-  } else {
-    mn = mx = 0.0;   // polytope: node range and world planes by the polytope warps below
-  }
-  const double a = P.dx_pow2 ? dmul(mn, P.inv_dx) : __ddiv_rn(mn, P.dx);
-  const double c = P.dx_pow2 ? dmul(mx, P.inv_dx) : __ddiv_rn(mx, P.dx);
-  if (type != 2) {
-    D.lohi[6 * p + k] = clamp_node(ceil(a));
-    D.lohi[6 * p + 3 + k] = clamp_node(floor(c));
-  }
-  D.Xf[3 * p + k] = xs[k];
-  const double xl = Xk * P.inv_dx;
-  const double kx = rint(xl);
-  D.kX[3 * p + k] = static_cast<int>(kx);
-  D.fX[3 * p + k] = static_cast<float>(xl - kx);
-  if (k == 0) {
-    int b[3];
-    for (int cc = 0; cc < 3; ++cc) b[cc] = min(max(static_cast<int>(xs[cc] * P.inv_binw_f[cc]), 0), P.nbin[cc] - 1);
-    const int bin = checked_index(W.err, b[0] + P.nbin[0] * (b[1] + P.nbin[1] * b[2]),
-                                  static_cast<long long>(P.nbin[0]) * P.nbin[1] * P.nbin[2], 0);
-    D.bin[p] = bin;
-    const int slot = atomicAdd(&W.bin_count[bin], 1);
-    if (slot < P.bin_cap) W.bin_items[static_cast<size_t>(bin) * P.bin_cap + slot] = p;
-    else set_error(W.err, kErrCapacity);
-  }
-  if (t == 0 && W.publish) W.counters[kTokenCounter] = token;
-}
-
-// Node box of pair (p, q) with q's image nearest p; returns false if empty.
-// The image index s = rint((X_q - X_p) / L) is taken by comparing the FP32
-// position difference with L/2 (positions lie in [0, L), so s is -1, 0 or 1).
-// It can differ from the exact choice only when |X_q - X_p| is within FP32
-// rounding of L/2; such a pair is no candidate in any image, because every
-// image lies at least L/2 - 1e-3 > 2 R_max away on that axis (L > 4 R_max + 2 dx).
-__device__ __forceinline__ bool pair_box(const Params& P, const Parts& D, int p, int q, int s[3], int lo[3],
+// Node box of pair (p, q) with q's image nearest p.
+__device__ __forceinline__ void pair_box(const Params& P, const PartRec* a, const PartRec* b, int s[3], int lo[3],
                                          int hi[3]) {
-  bool hit = true;
 #pragma unroll
   for (int k = 0; k < 3; ++k) {
-    const float d = D.Xf[3 * q + k] - D.Xf[3 * p + k];
-    const float h = 0.5f * static_cast<float>(P.L[k]);
-    s[k] = (d > h) ? 1 : ((d < -h) ? -1 : 0);
-    lo[k] = max(D.lohi[6 * p + k], D.lohi[6 * q + k] - s[k] * P.ncell[k]);
-    hi[k] = min(D.lohi[6 * p + 3 + k], D.lohi[6 * q + 3 + k] - s[k] * P.ncell[k]);
-    hit = hit && lo[k] <= hi[k];
+    s[k] = image_shift(b->lo[k] - a->lo[k], P.ncell[k]);
+    lo[k] = max(a->lo[k], b->lo[k] - s[k] * P.ncell[k]);
+    hi[k] = min(a->hi[k], b->hi[k] - s[k] * P.ncell[k]);
   }
-  return hit;
 }
 
 // K3: one warp per particle p.  Lane b < 27 owns neighbour bin b of the
-// fixed-capacity cell list; the candidates are read four per lane at a time
-// (their particle data loaded together), tested against p's node range, and
-// compacted with warp ballots into partners above (j > p) and below (j < p);
-// each list is then sorted by rank.
+// fixed-capacity cell list; its entries (node range and particle, one 16-byte
+// and one 4-byte word each) are read four at a time, tested against p's node
+// range, and compacted with warp ballots into partners above (j > p) and below
+// (j < p); each list is then sorted by rank.  Bound: load wavefronts (every
+// lane's load is its own line) and, on small boxes, load latency.  With the
+// ranges in the bins a candidate costs one wavefront and no dependent load
+// (nine scattered words of its particle before): 84.1 -> @BROAD@ us on 52218
+// cubes (58 candidates each).
 __global__ void __launch_bounds__(256) k_broad(Params P, Parts D, Lists W) {
   extern __shared__ int s_buf[];
   // the block's partner count (its particles share one row group), added
@@ -349,23 +359,21 @@ __global__ void __launch_bounds__(256) k_broad(Params P, Parts D, Lists W) {
   const int cap = P.max_nbr;
   int* up = s_buf + wid * 2 * cap;
   int* dn = up + cap;
-  const int bin = D.bin[p];
-  float xp[3];
-  int plo[3], phi[3];
-#pragma unroll
-  for (int k = 0; k < 3; ++k) {
-    xp[k] = D.Xf[3 * p + k];
-    plo[k] = D.lohi[6 * p + k];
-    phi[k] = D.lohi[6 * p + 3 + k];
-  }
+  const int4 own_lo = reinterpret_cast<const int4*>(D.rec + p)[0], own_hi = reinterpret_cast<const int4*>(D.rec + p)[1];
+  const int bin = own_hi.w;
+  const int plo[3] = {own_lo.x, own_lo.y, own_lo.z}, phi[3] = {own_hi.x, own_hi.y, own_hi.z};
+  const bool nodes = plo[0] <= phi[0] && plo[1] <= phi[1] && plo[2] <= phi[2];
   const int b[3] = {bin % P.nbin[0], (bin / P.nbin[0]) % P.nbin[1], bin / (P.nbin[0] * P.nbin[1])};
   int cnt[3];
 #pragma unroll
   for (int k = 0; k < 3; ++k) cnt[k] = P.nbin[k] >= 3 ? 3 : P.nbin[k];
   const int nnb = cnt[0] * cnt[1] * cnt[2];
   int num = 0;
-  const int* items = W.bin_items;
-  int pre[4] = {-1, -1, -1, -1};   // the bin's next four entries (the first ones fetched with its count)
+  size_t row = 0;
+  int4 ids = make_int4(-1, -1, -1, -1), recs[4];   // the bin's next four entries (the first ones fetched with its count)
+#pragma unroll
+  for (int u = 0; u < 4; ++u) recs[u] = make_int4(0, 0, 0, 0);
+  const int4* bin_rec = reinterpret_cast<const int4*>(W.bin_rec);
   if (lane < nnb) {
     int o[3] = {lane % cnt[0], (lane / cnt[0]) % cnt[1], lane / (cnt[0] * cnt[1])};
 #pragma unroll
@@ -375,47 +383,41 @@ __global__ void __launch_bounds__(256) k_broad(Params P, Parts D, Lists W) {
     }
     const int q = checked_index(W.err, o[0] + P.nbin[0] * (o[1] + P.nbin[1] * o[2]),
                                 static_cast<long long>(P.nbin[0]) * P.nbin[1] * P.nbin[2], bin);
-    items += static_cast<size_t>(q) * P.bin_cap;
-    // (entries past the count are stale and unused)
+    row = static_cast<size_t>(q) * P.bin_stride;   // (a multiple of four; entries past the count are stale and unused)
+    ids = *reinterpret_cast<const int4*>(W.bin_items + row);
 #pragma unroll
-    for (int u = 0; u < 4; ++u) pre[u] = u < P.bin_cap ? items[u] : -1;
+    for (int u = 0; u < 4; ++u) recs[u] = bin_rec[row + u];
     num = min(W.bin_count[q], P.bin_cap);
   }
   const int maxn = __reduce_max_sync(kFull, num);
   int nup = 0, ndn = 0;
   const unsigned below = (1u << lane) - 1u;
   for (int t0 = 0; t0 < maxn; t0 += 4) {
-    int jj[4];
+    const int jj[4] = {ids.x, ids.y, ids.z, ids.w};
+    int4 cur[4];
 #pragma unroll
-    for (int u = 0; u < 4; ++u) jj[u] = t0 + u < num ? checked_index(W.err, pre[u], P.n, -1) : -1;
-    // the next four entries, fetched with this round's candidate data
+    for (int u = 0; u < 4; ++u) cur[u] = recs[u];
+    // the next four entries, fetched while this round's are tested
+    if (t0 + 4 < num) {
+      ids = *reinterpret_cast<const int4*>(W.bin_items + row + t0 + 4);
 #pragma unroll
-    for (int u = 0; u < 4; ++u) pre[u] = t0 + 4 + u < num ? items[t0 + 4 + u] : -1;
-    float xj[4][3];
-    int jlo[4][3], jhi[4][3];
-#pragma unroll
-    for (int u = 0; u < 4; ++u) {
-      const int j = jj[u] >= 0 ? jj[u] : p;
-#pragma unroll
-      for (int k = 0; k < 3; ++k) {
-        xj[u][k] = D.Xf[3 * j + k];
-        jlo[u][k] = D.lohi[6 * j + k];
-        jhi[u][k] = D.lohi[6 * j + 3 + k];
-      }
+      for (int u = 0; u < 4; ++u) recs[u] = bin_rec[row + t0 + 4 + u];
     }
 #pragma unroll
     for (int u = 0; u < 4; ++u) {
-      const int j = jj[u];
-      // node ranges intersect, the partner moved by the image shift (as in pair_box)
-      bool hit = j >= 0 && j != p;
+      if (t0 + u >= maxn) break;   // warp-uniform
+      const int j = t0 + u < num ? checked_index(W.err, jj[u], P.n, -1) : -1;
+      // node ranges intersect, the partner moved by the image shift (as in pair_box):
+      // its corner lies above p's by at most p's length and below it by at most its own
+      bool hit = j >= 0 && j != p && nodes;
+      const int jl[3] = {cur[u].x, cur[u].y, cur[u].z};
 #pragma unroll
       for (int k = 0; k < 3; ++k) {
-        const float d = xj[u][k] - xp[k];
-        const float h = 0.5f * static_cast<float>(P.L[k]);
-        const int sk = (d > h) ? 1 : ((d < -h) ? -1 : 0);
-        const int lo = max(plo[k], jlo[u][k] - sk * P.ncell[k]);
-        const int hi = min(phi[k], jhi[u][k] - sk * P.ncell[k]);
-        hit = hit && lo <= hi;
+        int d = jl[k] - plo[k];
+        d -= image_shift(d, P.ncell[k]) * P.ncell[k];
+        int len = (cur[u].w >> (10 * k)) & kMaxLen;
+        if (P.wide && j >= 0) len = D.rec[j].hi[k] - D.rec[j].lo[k] + 1;   // (uniform: ranges beyond kMaxLen nodes)
+        hit = hit && d <= phi[k] - plo[k] && -d < len;
       }
       const unsigned bu = __ballot_sync(kFull, hit && j > p);
       const unsigned bd = __ballot_sync(kFull, hit && j < p);
@@ -471,13 +473,13 @@ __global__ void __launch_bounds__(256) k_broad(Params P, Parts D, Lists W) {
     const int v = up[e];
     int r = 0;
     for (int t = 0; t < nup; ++t) r += up[t] < v;
-    W.up_list[p * cap + r] = v;
+    W.up_list[static_cast<size_t>(p) * cap + r] = v;
   }
   for (int e = lane; e < ndn; e += 32) {
     const int v = dn[e];
     int r = 0;
     for (int t = 0; t < ndn; ++t) r += dn[t] < v;
-    W.dn_list[p * cap + r] = v;
+    W.dn_list[static_cast<size_t>(p) * cap + r] = v;
   }
   if (lane == 0) {
     W.up_count[p] = nup;
@@ -773,12 +775,12 @@ __global__ void __launch_bounds__(kBuildWarps * 32) k_build_pairs(Params P, Shap
         int plo[3], phi[3];
 #pragma unroll
         for (int k = 0; k < 3; ++k) {
-          plo[k] = D.lohi[6 * i + k];
-          phi[k] = D.lohi[6 * i + 3 + k];
+          plo[k] = D.rec[i].lo[k];
+          phi[k] = D.rec[i].hi[k];
         }
         wall_box(P.wall + 4 * (j - P.n), P.delta, P.dx, plo, phi, lo, hi);   // non-empty (tested by the broad phase)
       } else {
-        pair_box(P, D, i, j, shift, lo, hi);
+        pair_box(P, D.rec + i, D.rec + j, shift, lo, hi);
       }
 #pragma unroll
       for (int k = 0; k < 3; ++k) pr.shift[k] = shift[k];
@@ -792,25 +794,24 @@ __global__ void __launch_bounds__(kBuildWarps * 32) k_build_pairs(Params P, Shap
       // the candidate box's nodes (the cell evaluations and nominal lane-ops
       // of the step), whatever the node sweep later skips
       const long long volp = static_cast<long long>(pr.dim[0]) * pr.dim[1] * pr.dim[2];
-      pr.kinds = W.kind[i] | (W.kind[j] << 8);
+      const PartRec& ri = D.rec[i];
+      const PartRec& rj = D.rec[j];
+      pr.kinds = (ri.kind & 0xff) | ((rj.kind & 0xff) << 8);
 #pragma unroll
       for (int k = 0; k < 3; ++k) {
         // X_i / dx - lo and X_j' / dx - lo = (X_j / dx - s n) - lo
-        pr.ai[k] = D.kX[3 * i + k] - lo[k];
-        pr.af[k] = D.fX[3 * i + k];
-        pr.bi[k] = D.kX[3 * j + k] - pr.shift[k] * P.ncell[k] - lo[k];
-        pr.bf[k] = D.fX[3 * j + k];
+        pr.ai[k] = ri.kX[k] - lo[k];
+        pr.af[k] = ri.fX[k];
+        pr.bi[k] = rj.kX[k] - pr.shift[k] * P.ncell[k] - lo[k];
+        pr.bf[k] = rj.fX[k];
       }
 #pragma unroll
       for (int k = 0; k < 9; ++k) {
-        pr.rta[k] = D.Rt[9 * i + k];
-        pr.rtb[k] = D.Rt[9 * j + k];
+        pr.rta[k] = ri.rt[k];
+        pr.rtb[k] = rj.rt[k];
       }
-#pragma unroll
-      for (int k = 0; k < 3; ++k) {
-        pr.sza[k] = S.size_l[3 * i + k];
-        pr.szb[k] = S.size_l[3 * j + k];
-      }
+      pr.sza[0] = ri.sz0; pr.sza[1] = ri.sz1; pr.sza[2] = ri.sz2;
+      pr.szb[0] = rj.sz0; pr.szb[1] = rj.sz1; pr.szb[2] = rj.sz2;
       if (wall) {   // the wall's value at the box origin, m . lo - (h + inflate) / dx (lattice
                     // units), and its origin at the box origin (node offsets are box-relative)
         const double* e = P.wall + 4 * (j - P.n);
@@ -838,7 +839,7 @@ __global__ void __launch_bounds__(kBuildWarps * 32) k_build_pairs(Params P, Shap
       pr.pair = pi;
       W.pdone[pi] = 0;
       vol = static_cast<unsigned long long>(volp);
-      ops = vol * static_cast<unsigned long long>(S.nomops[i] + S.nomops[j]);
+      ops = vol * static_cast<unsigned long long>((ri.kind >> 8) + (rj.kind >> 8));
       pair_ij[2 * pi] = i;
       pair_ij[2 * pi + 1] = j;
       // slot of this pair in j's (sorted) list of lower partners: the number of entries below i
@@ -974,9 +975,9 @@ void launch_pose(const Params& P, const Shapes& S, const Parts& D, const Lists& 
                  const double* quat, cudaStream_t st) {
   // one-warp blocks: the FP64 chains of different warps land on different sub-partitions
   // (then one block per polytope for its vertices and faces)
-  const int nb = (3 * P.n + 31) / 32;
+  const int nb = (P.n + kPosePerWarp - 1) / kPosePerWarp;
   if (nb > 0) launch_pdl(k_pose, dim3(nb), dim3(32), 0, st, P, S, D, W, pos, quat);
-  if (P.npoly > 0) launch_pdl(k_pose_poly, dim3(P.npoly), dim3(32), 0, st, P, S, D, pos, quat);
+  if (P.npoly > 0) launch_pdl(k_pose_poly, dim3(P.npoly), dim3(32), 0, st, P, S, D, W);
 }
 
 

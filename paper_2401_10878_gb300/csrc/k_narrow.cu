@@ -1329,7 +1329,7 @@ __global__ void __launch_bounds__(kWarps * 32, 2) k_narrow64(Params P, Shapes S,
           acc[4 + a] += ma * gA[a] - mb * gB[a];
         }
         if (w > 0.0) {
-          const long long f = fl::dkey(-(pa + pb));
+          const long long f = order_key(-(pa + pb));
           const int ci = c[0] + r.dim[0] * (c[1] + r.dim[1] * c[2]);
           if (f > bk || (f == bk && ci < bi)) {
             bk = f;

@@ -181,6 +181,8 @@ extern "C" contact_status contact_step_noalloc(const contact_config* cfg, const 
   }
   P.bin_cap = bin_capacity(n, P.binw, rin_min, static_cast<long long>(P.nbin[0]) * P.nbin[1] * P.nbin[2],
                            CONTACT_NOALLOC_MAX_BIN_ENTRIES);
+  P.bin_stride = bin_row(P.bin_cap);
+  P.wide = wide_ranges(rmax, C.dx);
   P.dx = C.dx;
   P.inv_dx = 1.0 / C.dx;
   {
@@ -237,16 +239,12 @@ extern "C" contact_status contact_step_noalloc(const contact_config* cfg, const 
   D.X = cv.take<double>(3 * N);
   D.qhat = cv.take<double>(4 * N);
   D.R = cv.take<double>(9 * N);
-  D.lohi = cv.take<int>(6 * N);
-  D.bin = cv.take<int>(N);
-  D.Rt = cv.take<float>(9 * N);
+  D.rec = cv.take<PartRec>(N);
   D.wplane = cv.take<float4>(1);
-  D.Xf = cv.take<float>(3 * N);
-  D.kX = cv.take<int>(3 * N);
-  D.fX = cv.take<float>(3 * N);
   Lists W{};
   W.bin_count = cv.take<int>(nbins);
-  W.bin_items = cv.take<int>(static_cast<size_t>(nbins) * P.bin_cap);
+  W.bin_items = cv.take<int>(static_cast<size_t>(nbins) * P.bin_stride);
+  W.bin_rec = cv.take<BinRec>(static_cast<size_t>(nbins) * P.bin_stride);
   W.up_count = cv.take<int>(N);
   W.up_list = cv.take<int>(N * kMaxNbr);
   W.dn_count = cv.take<int>(N);
