@@ -282,11 +282,9 @@ struct Lists {
   double* hist_c;   // [2, N, max_nbr] its damping factor
   int* hist_n;      // [2, N] contacts per particle; buffer (steps & 1) is read, the other written
   double* hist_box; // [2, N, max_nbr, 6] box pipeline: each contact's corrected box relative to X_i (or null)
-  PairRec* pairs;   // [max_pairs]
   OvlRec* olist;    // [max_pairs] entry q: pair q's sums when it overlaps (oflag[q] = 1): the force law's work
-  int* oflag;       // [max_pairs] 1 when pair q overlaps (V > 0), else 0 (written by the node sweep or the
-                    // pair builder's separation test)
-  int* tile_pair;   // [max_tiles] pair of each tile
+  int* oflag;       // [max_pairs] 1 when pair q overlaps (V > 0), else 0 (cleared by the pair builder, set by the
+                    // node sweep)
   PairRec* tiles;   // [max_tiles] one record per tile (the pair's record with tile and pair set), the
                     // node sweep's list: a pair's tiles contiguous from its tile0
   float* partial;   // [max_tiles, kPartialFloats]
@@ -475,7 +473,7 @@ inline cudaError_t launch_pdl(void (*kernel)(KArgs...), dim3 grid, dim3 block, s
 void launch_pose(const Params& P, const Shapes& S, const Parts& D, const Lists& W, const double* pos,
                  const double* quat, cudaStream_t st);
 void launch_broad(const Params& P, const Parts& D, const Lists& W, cudaStream_t st);
-void launch_plan(const Params& P, const Shapes& S, const Parts& D, const Lists& W, int32_t* pair_ij, int32_t* n_pairs,
+void launch_plan(const Params& P, const Parts& D, const Lists& W, int32_t* pair_ij, int32_t* n_pairs,
                  double* pair_out, cudaStream_t st);
 constexpr int kRowGroup = 256;   // particles per group sum of the pair-row offsets
 // the row length of bin_cap entries, and whether BinRec's lengths suffice for particles of circumradius rmax

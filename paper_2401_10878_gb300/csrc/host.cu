@@ -250,7 +250,7 @@ void enqueue_step(contact_ctx* c, bool capturing, const double* pos, const doubl
   // bin counts are zero: contact_init clears them, every step's last kernel clears them again
   launch_pose(c->P, c->S, c->D, W, pos, quat, c->stream);
   launch_broad(c->P, c->D, W, c->stream);
-  launch_plan(c->P, c->S, c->D, W, pair_ij, n_pairs, pair_out, c->stream);
+  launch_plan(c->P, c->D, W, pair_ij, n_pairs, pair_out, c->stream);
   if (c->cfg.narrow_events) cudaEventRecordWithFlags(c->ev_narrow[0], c->stream, ev_flags);
   launch_narrow(c->P, c->S, c->D, W, vel, pair_out, c->grid_narrow, c->stream);
   // narrow_events = K > 1: K - 1 more launches of the node sweep, each
@@ -643,10 +643,8 @@ contact_status contact_init(const contact_config* cfg, const int32_t* shape_type
     // the box pipeline's warm start: each contact's corrected box relative to X_i
     if (C.box_mode == 1) GBC_TRY(dev_alloc(c, &W.hist_box, 2 * static_cast<size_t>(n) * max_nbr * 6));
   }
-  GBC_TRY(dev_alloc(c, &W.pairs, mp));
   GBC_TRY(dev_alloc(c, &W.olist, mp));
   GBC_TRY(dev_alloc(c, &W.oflag, mp));
-  GBC_TRY(dev_alloc(c, &W.tile_pair, mt));
   GBC_TRY(dev_alloc(c, &W.tiles, mt));
   GBC_TRY(dev_alloc(c, &W.partial, mt * kPartialFloats));
   if (C.precision == 1 && C.box_mode == 0) GBC_TRY(dev_alloc(c, &W.partial64, mt * kPartialDoubles));

@@ -69,17 +69,18 @@ __device__ __forceinline__ void cross3(const double a[3], const double b[3], dou
 // index on ties), component kc on lanes 0..2 of the pair's four (the layout
 // of k_adj_pre).  Called by the whole warp; `want` selects the pairs that
 // need it (the others get zeros).
-__device__ __forceinline__ void adj_depth_term(const Params& P, const Shapes& S, const Parts& D, const PairRec& pr,
-                                               const double* tp, double gd, bool want, double& dA, double& dcA,
+__device__ __forceinline__ void adj_depth_term(const Params& P, const Shapes& S, const Parts& D, const OvlRec& pr,
+                                               const double* tp, double gd, bool valid, bool want, double& dA, double& dcA,
                                                double& dB, double& dcB) {
   const int lane = threadIdx.x & 31;
   const int k = lane & 3, kc = k < 3 ? k : 0, b0 = lane & ~3;
   const int k1 = kc == 2 ? 0 : kc + 1, k2 = kc == 0 ? 2 : kc - 1;
   dA = dcA = dB = dcB = 0.0;
   if (__any_sync(kFull, want)) {
-    const int i = pr.i, j = pr.j;
-    const int d0 = pr.dim[0], d1 = pr.dim[1], d2 = pr.dim[2];
-    const int idx = min(max(static_cast<int>(tp[13]), 0), d0 * d1 * d2 - 1);
+    // (lanes of pairs without overlap take row 0's particles and a box of one node)
+    const int i = valid ? pr.i : 0, j = valid ? pr.j : 0;
+    const int d0 = valid ? pr.dim[0] : 1, d1 = valid ? pr.dim[1] : 1, d2 = valid ? pr.dim[2] : 1;
+    const int idx = valid ? min(max(static_cast<int>(tp[13]), 0), d0 * d1 * d2 - 1) : 0;
     const int ck = kc == 0 ? idx % d0 : (kc == 1 ? (idx / d0) % d1 : idx / (d0 * d1));
     const int lok = kc == 0 ? pr.lo[0] : (kc == 1 ? pr.lo[1] : pr.lo[2]);
     const int sh = kc == 0 ? pr.shift[0] : (kc == 1 ? pr.shift[1] : pr.shift[2]);
@@ -221,12 +222,13 @@ __global__ void __launch_bounds__(32) k_adj_pre(Params P, Shapes S, Parts D, Lis
     const int p = q0 + slot;
     const bool inr = p < np;
     const int pc = inr ? p : q0;
+    // (the tape and the overlap list hold the overlapping pairs only: flagged by the forward)
     const double* tp = W.tape + static_cast<size_t>(pc) * kTapeDoubles;
-    const PairRec& pr = W.pairs[pc];
-    const double S0 = tp[0];
-    const double fmag = tp[12];
-    const bool act = inr && S0 > 0.0 && record_in_bounds(P, W.err, pr, false);
-    const int i = act ? pr.i : 0, j = act ? pr.j : 0;
+    const OvlRec& pr = W.olist[pc];
+    const bool act = inr && W.oflag[pc] != 0;
+    const double S0 = act ? tp[0] : 1.0;
+    const double fmag = act ? tp[12] : 0.0;
+    const int i = act ? checked_index(W.err, pr.i, P.n, 0) : 0, j = act ? checked_index(W.err, pr.j, P.n + P.nwall, 0) : 0;
     const bool wallj = j >= P.n;   // a wall has no output and no velocity
     const double dx = P.dx;
     const double Lk = kc == 0 ? P.L[0] : (kc == 1 ? P.L[1] : P.L[2]);
@@ -342,7 +344,7 @@ __global__ void __launch_bounds__(32) k_adj_pre(Params P, Shapes S, Parts D, Lis
     }
     // the depth term at the deepest node (independent of the cell sums, so formed here)
     double dA, dcA, dB, dcB;
-    adj_depth_term(P, S, D, pr, tp, gd, act && gd != 0.0 && d > 0.0, dA, dcA, dB, dcB);
+    adj_depth_term(P, S, D, pr, tp, gd, act, act && gd != 0.0 && d > 0.0, dA, dcA, dB, dcB);
     gXA += dA;
     gXB += dB;
     // x_c = (lo + S1/S0) dx ; V = dx^3 S0

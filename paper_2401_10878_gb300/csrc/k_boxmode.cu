@@ -225,13 +225,6 @@ __device__ __forceinline__ float warp_sum_f(float v) {
   return v;
 }
 
-__device__ __forceinline__ void zero_pair(const Lists& W, double* pair_out, int q) {
-  const int lane = threadIdx.x & 31;
-  if (lane < 11) pair_out[static_cast<size_t>(q) * 11 + lane] = 0.0;
-  if (lane < kFtDoubles) W.ft[static_cast<size_t>(q) * kFtDoubles + lane] = 0.0;
-  if (lane < kTapeDoubles) W.tape[static_cast<size_t>(q) * kTapeDoubles + lane] = 0.0;
-}
-
 template <int SET>
 __global__ void __launch_bounds__(kBoxWarps * 32, 2) k_box_pairs(Params P, Shapes S, Parts D, Lists W,
                                                               const double* __restrict__ vel,
@@ -281,10 +274,7 @@ __global__ void __launch_bounds__(kBoxWarps * 32, 2) k_box_pairs(Params P, Shape
       mn[k] = __reduce_min_sync(kFull, mn[k]);
       mx[k] = __reduce_max_sync(kFull, mx[k]);
     }
-    if (mn[0] > mx[0]) {
-      zero_pair(W, pair_out, q);
-      continue;
-    }
+    if (mn[0] > mx[0]) continue;   // no rough contact: the pair builder's zero outputs stay
     // 2. B0 (physical, as the rough box's nodes +- sqrt(0.75) dx), then the lines
     const double s64 = sqrt(0.75) * P.dx;
     double b0lo[3], b0hi[3];
@@ -485,10 +475,7 @@ __global__ void __launch_bounds__(kBoxWarps * 32, 2) k_box_pairs(Params P, Shape
       const int kmax = __reduce_max_sync(kFull, key);
       bestidx = __reduce_min_sync(kFull, key == kmax ? bestidx : 0x7fffffff);
     }
-    if (!(cnt > 0.f)) {
-      zero_pair(W, pair_out, q);
-      continue;
-    }
+    if (!(cnt > 0.f)) continue;
     // 4. FP64 pair results and the force law: component k of every vector on
     // lane k < 3 (cross and dot products by shuffles; every FP64 warp
     // instruction costs the same however few lanes it has), the distances of
@@ -589,7 +576,6 @@ __global__ void __launch_bounds__(kBoxWarps * 32, 2) k_box_pairs(Params P, Shape
         o[7] = d;
         atomicAdd(&W.counters[5], 1);
       }
-      if (lane < kTapeDoubles) W.tape[static_cast<size_t>(q) * kTapeDoubles + lane] = 0.0;
       if (P.history) {   // this step's contact: j, c and the corrected box minus X_i
         const int wr = (W.counters[kStepCounter] & 1) ^ 1;
         int slot = 0;

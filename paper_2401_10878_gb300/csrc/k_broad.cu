@@ -307,17 +307,6 @@ __global__ void k_pose_poly(Params P, Shapes S, Parts D, Lists W) {
 // 4 R_max + 2 dx every range is shorter than n/2, so no other image can meet it.
 __device__ __forceinline__ int image_shift(int d, int n) { return d > (n >> 1) ? 1 : (d < -(n >> 1) ? -1 : 0); }
 
-// Node box of pair (p, q) with q's image nearest p.
-__device__ __forceinline__ void pair_box(const Params& P, const PartRec* a, const PartRec* b, int s[3], int lo[3],
-                                         int hi[3]) {
-#pragma unroll
-  for (int k = 0; k < 3; ++k) {
-    s[k] = image_shift(b->lo[k] - a->lo[k], P.ncell[k]);
-    lo[k] = max(a->lo[k], b->lo[k] - s[k] * P.ncell[k]);
-    hi[k] = min(a->hi[k], b->hi[k] - s[k] * P.ncell[k]);
-  }
-}
-
 // K3: one warp per particle p.  Lane b < 27 owns neighbour bin b of the
 // fixed-capacity cell list; its entries (node range and particle, one 16-byte
 // and one 4-byte word each) are read four at a time, tested against p's node
@@ -407,7 +396,7 @@ __global__ void __launch_bounds__(256) k_broad(Params P, Parts D, Lists W) {
     for (int u = 0; u < 4; ++u) {
       if (t0 + u >= maxn) break;   // warp-uniform
       const int j = t0 + u < num ? checked_index(W.err, jj[u], P.n, -1) : -1;
-      // node ranges intersect, the partner moved by the image shift (as in pair_box):
+      // node ranges intersect, the partner moved by the image shift (as in the pair builder):
       // its corner lies above p's by at most p's length and below it by at most its own
       bool hit = j >= 0 && j != p && nodes;
       const int jl[3] = {cur[u].x, cur[u].y, cur[u].z};
@@ -489,13 +478,28 @@ __global__ void __launch_bounds__(256) k_broad(Params P, Parts D, Lists W) {
 }
 
 
-// K4: one warp per particle row i, one lane per partner slot r: the pair
-// record of pair row_off[i] + r, its sweep layout and its node tiles.  Tiles
-// are allocated with one atomic per warp round; a pair's tiles are
-// contiguous, and its partial sums do not depend on where they land, so the
-// results are deterministic.  No FP64: centres come as integer node + FP32
-// remainder from the pose kernel.
-constexpr int kBuildWarps = 8;   // particle rows per block of the pair builder
+// K4: the candidate pairs of `rows` consecutive particles per one-warp block,
+// one lane per pair (their (row, partner) found in the rows' prefix sums): the
+// pair record of pair row_off[i] + r, its sweep layout and its node tiles.
+// Tiles are allocated with one atomic per round; a pair's tiles are contiguous,
+// and its partial sums do not depend on where they land, so the results are
+// deterministic.  No FP64 but for walls: centres come as integer node + FP32
+// remainder from the pose kernel.  Bound: instruction issue and load
+// wavefronts on large boxes, load latency on small ones.  One warp per row left
+// 28 of 32 lanes idle (3.4 partners a particle): 120 -> 27 us on 52218 cubes
+// with the lanes filled, the zero outputs stored by consecutive lanes and no
+// record kept of pairs without tiles.
+constexpr int kBuildRows = 8;   // most rows of a block
+constexpr int kUpAhead = 8;     // partners of a row fetched before its count is known
+// Rows per block: eight fill a warp at 3-4 partners a row (four in the box
+// pipeline, whose wider ranges give six); half as many while that leaves the
+// step with fewer than two blocks per SM sub-partition, where a block's latency
+// counts and not its lanes (1934 cubes: 6.4 us against
+// 9.6 us with sixteen rows on two warps).
+inline int build_rows(const Params& P) {
+  const int rows = P.box_mode == 1 ? 4 : 8;
+  return P.n < 2 * 608 * rows ? rows / 2 : rows;
+}
 
 // Store a pair record (with its tile index) as fourteen 16-byte stores from
 // registers, field by field (an aggregate copy would stage it in local memory).
@@ -641,62 +645,86 @@ __device__ unsigned pair_apart(const PairRec& r, float T) {
 // {phi_A < T} or {phi_B < T} is no rough-contact node, so the pair's node box
 // shrinks to the bounding box of the intersection of the two boxes grown by T
 // (half extents size + T).  The vertices of that intersection are end points
-// of the edges of either box clipped to the other one, so lane e < 24 clips
-// edge e (A's twelve, then B's) to the other box, grown by kCutSlack more, and
-// the bounds of the end points, widened by kCutSlack, are reduced over the
-// warp.  FP32 in box-relative lattice units: the rounding (~1e-5 cells) stays
-// far inside the slack, so every node with both distances below T is kept.
-// The whole warp calls this with the record in shared memory; false: the
+// of the edges of either box clipped to the other one, so each of the 24 edges
+// (A's twelve, then B's) is clipped to the other box, grown by kCutSlack more,
+// and the bounds of the end points are widened by kCutSlack.  FP32 in
+// box-relative lattice units: the rounding (~1e-5 cells) stays far inside the
+// slack, so every node with both distances below T is kept.  One lane per pair
+// (a warp per pair with the edges on its lanes took a pair after the other:
+// the kernel 26.3 -> 18.2 us on 1934 cubes).  Returns false when the
 // intersection is empty.
 constexpr float kCutSlack = 1e-2f;
 
-__device__ __forceinline__ bool cut_box(const PairRec& sr, float T, int nlo[3], int nhi[3]) {
-  const int lane = threadIdx.x & 31;
-  const bool onb = lane >= 12;
-  const int q = onb ? lane - 12 : lane;
-  const int m = min(q >> 2, 2), m1 = m == 2 ? 0 : m + 1, m2 = m1 == 2 ? 0 : m1 + 1;
-  const float s1 = (q & 1) ? 1.f : -1.f, s2 = (q & 2) ? 1.f : -1.f;
-  const float* ro = onb ? sr.rtb : sr.rta;   // the edge's box: body axis k = row k
-  const float* rx = onb ? sr.rta : sr.rtb;   // the other box
-  const float* eo = onb ? sr.szb : sr.sza;
-  const float* ex = onb ? sr.sza : sr.szb;
-  const int* io = onb ? sr.bi : sr.ai;
-  const int* ix = onb ? sr.ai : sr.bi;
-  const float* fo = onb ? sr.bf : sr.af;
-  const float* fx = onb ? sr.af : sr.bf;
-  const float e0 = eo[m] + T, e1 = eo[m1] + T, e2 = eo[m2] + T;
-  // edge p0 + t dv, t in [-1, 1]; rel = p0 minus the other box's centre
-  float p0[3], dv[3], rel[3];
+__device__ __forceinline__ bool cut_box(const PairRec& r, float T, int nlo[3], int nhi[3]) {
+  // M[a][b] = (A's body axis a) . (B's body axis b); d = centre of B - centre of A
+  float M[3][3], ca[3], cb[3], d[3];
 #pragma unroll
   for (int c = 0; c < 3; ++c) {
-    const float co = static_cast<float>(io[c]) + fo[c], cx = static_cast<float>(ix[c]) + fx[c];
-    p0[c] = fmaf(s2 * e2, ro[3 * m2 + c], fmaf(s1 * e1, ro[3 * m1 + c], co));
-    dv[c] = e0 * ro[3 * m + c];
-    rel[c] = p0[c] - cx;
+    ca[c] = static_cast<float>(r.ai[c]) + r.af[c];
+    cb[c] = static_cast<float>(r.bi[c]) + r.bf[c];
+    d[c] = cb[c] - ca[c];
   }
-  float t0 = -1.f, t1 = 1.f;
 #pragma unroll
-  for (int k = 0; k < 3; ++k) {
-    const float base = dot3(rx + 3 * k, rel), sl = dot3(rx + 3 * k, dv);
-    const float E = ex[k] + T + kCutSlack;
-    if (fabsf(sl) > 1e-6f) {
-      const float is = __fdividef(1.f, sl);
-      const float a = (-E - base) * is, b = (E - base) * is;
-      t0 = fmaxf(t0, fminf(a, b));
-      t1 = fminf(t1, fmaxf(a, b));
-    } else if (!(fabsf(base) <= E)) {
-      t1 = -2.f;
+  for (int a = 0; a < 3; ++a)
+#pragma unroll
+    for (int b = 0; b < 3; ++b) M[a][b] = dot3(r.rta + 3 * a, r.rtb + 3 * b);
+  float flo[3] = {FLT_MAX, FLT_MAX, FLT_MAX}, fhi[3] = {-FLT_MAX, -FLT_MAX, -FLT_MAX};
+#pragma unroll
+  for (int side = 0; side < 2; ++side) {   // A's edges against B's slabs, then B's against A's
+    const float* ro = side ? r.rtb : r.rta;
+    const float* rx = side ? r.rta : r.rtb;
+    const float* eo = side ? r.szb : r.sza;
+    const float* ex = side ? r.sza : r.szb;
+    const float* co = side ? cb : ca;
+    float base[3];   // the box's centre in the other's frame
+#pragma unroll
+    for (int k = 0; k < 3; ++k) base[k] = side ? dot3(rx + 3 * k, d) : -dot3(rx + 3 * k, d);
+#pragma unroll
+    for (int m = 0; m < 3; ++m) {   // edges along body axis m
+      const int m1 = m == 2 ? 0 : m + 1, m2 = m1 == 2 ? 0 : m1 + 1;
+      const float e0 = eo[m] + T, e1 = eo[m1] + T, e2 = eo[m2] + T;
+      float sl[3], is[3], b1[3], b2[3];
+#pragma unroll
+      for (int k = 0; k < 3; ++k) {
+        sl[k] = e0 * (side ? M[k][m] : M[m][k]);
+        is[k] = __fdividef(1.f, sl[k]);
+        b1[k] = e1 * (side ? M[k][m1] : M[m1][k]);
+        b2[k] = e2 * (side ? M[k][m2] : M[m2][k]);
+      }
+#pragma unroll
+      for (int q = 0; q < 4; ++q) {
+        const float s1 = (q & 1) ? 1.f : -1.f, s2 = (q & 2) ? 1.f : -1.f;
+        float t0 = -1.f, t1 = 1.f;   // p0 + t dv, t in [-1, 1]
+#pragma unroll
+        for (int k = 0; k < 3; ++k) {
+          const float p = fmaf(s2, b2[k], fmaf(s1, b1[k], base[k]));
+          const float E = ex[k] + T + kCutSlack;
+          if (fabsf(sl[k]) > 1e-6f) {
+            const float x = (-E - p) * is[k], y = (E - p) * is[k];
+            t0 = fmaxf(t0, fminf(x, y));
+            t1 = fminf(t1, fmaxf(x, y));
+          } else if (!(fabsf(p) <= E)) {
+            t1 = -2.f;
+          }
+        }
+        if (t0 <= t1) {
+#pragma unroll
+          for (int c = 0; c < 3; ++c) {
+            const float p0 = fmaf(s2 * e2, ro[3 * m2 + c], fmaf(s1 * e1, ro[3 * m1 + c], co[c]));
+            const float x = fmaf(t0 * e0, ro[3 * m + c], p0), y = fmaf(t1 * e0, ro[3 * m + c], p0);
+            flo[c] = fminf(flo[c], fminf(x, y));
+            fhi[c] = fmaxf(fhi[c], fmaxf(x, y));
+          }
+        }
+      }
     }
   }
-  const bool ok = lane < 24 && t0 <= t1;
   bool any = true;
 #pragma unroll
   for (int c = 0; c < 3; ++c) {
-    const float a = t0 * dv[c], b = t1 * dv[c];
-    const int lo = ok ? static_cast<int>(ceilf(p0[c] + fminf(a, b) - kCutSlack)) : 0x7fffffff;
-    const int hi = ok ? static_cast<int>(floorf(p0[c] + fmaxf(a, b) + kCutSlack)) : -0x7fffffff;
-    nlo[c] = __reduce_min_sync(kFull, lo);
-    nhi[c] = __reduce_max_sync(kFull, hi);
+    any = any && flo[c] <= fhi[c];
+    nlo[c] = any ? static_cast<int>(ceilf(flo[c] - kCutSlack)) : 1;
+    nhi[c] = any ? static_cast<int>(floorf(fhi[c] + kCutSlack)) : 0;
     any = any && nlo[c] <= nhi[c];
   }
   return any;
@@ -705,24 +733,26 @@ __device__ __forceinline__ bool cut_box(const PairRec& sr, float T, int nlo[3], 
 // BOXM: the box pipeline's variant (its separation test at the rough threshold,
 // the cut node boxes of two boxes, one list entry per kept pair).
 template <bool BOXM>
-__global__ void __launch_bounds__(kBuildWarps * 32) k_build_pairs(Params P, Shapes S, Parts D, Lists W,
-                                                                  int32_t* __restrict__ pair_ij,
-                                                                  int32_t* __restrict__ n_pairs_out,
-                                                                  double* __restrict__ pair_out) {
-  // per warp: tiles (exclusive prefix after the block scan)
-  __shared__ int s_w[kBuildWarps];
-  __shared__ int s_base;
-  __shared__ unsigned long long s_u64[kBuildWarps][2];
-  __shared__ __align__(16) PairRec s_pr[BOXM ? kBuildWarps : 1];   // a record being cut (cut_box)
+__global__ void __launch_bounds__(32) k_build_pairs(Params P, Parts D, Lists W, int rows,
+                                                               int32_t* __restrict__ pair_ij,
+                                                               int32_t* __restrict__ n_pairs_out,
+                                                               double* __restrict__ pair_out) {
+  __shared__ int s_off[kBuildRows + 1];             // pairs before each row of the block
+  __shared__ int s_up[kBuildRows][kUpAhead];        // the rows' first partners, fetched with their counts
   pdl_begin();
-  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-  const int i0 = blockIdx.x * kBuildWarps + wid;
-  const bool row_ok = i0 < P.n;
-  const int i = row_ok ? i0 : P.n - 1;   // rows past the end take part in the block's barriers only
+  const int lane = threadIdx.x;
+  const int row0 = blockIdx.x * rows;
+  const int nrow = min(rows, P.n - row0);
   const int cap = P.max_nbr;
-  // first pair of row i: the group sums before i's group plus the counts of
-  // the earlier particles of its group (both sets of loads in flight at once)
-  const int g = i / kRowGroup;
+#pragma unroll
+  for (int u = 0; u < kBuildRows * kUpAhead / 32; ++u) {   // (entries past a row's count are stale and unused)
+    const int x = lane + u * 32, rr = x / kUpAhead, k = x % kUpAhead;
+    if (rr < nrow && k < cap) s_up[rr][k] = W.up_list[static_cast<size_t>(row0 + rr) * cap + k];
+  }
+  // the rows' partner counts and their prefix; the first pair of row0: the group sums before its
+  // group plus the counts of the earlier particles of its group
+  int incl = lane < nrow ? W.up_count[row0 + lane] : 0;
+  const int g = row0 / kRowGroup;
   int acc = 0;
   for (int base = 0; base < g; base += 8 * 32) {
 #pragma unroll
@@ -734,88 +764,100 @@ __global__ void __launch_bounds__(kBuildWarps * 32) k_build_pairs(Params P, Shap
 #pragma unroll
   for (int u = 0; u < kRowGroup / 32; ++u) {
     const int e = g * kRowGroup + 32 * u + lane;
-    acc += e < i ? W.up_count[e] : 0;
+    acc += e < row0 ? W.up_count[e] : 0;
   }
-  const int cnt = row_ok ? W.up_count[i] : 0;
-  // the first 32 partners, fetched before the count is known (stale beyond it, unused)
-  const int jpre = lane < cap ? W.up_list[static_cast<size_t>(i) * cap + lane] : 0;
-  const int row = __reduce_add_sync(kFull, acc);
-  if (lane == 0 && row_ok) {
-    W.row_off[i] = row;
-    if (i == P.n - 1) {   // the pair count: the last row's offset plus its partners
-      const int total = row + cnt;
-      W.counters[0] = total;
-      W.row_off[P.n] = total;
-      *n_pairs_out = total;
-      if (total > P.max_pairs) set_error(W.err, kErrCapacity);
-    }
+#pragma unroll
+  for (int d = 1; d < kBuildRows; d <<= 1) {
+    const int v = __shfl_up_sync(kFull, incl, d);
+    if (lane >= d) incl += v;
   }
-  for (int base = 0; __syncthreads_or(base < cnt); base += 32) {   // block-uniform rounds of 32 partners
-    const int r = base + lane;
-    const bool active = r < cnt && (row + r) < P.max_pairs;
+  if (lane < kBuildRows) s_off[lane + 1] = incl;
+  if (lane == 0) s_off[0] = 0;
+  const int row_base = __reduce_add_sync(kFull, acc);
+  __syncwarp();
+  const int total = s_off[nrow];
+  if (lane < nrow) W.row_off[row0 + lane] = row_base + s_off[lane];
+  if (lane == 0 && row0 + nrow == P.n) {   // the pair count: the last row's offset plus its partners
+    const int all = row_base + total;
+    W.counters[0] = all;
+    W.row_off[P.n] = all;
+    *n_pairs_out = all;
+    if (all > P.max_pairs) set_error(W.err, kErrCapacity);
+  }
+  unsigned long long vol_sum = 0, ops_sum = 0;
+  for (int base = 0; base < total; base += 32) {   // warp-uniform rounds of 32 pairs
+    const int e = base + lane;
+    const int pi = row_base + e;
+    const bool active = e < total && pi < P.max_pairs;
     PairRec pr;
-    int pi = 0, ntiles = 0;
+    int ntiles = 0;
     bool skip = false, cut = false;
-    unsigned long long vol = 0, ops = 0;
     if (active) {
-      pi = row + r;
-      const int j = checked_index(W.err, base == 0 ? jpre : W.up_list[static_cast<size_t>(i) * cap + r],
+      int rr = 0;   // the last row that starts at or before the pair
+#pragma unroll
+      for (int d = kBuildRows / 2; d > 0; d >>= 1)
+        if (rr + d < nrow && s_off[rr + d] <= e) rr += d;
+      const int i = row0 + rr;
+      const int k_ = e - s_off[rr];
+      const int j = checked_index(W.err, k_ < kUpAhead ? s_up[rr][k_] : W.up_list[static_cast<size_t>(i) * cap + k_],
                                   P.n + P.nwall, i);
-      // j's lower-partner list, fetched with j's particle data (slot of this pair below);
-      // a wall (j >= n) has none
+      // j's lower-partner list, fetched with j's line (slot of this pair below); a wall (j >= n) has none
       const bool wall = j >= P.n;
       const int* dl = W.dn_list + static_cast<size_t>(wall ? 0 : j) * cap;
       const int dc = wall ? 0 : checked_index(W.err, W.dn_count[j], cap + 1, 0);
       int dpre[8];
 #pragma unroll
       for (int u = 0; u < 8; ++u) dpre[u] = u < cap ? dl[u] : 0;
-      int lo[3], hi[3];
-      int shift[3] = {0, 0, 0};
+      // both particles' lines, 16 bytes at a time
+      const int4* la = reinterpret_cast<const int4*>(D.rec + i);
+      const int4* lb = reinterpret_cast<const int4*>(D.rec + j);
+      const int4 a0 = la[0], a1 = la[1], a2 = la[2], a3 = la[3], a4 = la[4], a5 = la[5], a6 = la[6];
+      const int4 b0 = lb[0], b1 = lb[1], b2 = lb[2], b3 = lb[3], b4 = lb[4], b5 = lb[5], b6 = lb[6];
+      const int alo[3] = {a0.x, a0.y, a0.z}, ahi[3] = {a1.x, a1.y, a1.z};
+      const int blo[3] = {b0.x, b0.y, b0.z}, bhi[3] = {b1.x, b1.y, b1.z};
+      const int akx[3] = {a2.x, a2.y, a2.z}, bkx[3] = {b2.x, b2.y, b2.z};
+      const auto f = [](int x) { return __int_as_float(x); };
+      int lo[3], hi[3], shift[3] = {0, 0, 0};
       if (wall) {
-        int plo[3], phi[3];
+        wall_box(P.wall + 4 * (j - P.n), P.delta, P.dx, alo, ahi, lo, hi);   // non-empty (tested by the broad phase)
+      } else {
 #pragma unroll
         for (int k = 0; k < 3; ++k) {
-          plo[k] = D.rec[i].lo[k];
-          phi[k] = D.rec[i].hi[k];
+          shift[k] = image_shift(blo[k] - alo[k], P.ncell[k]);
+          lo[k] = max(alo[k], blo[k] - shift[k] * P.ncell[k]);
+          hi[k] = min(ahi[k], bhi[k] - shift[k] * P.ncell[k]);
         }
-        wall_box(P.wall + 4 * (j - P.n), P.delta, P.dx, plo, phi, lo, hi);   // non-empty (tested by the broad phase)
-      } else {
-        pair_box(P, D.rec + i, D.rec + j, shift, lo, hi);
       }
-#pragma unroll
-      for (int k = 0; k < 3; ++k) pr.shift[k] = shift[k];
       pr.i = i;
       pr.j = j;
 #pragma unroll
       for (int k = 0; k < 3; ++k) {
+        pr.shift[k] = shift[k];
         pr.lo[k] = lo[k];
         pr.dim[k] = hi[k] - lo[k] + 1;
+        // X_i / dx - lo and X_j' / dx - lo = (X_j / dx - s n) - lo
+        pr.ai[k] = akx[k] - lo[k];
+        pr.bi[k] = bkx[k] - shift[k] * P.ncell[k] - lo[k];
       }
       // the candidate box's nodes (the cell evaluations and nominal lane-ops
       // of the step), whatever the node sweep later skips
-      const long long volp = static_cast<long long>(pr.dim[0]) * pr.dim[1] * pr.dim[2];
-      const PartRec& ri = D.rec[i];
-      const PartRec& rj = D.rec[j];
-      pr.kinds = (ri.kind & 0xff) | ((rj.kind & 0xff) << 8);
-#pragma unroll
-      for (int k = 0; k < 3; ++k) {
-        // X_i / dx - lo and X_j' / dx - lo = (X_j / dx - s n) - lo
-        pr.ai[k] = ri.kX[k] - lo[k];
-        pr.af[k] = ri.fX[k];
-        pr.bi[k] = rj.kX[k] - pr.shift[k] * P.ncell[k] - lo[k];
-        pr.bf[k] = rj.fX[k];
-      }
-#pragma unroll
-      for (int k = 0; k < 9; ++k) {
-        pr.rta[k] = ri.rt[k];
-        pr.rtb[k] = rj.rt[k];
-      }
-      pr.sza[0] = ri.sz0; pr.sza[1] = ri.sz1; pr.sza[2] = ri.sz2;
-      pr.szb[0] = rj.sz0; pr.szb[1] = rj.sz1; pr.szb[2] = rj.sz2;
+      const unsigned long long vol =
+          static_cast<unsigned long long>(static_cast<long long>(pr.dim[0]) * pr.dim[1] * pr.dim[2]);
+      vol_sum += vol;
+      ops_sum += vol * static_cast<unsigned long long>((a0.w >> 8) + (b0.w >> 8));
+      pr.kinds = (a0.w & 0xff) | ((b0.w & 0xff) << 8);
+      pr.af[0] = f(a3.x); pr.af[1] = f(a3.y); pr.af[2] = f(a3.z);
+      pr.bf[0] = f(b3.x); pr.bf[1] = f(b3.y); pr.bf[2] = f(b3.z);
+      pr.rta[0] = f(a4.x); pr.rta[1] = f(a4.y); pr.rta[2] = f(a4.z); pr.rta[3] = f(a4.w);
+      pr.rta[4] = f(a5.x); pr.rta[5] = f(a5.y); pr.rta[6] = f(a5.z); pr.rta[7] = f(a5.w); pr.rta[8] = f(a6.x);
+      pr.rtb[0] = f(b4.x); pr.rtb[1] = f(b4.y); pr.rtb[2] = f(b4.z); pr.rtb[3] = f(b4.w);
+      pr.rtb[4] = f(b5.x); pr.rtb[5] = f(b5.y); pr.rtb[6] = f(b5.z); pr.rtb[7] = f(b5.w); pr.rtb[8] = f(b6.x);
+      pr.sza[0] = f(a2.w); pr.sza[1] = f(a3.w); pr.sza[2] = f(a6.y);
+      pr.szb[0] = f(b2.w); pr.szb[1] = f(b3.w); pr.szb[2] = f(b6.y);
       if (wall) {   // the wall's value at the box origin, m . lo - (h + inflate) / dx (lattice
                     // units), and its origin at the box origin (node offsets are box-relative)
-        const double* e = P.wall + 4 * (j - P.n);
-        const double p0 = ((e[0] * lo[0] + e[1] * lo[1]) + e[2] * lo[2]) - (e[3] + P.inflate) * P.inv_dx;
+        const double* w = P.wall + 4 * (j - P.n);
+        const double p0 = ((w[0] * lo[0] + w[1] * lo[1]) + w[2] * lo[2]) - (w[3] + P.inflate) * P.inv_dx;
         pr.szb[0] = static_cast<float>(p0);
 #pragma unroll
         for (int k = 0; k < 3; ++k) {
@@ -826,8 +868,8 @@ __global__ void __launch_bounds__(kBuildWarps * 32) k_build_pairs(Params P, Shap
       // the node sweeps skip pairs whose distance regions are apart, and
       // so does the box pipeline (regions at its rough-detection threshold;
       // a polytope's tabulated radii belong to the node sweep's threshold, so
-      // pairs with one are kept there); the skipped pairs' zero outputs are
-      // written below.  In the box pipeline two boxes' node box is also cut to
+      // pairs with one are kept there); the skipped pairs keep their zero
+      // outputs.  In the box pipeline two boxes' node box is also cut to
       // their regions' intersection (after the record is complete).
       const int ka = pr.kinds & 0xff, kb = pr.kinds >> 8;
       constexpr bool boxm = BOXM;
@@ -837,50 +879,37 @@ __global__ void __launch_bounds__(kBuildWarps * 32) k_build_pairs(Params P, Shap
       cut = boxm && !skip && (ka == KIND_CUBE || ka == KIND_CUBOID) && (kb == KIND_CUBE || kb == KIND_CUBOID);
       pr.tile = 0;
       pr.pair = pi;
-      W.pdone[pi] = 0;
-      vol = static_cast<unsigned long long>(volp);
-      ops = vol * static_cast<unsigned long long>((ri.kind >> 8) + (rj.kind >> 8));
-      pair_ij[2 * pi] = i;
-      pair_ij[2 * pi + 1] = j;
+      pair_ij[2 * static_cast<size_t>(pi)] = i;   // (the caller's array: 4-byte alignment)
+      pair_ij[2 * static_cast<size_t>(pi) + 1] = j;
       // slot of this pair in j's (sorted) list of lower partners: the number of entries below i
-      int a0 = 0;
+      int s0 = 0;
 #pragma unroll
-      for (int u = 0; u < 8; ++u) a0 += (u < dc && dpre[u] < i) ? 1 : 0;
-      for (int b = 8; b < dc; ++b) a0 += dl[b] < i ? 1 : 0;
-      if (!wall) W.dn_pair[static_cast<size_t>(j) * cap + checked_index(W.err, a0, cap, 0)] = pi;
+      for (int u = 0; u < 8; ++u) s0 += (u < dc && dpre[u] < i) ? 1 : 0;
+      for (int u = 8; u < dc; ++u) s0 += dl[u] < i ? 1 : 0;
+      if (!wall) W.dn_pair[static_cast<size_t>(j) * cap + checked_index(W.err, s0, cap, 0)] = pi;
     }
-    // the box pipeline's cut node boxes, one pair at a time for the whole
-    // warp (the record passes through shared memory); the box, the centres'
-    // integer parts and nothing else change, so every node keeps its FP32
-    // distances
-    for (unsigned todo = BOXM ? __ballot_sync(kFull, cut) : 0u; todo != 0u; todo &= todo - 1u) {
-      const int src = __ffs(todo) - 1;
-      if (lane == src) store_pair_rec(&s_pr[wid], pr, 0);
-      __syncwarp();
+    // the box pipeline's cut node boxes: the box, the centres' integer parts
+    // and nothing else change, so every node keeps its FP32 distances
+    if (BOXM && cut) {
       int nlo[3], nhi[3];
-      const bool any = cut_box(s_pr[wid], kRoughT, nlo, nhi);
-      if (lane == src) {
-        int a[3], b[3];
-        bool keep = any;
+      bool keep = cut_box(pr, kRoughT, nlo, nhi);
+#pragma unroll
+      for (int k = 0; k < 3; ++k) {
+        nlo[k] = max(nlo[k], 0);
+        nhi[k] = min(nhi[k], pr.dim[k] - 1);
+        keep = keep && nlo[k] <= nhi[k];
+      }
+      if (keep) {
 #pragma unroll
         for (int k = 0; k < 3; ++k) {
-          a[k] = max(nlo[k], 0);
-          b[k] = min(nhi[k], pr.dim[k] - 1);
-          keep = keep && a[k] <= b[k];
+          pr.lo[k] += nlo[k];
+          pr.dim[k] = nhi[k] - nlo[k] + 1;
+          pr.ai[k] -= nlo[k];
+          pr.bi[k] -= nlo[k];
         }
-        if (keep) {
-#pragma unroll
-          for (int k = 0; k < 3; ++k) {
-            pr.lo[k] += a[k];
-            pr.dim[k] = b[k] - a[k] + 1;
-            pr.ai[k] -= a[k];
-            pr.bi[k] -= a[k];
-          }
-        } else {
-          skip = true;   // no rough-contact node: zero outputs
-        }
+      } else {
+        skip = true;   // no rough-contact node: zero outputs
       }
-      __syncwarp();
     }
     if (active) {
       // sweep layout: whole node lines along the box's longest axis (the
@@ -898,74 +927,62 @@ __global__ void __launch_bounds__(kBuildWarps * 32) k_build_pairs(Params P, Shap
       // the box pipeline takes each kept pair as one entry of the tile list
       ntiles = skip ? 0 : (BOXM ? 1 : (pr.nitems + 32 * kTileItemsPerLane - 1) / (32 * kTileItemsPerLane));
       pr.ntiles = ntiles;
-      // a skipped pair's outputs, as the node sweep or the box pipeline would write them (zeros)
-      if (skip) {
-        double* po = pair_out + static_cast<size_t>(pi) * 11;
-        double* pf = W.ft + static_cast<size_t>(pi) * kFtDoubles;
-        double* pt = W.tape + static_cast<size_t>(pi) * kTapeDoubles;
-#pragma unroll
-        for (int k = 0; k < 11; ++k) po[k] = 0.0;
-#pragma unroll
-        for (int k = 0; k < kFtDoubles; ++k) pf[k] = 0.0;
-#pragma unroll
-        for (int k = 0; k < kTapeDoubles; ++k) pt[k] = 0.0;
-        W.oflag[pi] = 0;
-      }
     }
-    // allocations aggregated over the block (one atomic per counter and
-    // block, all in flight together): the pairs' tiles, contiguous per pair;
-    // tile k of a pair is entry tile0 + k of the node sweep's tile list
-    int incl = ntiles;
+    // allocation aggregated over the warp (one atomic per round): the pairs'
+    // tiles, contiguous per pair; tile k of a pair is entry tile0 + k of the
+    // node sweep's tile list
+    int tincl = ntiles;
 #pragma unroll
     for (int d = 1; d < 32; d <<= 1) {
-      const int v = __shfl_up_sync(kFull, incl, d);
-      if (lane >= d) incl += v;
+      const int v = __shfl_up_sync(kFull, tincl, d);
+      if (lane >= d) tincl += v;
     }
-    unsigned long long wv = vol, wo = ops;
-#pragma unroll
-    for (int d = 16; d > 0; d >>= 1) {
-      wv += __shfl_xor_sync(kFull, wv, d);
-      wo += __shfl_xor_sync(kFull, wo, d);
-    }
-    const int wtiles = __shfl_sync(kFull, incl, 31);
-    if (lane == 0) {
-      s_w[wid] = wtiles;
-      s_u64[wid][0] = wv;
-      s_u64[wid][1] = wo;
-    }
-    __syncthreads();
-    if (threadIdx.x == 0) {   // exclusive prefix over the warps, one atomic
-      int run = 0;
-      for (int w = 0; w < kBuildWarps; ++w) {
-        const int v = s_w[w];
-        s_w[w] = run;
-        run += v;
-      }
-      s_base = run > 0 ? atomicAdd(&W.counters[1], run) : 0;
-    } else if (threadIdx.x == 32) {
-      unsigned long long a = 0, b = 0;
-      for (int w = 0; w < kBuildWarps; ++w) { a += s_u64[w][0]; b += s_u64[w][1]; }
-      if (a > 0) {
-        atomicAdd(&W.u64[0], a);
-        atomicAdd(&W.u64[1], b);
+    const int wtiles = __shfl_sync(kFull, tincl, 31);
+    int tbase = 0;
+    if (lane == 0 && wtiles > 0) tbase = atomicAdd(&W.counters[1], wtiles);
+    // while the atomic is under way: the round's pairs' outputs start as zeros (what a pair without
+    // overlap keeps), consecutive lanes storing consecutive words
+    {
+      const size_t q0 = static_cast<size_t>(row_base) + base;
+      const int np = max(0, min(min(32, total - base), P.max_pairs - (row_base + base)));
+      double* po = pair_out + q0 * 11;
+      double* pf = W.ft + q0 * kFtDoubles;
+      for (int x = lane; x < 11 * np; x += 32) po[x] = 0.0;
+      for (int x = lane; x < kFtDoubles * np; x += 32) pf[x] = 0.0;
+      if (lane < np) {
+        W.oflag[q0 + lane] = 0;
+        W.pdone[q0 + lane] = 0;
       }
     }
-    __syncthreads();
-    const int tbase = s_base + s_w[wid];
-    if (active) {
-      pr.tile0 = tbase + incl - ntiles;
-      store_pair_rec(W.pairs + pi, pr, 0);
+    tbase = __shfl_sync(kFull, tbase, 0);
+    if (ntiles > 0) {
+      pr.tile0 = tbase + tincl - ntiles;
       // the tile records (beyond the tile capacity the step fails with
       // ECAPACITY and the node sweep does not run)
       for (int k = 0; k < ntiles; ++k) {
         if (pr.tile0 + k < P.max_tiles) {
-          W.tile_pair[pr.tile0 + k] = pi;
           store_pair_rec(W.tiles + pr.tile0 + k, pr, k);
         } else {
           set_error(W.err, kErrCapacity);
         }
       }
     }
+  }
+  // the step's node evaluations and nominal lane-ops, one atomic each per block
+  // (warp sums in 32 bits where they fit)
+  if (__all_sync(kFull, vol_sum < (1u << 26) && ops_sum < (1u << 26))) {
+    vol_sum = __reduce_add_sync(kFull, static_cast<unsigned>(vol_sum));
+    ops_sum = __reduce_add_sync(kFull, static_cast<unsigned>(ops_sum));
+  } else {
+#pragma unroll
+    for (int d = 16; d > 0; d >>= 1) {
+      vol_sum += __shfl_xor_sync(kFull, vol_sum, d);
+      ops_sum += __shfl_xor_sync(kFull, ops_sum, d);
+    }
+  }
+  if (lane == 0 && vol_sum > 0) {
+    atomicAdd(&W.u64[0], vol_sum);
+    atomicAdd(&W.u64[1], ops_sum);
   }
 }
 
@@ -988,11 +1005,12 @@ void launch_broad(const Params& P, const Parts& D, const Lists& W, cudaStream_t 
   if (nb > 0) launch_pdl(k_broad, dim3(nb), dim3(warps * 32), smem, st, P, D, W);
 }
 
-void launch_plan(const Params& P, const Shapes& S, const Parts& D, const Lists& W, int32_t* pair_ij, int32_t* n_pairs,
+void launch_plan(const Params& P, const Parts& D, const Lists& W, int32_t* pair_ij, int32_t* n_pairs,
                  double* pair_out, cudaStream_t st) {
-  const int nb = (P.n + kBuildWarps - 1) / kBuildWarps;   // one particle row per warp
-  launch_pdl(P.box_mode == 1 ? k_build_pairs<true> : k_build_pairs<false>, dim3(nb > 0 ? nb : 1),
-             dim3(kBuildWarps * 32), 0, st, P, S, D, W, pair_ij, n_pairs, pair_out);
+  const int rows = build_rows(P);
+  const int nb = (P.n + rows - 1) / rows;
+  launch_pdl(P.box_mode == 1 ? k_build_pairs<true> : k_build_pairs<false>, dim3(nb > 0 ? nb : 1), dim3(32), 0, st, P, D,
+             W, rows, pair_ij, n_pairs, pair_out);
 }
 
 }  // namespace gbc

@@ -833,26 +833,22 @@ __device__ __forceinline__ void flush_overlaps(const Params& P, const Shapes& S,
 
 // End of a pair (called by the whole warp once all its nodes are summed):
 // lanes c < 7 hold the FP64 sum of component c, every lane the deepest node.
-// A pair without overlap gets its zero outputs; an overlapping pair's sums go
-// to its entry of the overlap list, flagged for the force law (the next
-// kernel gathers the flagged entries, eight pairs per warp pass).
-__device__ __forceinline__ void pair_done(const Params& P, const Lists& W, const PairRec& r, double* pair_out,
-                                          double sv, int idx) {
+// A pair without overlap keeps the zero outputs of the pair builder; an
+// overlapping pair's sums go to its entry of the overlap list, flagged for the
+// force law (the next kernel gathers the flagged entries, eight pairs per warp
+// pass).
+__device__ __forceinline__ void pair_done(const Lists& W, const PairRec& r, double sv, int idx) {
   const int lane = threadIdx.x & 31;
   const int q = r.pair;
   const double s0 = __shfl_sync(kFull, sv, 0);
   const bool hit = __double_as_longlong(s0) > 0;   // V > 0
-  if (lane == 31) W.oflag[q] = hit ? 1 : 0;
   if (hit) {
+    if (lane == 31) W.oflag[q] = 1;
     OvlRec* e = W.olist + q;
     if (lane < 7) e->s[lane] = sv;
     if (lane == 7) e->q = q;
     if (lane == 8) e->idx = idx;
     if (lane >= 9 && lane < 20) (&e->i)[lane - 9] = reinterpret_cast<const int*>(&r)[lane - 9];   // i, j, lo, dim, shift
-  } else {
-    if (lane < 11) pair_out[static_cast<size_t>(q) * 11 + lane] = 0.0;
-    if (lane < kFtDoubles) W.ft[static_cast<size_t>(q) * kFtDoubles + lane] = 0.0;
-    if (lane < kTapeDoubles) W.tape[static_cast<size_t>(q) * kTapeDoubles + lane] = 0.0;
   }
 }
 
@@ -861,13 +857,12 @@ __device__ __forceinline__ void pair_done(const Params& P, const Lists& W, const
 // pair's last tile sums all of them in FP64 in a fixed order (4 tile slots x
 // 8 components per lane pattern, slots combined pairwise), whichever warp
 // that is.
-__device__ __forceinline__ void tile_done(const Params& P, const Lists& W, const PairRec& r, double* pair_out,
-                                          float v) {
+__device__ __forceinline__ void tile_done(const Lists& W, const PairRec& r, float v) {
   const int lane = threadIdx.x & 31;
   if (r.ntiles == 1) {
     const int idx = __shfl_sync(kFull, __float_as_int(v), 8);
     // (the hardware conversion: one issue slot on the node sweep's otherwise idle FP64 pipe)
-    pair_done(P, W, r, pair_out, lane < 7 ? static_cast<double>(v) : 0.0, idx);
+    pair_done(W, r, lane < 7 ? static_cast<double>(v) : 0.0, idx);
     return;
   }
   const size_t t0 = static_cast<size_t>(r.tile0);
@@ -914,7 +909,7 @@ __device__ __forceinline__ void tile_done(const Params& P, const Lists& W, const
     if (ob > bf || (ob == bf && oi < bi)) { bf = ob; bi = oi; }
   }
   if (lane == 0) W.pdone[r.pair] = 0;   // ready for a repeated sweep of the same tiles
-  pair_done(P, W, r, pair_out, acc, __shfl_sync(kFull, bi, 7));
+  pair_done(W, r, acc, __shfl_sync(kFull, bi, 7));
 }
 
 // Kernel variants: the full set of pair kinds, or spheres and cuboids only
@@ -997,9 +992,7 @@ __host__ __device__ constexpr int narrow_blocks() { return SET == SET_ALL ? 2 : 
 
 template <bool SMOOTH, int SET>
 __global__ void __launch_bounds__(narrow_warps<SET>() * 32, narrow_blocks<SET>()) k_narrow32(Params P, Shapes S,
-                                                                                             Parts D, Lists W,
-                                                                                             const double* vel,
-                                                                                             double* pair_out) {
+                                                                                             Parts D, Lists W) {
   constexpr int NW = narrow_warps<SET>();
   __shared__ __align__(16) PairRec s_rec[NW][2];
   // per evaluator: a polytope's planes, then its line clip's constants (a cube: the clip constants)
@@ -1025,7 +1018,7 @@ __global__ void __launch_bounds__(narrow_warps<SET>() * 32, narrow_blocks<SET>()
     if (record_in_bounds(P, W.err, r, true)) {
       const Partial o = dispatch<SMOOTH, SET>(P, S, D, r, r.tile, s_planes[wid][0], s_planes[wid][1],
                                               s_pk[SET == SET_ALL ? wid : 0], s_own[wid]);
-      tile_done(P, W, r, pair_out, o.touched ? reduce_tile<SMOOTH>(o) : empty_partial());
+      tile_done(W, r, o.touched ? reduce_tile<SMOOTH>(o) : empty_partial());
     }
     __syncwarp();
     if (tn < ntiles) store_rec_part(&s_rec[wid][buf ^ 1], lane, next);
@@ -1033,7 +1026,6 @@ __global__ void __launch_bounds__(narrow_warps<SET>() * 32, narrow_blocks<SET>()
     buf ^= 1;
     t = tn;
   }
-  (void)vel;   // the velocities enter with the force law (next kernel)
 }
 
 // The force law of the step's overlapping pairs, up to eight per warp pass
@@ -1163,11 +1155,10 @@ __device__ __forceinline__ double warp_sum8(const double v[8]) {
 
 // After a tile of the FP64 form (lane c < 7: component c of its sums; key, idx:
 // the deepest node on every lane): as tile_done, with FP64 partials.
-__device__ __forceinline__ void tile_done64(const Params& P, const Lists& W, const PairRec& r, double* pair_out,
-                                            double v, long long key, int idx) {
+__device__ __forceinline__ void tile_done64(const Lists& W, const PairRec& r, double v, long long key, int idx) {
   const int lane = threadIdx.x & 31;
   if (r.ntiles == 1) {
-    pair_done(P, W, r, pair_out, lane < 7 ? v : 0.0, idx);
+    pair_done(W, r, lane < 7 ? v : 0.0, idx);
     return;
   }
   const size_t t0 = static_cast<size_t>(r.tile0);
@@ -1211,17 +1202,15 @@ __device__ __forceinline__ void tile_done64(const Params& P, const Lists& W, con
     }
   }
   if (lane == 0) W.pdone[r.pair] = 0;   // ready for a repeated sweep of the same tiles
-  pair_done(P, W, r, pair_out, acc, __shfl_sync(kFull, bi, 7));
+  pair_done(W, r, acc, __shfl_sync(kFull, bi, 7));
 }
 
 template <bool SMOOTH>
-__global__ void __launch_bounds__(kWarps * 32, 2) k_narrow64(Params P, Shapes S, Parts D, Lists W, const double* vel,
-                                                             double* pair_out) {
+__global__ void __launch_bounds__(kWarps * 32, 2) k_narrow64(Params P, Shapes S, Parts D, Lists W) {
   __shared__ __align__(16) PairRec s_rec[kWarps];
   __shared__ float4 s_planes[kWarps][2][kMaxFaces];
   __shared__ unsigned s_pk[kWarps][kTileItemsPerLane * 32];   // clipped ranges: first node | count << 16
   __shared__ int s_excl[kWarps][32];                          // nodes before each lane's
-  (void)vel;
   pdl_begin();
   const int ntiles = W.counters[1];
   if (ntiles > P.max_tiles) return;   // capacity exceeded: the step reports ECAPACITY
@@ -1351,7 +1340,7 @@ __global__ void __launch_bounds__(kWarps * 32, 2) k_narrow64(Params P, Shapes S,
         }
       }
     }
-    tile_done64(P, W, r, pair_out, v, bk, bi);
+    tile_done64(W, r, v, bk, bi);
   }
 }
 
@@ -1401,20 +1390,20 @@ void launch_narrow(const Params& P, const Shapes& S, const Parts& D, const Lists
   }
   if (P.precision == 1) {
     if (P.smooth)
-      launch_pdl(k_narrow64<true>, dim3(grid), dim3(kWarps * 32), 0, st, P, S, D, W, vel, pair_out);
+      launch_pdl(k_narrow64<true>, dim3(grid), dim3(kWarps * 32), 0, st, P, S, D, W);
     else
-      launch_pdl(k_narrow64<false>, dim3(grid), dim3(kWarps * 32), 0, st, P, S, D, W, vel, pair_out);
+      launch_pdl(k_narrow64<false>, dim3(grid), dim3(kWarps * 32), 0, st, P, S, D, W);
     return;
   }
   const dim3 bc(narrow_warps<SET_CUBE>() * 32), bs(narrow_warps<SET_SC>() * 32), ba(narrow_warps<SET_ALL>() * 32);
   if (P.smooth) {
-    if (P.kind_set == SET_CUBE) launch_pdl(k_narrow32<true, SET_CUBE>, dim3(grid), bc, 0, st, P, S, D, W, vel, pair_out);
-    else if (P.kind_set == SET_SC) launch_pdl(k_narrow32<true, SET_SC>, dim3(grid), bs, 0, st, P, S, D, W, vel, pair_out);
-    else launch_pdl(k_narrow32<true, SET_ALL>, dim3(grid), ba, 0, st, P, S, D, W, vel, pair_out);
+    if (P.kind_set == SET_CUBE) launch_pdl(k_narrow32<true, SET_CUBE>, dim3(grid), bc, 0, st, P, S, D, W);
+    else if (P.kind_set == SET_SC) launch_pdl(k_narrow32<true, SET_SC>, dim3(grid), bs, 0, st, P, S, D, W);
+    else launch_pdl(k_narrow32<true, SET_ALL>, dim3(grid), ba, 0, st, P, S, D, W);
   } else {
-    if (P.kind_set == SET_CUBE) launch_pdl(k_narrow32<false, SET_CUBE>, dim3(grid), bc, 0, st, P, S, D, W, vel, pair_out);
-    else if (P.kind_set == SET_SC) launch_pdl(k_narrow32<false, SET_SC>, dim3(grid), bs, 0, st, P, S, D, W, vel, pair_out);
-    else launch_pdl(k_narrow32<false, SET_ALL>, dim3(grid), ba, 0, st, P, S, D, W, vel, pair_out);
+    if (P.kind_set == SET_CUBE) launch_pdl(k_narrow32<false, SET_CUBE>, dim3(grid), bc, 0, st, P, S, D, W);
+    else if (P.kind_set == SET_SC) launch_pdl(k_narrow32<false, SET_SC>, dim3(grid), bs, 0, st, P, S, D, W);
+    else launch_pdl(k_narrow32<false, SET_ALL>, dim3(grid), ba, 0, st, P, S, D, W);
   }
 }
 

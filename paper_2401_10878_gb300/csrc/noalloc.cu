@@ -252,10 +252,8 @@ extern "C" contact_status contact_step_noalloc(const contact_config* cfg, const 
   W.dn_pair = cv.take<int>(N * kMaxNbr);
   W.row_off = cv.take<int>(N + 1);
   W.grp_sum = cv.take<int>((N + kRowGroup - 1) / kRowGroup);
-  W.pairs = cv.take<PairRec>(MP);
   W.olist = cv.take<OvlRec>(MP);
   W.oflag = cv.take<int>(MP);
-  W.tile_pair = cv.take<int>(MT);
   W.tiles = cv.take<PairRec>(MT);
   W.partial = cv.take<float>(MT * kPartialFloats);
   W.pdone = cv.take<int>(MP);
@@ -281,7 +279,7 @@ extern "C" contact_status contact_step_noalloc(const contact_config* cfg, const 
   // the step's kernels, unchanged, on the scratch array
   launch_pose(P, S, D, W, pos, quat, s);
   launch_broad(P, D, W, s);
-  launch_plan(P, S, D, W, pair_ij, n_pairs, pair_out, s);
+  launch_plan(P, D, W, pair_ij, n_pairs, pair_out, s);
   launch_narrow(P, S, D, W, nullptr, pair_out, narrow_grid(P), s);
   launch_force(P, S, D, W, nullptr, pair_out, s);
   launch_particle_sum(P, D, W, force, torque, s);

@@ -39,3 +39,33 @@ def test_fp64_form_at_tile_edges(across, indicator, kind):
                indicator=indicator)
     rep, ref = _parity(st, 1)
     assert ref.n_pairs == 1 and ref.pair_out[0, 0] > 100.0
+
+
+def _crowd(n_small):
+    """A ball and n_small small ones around it: the first row holds n_small partners."""
+    k = np.arange(n_small) + 0.5
+    th, ph = np.arccos(1.0 - 2.0 * k / n_small), np.pi * (1.0 + 5.0 ** 0.5) * k
+    u = np.stack([np.sin(th) * np.cos(ph), np.sin(th) * np.sin(ph), np.cos(th)], 1)
+    c = np.array([31.13, 32.21, 30.87])
+    return state([W.SPHERE] * (n_small + 1), [[9.0, 0, 0]] + [[1.6, 0, 0]] * n_small,
+                 np.concatenate([c[None], c + u * 9.5]), n=64)
+
+
+# partners of one row: at and around the eight fetched ahead, and more than one warp round of pairs
+@pytest.mark.parametrize("n_small", [1, 7, 8, 9, 31, 33, 60])
+def test_pair_builder_rows(n_small):
+    st = _crowd(n_small)
+    rep, ref = _parity(st, 0)
+    assert np.sum(ref.pair_ij[:, 0] == 0) == n_small
+
+
+# node ranges whose length the ten bits of a bin entry hold, and ones they do not
+@pytest.mark.parametrize("half", [505.3, 511.3, 530.3])
+@pytest.mark.parametrize("gap", [7.1, 8.1])
+def test_broad_phase_long_ranges(half, gap):
+    """Axis-aligned rods across the periodic boundary, overlapping (7.1) or with ranges one node apart (8.1)."""
+    n = int(4 * half) + 60
+    st = state([W.CUBOID] * 3, [[half, 4.3, 4.2]] * 3,
+               [[5.2, 20.3, 40.4], [n - 300.3, 20.3 + gap, 41.7], [n / 2 + 3.3, 90.0, 40.1]], n=n)
+    rep, ref = _parity(st, 0)
+    assert ref.n_pairs == (1 if gap < 8.0 else 0) and np.all(ref.pair_out[:, 0] > 0)
