@@ -267,6 +267,21 @@ struct OvlRec {
 };
 static_assert(sizeof(OvlRec) == 128, "one overlap record per 128-byte line");
 
+// The box pipeline's pair: its corrected box (physical) and the sample spacing.
+// Its overlap record then holds sums over sample indices: idx is the deepest
+// sample, dim the samples per axis.
+struct BoxGeom {
+  double lo[3], hi[3], step[3];
+};
+
+// One pair with a rough contact, passed from kernel to kernel.
+struct __align__(16) BoxWork {
+  int t, bounds[6], pad0;   // entry of the tile list, rough box (nodes): lower, upper
+  BoxGeom box;              // the corrected box
+  double pad1;
+};
+static_assert(sizeof(BoxWork) % 16 == 0, "consecutive records stay aligned");
+
 struct Lists {
   int* bin_count;   // [nbins]
   int* bin_items;   // [nbins, bin_stride] particles of each bin, in arrival order
@@ -293,7 +308,8 @@ struct Lists {
   double* tape;     // [max_pairs, kTapeDoubles]
   double* ft;       // [max_pairs, kFtDoubles]
   const int* kind;  // [N] sweep kind of each particle (Kind, polytopes by face bucket)
-  int* counters;    // [16]: 0 pairs, 1 tiles, 2 box pipeline queue, 5 overlapping pairs, kStepCounter
+  BoxWork* box_work;   // [max_pairs] box pipeline: the pairs with a rough contact
+  int* counters;    // [16]: 0 pairs, 1 tiles, 2 box pipeline rough contacts, 5 overlapping pairs, kStepCounter
                     // steps completed (its parity selects the contact-history buffer)
   unsigned long long* u64;  // [4]: 0 node evaluations, 1 nominal lane-ops of the node sweep
   int* err;         // [1] sticky device error

@@ -39,6 +39,8 @@ struct ForceArgs {
   int* hn_wr;
   int* hj_wr;
   double* hc_wr;
+  double* hb_wr;                    // box pipeline: this step's corrected boxes (relative to X_i)
+  double gbox;                      // box pipeline: G of a cell = gbox * its volume * the band sum
   double damp_K;                    // c = damp_K / u0 for a contact's first step
   double mu_s_star, mu_k, inv_u_k;  // friction law of Eq. (contact_force_tangential)
 };
@@ -113,20 +115,48 @@ __device__ __forceinline__ double shape_value(int type, double prm0, double prmk
 
 }  // namespace fl
 
+__device__ __forceinline__ ForceArgs force_args(const Params& P, const Shapes& S, const Parts& D, const Lists& W,
+                                                const double* vel, double* pair_out) {
+  ForceArgs a;
+  a.X = D.X; a.R = D.R;
+  a.type = S.type; a.param = S.param; a.face_off = S.face_off; a.planes = S.planes; a.compl_ = S.compl_;
+  a.vel = vel; a.pair_out = pair_out; a.ft = W.ft; a.tape = W.tape;
+  for (int k = 0; k < 3; ++k) a.L[k] = P.L[k];
+  a.dx = P.dx; a.dx3 = P.dx3; a.gscale = P.gscale; a.g_min2 = P.g_min2; a.inflate = P.inflate;
+  a.damping_c = P.damping_c;
+  a.history = P.history; a.friction = P.friction; a.hist_cap = P.max_nbr;
+  a.n = P.n; a.rest6 = D.rest6;
+  a.damp_K = P.damp_K; a.mu_s_star = P.mu_s_star; a.mu_k = P.mu_k; a.inv_u_k = P.inv_u_k;
+  if (P.history) {   // buffer (steps & 1) holds the previous step's contacts
+    const int rd = W.counters[kStepCounter] & 1;
+    const size_t nn = static_cast<size_t>(P.n);
+    a.hn_rd = W.hist_n + rd * nn; a.hn_wr = W.hist_n + (rd ^ 1) * nn;
+    a.hj_rd = W.hist_j + rd * nn * P.max_nbr; a.hj_wr = W.hist_j + (rd ^ 1) * nn * P.max_nbr;
+    a.hc_rd = W.hist_c + rd * nn * P.max_nbr; a.hc_wr = W.hist_c + (rd ^ 1) * nn * P.max_nbr;
+  } else {
+    a.hn_rd = a.hj_rd = nullptr; a.hc_rd = nullptr; a.hn_wr = a.hj_wr = nullptr; a.hc_wr = nullptr;
+  }
+  a.hb_wr = nullptr;
+  a.gbox = 0.0;
+  return a;
+}
+
 constexpr int kForcePairsPerPass = 8;   // pairs one call handles (four lanes each)
 
-// The whole warp calls this for the n <= 8 pairs e[0..n) (shared memory).
+// The whole warp calls this for the n <= 8 pairs e[0..n), in the box pipeline
+// (BOX) with their boxes bx[0..n) (shared memory).
 // SET: the context's kind set (as shape_value).  LAW: false when the step has
 // no contact history, no friction and no velocity-driven damping (the
 // relative-velocity, history and friction code is then compiled out).
-template <int SET, bool LAW>
-__device__ __forceinline__ void pair_force_law(ForceArgs a, const OvlRec* e, int n) {
+template <int SET, bool LAW, bool BOX = false>
+__device__ __forceinline__ void pair_force_law(ForceArgs a, const OvlRec* e, int n, const BoxGeom* bx = nullptr) {
   using namespace fl;
   const int lane = threadIdx.x & 31;
   const int slot = lane >> 2, k = lane & 3, kc = k < 3 ? k : 0, b0 = lane & ~3;
   {
     const bool act = slot < n;
-    const OvlRec& er = e[act ? slot : 0];
+    const int at = act ? slot : 0;
+    const OvlRec& er = e[at];
     const int q = er.q;
     const int i = er.i, j = er.j;
     const int lok = er.lo[kc], d0 = er.dim[0], d1 = er.dim[1], d2 = er.dim[2], sh = er.shift[kc];
@@ -147,8 +177,16 @@ __device__ __forceinline__ void pair_force_law(ForceArgs a, const OvlRec* e, int
     const double Lsel = sh == 0 ? 0.0 : (sh > 0 ? Lk : -Lk);
     const double XB = Xj - Lsel;   // X_j - s L, s in {-1, 0, 1}
     const double s0 = sm[0];
-    const double V = a.dx3 * s0;
-    const double Gk = a.gscale * sm[4 + kc];
+    // a sample's volume and the scale of G: a node's dx^3, or in the box pipeline a cell of the corrected box
+    double blo = 0.0, bst = 0.0, cell = a.dx3, gscale = a.gscale;
+    if constexpr (BOX) {
+      blo = bx[at].lo[kc];
+      bst = bx[at].step[kc];
+      cell = bx[at].step[0] * bx[at].step[1] * bx[at].step[2];
+      gscale = a.gbox * cell;
+    }
+    const double V = cell * s0;
+    const double Gk = gscale * sm[4 + kc];
     const double G0 = __shfl_sync(kFull, Gk, b0), G1 = __shfl_sync(kFull, Gk, b0 + 1),
                    G2 = __shfl_sync(kFull, Gk, b0 + 2);
     const double gn2 = fma(G2, G2, fma(G1, G1, G0 * G0));
@@ -156,7 +194,7 @@ __device__ __forceinline__ void pair_force_law(ForceArgs a, const OvlRec* e, int
     // indentation depth: FP64 re-evaluation at the deepest node
     const int idx = min(max(er.idx, 0), d0 * d1 * d2 - 1);
     const int ck = kc == 0 ? idx % d0 : (kc == 1 ? (idx / d0) % d1 : idx / (d0 * d1));
-    const double xk = int_to_double(lok + ck) * a.dx;
+    const double xk = BOX ? fma(int_to_double(ck) + 0.5, bst, blo) : int_to_double(lok + ck) * a.dx;
     const double rAk = xk - XA, rBk = xk - XB;
     double rA[3], rB[3], yA[3], yB[3];
 #pragma unroll
@@ -188,7 +226,8 @@ __device__ __forceinline__ void pair_force_law(ForceArgs a, const OvlRec* e, int
                    y2 = __shfl_sync(kFull, y, b0 + 2), y3 = __shfl_sync(kFull, y, b0 + 3);
     const double inv_s0 = y0 * y0;
     const double estar = y1 * y1;
-    const double xck = fma(sm[1 + kc], inv_s0, int_to_double(lok)) * a.dx;
+    const double xck = BOX ? fma(fma(sm[1 + kc], inv_s0, 0.5), bst, blo)
+                           : fma(sm[1 + kc], inv_s0, int_to_double(lok)) * a.dx;
     double nk = Gk * y2;
     double fallback = 0.0;
     if (__any_sync(kFull, act && !gok)) {   // centre-line fallback normal (a wall: -m)
@@ -298,20 +337,33 @@ __device__ __forceinline__ void pair_force_law(ForceArgs a, const OvlRec* e, int
       if (k < 3) {
         o[1 + k] = xck; o[4 + k] = nk; o[8 + k] = Fk;
         f[k] = Fk; f[3 + k] = TAk; f[6 + k] = TBk;
-        tp[1 + k] = xck; tp[4 + k] = nk;
+        if (!BOX) {
+          tp[1 + k] = xck; tp[4 + k] = nk;
+        }
       }
       if (k == 0) {
         o[0] = V; o[7] = d;
-        tp[0] = s0; tp[7] = d; tp[8] = gn; tp[9] = fallback;
-      } else if (k == 3) {
+        if (!BOX) {
+          tp[0] = s0; tp[7] = d; tp[8] = gn; tp[9] = fallback;
+        }
+      } else if (k == 3 && !BOX) {
         tp[10] = estar; tp[11] = damp; tp[12] = fmag; tp[13] = int_to_double(idx);
         tp[14] = cdamp; tp[15] = 0.0;
       }
-      if (LAW && a.history && k == 0) {   // this step's contact list of i
-        const int slot = atomicAdd(a.hn_wr + i, 1);
-        if (slot < a.hist_cap) {
-          a.hj_wr[static_cast<size_t>(i) * a.hist_cap + slot] = j;
-          a.hc_wr[static_cast<size_t>(i) * a.hist_cap + slot] = cdamp;
+    }
+    if (LAW && a.history) {   // this step's contact list of i
+      int hs = -1;
+      if (act && k == 0) hs = atomicAdd(a.hn_wr + i, 1);
+      if constexpr (BOX) hs = __shfl_sync(kFull, hs, b0);
+      const size_t he = static_cast<size_t>(i) * a.hist_cap + (hs < 0 ? 0 : hs);
+      if (hs >= 0 && hs < a.hist_cap) {
+        if (k == 0) {
+          a.hj_wr[he] = j;
+          a.hc_wr[he] = cdamp;
+        }
+        if (BOX && k < 3) {   // the corrected box minus X_i: the next step's warm start
+          a.hb_wr[6 * he + k] = __dsub_rn(blo, XA);
+          a.hb_wr[6 * he + 3 + k] = __dsub_rn(bx[at].hi[k], XA);
         }
       }
     }

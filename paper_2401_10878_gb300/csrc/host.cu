@@ -645,6 +645,7 @@ contact_status contact_init(const contact_config* cfg, const int32_t* shape_type
   }
   GBC_TRY(dev_alloc(c, &W.olist, mp));
   GBC_TRY(dev_alloc(c, &W.oflag, mp));
+  if (C.box_mode == 1) GBC_TRY(dev_alloc(c, &W.box_work, mp));
   GBC_TRY(dev_alloc(c, &W.tiles, mt));
   GBC_TRY(dev_alloc(c, &W.partial, mt * kPartialFloats));
   if (C.precision == 1 && C.box_mode == 0) GBC_TRY(dev_alloc(c, &W.partial64, mt * kPartialDoubles));
@@ -922,7 +923,8 @@ contact_status contact_history_reset(contact_ctx* c) {
 
 int32_t contact_kernels_per_step(const contact_ctx* c) {
   if (c == nullptr) return 0;
-  return 5 + (c->P.npoly > 0 ? 1 : 0) + (c->P.box_mode == 0 ? 1 : 0);   // + polytope pose, + force law
+  // + polytope pose; node sweep and force law, or the box pipeline's three kernels
+  return (c->P.box_mode == 0 ? 6 : 7) + (c->P.npoly > 0 ? 1 : 0);
 }
 int32_t contact_kernels_per_backward(const contact_ctx*) { return 3; }
 

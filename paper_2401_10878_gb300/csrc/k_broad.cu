@@ -54,7 +54,7 @@ __global__ void k_pose(Params P, Shapes S, Parts D, Lists W, const double* __res
   if (t == 0) {
     W.counters[0] = 0;   // pairs (written by the pair builder)
     W.counters[1] = 0;   // tiles allocated
-    W.counters[2] = 0;   // box pipeline queue head
+    W.counters[2] = 0;   // box pipeline: pairs with a rough contact
     W.counters[5] = 0;   // pairs with V > 0
     W.u64[0] = 0;        // node evaluations
     W.u64[1] = 0;        // nominal lane-ops

@@ -10,6 +10,8 @@ import oracle
 from paper_2401_10878_gb300 import workloads as W
 from tests.helpers import cube_planes, quat_axis_angle, state
 from tests.parity import compare, gpu_step
+from tests.test_gpu_box_pipeline import boxed
+from tests.test_gpu_box_pipeline import run as run_box
 
 torch = pytest.importorskip("torch")
 pytestmark = pytest.mark.gpu
@@ -69,3 +71,25 @@ def test_broad_phase_long_ranges(half, gap):
                [[5.2, 20.3, 40.4], [n - 300.3, 20.3 + gap, 41.7], [n / 2 + 3.3, 90.0, 40.1]], n=n)
     rep, ref = _parity(st, 0)
     assert ref.n_pairs == (1 if gap < 8.0 else 0) and np.all(ref.pair_out[:, 0] > 0)
+
+
+# one line and sample per direction up to the most, around the 32 lanes of a warp
+@pytest.mark.parametrize("nc", [1, 2, 5, 6, 7, 33])
+@pytest.mark.parametrize("kinds", ["grid", "cubes_walls", "polytopes"])
+def test_box_pipeline_line_grids(nc, kinds):
+    """Spheres with cubes, cubes with walls (every line of a wall's face ties)
+    and polytopes, each kernel variant of the box pipeline."""
+    if kinds == "grid":
+        st = W.mixed_grid_27()
+    elif kinds == "cubes_walls":
+        st = W.floor_and_ceiling(state([W.CUBOID] * 3, [[6.0, 6.0, 6.0]] * 3,
+                                       [[20.3, 20.6, 20.2], [31.1, 20.9, 21.3], [44.4, 44.1, 43.7]],
+                                       quat=[[1.0, 0.0, 0.0, 0.0], quat_axis_angle([0.2, 1.0, 0.1], 0.3),
+                                             quat_axis_angle([1.0, 0.3, 0.5], 0.7)]), gap=4.0)
+    else:
+        rng = np.random.default_rng(5)
+        pl = [W.random_polytope(rng, 14, 9.0)[0] for _ in range(2)]
+        st = state([W.POLYTOPE] * 2, [[0, 0, 0]] * 2, [[25.2, 26.1, 25.7], [33.4, 29.3, 27.4]], n=64, planes=pl,
+                   quat=W.random_quaternions(rng, 2))
+    rep, ref = run_box(boxed(st, nc))
+    assert ref.n_pairs > 0
