@@ -33,6 +33,7 @@ __device__ __forceinline__ bool sweep_swap(int ka, int kb) {
 // rough-detection threshold (Sec. 3.3.1).
 constexpr float kRoughT = 0.8660254037844386f;
 
+constexpr int kSms = 152;             // SMs of the GPU (rules on how to split the work; any other count runs too)
 constexpr int kMaxFaces = 32;         // faces of one polytope
 constexpr int kTileItemsPerLane = 4;  // node lines per lane per tile
 constexpr int kPartialFloats = 12;    // FP32 partial sums per tile
@@ -142,7 +143,7 @@ struct __align__(128) PartRec {
   int lo[3];       // node range of the offset shape, lower ...
   int kind;        // sweep kind | nominal lane-ops of one signed-distance test << 8
   int hi[3];       // ... and upper corner
-  int bin;         // cell-list bin
+  int bin;         // cell-list bin: its coordinates, eight bits each
   int kX[3];       // nearest node of X / dx
   float sz0;       // size_l: lattice units incl. inflate (Shapes::size_l)
   float fX[3];     // X / dx - kX, in [-1/2, 1/2] (FP64 difference, rounded once)

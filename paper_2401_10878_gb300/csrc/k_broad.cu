@@ -15,17 +15,18 @@ namespace {
 
 constexpr unsigned kFull = 0xffffffffu;
 
-constexpr int kPosePerWarp = 10;   // particles of one pose warp (three lanes each, lanes 30 and 31 idle)
-
 // Enter particle p with the given node range into its bin's row (one lane).
+// bin: its coordinates, eight bits each.
 __device__ __forceinline__ void bin_insert(const Params& P, const Lists& W, int p, int bin, const int lo[3],
                                            const int hi[3]) {
-  const int slot = atomicAdd(&W.bin_count[bin], 1);
+  const int b = checked_index(W.err, (bin & 0xff) + P.nbin[0] * (((bin >> 8) & 0xff) + P.nbin[1] * (bin >> 16)),
+                              static_cast<long long>(P.nbin[0]) * P.nbin[1] * P.nbin[2], 0);
+  const int slot = atomicAdd(&W.bin_count[b], 1);
   if (slot >= P.bin_cap) {
     set_error(W.err, kErrCapacity);
     return;
   }
-  const size_t at = static_cast<size_t>(bin) * P.bin_stride + slot;
+  const size_t at = static_cast<size_t>(b) * P.bin_stride + slot;
   const bool empty = hi[0] < lo[0] || hi[1] < lo[1] || hi[2] < lo[2];
   unsigned len = 0;
 #pragma unroll
@@ -35,16 +36,21 @@ __device__ __forceinline__ void bin_insert(const Params& P, const Lists& W, int 
 }
 
 // ---------------------------------------------------------------------------
-// K1: three lanes per particle (lane k: axis k), ten particles per warp: row k
-// of the rotation, the node range along k and the FP32 sweep geometry; lane 0
-// enters the particle into its bin.  Bound: the FP64 pipe (64 cycles a warp
-// instruction).  FP64 is kept to what the bit-exact node range needs, the same
-// instruction for the three rows (a branch per row ran all three in turn), and
-// conversions, roundings and comparisons are integer operations: 29.8 -> 22.9 us
-// on 52218 cubes.
+// K1: rotation, node range and FP32 sweep geometry of every particle, and its
+// bin entry.  ROWS = 1: three lanes per particle (lane k: axis k), ten particles
+// per warp; ROWS = 3: one lane per particle.  Bound: the FP64 pipe (64 cycles a
+// warp instruction).  FP64 is kept to what the bit-exact node range needs, the
+// same instruction for the three rows (a branch per row ran all three in turn),
+// and conversions, roundings and comparisons are integer operations.  Three
+// lanes give the shorter chain while every warp has a sub-partition to itself;
+// above that (6080 particles) what is common to the three rows is done once for
+// 32 particles instead of ten: 52218 cubes 29.8 -> 22.9 us with three lanes,
+// 17.7 us with one.
+template <int ROWS>
 __global__ void k_pose(Params P, Shapes S, Parts D, Lists W, const double* __restrict__ pos,
                        const double* __restrict__ quat) {
-  __shared__ __align__(16) int s_rec[kPosePerWarp][4 * kPartRecParts];
+  constexpr int kPer = ROWS == 1 ? 10 : 32;   // particles of one warp
+  __shared__ __align__(16) int s_rec[kPer][4 * kPartRecParts];
   pdl_begin();
   const int lane = threadIdx.x;   // one-warp blocks
   const int t = blockIdx.x * 32 + lane;
@@ -62,17 +68,17 @@ __global__ void k_pose(Params P, Shapes S, Parts D, Lists W, const double* __res
   if (t < (P.n + kRowGroup - 1) / kRowGroup) W.grp_sum[t] = 0;
   // contact history: this step's lists (the buffer not read) start empty
   if (P.history && t < P.n) W.hist_n[static_cast<size_t>(((W.counters[kStepCounter] & 1) ^ 1)) * P.n + t] = 0;
-  const int g = min(lane / 3, kPosePerWarp - 1), k = lane - 3 * g;   // (lanes 30, 31: k = 3, 4, no stores)
-  const int p_ = blockIdx.x * kPosePerWarp + g;
-  const bool act = k < 3 && p_ < P.n;
-  const int p = min(p_, P.n - 1), kc = k < 3 ? k : 0;
-  const int k1 = kc == 2 ? 0 : kc + 1;
+  const int g = ROWS == 1 ? min(lane / 3, kPer - 1) : lane;   // the particle's place in the warp
+  const int k0 = ROWS == 1 ? lane - 3 * g : 0;                // (lanes 30, 31: k = 3, 4, no stores)
+  const int p_ = blockIdx.x * kPer + g;
+  const bool act = k0 < 3 && p_ < P.n;
+  const int p = min(p_, P.n - 1);
   double q[4];
 #pragma unroll
   for (int c = 0; c < 4; ++c) q[c] = quat[4 * p + c];
   // position check by bit patterns: 0 <= X < L (NaN and negatives fail; -0.0 counts as 0)
   bool bad = false;
-  double Xk = 0.0;
+  double X[3];
 #pragma unroll
   for (int c = 0; c < 3; ++c) {
     const double v = pos[3 * p + c];
@@ -80,7 +86,7 @@ __global__ void k_pose(Params P, Shapes S, Parts D, Lists W, const double* __res
     if (b == static_cast<long long>(0x8000000000000000ULL)) b = 0;
     const bool ok = b >= 0 && b < __double_as_longlong(P.L[c]);
     bad = bad || !ok;
-    if (c == kc) Xk = ok ? __longlong_as_double(b) : 0.0;
+    X[c] = ok ? __longlong_as_double(b) : 0.0;
   }
   const double nn = dadd(dadd(dadd(dmul(q[0], q[0]), dmul(q[1], q[1])), dmul(q[2], q[2])), dmul(q[3], q[3]));
   // 1e-24 < nn < 1e300 (nn >= 0 or NaN: its bits order as its values, a NaN's above every number's)
@@ -88,69 +94,85 @@ __global__ void k_pose(Params P, Shapes S, Parts D, Lists W, const double* __res
     bad = true;
     q[0] = 1.0; q[1] = q[2] = q[3] = 0.0;
   }
-  if (bad && act && k == 0) set_error(W.err, kErrInval);
+  if (bad && act && k0 == 0) set_error(W.err, kErrInval);
   const double s = bad ? 2.0 : dmul(2.0, __drcp_rn(nn));
-  // row k of the rotation (rotation_row_rn with the row's cyclic axes k, k1, k2):
-  // 1 - s (q_k1^2 + q_k2^2), s (q_k q_k1 - w q_k2), s (q_k q_k2 + w q_k1)
-  const double qk = kc == 0 ? q[1] : (kc == 1 ? q[2] : q[3]);
-  const double qk1 = kc == 0 ? q[2] : (kc == 1 ? q[3] : q[1]);
-  const double qk2 = kc == 0 ? q[3] : (kc == 1 ? q[1] : q[2]);
-  const double rd = dsub(1.0, dmul(s, dadd(dmul(qk1, qk1), dmul(qk2, qk2))));
-  const double r1 = dmul(s, dsub(dmul(qk, qk1), dmul(q[0], qk2)));
-  const double r2 = dmul(s, dadd(dmul(qk, qk2), dmul(q[0], qk1)));
-  double r[3];   // by world column c
+  if (act && k0 == 0)
 #pragma unroll
-  for (int c = 0; c < 3; ++c) r[c] = c == kc ? rd : (c == k1 ? r1 : r2);
-  if (act) {
-    D.X[3 * p + k] = Xk;
-    if (k == 0)
-#pragma unroll
-      for (int c = 0; c < 4; ++c) D.qhat[4 * p + c] = q[c];   // raw quaternion of the step (adjoint tape)
-#pragma unroll
-    for (int c = 0; c < 3; ++c) D.R[9 * p + 3 * k + c] = r[c];
-  }
-  // extent along k of the offset shape {phi <= delta} (explicit rounding: compared bit for bit);
-  // a polytope's node range and bin entry come from its own warp (k_pose_poly)
+    for (int c = 0; c < 4; ++c) D.qhat[4 * p + c] = q[c];   // raw quaternion of the step (adjoint tape)
   const int type = S.type[p];
   const double* e = S.ext + 3 * p;
-  double ext = dadd(dadd(dmul(fabs(r[0]), e[0]), dmul(fabs(r[1]), e[1])), dmul(fabs(r[2]), e[2]));
-  if (type == 0) ext = e[0];
-  const double mn = dsub(Xk, ext), mx = dadd(Xk, ext);
-  const int lo = ceil_node(P.dx_pow2 ? dmul(mn, P.inv_dx) : __ddiv_rn(mn, P.dx));
-  const int hi = floor_node(P.dx_pow2 ? dmul(mx, P.inv_dx) : __ddiv_rn(mx, P.dx));
-  // nearest node of X / dx (round to even) by the 1.5 2^52 shift, and the remainder
-  const double xl = Xk * P.inv_dx;
-  const double sh = __dadd_rn(xl, 6755399441055744.0);
-  const int kx = __double2loint(sh);
-  const float fx = narrow(__dsub_rn(xl, __dsub_rn(sh, 6755399441055744.0)));
-  // cell-list bin
-  const int b = min(max(static_cast<int>(narrow(Xk) * P.inv_binw_f[kc]), 0), P.nbin[kc] - 1);
-  const int l0 = 3 * g;
-  const int b0 = __shfl_sync(kFull, b, l0), b1 = __shfl_sync(kFull, b, l0 + 1), b2 = __shfl_sync(kFull, b, l0 + 2);
-  const int los[3] = {__shfl_sync(kFull, lo, l0), __shfl_sync(kFull, lo, l0 + 1), __shfl_sync(kFull, lo, l0 + 2)};
-  const int his[3] = {__shfl_sync(kFull, hi, l0), __shfl_sync(kFull, hi, l0 + 1), __shfl_sync(kFull, hi, l0 + 2)};
-  const int bin = checked_index(W.err, b0 + P.nbin[0] * (b1 + P.nbin[1] * b2),
-                                static_cast<long long>(P.nbin[0]) * P.nbin[1] * P.nbin[2], 0);
-  if (act && k == 0 && type != 2) bin_insert(P, W, p, bin, los, his);
-  // the particle's line, staged so that the warp stores whole 16-byte pieces
-  if (act) {
-    int* w = s_rec[g];
-    w[k] = lo;
-    w[4 + k] = hi;
-    w[8 + k] = kx;
-    w[11 + 4 * k + (k == 2 ? 6 : 0)] = __float_as_int(S.size_l[3 * p + k]);   // words 11, 15, 25
-    w[12 + k] = __float_as_int(fx);
+  const double e0 = e[0], e1 = e[1], e2 = e[2];
+  int los[3], his[3], bins[3];
 #pragma unroll
-    for (int c = 0; c < 3; ++c) w[16 + 3 * c + k] = __float_as_int(narrow(r[c]));   // R^T row c, column k
-    if (k == 0) w[3] = W.kind[p] | (S.nomops[p] << 8);
-    if (k == 1) w[7] = bin;
-    if (k == 2) w[26] = w[27] = 0;
+  for (int row = 0; row < ROWS; ++row) {
+    const int k = ROWS == 1 ? (k0 < 3 ? k0 : 0) : row;
+    const int k1 = k == 2 ? 0 : k + 1;
+    const double Xk = k == 0 ? X[0] : (k == 1 ? X[1] : X[2]);
+    // row k of the rotation (rotation_row_rn with the row's cyclic axes k, k1, k2):
+    // 1 - s (q_k1^2 + q_k2^2), s (q_k q_k1 - w q_k2), s (q_k q_k2 + w q_k1)
+    const double qk = k == 0 ? q[1] : (k == 1 ? q[2] : q[3]);
+    const double qk1 = k == 0 ? q[2] : (k == 1 ? q[3] : q[1]);
+    const double qk2 = k == 0 ? q[3] : (k == 1 ? q[1] : q[2]);
+    const double rd = dsub(1.0, dmul(s, dadd(dmul(qk1, qk1), dmul(qk2, qk2))));
+    const double r1 = dmul(s, dsub(dmul(qk, qk1), dmul(q[0], qk2)));
+    const double r2 = dmul(s, dadd(dmul(qk, qk2), dmul(q[0], qk1)));
+    double r[3];   // by world column c
+#pragma unroll
+    for (int c = 0; c < 3; ++c) r[c] = c == k ? rd : (c == k1 ? r1 : r2);
+    // extent along k of the offset shape {phi <= delta} (explicit rounding: compared bit for bit);
+    // a polytope's node range and bin entry come from its own warp (k_pose_poly)
+    double ext = dadd(dadd(dmul(fabs(r[0]), e0), dmul(fabs(r[1]), e1)), dmul(fabs(r[2]), e2));
+    if (type == 0) ext = e0;
+    const double mn = dsub(Xk, ext), mx = dadd(Xk, ext);
+    const int lo = ceil_node(P.dx_pow2 ? dmul(mn, P.inv_dx) : __ddiv_rn(mn, P.dx));
+    const int hi = floor_node(P.dx_pow2 ? dmul(mx, P.inv_dx) : __ddiv_rn(mx, P.dx));
+    // nearest node of X / dx (round to even) by the 1.5 2^52 shift, and the remainder
+    const double xl = Xk * P.inv_dx;
+    const double sh = __dadd_rn(xl, 6755399441055744.0);
+    const int kx = __double2loint(sh);
+    const float fx = narrow(__dsub_rn(xl, __dsub_rn(sh, 6755399441055744.0)));
+    // cell-list bin
+    const int b = min(max(static_cast<int>(narrow(Xk) * P.inv_binw_f[k]), 0), P.nbin[k] - 1);
+    if (ROWS == 1) {
+#pragma unroll
+      for (int c = 0; c < 3; ++c) {
+        los[c] = __shfl_sync(kFull, lo, 3 * g + c);
+        his[c] = __shfl_sync(kFull, hi, 3 * g + c);
+        bins[c] = __shfl_sync(kFull, b, 3 * g + c);
+      }
+    } else {
+      los[row] = lo;
+      his[row] = hi;
+      bins[row] = b;
+    }
+    if (act) {
+      D.X[3 * p + k] = Xk;
+#pragma unroll
+      for (int c = 0; c < 3; ++c) D.R[9 * p + 3 * k + c] = r[c];
+      // the particle's line, staged so that the warp stores whole 16-byte pieces
+      int* w = s_rec[g];
+      w[k] = lo;
+      w[4 + k] = hi;
+      w[8 + k] = kx;
+      w[11 + 4 * k + (k == 2 ? 6 : 0)] = __float_as_int(S.size_l[3 * p + k]);   // words 11, 15, 25
+      w[12 + k] = __float_as_int(fx);
+#pragma unroll
+      for (int c = 0; c < 3; ++c) w[16 + 3 * c + k] = __float_as_int(narrow(r[c]));   // R^T row c, column k
+    }
+  }
+  if (act && k0 == 0) {
+    const int bin = bins[0] | (bins[1] << 8) | (bins[2] << 16);   // (at most 256 bins per axis)
+    int* w = s_rec[g];
+    w[3] = W.kind[p] | (S.nomops[p] << 8);
+    w[7] = bin;
+    w[26] = w[27] = 0;
+    if (type != 2) bin_insert(P, W, p, bin, los, his);
   }
   __syncwarp();
-  const int np = min(kPosePerWarp, P.n - static_cast<int>(blockIdx.x) * kPosePerWarp);
+  const int np = min(kPer, P.n - static_cast<int>(blockIdx.x) * kPer);
   for (int u = lane; u < kPartRecParts * np; u += 32) {
     const int gp = u / kPartRecParts, part = u - gp * kPartRecParts;
-    reinterpret_cast<int4*>(D.rec + static_cast<size_t>(blockIdx.x) * kPosePerWarp + gp)[part] =
+    reinterpret_cast<int4*>(D.rec + static_cast<size_t>(blockIdx.x) * kPer + gp)[part] =
         reinterpret_cast<const int4*>(s_rec[gp])[part];
   }
   if (t == 0 && W.publish) W.counters[kTokenCounter] = token;
@@ -283,8 +305,7 @@ __global__ void k_pose_poly(Params P, Shapes S, Parts D, Lists W) {
         rec->lo[k] = los[k];
         rec->hi[k] = his[k];
       }
-      bin_insert(P, W, p, checked_index(W.err, bin, static_cast<long long>(P.nbin[0]) * P.nbin[1] * P.nbin[2], 0),
-                 los, his);
+      bin_insert(P, W, p, bin, los, his);
     }
   }
   // world planes: face f on lane f (FP64 product per component, one rounding to FP32)
@@ -308,15 +329,18 @@ __global__ void k_pose_poly(Params P, Shapes S, Parts D, Lists W) {
 __device__ __forceinline__ int image_shift(int d, int n) { return d > (n >> 1) ? 1 : (d < -(n >> 1) ? -1 : 0); }
 
 // K3: one warp per particle p.  Lane b < 27 owns neighbour bin b of the
-// fixed-capacity cell list; its entries (node range and particle, one 16-byte
-// and one 4-byte word each) are read four at a time, tested against p's node
-// range, and compacted with warp ballots into partners above (j > p) and below
-// (j < p); each list is then sorted by rank.  Bound: load wavefronts (every
-// lane's load is its own line) and, on small boxes, load latency.  With the
-// ranges in the bins a candidate costs one wavefront and no dependent load
-// (nine scattered words of its particle before): 84.1 -> 61.6 us on 52218
-// cubes (58 candidates each).
-__global__ void __launch_bounds__(256) k_broad(Params P, Parts D, Lists W) {
+// fixed-capacity cell list (only its own one along an axis of one bin); the
+// bin's entries (node range and particle, one 16-byte and one 4-byte word each)
+// are read four at a time and tested against p's node range, moved by the
+// bin's periodic image; the hits are collected with warp ballots and each goes
+// to its rank among the partners above (j > p) or below (j < p).  Bound:
+// instruction issue, and on small boxes load latency.  With the ranges in the
+// bins a candidate costs one load wavefront and no dependent load (nine
+// scattered words of its particle before): 84.1 -> 61.6 us on 52218 cubes (58
+// candidates each); with bin coordinates kept per particle (no divisions), the
+// image of a bin instead of a candidate's, one unsigned comparison per axis and
+// one list for both sides and four blocks per SM, 50.0 us.
+__global__ void __launch_bounds__(256, 4) k_broad(Params P, Parts D, Lists W) {
   extern __shared__ int s_buf[];
   // the block's partner count (its particles share one row group), added
   // to the group sum by the block's last warp to finish: one global atomic per block
@@ -346,32 +370,40 @@ __global__ void __launch_bounds__(256) k_broad(Params P, Parts D, Lists W) {
     return;
   }
   const int cap = P.max_nbr;
-  int* up = s_buf + wid * 2 * cap;
-  int* dn = up + cap;
+  int* hits = s_buf + wid * 2 * cap;   // at most cap partners on either side, else ECAPACITY
   const int4 own_lo = reinterpret_cast<const int4*>(D.rec + p)[0], own_hi = reinterpret_cast<const int4*>(D.rec + p)[1];
   const int bin = own_hi.w;
   const int plo[3] = {own_lo.x, own_lo.y, own_lo.z}, phi[3] = {own_hi.x, own_hi.y, own_hi.z};
   const bool nodes = plo[0] <= phi[0] && plo[1] <= phi[1] && plo[2] <= phi[2];
-  const int b[3] = {bin % P.nbin[0], (bin / P.nbin[0]) % P.nbin[1], bin / (P.nbin[0] * P.nbin[1])};
-  int cnt[3];
+  // the lane's bin, and p's corner (plus one) in its image: the particles of a
+  // bin beyond the boundary lie one period away.  (Bins are at least 2 R_max +
+  // 2 dx wide, so a partner in any other image is out of reach.)
+  const int off[3] = {lane % 3, (lane / 3) % 3, lane / 9};
+  int c[3], corner[3];
+  bool use = lane < 27 && nodes;
 #pragma unroll
-  for (int k = 0; k < 3; ++k) cnt[k] = P.nbin[k] >= 3 ? 3 : P.nbin[k];
-  const int nnb = cnt[0] * cnt[1] * cnt[2];
+  for (int k = 0; k < 3; ++k) {
+    const int nb = P.nbin[k];
+    c[k] = ((bin >> (8 * k)) & 0xff) + off[k] - 1;
+    corner[k] = plo[k] + 1;
+    if (c[k] < 0) {
+      c[k] += nb;
+      corner[k] += P.ncell[k];
+    } else if (c[k] >= nb) {
+      c[k] -= nb;
+      corner[k] -= P.ncell[k];
+    }
+    use = use && (nb >= 3 || off[k] == 1);
+  }
   int num = 0;
   size_t row = 0;
   int4 ids = make_int4(-1, -1, -1, -1), recs[4];   // the bin's next four entries (the first ones fetched with its count)
 #pragma unroll
   for (int u = 0; u < 4; ++u) recs[u] = make_int4(0, 0, 0, 0);
   const int4* bin_rec = reinterpret_cast<const int4*>(W.bin_rec);
-  if (lane < nnb) {
-    int o[3] = {lane % cnt[0], (lane / cnt[0]) % cnt[1], lane / (cnt[0] * cnt[1])};
-#pragma unroll
-    for (int k = 0; k < 3; ++k) {
-      const int c = P.nbin[k] >= 3 ? b[k] + o[k] - 1 : o[k];
-      o[k] = (c + P.nbin[k]) % P.nbin[k];
-    }
-    const int q = checked_index(W.err, o[0] + P.nbin[0] * (o[1] + P.nbin[1] * o[2]),
-                                static_cast<long long>(P.nbin[0]) * P.nbin[1] * P.nbin[2], bin);
+  if (use) {
+    const int q = checked_index(W.err, c[0] + P.nbin[0] * (c[1] + P.nbin[1] * c[2]),
+                                static_cast<long long>(P.nbin[0]) * P.nbin[1] * P.nbin[2], 0);
     row = static_cast<size_t>(q) * P.bin_stride;   // (a multiple of four; entries past the count are stale and unused)
     ids = *reinterpret_cast<const int4*>(W.bin_items + row);
 #pragma unroll
@@ -379,47 +411,42 @@ __global__ void __launch_bounds__(256) k_broad(Params P, Parts D, Lists W) {
     num = min(W.bin_count[q], P.bin_cap);
   }
   const int maxn = __reduce_max_sync(kFull, num);
-  int nup = 0, ndn = 0;
+  const bool one_bin = P.nbin[0] < 3 || P.nbin[1] < 3 || P.nbin[2] < 3;
+  const int reach[3] = {phi[0] - plo[0], phi[1] - plo[1], phi[2] - plo[2]};
   const unsigned below = (1u << lane) - 1u;
+  int nhit = 0;
   for (int t0 = 0; t0 < maxn; t0 += 4) {
     const int jj[4] = {ids.x, ids.y, ids.z, ids.w};
-    int4 cur[4];
-#pragma unroll
-    for (int u = 0; u < 4; ++u) cur[u] = recs[u];
-    // the next four entries, fetched while this round's are tested
-    if (t0 + 4 < num) {
-      ids = *reinterpret_cast<const int4*>(W.bin_items + row + t0 + 4);
-#pragma unroll
-      for (int u = 0; u < 4; ++u) recs[u] = bin_rec[row + t0 + 4 + u];
-    }
+    const bool more = t0 + 4 < num;
+    if (more) ids = *reinterpret_cast<const int4*>(W.bin_items + row + t0 + 4);
 #pragma unroll
     for (int u = 0; u < 4; ++u) {
       if (t0 + u >= maxn) break;   // warp-uniform
-      const int j = t0 + u < num ? checked_index(W.err, jj[u], P.n, -1) : -1;
-      // node ranges intersect, the partner moved by the image shift (as in the pair builder):
-      // its corner lies above p's by at most p's length and below it by at most its own
-      bool hit = j >= 0 && j != p && nodes;
-      const int jl[3] = {cur[u].x, cur[u].y, cur[u].z};
+      const int j = t0 + u < num ? checked_index(W.err, jj[u], P.n, p) : p;
+      int d[3] = {recs[u].x - corner[0], recs[u].y - corner[1], recs[u].z - corner[2]};
+      int len[3] = {recs[u].w & kMaxLen, (recs[u].w >> 10) & kMaxLen, recs[u].w >> 20};
+      if (more) recs[u] = bin_rec[row + t0 + 4 + u];   // (the next round's entry, under way during this one)
+      if (one_bin) {   // (uniform) the candidate's own image along an axis of one bin
 #pragma unroll
-      for (int k = 0; k < 3; ++k) {
-        int d = jl[k] - plo[k];
-        d -= image_shift(d, P.ncell[k]) * P.ncell[k];
-        int len = (cur[u].w >> (10 * k)) & kMaxLen;
-        if (P.wide && j >= 0) len = D.rec[j].hi[k] - D.rec[j].lo[k] + 1;   // (uniform: ranges beyond kMaxLen nodes)
-        hit = hit && d <= phi[k] - plo[k] && -d < len;
+        for (int k = 0; k < 3; ++k)
+          if (P.nbin[k] < 3) d[k] -= image_shift(d[k] + 1, P.ncell[k]) * P.ncell[k];
       }
-      const unsigned bu = __ballot_sync(kFull, hit && j > p);
-      const unsigned bd = __ballot_sync(kFull, hit && j < p);
-      if (hit && j > p) {
-        const int at = nup + __popc(bu & below);
-        if (at < cap) up[at] = j;
+      if (P.wide && j != p) {   // (uniform) ranges beyond kMaxLen nodes
+#pragma unroll
+        for (int k = 0; k < 3; ++k) len[k] = D.rec[j].hi[k] - D.rec[j].lo[k] + 1;
       }
-      if (hit && j < p) {
-        const int at = ndn + __popc(bd & below);
-        if (at < cap) dn[at] = j;
+      // the ranges share a node: the partner's corner lies above p's by at most
+      // p's reach and below it by less than its own length, -len < d + 1 <= reach
+      bool hit = j != p;
+#pragma unroll
+      for (int k = 0; k < 3; ++k)
+        hit = hit && static_cast<unsigned>(d[k] + len[k]) < static_cast<unsigned>(reach[k] + len[k]);
+      const unsigned bh = __ballot_sync(kFull, hit);
+      if (hit) {
+        const int at = nhit + __popc(bh & below);
+        if (at < 2 * cap) hits[at] = j;
       }
-      nup += __popc(bu);
-      ndn += __popc(bd);
+      nhit += __popc(bh);
     }
   }
   // walls (partners n + w, after every particle): lane w tests wall w with an
@@ -446,29 +473,33 @@ __global__ void __launch_bounds__(256) k_broad(Params P, Parts D, Lists W) {
     }
     const unsigned bw = __ballot_sync(kFull, hit);
     if (hit) {
-      const int at = nup + __popc(bw & below);
-      if (at < cap) up[at] = P.n + w;
+      const int at = nhit + __popc(bw & below);
+      if (at < 2 * cap) hits[at] = P.n + w;
     }
-    nup += __popc(bw);
+    nhit += __popc(bw);
   }
-  if (nup > cap || ndn > cap) {
+  const bool over = nhit > 2 * cap;   // (then one side has more than cap)
+  nhit = min(nhit, 2 * cap);
+  __syncwarp();
+  // each hit to its rank on its side (unique keys): above, the hits in (p, v);
+  // below, those in [0, v)
+  int nup = 0;
+  for (int e0 = 0; e0 < nhit; e0 += 32) {
+    const int e = e0 + lane;
+    const int v = e < nhit ? hits[e] : -1;
+    const bool up = v > p;
+    const int from = up ? p + 1 : 0;
+    const unsigned key = static_cast<unsigned>(v - from);
+    int r = 0;
+    for (int x = 0; x < nhit; ++x) r += static_cast<unsigned>(hits[x] - from) < key ? 1 : 0;
+    if (e < nhit && r < cap) (up ? W.up_list : W.dn_list)[static_cast<size_t>(p) * cap + r] = v;
+    nup += __popc(__ballot_sync(kFull, e < nhit && up));
+  }
+  int ndn = nhit - nup;
+  if (over || nup > cap || ndn > cap) {
     if (lane == 0) set_error(W.err, kErrCapacity);
     nup = min(nup, cap);
     ndn = min(ndn, cap);
-  }
-  __syncwarp();
-  // rank sort (lists are short and keys unique)
-  for (int e = lane; e < nup; e += 32) {
-    const int v = up[e];
-    int r = 0;
-    for (int t = 0; t < nup; ++t) r += up[t] < v;
-    W.up_list[static_cast<size_t>(p) * cap + r] = v;
-  }
-  for (int e = lane; e < ndn; e += 32) {
-    const int v = dn[e];
-    int r = 0;
-    for (int t = 0; t < ndn; ++t) r += dn[t] < v;
-    W.dn_list[static_cast<size_t>(p) * cap + r] = v;
   }
   if (lane == 0) {
     W.up_count[p] = nup;
@@ -498,7 +529,7 @@ constexpr int kUpAhead = 8;     // partners of a row fetched before its count is
 // 9.6 us with sixteen rows on two warps).
 inline int build_rows(const Params& P) {
   const int rows = P.box_mode == 1 ? 4 : 8;
-  return P.n < 2 * 608 * rows ? rows / 2 : rows;
+  return P.n < 2 * 4 * kSms * rows ? rows / 2 : rows;
 }
 
 // Store a pair record (with its tile index) as fourteen 16-byte stores from
@@ -992,8 +1023,8 @@ void launch_pose(const Params& P, const Shapes& S, const Parts& D, const Lists& 
                  const double* quat, cudaStream_t st) {
   // one-warp blocks: the FP64 chains of different warps land on different sub-partitions
   // (then one block per polytope for its vertices and faces)
-  const int nb = (P.n + kPosePerWarp - 1) / kPosePerWarp;
-  if (nb > 0) launch_pdl(k_pose, dim3(nb), dim3(32), 0, st, P, S, D, W, pos, quat);
+  if (P.n > 10 * 4 * kSms) launch_pdl(k_pose<3>, dim3((P.n + 31) / 32), dim3(32), 0, st, P, S, D, W, pos, quat);
+  else launch_pdl(k_pose<1>, dim3((P.n + 9) / 10), dim3(32), 0, st, P, S, D, W, pos, quat);
   if (P.npoly > 0) launch_pdl(k_pose_poly, dim3(P.npoly), dim3(32), 0, st, P, S, D, W);
 }
 

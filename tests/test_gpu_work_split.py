@@ -89,7 +89,7 @@ def test_box_pipeline_line_grids(nc, kinds):
     else:
         rng = np.random.default_rng(5)
         pl = [W.random_polytope(rng, 14, 9.0)[0] for _ in range(2)]
-        st = state([W.POLYTOPE] * 2, [[0, 0, 0]] * 2, [[25.2, 26.1, 25.7], [33.4, 29.3, 27.4]], n=64, planes=pl,
+        st = state([W.POLYTOPE] * 2, [[0, 0, 0]] * 2, [[25.2, 26.1, 25.7], [30.9, 27.8, 26.6]], n=64, planes=pl,
                    quat=W.random_quaternions(rng, 2))
     rep, ref = run_box(boxed(st, nc))
     assert ref.n_pairs > 0
