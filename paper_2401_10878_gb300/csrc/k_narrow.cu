@@ -319,6 +319,19 @@ struct CubeEval {
     gb2 += (!s0 && !s1) ? copysignf(m, y2) : 0.f;
   }
   __device__ __forceinline__ void end_line() {}
+  // what grad(m) adds for the current node, and the same additions later (shared tiles)
+  __device__ __forceinline__ float4 record(float m) const {
+    const float a0 = fabsf(y0), a1 = fabsf(y1), a2 = fabsf(y2);
+    const bool s0 = a0 >= a1 && a0 >= a2;
+    const bool s1 = !s0 && a1 >= a2;
+    return make_float4(1.f, s0 ? copysignf(m, y0) : 0.f, s1 ? copysignf(m, y1) : 0.f,
+                       (!s0 && !s1) ? copysignf(m, y2) : 0.f);
+  }
+  __device__ __forceinline__ void replay(const float4& e) {
+    gb0 += e.y;
+    gb1 += e.z;
+    gb2 += e.w;
+  }
   __device__ float world(int c, const Local&, const PairRec& r, bool second) const {
     const float* rt = second ? r.rtb : r.rta;
     return rt[c] * gb0 + rt[3 + c] * gb1 + rt[6 + c] * gb2;
@@ -535,7 +548,22 @@ struct Partial {
   float cnt, mx, my, mz, gx, gy, gz, bestf;
   int bestidx;
   bool touched;   // warp-uniform: some lane evaluated a node (else every sum is zero)
+  bool deferred;  // warp-uniform: more clipped nodes than the limit, nothing evaluated
+  int nown, total;   // deferred: lanes with nodes, clipped nodes
 };
+
+// A tile shared by the block's warps (COOP), clipped by one of them (its record,
+// staged constants and node table in shared memory; nown lanes with nodes,
+// total nodes): warp w evaluates node passes w, w + 8, ... and leaves what each
+// node adds in shared memory; warp 0 makes the additions pass by pass, in the
+// order of a tile swept by one warp, so the sums are the same bit for bit.
+struct CoopNode {
+  float4 ga, gb;        // both evaluators' band terms (record)
+  float4 mom;           // weight and node (u, v, w)
+  float f;              // depth and node index
+  int idx;
+};
+constexpr int kShareNodes = 128;   // a tile of more clipped nodes is shared when every warp has at most one tile
 
 // Order-preserving map of FP32 values to signed ints (for integer max).
 __device__ __forceinline__ int float_key(float f) {
@@ -556,11 +584,11 @@ __device__ __forceinline__ float key_float(int k) { return __int_as_float(k >= 0
 // ROLL (the kernel with every kind, nine kind pairs): the slot loops stay
 // rolled, with the slots' clipped ranges in shared memory, to keep the
 // kernel's code small; otherwise they are unrolled over registers.
-template <bool SMOOTH, bool ROLL, class EA, class EB>
+template <bool SMOOTH, bool ROLL, bool COOP, class EA, class EB>
 __device__ __forceinline__ Partial sweep_tile(const Params& P, const Shapes& S, const Parts& D, const PairRec& r,
                                               bool swap, int tl, float4* smA, float4* smB, unsigned* spk,
-                                              int4* own) {
-  const int lane = threadIdx.x & 31;
+                                              int4* own, int limit, CoopNode* coop, int nown, int total_in) {
+  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5, nwarp = blockDim.x >> 5;
   const Local L = make_local(r);
   EA A;
   EB B;
@@ -571,7 +599,8 @@ __device__ __forceinline__ Partial sweep_tile(const Params& P, const Shapes& S, 
   const float inv_w = P.inv_w, hw = 0.5f * P.wdx_l, T = hw + kClipMargin;
   // evaluators with a staged line clip keep its constants in their (otherwise
   // unused) plane buffer
-  if constexpr (std::is_same<EA, CubeEval>::value && std::is_same<EB, CubeEval>::value) {
+  if constexpr (COOP) {
+  } else if constexpr (std::is_same<EA, CubeEval>::value && std::is_same<EB, CubeEval>::value) {
     // two cubes in one pass: lanes 0 .. 3 form A's constants, lanes 4 .. 7 B's
     const bool isb = (lane & 4) != 0;
     CubeEval::prep_lanes(r, isb ? !swap : swap, L, T, isb ? smB : smA, lane < 8 ? (lane & 3) : 4);
@@ -588,79 +617,95 @@ __device__ __forceinline__ Partial sweep_tile(const Params& P, const Shapes& S, 
   int bestidx = 0x7fffffff;
   const int it0 = tl * 32 * kTileItemsPerLane;
   const int ns = min(kTileItemsPerLane, (r.nitems - it0 + 31) >> 5);   // slots of this tile (warp-uniform)
-  // (A) per slot: first clipped node (low 16 bits) and count (high 16 bits);
-  // a pair box is below 2^16 nodes along an axis
-  unsigned pk[kTileItemsPerLane];
-  int nl = 0;
-  // line it0 + 32 s + lane as (cv, cw) = its remainder and quotient by dv:
-  // unrolled, one division for slot 0, then steps of 32 = q32 dv + r32; the
-  // rolled loop divides per slot (fewer live registers)
-  int cv = 0, r32 = 0, q32 = 0;
-  int cw = 0;
-  if constexpr (!ROLL) {
-    cw = div_small(it0 + lane, dv, inv_dv, &cv);
-    q32 = div_small(32, dv, inv_dv, &r32);
-  }
-#pragma unroll(ROLL ? 1 : kTileItemsPerLane)
-  for (int s = 0; s < kTileItemsPerLane; ++s) {
-    if (!ROLL) pk[s] = 0u;
-    if (s < ns) {
-      const int it = it0 + s * 32 + lane;
-      if constexpr (ROLL) cw = div_small(it, dv, inv_dv, &cv);
-      const int len = it < r.nitems ? du : 0;
-      float clo = 0.f, chi = static_cast<float>(len - 1);
-      clip_line_of(A, r, swap, L, csA, cv, cw, T, clo, chi, 0);
-      clip_line_of(B, r, !swap, L, csB, cv, cw, T, clo, chi, 0);
-      int ub;
-      const int nk = clip_nodes(clo, chi, 0, len, &ub);
-      const unsigned v = static_cast<unsigned>(ub) | (static_cast<unsigned>(nk) << 16);
-      if constexpr (ROLL) spk[s * 32 + lane] = v;
-      else pk[s] = v;
-      nl += nk;
-    }
+  int total = total_in, excl = 0;
+  bool has = false;
+  if constexpr (COOP) {   // (only counts of first nodes matter below: lane k stands for entry k of own)
+    has = lane < nown;
+    excl = has ? own[lane].y : 0;
+  } else {
+    // (A) per slot: first clipped node (low 16 bits) and count (high 16 bits);
+    // a pair box is below 2^16 nodes along an axis
+    unsigned pk[kTileItemsPerLane];
+    int nl = 0;
+    // line it0 + 32 s + lane as (cv, cw) = its remainder and quotient by dv:
+    // unrolled, one division for slot 0, then steps of 32 = q32 dv + r32; the
+    // rolled loop divides per slot (fewer live registers)
+    int cv = 0, r32 = 0, q32 = 0;
+    int cw = 0;
     if constexpr (!ROLL) {
-      cv += r32;
-      cw += q32;
-      if (cv >= dv) {
-        cv -= dv;
-        ++cw;
+      cw = div_small(it0 + lane, dv, inv_dv, &cv);
+      q32 = div_small(32, dv, inv_dv, &r32);
+    }
+#pragma unroll(ROLL ? 1 : kTileItemsPerLane)
+    for (int s = 0; s < kTileItemsPerLane; ++s) {
+      if (!ROLL) pk[s] = 0u;
+      if (s < ns) {
+        const int it = it0 + s * 32 + lane;
+        if constexpr (ROLL) cw = div_small(it, dv, inv_dv, &cv);
+        const int len = it < r.nitems ? du : 0;
+        float clo = 0.f, chi = static_cast<float>(len - 1);
+        clip_line_of(A, r, swap, L, csA, cv, cw, T, clo, chi, 0);
+        clip_line_of(B, r, !swap, L, csB, cv, cw, T, clo, chi, 0);
+        int ub;
+        const int nk = clip_nodes(clo, chi, 0, len, &ub);
+        const unsigned v = static_cast<unsigned>(ub) | (static_cast<unsigned>(nk) << 16);
+        if constexpr (ROLL) spk[s * 32 + lane] = v;
+        else pk[s] = v;
+        nl += nk;
+      }
+      if constexpr (!ROLL) {
+        cv += r32;
+        cw += q32;
+        if (cv >= dv) {
+          cv -= dv;
+          ++cw;
+        }
       }
     }
-  }
-  if (ROLL) __syncwarp();
-  int incl = nl;
+    if (ROLL) __syncwarp();
+    int incl = nl;
 #pragma unroll
-  for (int d = 1; d < 32; d <<= 1) {
-    const int v = __shfl_up_sync(kFull, incl, d);
-    if (lane >= d) incl += v;
-  }
-  const int total = __shfl_sync(kFull, incl, 31);
-  const int excl = incl - nl;
-  // the lanes with nodes, in lane order (their first nodes strictly
-  // increase): entry k of own holds the k-th one's lane, first node and
-  // clipped ranges
-  const bool has = nl > 0;
-  if (total > 0) {
-    const int rank = __popc(__ballot_sync(kFull, has) & ((1u << lane) - 1u));
-    if (has) {
-      if constexpr (ROLL) {
-        own[rank] = make_int4(lane, excl, 0, 0);
-      } else {
-        static_assert(kTileItemsPerLane == 4, "own holds four clipped ranges per lane");
-        // and the lane's node counts before slots 2 and 3
-        const int c2 = static_cast<int>(pk[0] >> 16) + static_cast<int>(pk[1] >> 16);
-        own[rank] = make_int4(lane, excl, static_cast<int>(pk[0]), static_cast<int>(pk[1]));
-        own[32 + rank] = make_int4(static_cast<int>(pk[2]), static_cast<int>(pk[3]), c2,
-                                   c2 + static_cast<int>(pk[2] >> 16));
-      }
+    for (int d = 1; d < 32; d <<= 1) {
+      const int v = __shfl_up_sync(kFull, incl, d);
+      if (lane >= d) incl += v;
     }
-    __syncwarp();
+    total = __shfl_sync(kFull, incl, 31);
+    excl = incl - nl;
+    // the lanes with nodes, in lane order (their first nodes strictly
+    // increase): entry k of own holds the k-th one's lane, first node and
+    // clipped ranges
+    has = nl > 0;
+    if (total > 0) {
+      const int rank = __popc(__ballot_sync(kFull, has) & ((1u << lane) - 1u));
+      if (has) {
+        if constexpr (ROLL) {
+          own[rank] = make_int4(lane, excl, 0, 0);
+        } else {
+          static_assert(kTileItemsPerLane == 4, "own holds four clipped ranges per lane");
+          // and the lane's node counts before slots 2 and 3
+          const int c2 = static_cast<int>(pk[0] >> 16) + static_cast<int>(pk[1] >> 16);
+          own[rank] = make_int4(lane, excl, static_cast<int>(pk[0]), static_cast<int>(pk[1]));
+          own[32 + rank] = make_int4(static_cast<int>(pk[2]), static_cast<int>(pk[3]), c2,
+                                     c2 + static_cast<int>(pk[2] >> 16));
+        }
+      }
+      __syncwarp();
+    }
+    if (total > limit) {
+      Partial o{};
+      o.deferred = true;
+      o.nown = __popc(__ballot_sync(kFull, has));
+      o.total = total;
+      return o;
+    }
   }
   // (B) node g of the tile's clipped nodes on lane g mod 32; its owner is the
   // last lane with nodes whose first node is <= g, i.e. entry (number of such
   // lanes) - 1 of own, counted from the lanes that start before the pass and
   // a mask of the first nodes inside it
-  for (int base = 0; base < total; base += 32) {
+  const int step = COOP ? 32 * nwarp : 32;
+  for (int base0 = 0; base0 < total; base0 += step) {
+    const int base = COOP ? base0 + 32 * wid : base0;
     const int g = base + lane;
     const unsigned before = __ballot_sync(kFull, has && excl < base);
     const unsigned inside =
@@ -715,20 +760,51 @@ __device__ __forceinline__ Partial sweep_tile(const Params& P, const Shapes& S, 
       ma = (any && fb <= 0.f) ? fmaf(-ta, ta, ta) : 0.f;
       mb = (any && fa <= 0.f) ? fmaf(-tb, tb, tb) : 0.f;
     }
-    cnt += w;
-    mu = fmaf(w, static_cast<float>(u), mu);
-    mv = fmaf(w, static_cast<float>(ocv), mv);
-    mw = fmaf(w, static_cast<float>(ocw), mw);
-    const float f = -(fa + fb);
-    const int idx = u * L.su + ocv * L.sv + ocw * L.sw;
-    if (w > 0.f && (f > bestf || (f == bestf && idx < bestidx))) {
-      bestf = f;
-      bestidx = idx;
+    float f = -(fa + fb);
+    int idx = u * L.su + ocv * L.sv + ocw * L.sw;
+    if constexpr (COOP) {
+      if (base < total) {   // warp-uniform
+        CoopNode& c = coop[32 * wid + lane];
+        c.ga = A.record(ma);
+        c.gb = B.record(mb);
+        c.mom = make_float4(w, static_cast<float>(u), static_cast<float>(ocv), static_cast<float>(ocw));
+        c.f = f;
+        c.idx = idx;
+      }
+      __syncthreads();
+      if (wid == 0) {
+        for (int q = 0; q < nwarp && base0 + 32 * q < total; ++q) {
+          const CoopNode& c = coop[32 * q + lane];
+          const float4 m = c.mom;
+          cnt += m.x;
+          mu = fmaf(m.x, m.y, mu);
+          mv = fmaf(m.x, m.z, mv);
+          mw = fmaf(m.x, m.w, mw);
+          f = c.f;
+          idx = c.idx;
+          if (m.x > 0.f && (f > bestf || (f == bestf && idx < bestidx))) {
+            bestf = f;
+            bestidx = idx;
+          }
+          A.replay(c.ga);
+          B.replay(c.gb);
+        }
+      }
+      __syncthreads();
+    } else {
+      cnt += w;
+      mu = fmaf(w, static_cast<float>(u), mu);
+      mv = fmaf(w, static_cast<float>(ocv), mv);
+      mw = fmaf(w, static_cast<float>(ocw), mw);
+      if (w > 0.f && (f > bestf || (f == bestf && idx < bestidx))) {
+        bestf = f;
+        bestidx = idx;
+      }
+      A.grad(ma);
+      B.grad(mb);
+      A.end_line();
+      B.end_line();
     }
-    A.grad(ma);
-    B.grad(mb);
-    A.end_line();
-    B.end_line();
   }
   Partial o;
   o.cnt = cnt;
@@ -741,6 +817,7 @@ __device__ __forceinline__ Partial sweep_tile(const Params& P, const Shapes& S, 
   o.bestf = bestf;
   o.bestidx = bestidx;
   o.touched = total > 0;
+  o.deferred = false;
   return o;
 }
 
@@ -898,9 +975,10 @@ __device__ __forceinline__ void tile_done(const Lists& W, const PairRec& r, floa
 // (chosen at init when no polytope is present; fewer registers, no spills).
 enum KindSet : int { SET_ALL = 0, SET_SC = 1, SET_CUBE = 2 };
 
-template <bool SMOOTH, int SET>
+template <bool SMOOTH, int SET, bool COOP>
 __device__ __forceinline__ Partial dispatch(const Params& P, const Shapes& S, const Parts& D, const PairRec& r,
-                                            int tl, float4* smA, float4* smB, unsigned* spk, int4* own) {
+                                            int tl, float4* smA, float4* smB, unsigned* spk, int4* own, int limit,
+                                            CoopNode* coop, int nown, int total) {
   int ka = r.kinds & 0xff, kb = r.kinds >> 8;
   // evaluate the cheaper kind as A (G's sign flips back below); two cubes keep the record's order
   const bool swap = SET == SET_CUBE ? false : sweep_swap(ka, kb);
@@ -911,14 +989,16 @@ __device__ __forceinline__ Partial dispatch(const Params& P, const Shapes& S, co
     ka = ka == KIND_CUBE ? KIND_CUBOID : ka;
     kb = kb == KIND_CUBE ? KIND_CUBOID : kb;
   }
-  Partial o{0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, -FLT_MAX, 0x7fffffff, false};
+  Partial o{0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, -FLT_MAX, 0x7fffffff, false, false, 0, 0};
+  if constexpr (SET == SET_CUBE) {
+    return sweep_tile<SMOOTH, false, COOP, CubeEval, CubeEval>(P, S, D, r, swap, tl, smA, smB, spk, own, limit, coop,
+                                                               nown, total);
+  }
 #define GBC_CASE(KA, KB, TA, TB)                                                  \
   case (KA) * 8 + (KB):                                                          \
-    o = sweep_tile<SMOOTH, SET == SET_ALL, TA, TB>(P, S, D, r, swap, tl, smA, smB, spk, own); \
+    o = sweep_tile<SMOOTH, SET == SET_ALL, false, TA, TB>(P, S, D, r, swap, tl, smA, smB, spk, own, limit, nullptr, 0, 0); \
     break;
-  if constexpr (SET == SET_CUBE) {
-    o = sweep_tile<SMOOTH, false, CubeEval, CubeEval>(P, S, D, r, swap, tl, smA, smB, spk, own);
-  } else if constexpr (SET == SET_SC) {
+  if constexpr (SET == SET_SC) {
     switch (ka * 8 + kb) {
       GBC_CASE(0, 0, SphereEval, SphereEval)
       GBC_CASE(0, 4, SphereEval, CubeEval)
@@ -932,7 +1012,7 @@ __device__ __forceinline__ Partial dispatch(const Params& P, const Shapes& S, co
       default:
         break;
     }
-  } else {
+  } else if constexpr (SET == SET_ALL) {
     switch (ka * 8 + kb) {
       GBC_CASE(0, 0, SphereEval, SphereEval)
       GBC_CASE(0, 1, SphereEval, CuboidEval)
@@ -981,15 +1061,31 @@ __global__ void __launch_bounds__(narrow_warps<SET>() * 32, narrow_blocks<SET>()
   __shared__ float4 s_planes[NW][2][SET == SET_CUBE ? 8 : 2 * kMaxFaces];
   __shared__ unsigned s_pk[SET == SET_ALL ? NW : 1][kTileItemsPerLane * 32];   // clipped ranges (rolled sweep)
   __shared__ int4 s_own[NW][64];   // the lanes with clipped nodes (sweep_tile)
+  // tiles shared by the block: in the cubes-only variant (the others hold nine
+  // kind pairs, and the second sweep of each would cost their instruction
+  // fetches more than it gives: 10.8 -> 11.1 us on 1934 mixed particles)
+  constexpr bool kShare = SET == SET_CUBE;
+  __shared__ CoopNode s_coop[kShare ? NW * 32 : 1];   // a shared tile's nodes
+  __shared__ int3 s_deferred[NW];   // warp that clipped it, lanes with nodes, clipped nodes
+  __shared__ int s_ndeferred;
   pdl_begin();
   const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
   const int ntiles = W.counters[1];
-  // tiles w, w + W, ... of the list (W warps); the first record is fetched
-  // with the tile count, the next one while a tile runs
+  // tiles w, w + W, ... of the list (W warps, numbered across the blocks first:
+  // consecutive tiles, often of one pair, run on different SMs); the first
+  // record is fetched with the tile count, the next one while a tile runs
   const int nwarps = gridDim.x * NW;
-  int t = blockIdx.x * NW + wid;
+  int t = blockIdx.x + gridDim.x * wid;
   const int4 first = t < P.max_tiles ? load_rec_part(W.tiles + t, lane) : make_int4(0, 0, 0, 0);
   if (ntiles > P.max_tiles) return;   // capacity exceeded: the step reports ECAPACITY
+  // with at most one tile per warp a tile of many node passes would be the
+  // kernel's tail: it is left for the whole block, whose other warps are done
+  // (400 cubes, one in seven pressed into a neighbour: 16.0 -> @COOP@ us)
+  const bool share = kShare && ntiles <= nwarps;
+  if (share) {
+    if (threadIdx.x == 0) s_ndeferred = 0;
+    __syncthreads();
+  }
   if (t < ntiles) store_rec_part(&s_rec[wid][0], lane, first);
   __syncwarp();
   int buf = 0;
@@ -998,15 +1094,30 @@ __global__ void __launch_bounds__(narrow_warps<SET>() * 32, narrow_blocks<SET>()
     const int4 next = tn < ntiles ? load_rec_part(W.tiles + tn, lane) : make_int4(0, 0, 0, 0);
     const PairRec& r = s_rec[wid][buf];
     if (record_in_bounds(P, W.err, r, true)) {
-      const Partial o = dispatch<SMOOTH, SET>(P, S, D, r, r.tile, s_planes[wid][0], s_planes[wid][1],
-                                              s_pk[SET == SET_ALL ? wid : 0], s_own[wid]);
-      tile_done(W, r, o.touched ? reduce_tile<SMOOTH>(o) : empty_partial());
+      const Partial o = dispatch<SMOOTH, SET, false>(P, S, D, r, r.tile, s_planes[wid][0], s_planes[wid][1],
+                                                     s_pk[SET == SET_ALL ? wid : 0], s_own[wid],
+                                                     share ? kShareNodes : 0x7fffffff, nullptr, 0, 0);
+      if (!o.deferred) tile_done(W, r, o.touched ? reduce_tile<SMOOTH>(o) : empty_partial());
+      else if (lane == 0) s_deferred[atomicAdd_block(&s_ndeferred, 1)] = make_int3(wid, o.nown, o.total);
     }
+    if (share) break;   // (one tile per warp at most: what it staged stays for the block)
     __syncwarp();
     if (tn < ntiles) store_rec_part(&s_rec[wid][buf ^ 1], lane, next);
     __syncwarp();
     buf ^= 1;
     t = tn;
+  }
+  if constexpr (kShare) {
+    if (!share) return;
+    __syncthreads();
+    const int nd = s_ndeferred;
+    for (int d = 0; d < nd; ++d) {
+      const int3 e = s_deferred[d];
+      const PairRec& r = s_rec[e.x][0];
+      const Partial o = dispatch<SMOOTH, SET, true>(P, S, D, r, r.tile, s_planes[e.x][0], s_planes[e.x][1], s_pk[0],
+                                                    s_own[e.x], 0, s_coop, e.y, e.z);
+      if (wid == 0) tile_done(W, r, reduce_tile<SMOOTH>(o));
+    }
   }
 }
 

@@ -93,3 +93,18 @@ def test_box_pipeline_line_grids(nc, kinds):
                    quat=W.random_quaternions(rng, 2))
     rep, ref = run_box(boxed(st, nc))
     assert ref.n_pairs > 0
+
+
+# clipped nodes per tile: about one per line (at the limit above which a block shares a tile), several, many
+@pytest.mark.parametrize("pen", [0.6, 1.1, 1.6, 3.2, 9.0])
+@pytest.mark.parametrize("indicator", [0, 1])
+@pytest.mark.parametrize("half", [5.6, 5.9, 12.0])
+def test_shared_tiles_of_cubes(pen, indicator, half):
+    """Cubes pressed together over a whole face, alone and with a third one
+    aside: few tiles of many node passes."""
+    q = [quat_axis_angle([0.3, 1.0, 0.2], 0.004), quat_axis_angle([1.0, 0.1, 0.4], 0.006), quat_axis_angle([1, 1, 0], 0.9)]
+    c = np.array([40.23, 41.31, 42.17])
+    st = state([W.CUBOID] * 3, [[half] * 3] * 3, [c, c + [2 * half - pen, 0.21, -0.17], c + [0.3, 1.9 * half, 7.7]],
+               quat=q, n=128, indicator=indicator)
+    rep, ref = _parity(st, 0)
+    assert ref.pair_out[0, 0] > 0.0
