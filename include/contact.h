@@ -239,6 +239,14 @@ contact_status contact_backward(contact_ctx* ctx, const double* grad_force, cons
 /* Synchronises the context stream and returns the sticky device error (the
  * error stays set; contact_clear_error resets it). */
 contact_status contact_check(contact_ctx* ctx);
+
+/* Synchronises the context stream and writes the pair count of the last
+ * completed step (the step's n_pairs: above max_pairs after a step that failed
+ * with CONTACT_ECAPACITY; 0 before the first step), without a device copy.
+ * Reports no device error (contact_check does).
+ *   n_pairs  host out
+ * CONTACT_EINVAL for a null argument. */
+contact_status contact_pair_count(contact_ctx* ctx, int32_t* n_pairs);
 void contact_clear_error(contact_ctx* ctx);
 
 /* Human-readable description of the last error of the context (never NULL). */

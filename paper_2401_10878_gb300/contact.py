@@ -33,7 +33,7 @@ EXPORTS = ["contact_config_default", "contact_init", "contact_step", "contact_ba
            "contact_kernels_per_backward", "contact_destroy", "contact_step_noalloc", "contact_step_host",
            "contact_history_get", "contact_history_set", "contact_history_reset", "contact_polytope_centroid",
            "contact_polytope_shift", "contact_fp32_ffma_rate", "contact_fp64_dfma_rate",
-           "contact_adjoint_time", "contact_bounds_selftest"]
+           "contact_adjoint_time", "contact_bounds_selftest", "contact_pair_count"]
 
 
 class Config(ctypes.Structure):
@@ -84,6 +84,8 @@ def load_library(build_if_missing: bool = True, checks: bool = False):
     lib.contact_backward.restype = I32
     lib.contact_check.argtypes = [P]
     lib.contact_check.restype = I32
+    lib.contact_pair_count.argtypes = [P, P]
+    lib.contact_pair_count.restype = I32
     lib.contact_clear_error.argtypes = [P]
     lib.contact_clear_error.restype = None
     lib.contact_last_error.argtypes = [P]
@@ -202,6 +204,8 @@ class Contact:
         self.n_pairs = torch.zeros(1, dtype=torch.int32, device=dev)
         self.force = torch.zeros((n, 3), dtype=torch.float64, device=dev)
         self.torque = torch.zeros((n, 3), dtype=torch.float64, device=dev)
+        # recorded on the caller's stream, waited for by the context's (one event, recorded anew on each call)
+        self._inputs_ready = torch.cuda.Event()
 
     @classmethod
     def from_state(cls, st, **kw):
@@ -296,31 +300,42 @@ class Contact:
         if rc != OK:
             self._raise(rc, "contact_step")
 
+    def _wait_for_inputs(self):
+        """Order the context's stream after the work enqueued on the caller's."""
+        self._inputs_ready.record(torch.cuda.current_stream(self.device))
+        self.stream.wait_event(self._inputs_ready)
+
     def step(self, pos, quat, vel=None, check=True):
-        """contact_step; waits for the result when check is True."""
-        cur = torch.cuda.current_stream(self.device)
-        self.stream.wait_stream(cur)
+        """contact_step; returns when the step is done (its pair count is read
+        on the host), raising its device error when check is True."""
+        self._wait_for_inputs()
         self.step_async(pos, quat, vel)
-        cur.wait_stream(self.stream)
         if check:
             self.check()
-        P = int(self.n_pairs.item())
-        P = min(P, self.max_pairs)
+        count = ctypes.c_int32()
+        rc = self.lib.contact_pair_count(self.ctx, ctypes.byref(count))   # waits for the step
+        if rc != OK:
+            self._raise(rc, "contact_pair_count")
+        P = min(count.value, self.max_pairs)
         return dict(pair_ij=self.pair_ij[:P], pair_out=self.pair_out[:P], force=self.force, torque=self.torque,
                     n_pairs=P)
 
     def backward(self, grad_force, grad_torque, check=True):
-        gp = torch.zeros((self.n, 3), dtype=torch.float64, device=self.device)
-        gq = torch.zeros((self.n, 4), dtype=torch.float64, device=self.device)
-        cur = torch.cuda.current_stream(self.device)
-        self.stream.wait_stream(cur)
-        rc = self.lib.contact_backward(self.ctx, _ptr(grad_force.contiguous()), _ptr(grad_torque.contiguous()),
-                                       _ptr(gp), _ptr(gq))
+        # (every entry is written: a particle without contacts gets zeros)
+        gp = torch.empty((self.n, 3), dtype=torch.float64, device=self.device)
+        gq = torch.empty((self.n, 4), dtype=torch.float64, device=self.device)
+        gf, gt = grad_force.contiguous(), grad_torque.contiguous()
+        self._wait_for_inputs()
+        rc = self.lib.contact_backward(self.ctx, _ptr(gf), _ptr(gt), _ptr(gp), _ptr(gq))
         if rc != OK:
             self._raise(rc, "contact_backward")
-        cur.wait_stream(self.stream)
         if check:
-            self.check()
+            self.check()   # waits: the results and the inputs' memory are the caller's stream's again
+        else:
+            cur = torch.cuda.current_stream(self.device)
+            for t in (gf, gt):
+                t.record_stream(self.stream)
+            cur.wait_stream(self.stream)
         return gp, gq
 
     def check(self):
@@ -448,27 +463,32 @@ def polytope_centroid(planes) -> np.ndarray:
 
 class ContactFunction(torch.autograd.Function):
     """(pos, quat, vel) -> (force, torque, pair_ij, pair_out) with the
-    library's adjoint as backward.  vel (or None) enters the damping and the
-    friction and is not differentiated; the pair outputs carry no gradient."""
+    library's adjoint as backward; with pairs=False (force, torque) alone.
+    vel (or None) enters the damping and the friction and is not
+    differentiated; the pair outputs carry no gradient."""
 
     @staticmethod
-    def forward(ctx, model, pos, quat, vel):
+    def forward(ctx, model, pos, quat, vel, pairs=True):
         v = None if vel is None else vel.detach().to(torch.float64).contiguous()
         out = model.step(pos.detach().to(torch.float64).contiguous(), quat.detach().to(torch.float64).contiguous(), v)
         ctx.model = model
         ctx.step_id = model.steps
         ctx.vel = v   # the adjoint reads the step's velocities: they stay alive until backward
+        # the model's own buffers are written by its next step
+        force, torque = out["force"].clone(), out["torque"].clone()
+        if not pairs:
+            return force, torque
         pij, pout = out["pair_ij"].clone(), out["pair_out"].clone()
         ctx.mark_non_differentiable(pij, pout)
-        return out["force"].clone(), out["torque"].clone(), pij, pout
+        return force, torque, pij, pout
 
     @staticmethod
-    def backward(ctx, gF, gT, _g_ij, _g_out):
+    def backward(ctx, gF, gT, *_g_pairs):
         if ctx.model.steps != ctx.step_id:
             raise RuntimeError("contact_forces: the model stepped again after this forward; the adjoint "
                                "differentiates the model's last step only")
         gp, gq = ctx.model.backward(gF.to(torch.float64).contiguous(), gT.to(torch.float64).contiguous())
-        return None, gp, gq, None
+        return (None, gp, gq, None, None)[:len(ctx.needs_input_grad)]
 
 
 def contact_forces(model: Contact, pos: torch.Tensor, quat: torch.Tensor, vel: torch.Tensor = None,
@@ -478,10 +498,10 @@ def contact_forces(model: Contact, pos: torch.Tensor, quat: torch.Tensor, vel: t
     damping and friction (not differentiated).  With pairs=True also returns
     dict(pair_ij [P,2], pair_out [P,11]) of the step.  A backward must come
     before the model's next step."""
-    force, torque, pij, pout = ContactFunction.apply(model, pos, quat, vel)
     if pairs:
+        force, torque, pij, pout = ContactFunction.apply(model, pos, quat, vel, True)
         return force, torque, dict(pair_ij=pij, pair_out=pout)
-    return force, torque
+    return ContactFunction.apply(model, pos, quat, vel, False)
 
 
 def fp32_ffma_rate(iters: int = 2000) -> float:

@@ -314,9 +314,9 @@ struct Lists {
                     // steps completed (its parity selects the contact-history buffer)
   unsigned long long* u64;  // [4]: 0 node evaluations, 1 nominal lane-ops of the node sweep
   int* err;         // [1] sticky device error
-  int* err_host;    // [3] mapped host words: 0 mirrors err; 1 the token of the last completed step
+  int* err_host;    // [4] mapped host words: 0 mirrors err; 1 the token of the last completed step
                     // (written by the step's last block); 2 the token the host gave the step being
-                    // launched (read by k_pose into counters[kTokenCounter])
+                    // launched (read by k_pose into counters[kTokenCounter]); 3 the last step's pairs
   int publish;      // 1 in a host-buffer step that returns on its token: k_pose reads the token, the
                     // particle sums' last block mirrors err and publishes it (0: err mirrored at the
                     // start of the particle sums, no token)
@@ -507,6 +507,7 @@ void launch_force(const Params& P, const Shapes& S, const Parts& D, const Lists&
 void launch_particle_sum(const Params& P, const Parts& D, const Lists& W, double* force, double* torque,
                          cudaStream_t st);
 size_t adjoint_scratch_doubles(int max_pairs, int max_tiles);
+int adjoint_grid(const Params& P);   // blocks of the adjoint's cell sweep: every resident slot
 void launch_adjoint(const Params& P, const Shapes& S, const Parts& D, const Lists& W, const double* vel,
                     const double* gF, const double* gT, double* gpos, double* gquat, double* scratch,
                     int grid, cudaStream_t st, cudaEvent_t ev0 = nullptr, cudaEvent_t ev1 = nullptr);

@@ -668,14 +668,14 @@ contact_status contact_init(const contact_config* cfg, const int32_t* shape_type
   GBC_TRY(cudaEventCreate(&c->ev_narrow[1]));
   GBC_TRY(cudaEventCreate(&c->ev_adj[0]));
   GBC_TRY(cudaEventCreate(&c->ev_adj[1]));
-  GBC_TRY(cudaHostAlloc(reinterpret_cast<void**>(&c->err_host), 3 * sizeof(int), cudaHostAllocMapped));
-  c->err_host[0] = c->err_host[1] = c->err_host[2] = 0;
+  GBC_TRY(cudaHostAlloc(reinterpret_cast<void**>(&c->err_host), 4 * sizeof(int), cudaHostAllocMapped));
+  for (int k = 0; k < 4; ++k) c->err_host[k] = 0;
   int* err_dev_view = nullptr;
   GBC_TRY(cudaHostGetDevicePointer(reinterpret_cast<void**>(&err_dev_view), c->err_host, 0));
   W.err_host = err_dev_view;
 #undef GBC_TRY
   c->grid_narrow = narrow_grid(P);
-  c->grid_adjoint = c->grid_narrow;
+  c->grid_adjoint = adjoint_grid(P);
   *out = c;
   return CONTACT_OK;
 }
@@ -759,11 +759,21 @@ contact_status contact_check(contact_ctx* c) {
   if (c == nullptr) return CONTACT_EINVAL;
   cudaError_t e = cudaStreamSynchronize(c->stream);
   if (e != cudaSuccess) return cuda_fail(c, e, "cudaStreamSynchronize");
+#ifdef CONTACT_CHECKS   // (the index checks may also fail in the particle sums and in the backward kernels)
   int err = 0;
   e = cudaMemcpy(&err, c->W.err, sizeof(int), cudaMemcpyDeviceToHost);
   if (e != cudaSuccess) return cuda_fail(c, e, "cudaMemcpy");
   *c->err_host = err;
-  return check_sticky(c);
+#endif
+  return check_sticky(c);   // every step's last kernel has mirrored the error word
+}
+
+contact_status contact_pair_count(contact_ctx* c, int32_t* n_pairs) {
+  if (c == nullptr || n_pairs == nullptr) return CONTACT_EINVAL;
+  const cudaError_t e = cudaStreamSynchronize(c->stream);
+  if (e != cudaSuccess) return cuda_fail(c, e, "cudaStreamSynchronize");
+  *n_pairs = reinterpret_cast<const volatile int*>(c->err_host)[3];
+  return CONTACT_OK;
 }
 
 contact_status contact_bounds_selftest(contact_ctx* c) {

@@ -999,7 +999,18 @@ size_t adjoint_scratch_doubles(int max_pairs, int max_tiles) {
          static_cast<size_t>(max_pairs) * kPairGrad + static_cast<size_t>(max_pairs) / 2 + 16;
 }
 
-// ev0 / ev1 (nullable): events recorded around the cell sweep's launch.
+int adjoint_grid(const Params& P) {
+  // compiled per kind set, as the node sweep (2 cubes only, 1 spheres / cuboids / walls, 0 every kind)
+  auto cells = P.kind_set == 2 ? k_adj_cells<2> : (P.kind_set == 1 ? k_adj_cells<1> : k_adj_cells<0>);
+  int dev = 0, sms = 0, per_sm = 0;
+  cudaGetDevice(&dev);
+  cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+  cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, cells, kAdjWarps * 32, 0);
+  return (per_sm > 0 ? per_sm : 1) * (sms > 0 ? sms : 1);
+}
+
+// grid: adjoint_grid (formed once per context: the occupancy queries cost the
+// host more than a launch).  ev0 / ev1 (nullable): events recorded around the cell sweep's launch.
 void launch_adjoint(const Params& P, const Shapes& S, const Parts& D, const Lists& W, const double* vel,
                     const double* gF, const double* gT, double* gpos, double* gquat, double* scratch, int grid,
                     cudaStream_t st, cudaEvent_t ev0, cudaEvent_t ev1) {
@@ -1008,20 +1019,13 @@ void launch_adjoint(const Params& P, const Shapes& S, const Parts& D, const List
   B.seeds = B.partial + static_cast<size_t>(P.max_tiles) * kAdjPartial;
   B.pgrad = reinterpret_cast<double*>(B.seeds + static_cast<size_t>(P.max_pairs) * kSeedFloats + 8);
   B.done = reinterpret_cast<int*>(B.pgrad + static_cast<size_t>(P.max_pairs) * kPairGrad);
-  int dev = 0, sms = 0;
-  cudaGetDevice(&dev);
-  cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
   const int wneed0 = (P.max_pairs + 7) / 8;   // pre: eight pairs per warp pass
-  const int wgrid0 = wneed0 < 8 * sms ? (wneed0 > 0 ? wneed0 : 1) : 8 * sms;
+  const int wgrid0 = wneed0 < 8 * kSms ? (wneed0 > 0 ? wneed0 : 1) : 8 * kSms;
   launch_pdl(k_adj_pre, dim3(wgrid0), dim3(32), 0, st, P, S, D, W, B, vel, gF, gT);
   // compiled per kind set, as the node sweep (2 cubes only, 1 spheres / cuboids / walls, 0 every kind)
   auto cells = P.kind_set == 2 ? k_adj_cells<2> : (P.kind_set == 1 ? k_adj_cells<1> : k_adj_cells<0>);
-  int per_sm = 0;
-  cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, cells, kAdjWarps * 32, 0);
-  const int cgrid = (per_sm > 0 ? per_sm : 1) * sms;   // persistent: every resident slot pulls tiles
-  (void)grid;
   if (ev0 != nullptr) cudaEventRecord(ev0, st);
-  launch_pdl(cells, dim3(cgrid), dim3(kAdjWarps * 32), 0, st, P, S, D, W, B);
+  launch_pdl(cells, dim3(grid), dim3(kAdjWarps * 32), 0, st, P, S, D, W, B);
   if (ev1 != nullptr) cudaEventRecord(ev1, st);
   launch_pdl(k_adj_scatter, dim3((8 * P.n + 31) / 32), dim3(32), 0, st, P, D, W, B, gpos, gquat);
 }

@@ -57,6 +57,7 @@ __global__ void __launch_bounds__(32) k_particle_sum(Params P, Parts D, Lists W,
   const int t = blockIdx.x * blockDim.x + threadIdx.x;
   if (t == 0) {
     if (!W.publish) *W.err_host = *W.err;
+    W.err_host[3] = W.counters[0];   // (contact_pair_count)
     ++W.counters[kStepCounter];   // the contact history written this step is read by the next
   }
   // the cell list's bin counts start the next step at zero

@@ -108,3 +108,25 @@ def test_shared_tiles_of_cubes(pen, indicator, half):
                quat=q, n=128, indicator=indicator)
     rep, ref = _parity(st, 0)
     assert ref.pair_out[0, 0] > 0.0
+
+
+@pytest.mark.parametrize("max_pairs", [None, 8])
+def test_pair_count_of_the_last_step(max_pairs):
+    """contact_pair_count is the step's n_pairs, also beyond the capacity (0 before the first step)."""
+    import ctypes
+
+    from paper_2401_10878_gb300.contact import ECAPACITY, Contact, ContactError
+    st = W.mixed_grid_27()
+    m = Contact.from_state(st, max_pairs=max_pairs)
+    n = ctypes.c_int32(-1)
+    assert m.lib.contact_pair_count(m.ctx, ctypes.byref(n)) == 0 and n.value == 0
+    pos, quat = torch.tensor(st.pos, device="cuda"), torch.tensor(st.quat, device="cuda")
+    if max_pairs is None:
+        assert m.step(pos, quat)["n_pairs"] == int(m.n_pairs.item())
+    else:
+        assert m.step(pos, quat, check=False)["n_pairs"] == max_pairs
+        with pytest.raises(ContactError) as e:
+            m.step(pos, quat)
+        assert e.value.code == ECAPACITY
+    assert m.lib.contact_pair_count(m.ctx, ctypes.byref(n)) == 0 and n.value == int(m.n_pairs.item()) > 8
+    m.close()
