@@ -75,117 +75,6 @@ __device__ __forceinline__ float world_comp(int c, const Local& L, float au, flo
 // lattice units, relative to the pair box origin; it reads the pair record
 // from shared memory (second = the record's particle j).
 
-struct SphereEval {
-  int iu, iv, iw;
-  float fu, fv, fw, rad;
-  float cnt_u, rv, rw, rho2, ru, q;
-  float gu, gv, gw, gl;
-  __device__ void load(const PairRec& r, bool second, const Shapes&, const Parts&, const Local& L, float4*) {
-    const int* ci = second ? r.bi : r.ai;
-    const float* cf = second ? r.bf : r.af;
-    iu = ci[L.u]; iv = ci[L.v]; iw = ci[L.w];
-    fu = cf[L.u]; fv = cf[L.v]; fw = cf[L.w];
-    rad = second ? r.szb[0] : r.sza[0];
-    gu = gv = gw = 0.f;
-  }
-  __device__ __forceinline__ void begin_line(int cv, int cw, int u0) {
-    rv = static_cast<float>(cv - iv) - fv;
-    rw = static_cast<float>(cw - iw) - fw;
-    rho2 = fmaf(rv, rv, rw * rw);
-    gl = 0.f;
-    cnt_u = static_cast<float>(u0 - iu) - 1.f;
-  }
-  // [lo, hi] (line coordinates) cut to where phi < T on the current line
-  __device__ __forceinline__ void clip(float T, float& lo, float& hi) const {
-    const float o = static_cast<float>(iu);
-    float l = lo - o, h = hi - o;
-    clip_ball(fu, rho2, rad, T, l, h);
-    lo = l + o;
-    hi = h + o;
-  }
-  __device__ __forceinline__ float phi() {
-    cnt_u += 1.f;
-    ru = cnt_u - fu;
-    q = fmaf(ru, ru, rho2);
-    return sqrtf(q) - rad;
-  }
-  __device__ __forceinline__ void grad(float m) {
-    const float mi = m * (q > 0.f ? rsqrtf(q) : 0.f);
-    gu = fmaf(mi, ru, gu);
-    gl += mi;
-  }
-  __device__ __forceinline__ void end_line() {
-    gv = fmaf(gl, rv, gv);
-    gw = fmaf(gl, rw, gw);
-  }
-  __device__ float world(int c, const Local& L, const PairRec&, bool) const { return world_comp(c, L, gu, gv, gw); }
-};
-
-struct CuboidEval {
-  int iu, iv, iw;
-  float fu, fv, fw;
-  float tu[3], tv[3], tw[3], h[3], itu[3];
-  float cnt_u, p[3], y[3], a[3];
-  float gb[3];
-  __device__ void load(const PairRec& r, bool second, const Shapes&, const Parts&, const Local& L, float4*) {
-    const int* ci = second ? r.bi : r.ai;
-    const float* cf = second ? r.bf : r.af;
-    const float* rt = second ? r.rtb : r.rta;
-    const float* sz = second ? r.szb : r.sza;
-    iu = ci[L.u]; iv = ci[L.v]; iw = ci[L.w];
-    fu = cf[L.u]; fv = cf[L.v]; fw = cf[L.w];
-#pragma unroll
-    for (int k = 0; k < 3; ++k) {
-      tu[k] = rt[3 * k + L.u];
-      tv[k] = rt[3 * k + L.v];
-      tw[k] = rt[3 * k + L.w];
-      h[k] = sz[k];
-      itu[k] = clip_inv(tu[k]);
-      gb[k] = 0.f;
-    }
-  }
-  __device__ __forceinline__ void begin_line(int cv, int cw, int u0) {
-    const float rv = static_cast<float>(cv - iv) - fv;
-    const float rw = static_cast<float>(cw - iw) - fw;
-    // y_k = tu_k (m - fu) + tv_k rv + tw_k rw with m = cu - iu: the constant
-    // part is folded once per line, a node costs one FMA per axis
-#pragma unroll
-    for (int k = 0; k < 3; ++k) p[k] = fmaf(-tu[k], fu, fmaf(tv[k], rv, tw[k] * rw));
-    cnt_u = static_cast<float>(u0 - iu) - 1.f;
-  }
-  __device__ __forceinline__ void clip(float T, float& lo, float& hi) const {
-    const float o = static_cast<float>(iu);
-    float l = lo - o, hh = hi - o;
-#pragma unroll
-    for (int k = 0; k < 3; ++k) clip_slab(tu[k], itu[k], p[k], h[k] + T, l, hh);
-    lo = l + o;
-    hi = hh + o;
-  }
-  __device__ __forceinline__ float phi() {
-    cnt_u += 1.f;
-#pragma unroll
-    for (int k = 0; k < 3; ++k) {
-      y[k] = fmaf(tu[k], cnt_u, p[k]);
-      a[k] = fabsf(y[k]) - h[k];
-    }
-    return fmaxf(a[0], fmaxf(a[1], a[2]));
-  }
-  __device__ __forceinline__ void grad(float m) {
-    // active face: first maximal axis; gradient sign(y_k) e_k (body frame)
-    const bool s0 = a[0] >= a[1] && a[0] >= a[2];
-    const bool s1 = !s0 && a[1] >= a[2];
-    gb[0] += s0 ? copysignf(m, y[0]) : 0.f;
-    gb[1] += s1 ? copysignf(m, y[1]) : 0.f;
-    gb[2] += (!s0 && !s1) ? copysignf(m, y[2]) : 0.f;
-  }
-  __device__ __forceinline__ void end_line() {}
-  // world component c of R gb, R^T row k = body axis k in world
-  __device__ float world(int c, const Local&, const PairRec& r, bool second) const {
-    const float* rt = second ? r.rtb : r.rta;
-    return rt[c] * gb[0] + rt[3 + c] * gb[1] + rt[6 + c] * gb[2];
-  }
-};
-
 // Cube (equal half extents h): phi = max_k |y_k| - h.  Only what the node
 // loop needs stays in registers; the cross-axis terms are re-read from the
 // shared-memory pair record at each line start.  The line clip reads per-tile
@@ -198,10 +87,8 @@ struct CubeEval {
   bool flat;   // a slab parallel to the lines (|tu_k| <= kClipFlat): the general clip
   float cnt_u, p0, p1, p2, y0, y1, y2;
   float gb0, gb1, gb2;
-  // the geometry comes with the staged constants (prep_clip, then fetch)
-  __device__ void load(const PairRec&, bool, const Shapes&, const Parts&, const Local&, float4*) {
-    gb0 = gb1 = gb2 = 0.f;
-  }
+  // (the geometry comes with the staged constants: prep_lanes, then fetch)
+  __device__ __forceinline__ void clear() { gb0 = gb1 = gb2 = 0.f; }
   __device__ __forceinline__ void begin_line_rec(const PairRec& r, bool second, const Local& L, int cv, int cw,
                                                  int u0) {
     const int* ci = second ? r.bi : r.ai;
@@ -231,9 +118,6 @@ struct CubeEval {
   // centre and size (two cubes: lanes 4 .. 7 form B's in the same pass); the
   // caller syncs the warp once for both evaluators and every lane then
   // fetches its registers.
-  __device__ __forceinline__ void prep_clip(const PairRec& r, bool second, const Local& L, float T, float4* cs) {
-    prep_lanes(r, second, L, T, cs, threadIdx.x & 31);
-  }
   // the stores of lane q of the group that forms the constants (q < 3: axis
   // q's entries, q = 3: the centre and size, q > 3: none)
   static __device__ __forceinline__ void prep_lanes(const PairRec& r, bool second, const Local& L, float T,
@@ -318,7 +202,6 @@ struct CubeEval {
     gb1 += s1 ? copysignf(m, y1) : 0.f;
     gb2 += (!s0 && !s1) ? copysignf(m, y2) : 0.f;
   }
-  __device__ __forceinline__ void end_line() {}
   // what grad(m) adds for the current node, and the same additions later (shared tiles)
   __device__ __forceinline__ float4 record(float m) const {
     const float a0 = fabsf(y0), a1 = fabsf(y1), a2 = fabsf(y2);
@@ -360,186 +243,191 @@ __device__ __forceinline__ int stage_planes(const Shapes& S, const Parts& D, int
   return nf;
 }
 
-// Polytopes: planes read from shared memory (sp[0 .. nf)); phi keeps the index
-// of the first maximal face for the gradient.  The line clip reads per-tile
-// half-line bounds (prep_clip) from sp[kMaxFaces ..): along the line, face f
-// of slope m = e.x bounds the node counter c - iu by
-// C_f - sy_f rv - sz_f rw (above for m > 0, below for m < 0) with
-// sy_f = e.y / m, sz_f = e.z / m, C_f = (T + e.w) / m + fu; a face parallel
-// to the line (|m| <= kClipFlat) keeps or empties the whole line.
-struct PolyEval {
-  int iu, iv, iw, nf, nup, ndn, kbest;
+// Any kind, chosen at run time (the variant with every kind): what the other
+// evaluators keep in registers stays in the warp's shared memory, so one copy of
+// the code serves every pair of kinds.  With a sweep compiled per kind pair the
+// warps of an SM, each on its own pair, waited on instruction fetches for most
+// of the time (16 of 23 stalled cycles per instruction: 82 us for 15472
+// smoothed mixed particles, 10.8 us for 1934 sharp ones; 39.5 and 8.9 us with
+// one copy).  The arithmetic of a line and of a node is that of the evaluators
+// above, operation for operation.
+// cs: sphere (radius); cuboid (tu, tv, tw, h) per axis, then 1 / tu; wall
+// (mu, mv, mw, p0), then 1 / mu (p0 = the wall's value at the box origin,
+// inflate included, formed in FP64 by the pair builder: box-relative values
+// stay small, so FP32 keeps them to ~1e-6); polytope its planes in local axes
+// and, from kMaxFaces, the half-line bounds of its faces: along the line, face
+// f of slope m = e.x bounds the node counter c - iu by C_f - sy_f rv - sz_f rw
+// (above for m > 0, below for m < 0) with sy_f = e.y / m, sz_f = e.z / m, C_f =
+// (T + e.w) / m + fu, sorted into upper, lower and parallel faces (|m| <=
+// kClipFlat: the plane, which keeps or empties the whole line).  POLY: there
+// are polytopes; CUBE: cubes are swept as CubeEval does (its constants in cs),
+// else as cuboids.
+template <bool POLY, bool CUBE>
+struct AnyEval {
+  int kind, iu, iv, iw, nf, nup, ndn;
   float fu, fv, fw;
-  const float4* sp;
-  float cnt_u, ru, rv, rw;
-  float gu, gv, gw;
-  __device__ void load(const PairRec& r, bool second, const Shapes& S, const Parts& D, const Local& L,
+  const float4* cs;
+  float g0, g1, g2;   // band sum: local axes (sphere, polytope), body axes (cuboid), along the normal (wall)
+  __device__ void load(const PairRec& r, bool second, const Shapes& S, const Parts& D, const Local& L, float T,
                        float4* sm) {
+    const int lane = threadIdx.x & 31;
+    kind = second ? r.kinds >> 8 : r.kinds & 0xff;
     const int* ci = second ? r.bi : r.ai;
     const float* cf = second ? r.bf : r.af;
+    const float* rt = second ? r.rtb : r.rta;
+    const float* sz = second ? r.szb : r.sza;
     iu = ci[L.u]; iv = ci[L.v]; iw = ci[L.w];
     fu = cf[L.u]; fv = cf[L.v]; fw = cf[L.w];
-    nf = stage_planes(S, D, second ? r.j : r.i, L, sm, kMaxFaces);
-    sp = sm;
-    gu = gv = gw = 0.f;
-  }
-  __device__ __forceinline__ void begin_line(int cv, int cw, int u0) {
-    rv = static_cast<float>(cv - iv) - fv;
-    rw = static_cast<float>(cw - iw) - fw;
-    cnt_u = static_cast<float>(u0 - iu) - 1.f;
-  }
-  // the half-line bounds of the tile's faces in sp[kMaxFaces ..): faces
-  // bounding from above, then from below, then parallel ones (their planes)
-  __device__ __forceinline__ void prep_clip(const PairRec&, bool, const Local&, float T, float4* cs) {
-    const int lane = threadIdx.x & 31;
-    const bool act = lane < nf;
-    const float4 e = sp[act ? lane : 0];
-    const bool up = act && e.x > kClipFlat, dn = act && e.x < -kClipFlat, par = act && !up && !dn;
-    const unsigned bu = __ballot_sync(kFull, up), bd = __ballot_sync(kFull, dn), bp = __ballot_sync(kFull, par);
-    nup = __popc(bu);
-    ndn = __popc(bd);
-    const unsigned lt = (1u << lane) - 1u;
-    const int pos = up ? __popc(bu & lt) : (dn ? nup + __popc(bd & lt) : nup + ndn + __popc(bp & lt));
-    if (act) {
-      float4 c = e;
-      if (!par) {
-        const float im = __fdividef(1.f, e.x);
-        c = make_float4(e.y * im, e.z * im, fmaf(T + e.w, im, fu), 0.f);
+    cs = sm;
+    nf = nup = ndn = 0;
+    g0 = g1 = g2 = 0.f;
+    if (CUBE && kind == KIND_CUBE) {
+      CubeEval::prep_lanes(r, second, L, T, sm, lane);
+    } else if (POLY && kind == KIND_POLY) {
+      nf = stage_planes(S, D, second ? r.j : r.i, L, sm, kMaxFaces);
+      const bool act = lane < nf;
+      const float4 e = sm[act ? lane : 0];
+      const bool up = act && e.x > kClipFlat, dn = act && e.x < -kClipFlat, par = act && !up && !dn;
+      const unsigned bu = __ballot_sync(kFull, up), bd = __ballot_sync(kFull, dn), bp = __ballot_sync(kFull, par);
+      nup = __popc(bu);
+      ndn = __popc(bd);
+      const unsigned lt = (1u << lane) - 1u;
+      const int pos = up ? __popc(bu & lt) : (dn ? nup + __popc(bd & lt) : nup + ndn + __popc(bp & lt));
+      if (act) {
+        float4 c = e;
+        if (!par) {
+          const float im = __fdividef(1.f, e.x);
+          c = make_float4(e.y * im, e.z * im, fmaf(T + e.w, im, fu), 0.f);
+        }
+        sm[kMaxFaces + pos] = c;
       }
-      cs[kMaxFaces + pos] = c;
+    } else if (kind == KIND_SPHERE) {
+      if (lane == 0) sm[0] = make_float4(sz[0], 0.f, 0.f, 0.f);
+    } else if (kind == KIND_WALL) {
+      if (lane == 0) sm[0] = make_float4(rt[L.u], rt[L.v], rt[L.w], sz[0]);
+      if (lane == 1) sm[1] = make_float4(clip_inv(rt[L.u]), 0.f, 0.f, 0.f);
+    } else {   // cuboids and cubes
+      if (lane < 3) {
+        sm[lane] = make_float4(rt[3 * lane + L.u], rt[3 * lane + L.v], rt[3 * lane + L.w], sz[lane]);
+        reinterpret_cast<float*>(sm + 3)[lane] = clip_inv(rt[3 * lane + L.u]);
+      }
     }
-    __syncwarp();
   }
-  __device__ __forceinline__ void clip_line(const PairRec&, bool, const Local&, const float4*, int cv, int cw,
+  // [lo, hi] (line coordinates) cut to where phi < T on the line (cv, cw)
+  __device__ __forceinline__ void clip_line(const PairRec& r, bool second, const Local& L, const float4*, int cv, int cw,
                                             float T, float& lo, float& hi) const {
-    const float lrv = static_cast<float>(cv - iv) - fv, lrw = static_cast<float>(cw - iw) - fw;
+    if (CUBE && kind == KIND_CUBE) {
+      CubeEval e;
+      e.fetch(cs);
+      e.clip_line(r, second, L, cs, cv, cw, T, lo, hi);
+      return;
+    }
+    const float rv = static_cast<float>(cv - iv) - fv;
+    const float rw = static_cast<float>(cw - iw) - fw;
     const float o = static_cast<float>(iu);
-    const float4* cl = sp + kMaxFaces;
+    if (kind == KIND_WALL) {
+      const float4 m = cs[0];
+      clip_half(m.x, cs[1].x, fmaf(m.y, static_cast<float>(cv), fmaf(m.z, static_cast<float>(cw), m.w)), T, lo, hi);
+      return;
+    }
     float l = lo - o, h = hi - o;
-    int f = 0;
-    for (; f < nup; ++f) {
-      const float4 c = cl[f];
-      h = fminf(h, fmaf(-c.x, lrv, fmaf(-c.y, lrw, c.z)));
-    }
-    for (; f < nup + ndn; ++f) {
-      const float4 c = cl[f];
-      l = fmaxf(l, fmaf(-c.x, lrv, fmaf(-c.y, lrw, c.z)));
-    }
-    for (; f < nf; ++f) {
-      const float4 e = cl[f];
-      if (!(fmaf(-e.x, fu, fmaf(e.y, lrv, fmaf(e.z, lrw, -e.w))) < T)) l = kClipEmpty;
+    if (kind == KIND_SPHERE) {
+      clip_ball(fu, fmaf(rv, rv, rw * rw), cs[0].x, T, l, h);
+    } else if (POLY && kind == KIND_POLY) {
+      const float4* cl = cs + kMaxFaces;
+      int f = 0;
+      for (; f < nup; ++f) {
+        const float4 c = cl[f];
+        h = fminf(h, fmaf(-c.x, rv, fmaf(-c.y, rw, c.z)));
+      }
+      for (; f < nup + ndn; ++f) {
+        const float4 c = cl[f];
+        l = fmaxf(l, fmaf(-c.x, rv, fmaf(-c.y, rw, c.z)));
+      }
+      for (; f < nf; ++f) {
+        const float4 e = cl[f];
+        if (!(fmaf(-e.x, fu, fmaf(e.y, rv, fmaf(e.z, rw, -e.w))) < T)) l = kClipEmpty;
+      }
+    } else {
+      const float4 it = cs[3];
+#pragma unroll
+      for (int k = 0; k < 3; ++k) {
+        const float4 e = cs[k];
+        const float p = fmaf(-e.x, fu, fmaf(e.y, rv, e.z * rw));
+        clip_slab(e.x, k == 0 ? it.x : (k == 1 ? it.y : it.z), p, e.w + T, l, h);
+      }
     }
     lo = l + o;
     hi = h + o;
   }
-  __device__ __forceinline__ float value(int f) const {
-    const float4 e = sp[f];
-    return fmaf(e.x, ru, fmaf(e.y, rv, fmaf(e.z, rw, -e.w)));
-  }
-  __device__ __forceinline__ float phi() {
-    cnt_u += 1.f;
-    ru = cnt_u - fu;
-    int k = 0;
-    float best = value(0);
-    for (int f = 1; f < nf; ++f) {
-      const float v = value(f);
-      if (v > best) { best = v; k = f; }
+  // phi at node (u, cv, cw), and d: the direction that add(m, d) adds m times
+  // (a sphere's d.w scales m)
+  __device__ __forceinline__ float phi(int u, int cv, int cw, float4& d) const {
+    if (CUBE && kind == KIND_CUBE) {
+      CubeEval e;
+      e.fetch(cs);
+      e.begin_node(cs, cv, cw, u);
+      const float f = e.phi();
+      d = e.record(1.f);
+      d = make_float4(d.y, d.z, d.w, 1.f);
+      return f;
     }
-    kbest = k;
-    return best;
+    if (kind == KIND_WALL) {
+      const float4 m = cs[0];
+      d = make_float4(1.f, 0.f, 0.f, 1.f);
+      return fmaf(m.x, static_cast<float>(u), fmaf(m.y, static_cast<float>(cv), fmaf(m.z, static_cast<float>(cw), m.w)));
+    }
+    const float rv = static_cast<float>(cv - iv) - fv;
+    const float rw = static_cast<float>(cw - iw) - fw;
+    const float cnt_u = static_cast<float>(u - iu);
+    if (kind == KIND_SPHERE) {
+      const float ru = cnt_u - fu;
+      const float q = fmaf(ru, ru, fmaf(rv, rv, rw * rw));
+      d = make_float4(ru, rv, rw, q > 0.f ? rsqrtf(q) : 0.f);
+      return sqrtf(q) - cs[0].x;
+    }
+    if (POLY && kind == KIND_POLY) {
+      const float ru = cnt_u - fu;
+      float4 e = cs[0];
+      float best = fmaf(e.x, ru, fmaf(e.y, rv, fmaf(e.z, rw, -e.w)));
+      int k = 0;
+      for (int f = 1; f < nf; ++f) {
+        e = cs[f];
+        const float v = fmaf(e.x, ru, fmaf(e.y, rv, fmaf(e.z, rw, -e.w)));
+        if (v > best) { best = v; k = f; }
+      }
+      e = cs[k];
+      d = make_float4(e.x, e.y, e.z, 1.f);
+      return best;
+    }
+    float y[3], a[3];
+#pragma unroll
+    for (int k = 0; k < 3; ++k) {
+      const float4 e = cs[k];
+      y[k] = fmaf(e.x, cnt_u, fmaf(-e.x, fu, fmaf(e.y, rv, e.z * rw)));
+      a[k] = fabsf(y[k]) - e.w;
+    }
+    // active face: first maximal axis; gradient sign(y_k) e_k (body frame)
+    const bool s0 = a[0] >= a[1] && a[0] >= a[2];
+    const bool s1 = !s0 && a[1] >= a[2];
+    d = make_float4(s0 ? copysignf(1.f, y[0]) : 0.f, s1 ? copysignf(1.f, y[1]) : 0.f,
+                    (!s0 && !s1) ? copysignf(1.f, y[2]) : 0.f, 1.f);
+    return fmaxf(a[0], fmaxf(a[1], a[2]));
   }
-  __device__ __forceinline__ void grad(float m) {
-    const float4 e = sp[kbest];
-    gu = fmaf(m, e.x, gu);
-    gv = fmaf(m, e.y, gv);
-    gw = fmaf(m, e.z, gw);
+  __device__ __forceinline__ void add(float m, const float4& d) {
+    const float mi = m * d.w;
+    g0 = fmaf(mi, d.x, g0);
+    g1 = fmaf(mi, d.y, g1);
+    g2 = fmaf(mi, d.z, g2);
   }
-  __device__ __forceinline__ void end_line() {}
-  __device__ float world(int c, const Local& L, const PairRec&, bool) const { return world_comp(c, L, gu, gv, gw); }
+  // component c of the band sum in the world frame
+  __device__ float world(int c, const Local& L, const PairRec& r, bool second) const {
+    const float* rt = second ? r.rtb : r.rta;
+    if (kind == KIND_WALL) return rt[c] * g0;
+    if (kind == KIND_SPHERE || (POLY && kind == KIND_POLY)) return world_comp(c, L, g0, g1, g2);
+    return rt[c] * g0 + rt[3 + c] * g1 + rt[6 + c] * g2;
+  }
 };
-
-// Fixed wall m . x <= h: phi = m . c + p0 at box-relative node c (lattice
-// units; p0 = the value at the box origin, inflate included, computed in
-// FP64 by the pair builder and kept in the record's size slot; the record's
-// centre of a wall is the box origin).  Box-relative values stay small, so
-// FP32 keeps them to ~1e-6.
-struct WallEval {
-  float mu_, mv_, mw_, p0, imu_;
-  float base, cnt_u, g;
-  __device__ void load(const PairRec& r, bool second, const Shapes&, const Parts&, const Local& L, float4*) {
-    const float* rt = second ? r.rtb : r.rta;   // row 0: the wall normal m (world)
-    mu_ = rt[L.u]; mv_ = rt[L.v]; mw_ = rt[L.w];
-    imu_ = clip_inv(mu_);
-    p0 = second ? r.szb[0] : r.sza[0];
-    g = 0.f;
-  }
-  __device__ __forceinline__ void begin_line(int cv, int cw, int u0) {
-    base = fmaf(mv_, static_cast<float>(cv), fmaf(mw_, static_cast<float>(cw), p0));
-    cnt_u = static_cast<float>(u0) - 1.f;
-  }
-  __device__ __forceinline__ void clip(float T, float& lo, float& hi) const { clip_half(mu_, imu_, base, T, lo, hi); }
-  __device__ __forceinline__ float phi() {
-    cnt_u += 1.f;
-    return fmaf(mu_, cnt_u, base);
-  }
-  __device__ __forceinline__ void grad(float m) { g += m; }
-  __device__ __forceinline__ void end_line() {}
-  __device__ float world(int c, const Local&, const PairRec& r, bool second) const {
-    return (second ? r.rtb : r.rta)[c] * g;
-  }
-};
-
-// Line start of an evaluator: from the shared-memory record when the
-// evaluator re-reads its cross-axis terms there, else from its registers.
-template <class E>
-__device__ __forceinline__ auto begin_line_of(E& e, const PairRec& r, bool second, const Local& L, int cv, int cw,
-                                              int u0, int) -> decltype(e.begin_line_rec(r, second, L, cv, cw, u0)) {
-  e.begin_line_rec(r, second, L, cv, cw, u0);
-}
-template <class E>
-__device__ __forceinline__ void begin_line_of(E& e, const PairRec&, bool, const Local&, int cv, int cw, int u0, long) {
-  e.begin_line(cv, cw, u0);
-}
-
-// Line clip of an evaluator: its own clip_line (per-tile constants staged by
-// prep_clip) where it has one, else the line start and the general clip.
-template <class E>
-__device__ __forceinline__ auto prep_clip_of(E& e, const PairRec& r, bool second, const Local& L, float T, float4* cs,
-                                             int) -> decltype(e.prep_clip(r, second, L, T, cs)) {
-  e.prep_clip(r, second, L, T, cs);
-}
-template <class E>
-__device__ __forceinline__ void prep_clip_of(E&, const PairRec&, bool, const Local&, float, float4*, long) {}
-// Registers from the staged constants (after the warp's sync), where the evaluator keeps them there.
-template <class E>
-__device__ __forceinline__ auto fetch_of(E& e, const float4* cs, int) -> decltype(e.fetch(cs)) {
-  e.fetch(cs);
-}
-template <class E>
-__device__ __forceinline__ void fetch_of(E&, const float4*, long) {}
-template <class E>
-__device__ __forceinline__ auto clip_line_of(E& e, const PairRec& r, bool second, const Local& L, const float4* cs,
-                                             int cv, int cw, float T, float& lo, float& hi, int)
-    -> decltype(e.clip_line(r, second, L, cs, cv, cw, T, lo, hi)) {
-  e.clip_line(r, second, L, cs, cv, cw, T, lo, hi);
-}
-template <class E>
-__device__ __forceinline__ void clip_line_of(E& e, const PairRec& r, bool second, const Local& L, const float4*, int cv,
-                                             int cw, float T, float& lo, float& hi, long) {
-  begin_line_of(e, r, second, L, cv, cw, 0, 0);
-  e.clip(T, lo, hi);
-}
-
-template <class E>
-__device__ __forceinline__ auto node_line_of(E& e, const PairRec&, bool, const Local&, const float4* cs, int cv, int cw,
-                                             int u0, int) -> decltype(e.begin_node(cs, cv, cw, u0)) {
-  e.begin_node(cs, cv, cw, u0);
-}
-template <class E>
-__device__ __forceinline__ void node_line_of(E& e, const PairRec& r, bool second, const Local& L, const float4*,
-                                             int cv, int cw, int u0, long) {
-  begin_line_of(e, r, second, L, cv, cw, u0, 0);
-}
 
 // ---------------------------------------------------------------- tile sweep
 // Per-lane partials of a tile: node count and first moments (exact integers
@@ -581,36 +469,37 @@ __device__ __forceinline__ float key_float(int k) { return __int_as_float(k >= 0
 // of the lanes with nodes, the slot by the owner's counts, and the evaluators
 // start that node's line at the node itself, so the node gets exactly the
 // arithmetic of a node walk (the same FP32 distances, bit for bit).
-// ROLL (the kernel with every kind, nine kind pairs): the slot loops stay
-// rolled, with the slots' clipped ranges in shared memory, to keep the
-// kernel's code small; otherwise they are unrolled over registers.
-template <bool SMOOTH, bool ROLL, bool COOP, class EA, class EB>
+// E: the evaluator of both particles.  With AnyEval the slot loops stay rolled,
+// with the slots' clipped ranges in shared memory, to keep the kernel's code
+// small (unrolled: 38.8 -> 61.8 us on 15472 mixed particles); for two cubes they
+// are unrolled over registers.
+template <bool SMOOTH, bool COOP, class E>
 __device__ __forceinline__ Partial sweep_tile(const Params& P, const Shapes& S, const Parts& D, const PairRec& r,
                                               bool swap, int tl, float4* smA, float4* smB, unsigned* spk,
                                               int4* own, int limit, CoopNode* coop, int nown, int total_in) {
   const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5, nwarp = blockDim.x >> 5;
   const Local L = make_local(r);
-  EA A;
-  EB B;
-  A.load(r, swap, S, D, L, smA);
-  B.load(r, !swap, S, D, L, smB);
+  constexpr bool ROLL = !std::is_same<E, CubeEval>::value;
+  E A, B;
   const int du = r.dim[L.u], dv = r.dim[L.v];
   const float inv_dv = __fdividef(1.f, static_cast<float>(dv));
   const float inv_w = P.inv_w, hw = 0.5f * P.wdx_l, T = hw + kClipMargin;
-  // evaluators with a staged line clip keep its constants in their (otherwise
-  // unused) plane buffer
-  if constexpr (COOP) {
-  } else if constexpr (std::is_same<EA, CubeEval>::value && std::is_same<EB, CubeEval>::value) {
-    // two cubes in one pass: lanes 0 .. 3 form A's constants, lanes 4 .. 7 B's
-    const bool isb = (lane & 4) != 0;
-    CubeEval::prep_lanes(r, isb ? !swap : swap, L, T, isb ? smB : smA, lane < 8 ? (lane & 3) : 4);
+  if constexpr (ROLL) {
+    A.load(r, swap, S, D, L, T, smA);
+    B.load(r, !swap, S, D, L, T, smB);
+    __syncwarp();
   } else {
-    prep_clip_of(A, r, swap, L, T, smA, 0);
-    prep_clip_of(B, r, !swap, L, T, smB, 0);
+    A.clear();
+    B.clear();
+    if constexpr (!COOP) {
+      // two cubes in one pass: lanes 0 .. 3 form A's constants, lanes 4 .. 7 B's
+      const bool isb = (lane & 4) != 0;
+      CubeEval::prep_lanes(r, isb ? !swap : swap, L, T, isb ? smB : smA, lane < 8 ? (lane & 3) : 4);
+    }
+    __syncwarp();
+    A.fetch(smA);
+    B.fetch(smB);
   }
-  __syncwarp();
-  fetch_of(A, smA, 0);
-  fetch_of(B, smB, 0);
   const float4* csA = smA;
   const float4* csB = smB;
   float cnt = 0.f, mu = 0.f, mv = 0.f, mw = 0.f, bestf = -FLT_MAX;
@@ -644,8 +533,8 @@ __device__ __forceinline__ Partial sweep_tile(const Params& P, const Shapes& S, 
         if constexpr (ROLL) cw = div_small(it, dv, inv_dv, &cv);
         const int len = it < r.nitems ? du : 0;
         float clo = 0.f, chi = static_cast<float>(len - 1);
-        clip_line_of(A, r, swap, L, csA, cv, cw, T, clo, chi, 0);
-        clip_line_of(B, r, !swap, L, csB, cv, cw, T, clo, chi, 0);
+        A.clip_line(r, swap, L, csA, cv, cw, T, clo, chi);
+        B.clip_line(r, !swap, L, csB, cv, cw, T, clo, chi);
         int ub;
         const int nk = clip_nodes(clo, chi, 0, len, &ub);
         const unsigned v = static_cast<unsigned>(ub) | (static_cast<unsigned>(nk) << 16);
@@ -740,10 +629,17 @@ __device__ __forceinline__ Partial sweep_tile(const Params& P, const Shapes& S, 
     }
     int ocv;
     const int ocw = div_small(it0 + os * 32 + o, dv, inv_dv, &ocv);
-    node_line_of(A, r, swap, L, csA, ocv, ocw, u, 0);
-    node_line_of(B, r, !swap, L, csB, ocv, ocw, u, 0);
-    const float fa = A.phi();
-    const float fb = B.phi();
+    float fa, fb;
+    float4 da, db;
+    if constexpr (ROLL) {
+      fa = A.phi(u, ocv, ocw, da);
+      fb = B.phi(u, ocv, ocw, db);
+    } else {
+      A.begin_node(csA, ocv, ocw, u);
+      B.begin_node(csB, ocv, ocw, u);
+      fa = A.phi();
+      fb = B.phi();
+    }
     // W > 0, or a band term of the normal: max < w/2 and (sharp) min <= 0
     const bool any = g < total && fmaxf(fa, fb) < hw && (SMOOTH || fminf(fa, fb) <= 0.f);
     const float ta = __saturatef(fmaf(fa, -inv_w, 0.5f));
@@ -800,10 +696,13 @@ __device__ __forceinline__ Partial sweep_tile(const Params& P, const Shapes& S, 
         bestf = f;
         bestidx = idx;
       }
-      A.grad(ma);
-      B.grad(mb);
-      A.end_line();
-      B.end_line();
+      if constexpr (ROLL) {
+        A.add(ma, da);
+        B.add(mb, db);
+      } else {
+        A.grad(ma);
+        B.grad(mb);
+      }
     }
   }
   Partial o;
@@ -979,55 +878,10 @@ template <bool SMOOTH, int SET, bool COOP>
 __device__ __forceinline__ Partial dispatch(const Params& P, const Shapes& S, const Parts& D, const PairRec& r,
                                             int tl, float4* smA, float4* smB, unsigned* spk, int4* own, int limit,
                                             CoopNode* coop, int nown, int total) {
-  int ka = r.kinds & 0xff, kb = r.kinds >> 8;
   // evaluate the cheaper kind as A (G's sign flips back below); two cubes keep the record's order
-  const bool swap = SET == SET_CUBE ? false : sweep_swap(ka, kb);
-  if (swap) {
-    const int t = ka; ka = kb; kb = t;
-  }
-  if (SET == SET_ALL) {   // the full variant sweeps cubes as cuboids
-    ka = ka == KIND_CUBE ? KIND_CUBOID : ka;
-    kb = kb == KIND_CUBE ? KIND_CUBOID : kb;
-  }
-  Partial o{0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, -FLT_MAX, 0x7fffffff, false, false, 0, 0};
-  if constexpr (SET == SET_CUBE) {
-    return sweep_tile<SMOOTH, false, COOP, CubeEval, CubeEval>(P, S, D, r, swap, tl, smA, smB, spk, own, limit, coop,
-                                                               nown, total);
-  }
-#define GBC_CASE(KA, KB, TA, TB)                                                  \
-  case (KA) * 8 + (KB):                                                          \
-    o = sweep_tile<SMOOTH, SET == SET_ALL, false, TA, TB>(P, S, D, r, swap, tl, smA, smB, spk, own, limit, nullptr, 0, 0); \
-    break;
-  if constexpr (SET == SET_SC) {
-    switch (ka * 8 + kb) {
-      GBC_CASE(0, 0, SphereEval, SphereEval)
-      GBC_CASE(0, 4, SphereEval, CubeEval)
-      GBC_CASE(0, 1, SphereEval, CuboidEval)
-      GBC_CASE(4, 4, CubeEval, CubeEval)
-      GBC_CASE(4, 1, CubeEval, CuboidEval)
-      GBC_CASE(1, 1, CuboidEval, CuboidEval)
-      GBC_CASE(5, 0, WallEval, SphereEval)
-      GBC_CASE(5, 4, WallEval, CubeEval)
-      GBC_CASE(5, 1, WallEval, CuboidEval)
-      default:
-        break;
-    }
-  } else if constexpr (SET == SET_ALL) {
-    switch (ka * 8 + kb) {
-      GBC_CASE(0, 0, SphereEval, SphereEval)
-      GBC_CASE(0, 1, SphereEval, CuboidEval)
-      GBC_CASE(0, 3, SphereEval, PolyEval)
-      GBC_CASE(1, 1, CuboidEval, CuboidEval)
-      GBC_CASE(1, 3, CuboidEval, PolyEval)
-      GBC_CASE(3, 3, PolyEval, PolyEval)
-      GBC_CASE(5, 0, WallEval, SphereEval)
-      GBC_CASE(5, 1, WallEval, CuboidEval)
-      GBC_CASE(5, 3, WallEval, PolyEval)
-      default:
-        break;
-    }
-  }
-#undef GBC_CASE
+  const bool swap = SET == SET_CUBE ? false : sweep_swap(r.kinds & 0xff, r.kinds >> 8);
+  using E = typename std::conditional<SET == SET_CUBE, CubeEval, AnyEval<SET == SET_ALL, SET == SET_SC>>::type;
+  Partial o = sweep_tile<SMOOTH, COOP, E>(P, S, D, r, swap, tl, smA, smB, spk, own, limit, coop, nown, total);
   if (swap) {
     o.gx = -o.gx; o.gy = -o.gy; o.gz = -o.gz;
   }
@@ -1058,8 +912,8 @@ __global__ void __launch_bounds__(narrow_warps<SET>() * 32, narrow_blocks<SET>()
   constexpr int NW = narrow_warps<SET>();
   __shared__ __align__(16) PairRec s_rec[NW][2];
   // per evaluator: a polytope's planes, then its line clip's constants (a cube: the clip constants)
-  __shared__ float4 s_planes[NW][2][SET == SET_CUBE ? 8 : 2 * kMaxFaces];
-  __shared__ unsigned s_pk[SET == SET_ALL ? NW : 1][kTileItemsPerLane * 32];   // clipped ranges (rolled sweep)
+  __shared__ float4 s_planes[NW][2][SET == SET_ALL ? 2 * kMaxFaces : 8];
+  __shared__ unsigned s_pk[SET == SET_CUBE ? 1 : NW][kTileItemsPerLane * 32];   // clipped ranges (rolled sweep)
   __shared__ int4 s_own[NW][64];   // the lanes with clipped nodes (sweep_tile)
   // tiles shared by the block: in the cubes-only variant (the others hold nine
   // kind pairs, and the second sweep of each would cost their instruction
@@ -1095,7 +949,7 @@ __global__ void __launch_bounds__(narrow_warps<SET>() * 32, narrow_blocks<SET>()
     const PairRec& r = s_rec[wid][buf];
     if (record_in_bounds(P, W.err, r, true)) {
       const Partial o = dispatch<SMOOTH, SET, false>(P, S, D, r, r.tile, s_planes[wid][0], s_planes[wid][1],
-                                                     s_pk[SET == SET_ALL ? wid : 0], s_own[wid],
+                                                     s_pk[SET == SET_CUBE ? 0 : wid], s_own[wid],
                                                      share ? kShareNodes : 0x7fffffff, nullptr, 0, 0);
       if (!o.deferred) tile_done(W, r, o.touched ? reduce_tile<SMOOTH>(o) : empty_partial());
       else if (lane == 0) s_deferred[atomicAdd_block(&s_ndeferred, 1)] = make_int3(wid, o.nown, o.total);
@@ -1228,40 +1082,6 @@ __global__ void __launch_bounds__(kWarps * 32, 1) k_force(Params P, Shapes S, Pa
 // node of the pair box in FP64 spent 1006 us on 1934 cubes at 30 % (2.64e6
 // nodes, 1 % of which add to the sums); the clipped sweep takes 31 us.
 
-// [lo, hi] (line coordinates) cut to where one particle's distance lies below
-// T on the line (cv, cw); sp: a polytope's planes in local axes (stage_planes).
-template <class E>
-__device__ __forceinline__ void clip_with(const Shapes& S, const Parts& D, const PairRec& r, bool second,
-                                          const Local& L, int cv, int cw, float T, float& lo, float& hi) {
-  E e;
-  e.load(r, second, S, D, L, nullptr);
-  e.begin_line(cv, cw, 0);
-  e.clip(T, lo, hi);
-}
-__device__ __forceinline__ void clip_any(const Shapes& S, const Parts& D, const PairRec& r, bool second,
-                                         const Local& L, const float4* sp, int nf, int cv, int cw, float T, float& lo,
-                                         float& hi) {
-  switch (second ? r.kinds >> 8 : r.kinds & 0xff) {   // warp-uniform
-    case KIND_SPHERE: clip_with<SphereEval>(S, D, r, second, L, cv, cw, T, lo, hi); break;
-    case KIND_WALL: clip_with<WallEval>(S, D, r, second, L, cv, cw, T, lo, hi); break;
-    case KIND_POLY: {
-      const int* ci = second ? r.bi : r.ai;
-      const float* cf = second ? r.bf : r.af;
-      const float rv = static_cast<float>(cv - ci[L.v]) - cf[L.v], rw = static_cast<float>(cw - ci[L.w]) - cf[L.w];
-      const float o = static_cast<float>(ci[L.u]), fu = cf[L.u];
-      float l = lo - o, h = hi - o;
-      for (int f = 0; f < nf; ++f) {
-        const float4 e = sp[f];
-        clip_half(e.x, clip_inv(e.x), fmaf(-e.x, fu, fmaf(e.y, rv, fmaf(e.z, rw, -e.w))), T, l, h);
-      }
-      lo = l + o;
-      hi = h + o;
-      break;
-    }
-    default: clip_with<CuboidEval>(S, D, r, second, L, cv, cw, T, lo, hi); break;   // cubes and cuboids
-  }
-}
-
 // Sums of v[0 .. 8) over the warp by halving exchanges (nine FP64 additions):
 // lane c < 8 returns the sum of component c.
 __device__ __forceinline__ double warp_sum8(const double v[8]) {
@@ -1334,7 +1154,7 @@ __device__ __forceinline__ void tile_done64(const Lists& W, const PairRec& r, do
 template <bool SMOOTH>
 __global__ void __launch_bounds__(kWarps * 32, 2) k_narrow64(Params P, Shapes S, Parts D, Lists W) {
   __shared__ __align__(16) PairRec s_rec[kWarps];
-  __shared__ float4 s_planes[kWarps][2][kMaxFaces];
+  __shared__ float4 s_planes[kWarps][2][2 * kMaxFaces];       // the clips' constants
   __shared__ unsigned s_pk[kWarps][kTileItemsPerLane * 32];   // clipped ranges: first node | count << 16
   __shared__ int s_excl[kWarps][32];                          // nodes before each lane's
   pdl_begin();
@@ -1352,9 +1172,10 @@ __global__ void __launch_bounds__(kWarps * 32, 2) k_narrow64(Params P, Shapes S,
     if (!record_in_bounds(P, W.err, r, true)) continue;   // warp-uniform (checked build only)
     const Local L = make_local(r);
     const int i = r.i, j = r.j;
-    const int ka = r.kinds & 0xff, kb = r.kinds >> 8;
-    const int fa = ka == KIND_POLY ? stage_planes(S, D, i, L, s_planes[wid][0], kMaxFaces) : 0;
-    const int fb = kb == KIND_POLY ? stage_planes(S, D, j, L, s_planes[wid][1], kMaxFaces) : 0;
+    AnyEval<true, false> A, B;
+    A.load(r, false, S, D, L, T, s_planes[wid][0]);
+    B.load(r, true, S, D, L, T, s_planes[wid][1]);
+    __syncwarp();
     // both particles in FP64 (the same address on every lane)
     double XA[3], XB[3], RA[9], RB[9];
 #pragma unroll
@@ -1383,8 +1204,8 @@ __global__ void __launch_bounds__(kWarps * 32, 2) k_narrow64(Params P, Shapes S,
       const int cw = div_small(it, dv, inv_dv, &cv);
       const int len = it < r.nitems ? du : 0;
       float clo = 0.f, chi = static_cast<float>(len - 1);
-      clip_any(S, D, r, false, L, s_planes[wid][0], fa, cv, cw, T, clo, chi);
-      clip_any(S, D, r, true, L, s_planes[wid][1], fb, cv, cw, T, clo, chi);
+      A.clip_line(r, false, L, nullptr, cv, cw, T, clo, chi);
+      B.clip_line(r, true, L, nullptr, cv, cw, T, clo, chi);
       int ub;
       const int nk = clip_nodes(clo, chi, 0, len, &ub);
       s_pk[wid][s * 32 + lane] = static_cast<unsigned>(ub) | (static_cast<unsigned>(nk) << 16);
