@@ -42,6 +42,7 @@ constexpr int kTapeDoubles = 16;      // FP64 per-pair values kept for the adjoi
 constexpr int kStepCounter = 12;      // counters[] slot of the completed-step count
 constexpr int kDoneCounter = 13;      // counters[] slot: particle-sum blocks finished (the last resets it)
 constexpr int kTokenCounter = 14;     // counters[] slot: the host's token of this step
+constexpr int kAdjCounter = 15;       // counters[] slot: tiles the adjoint's cell sweep took from its queue
 constexpr int kFtDoubles = 9;         // per-pair F, T_A, T_B
 
 // Error codes written by kernels (same numbering as contact_status).

@@ -270,15 +270,22 @@ __device__ __forceinline__ void pair_force_law(ForceArgs a, const OvlRec* e, int
                      t2b = __shfl_sync(kFull, t2, b0 + 2);
       utn2 = (t0 + t1) + t2b;
     }
-    // two more reciprocal square roots: of ddot_n (lane 0, a new contact's
-    // c = damp_K / ddot_n) and of |u_t|^2 (lane 1)
-    double inv_ddot = 0.0, inv_utn = 0.0;
+    // three more reciprocal square roots: of ddot_n (lane 0, a new contact's
+    // c = damp_K / ddot_n), of |u_t|^2 (lane 1) and of the friction law's
+    // denominator (a^4 + 1)(a^2 + 1), a = |u_t| / u_k (lane 2: an FP64 division
+    // costs as many instructions as all three)
+    double inv_ddot = 0.0, inv_utn = 0.0, inv_den = 0.0, a2 = 0.0, den1 = 1.0, den2 = 1.0;
     const bool dpos = __double_as_longlong(ddot) > 0, upos = __double_as_longlong(utn2) > 0;
     if (LAW && (a.history || a.friction)) {
-      const double y5 = nr_rsqrt(k == 0 ? (dpos ? ddot : 1.0) : (upos ? utn2 : 1.0));
-      const double ya = __shfl_sync(kFull, y5, b0), yb = __shfl_sync(kFull, y5, b0 + 1);
+      a2 = utn2 * (a.inv_u_k * a.inv_u_k);
+      den1 = fma(a2, a2, 1.0);
+      den2 = a2 + 1.0;
+      const bool fast = a2 < 1e30;   // (above, the coefficient is mu_k)
+      const double y5 = nr_rsqrt(k == 0 ? (dpos ? ddot : 1.0) : (k == 1 ? (upos ? utn2 : 1.0) : (fast ? den1 * den2 : 1.0)));
+      const double ya = __shfl_sync(kFull, y5, b0), yb = __shfl_sync(kFull, y5, b0 + 1), yc = __shfl_sync(kFull, y5, b0 + 2);
       inv_ddot = dpos ? ya * ya : 0.0;
       inv_utn = upos ? yb : 0.0;
+      inv_den = fast ? yc * yc : 0.0;
     }
     double cdamp = a.damping_c;   // c of Eq. (damping_factor) for this pair
     if (LAW && a.history) {
@@ -317,13 +324,8 @@ __device__ __forceinline__ void pair_force_law(ForceArgs a, const OvlRec* e, int
     if (LAW && a.friction && __double_as_longlong(fmag) > 0 && upos) {
       // Eq. (contact_force_tangential): B receives +f(a) |F_n| t, a = |u_t| / u_k,
       // f = (2 mu_s* - mu_k) a^2 / (a^4 + 1) + mu_k a^2 / (a^2 + 1)
-      const double sa = utn2 * inv_utn * a.inv_u_k;
-      const double a2 = sa * sa;
       double coef = a.mu_k;
-      if (a2 < 1e30) {
-        const double den1 = fma(a2, a2, 1.0), den2 = a2 + 1.0;
-        coef = a2 * fma(2.0 * a.mu_s_star - a.mu_k, den2, a.mu_k * den1) / (den1 * den2);
-      }
+      if (a2 < 1e30) coef = a2 * fma(2.0 * a.mu_s_star - a.mu_k, den2, a.mu_k * den1) * inv_den;
       Fk = fma(coef * fmag, utk * inv_utn, Fk);
     }
     const double F1 = __shfl_sync(kFull, Fk, b0 + k1), F2 = __shfl_sync(kFull, Fk, b0 + k2);

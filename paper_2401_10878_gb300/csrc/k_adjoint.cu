@@ -255,23 +255,36 @@ __device__ __forceinline__ void adj_pre_pass(const Params& P, const Shapes& S, c
     }
     // friction, Eq. (contact_force_tangential): F = fmag (n + f(a) t), t = u_t / |u_t|,
     // u_t = u_AB - ddot_n n, a = |u_t| / u_k
+    // (1 / |u_t| and the reciprocals of a^4 + 1, a^2 + 1 and the damping factor by
+    // one reciprocal square root each, on lanes 0 .. 3: the divisions and the square
+    // root cost about a hundred FP64 instructions a pass)
     bool fric = false;
-    double tdir = 0.0, coef = 0.0, dcoef = 0.0, utn = 0.0;
-    if (P.friction && vel != nullptr) {
+    double tdir = 0.0, coef = 0.0, dcoef = 0.0, inv_utn = 0.0, inv_damp = 0.0;
+    if (vel != nullptr) {
       const double ut = uab - ddot * nk;
-      const double utn2 = sum3(ut * ut);
+      double utn2 = 0.0, a2 = 0.0;
+      if (P.friction) {
+        utn2 = sum3(ut * ut);
+        a2 = utn2 * (P.inv_u_k * P.inv_u_k);
+      }
       fric = fmag > 0.0 && utn2 > 0.0;
+      const bool slip = a2 < 1e30;   // (above, the coefficient is mu_k)
+      const double den1 = fma(a2, a2, 1.0), den2 = a2 + 1.0;
+      const double arg = k == 0 ? utn2 : (k == 1 ? den1 : (k == 2 ? den2 : damp));
+      const double yr = fl::nr_rsqrt(arg > 0.0 && arg < 1e60 ? arg : 1.0);
+      inv_utn = at(yr, 0);
+      const double i1 = at(yr, 1) * at(yr, 1), i2 = at(yr, 2) * at(yr, 2);
+      inv_damp = __shfl_sync(kFull, yr, b0 + 3);
+      inv_damp *= inv_damp;
       if (fric) {
-        utn = sqrt(utn2);
-        tdir = ut / utn;
-        const double a = utn * P.inv_u_k, a2 = a * a;
+        tdir = ut * inv_utn;
         const double A = 2.0 * P.mu_s_star - P.mu_k;
         coef = P.mu_k;
-        if (a2 < 1e30) {
-          const double den1 = a2 * a2 + 1.0, den2 = a2 + 1.0;
-          coef = a2 * (A * den2 + P.mu_k * den1) / (den1 * den2);
+        if (slip) {
+          const double a = utn2 * inv_utn * P.inv_u_k;
+          coef = a2 * (A * den2 + P.mu_k * den1) * (i1 * i2);
           // f'(a) = 2a [A (1 - a^4) / (a^4 + 1)^2 + mu_k / (a^2 + 1)^2]
-          dcoef = 2.0 * a * (A * (1.0 - a2 * a2) / (den1 * den1) + P.mu_k / (den2 * den2));
+          dcoef = 2.0 * a * (A * (1.0 - a2 * a2) * (i1 * i1) + P.mu_k * (i2 * i2));
         }
         Fk += fmag * coef * tdir;
       }
@@ -290,7 +303,7 @@ __device__ __forceinline__ void adj_pre_pass(const Params& P, const Shapes& S, c
     double guab = 0.0;   // dL/du_AB
     if (__any_sync(kFull, fric)) {
       // through t (projected on its normal plane) and through f(a)
-      const double s_dir = fric ? fmag * coef / utn : 0.0, s_mag = fmag * Lt * dcoef * P.inv_u_k;
+      const double s_dir = fric ? fmag * coef * inv_utn : 0.0, s_mag = fmag * Lt * dcoef * P.inv_u_k;
       const double gut = s_dir * (Lam - Lt * tdir) + s_mag * tdir;
       const double gun = sum3(gut * nk);
       if (fric) {
@@ -310,7 +323,7 @@ __device__ __forceinline__ void adj_pre_pass(const Params& P, const Shapes& S, c
       gV = half_lf * inv_S0 * (P.inv_dx * P.inv_dx * P.inv_dx);
       gd = half_lf * (yd * yd);
       if (vel != nullptr && cdamp != 0.0 && damp > 0.0) {
-        const double gdd = Lm * fmag * cdamp / damp;   // dL/d(ddot_n)
+        const double gdd = Lm * fmag * cdamp * inv_damp;   // dL/d(ddot_n)
         gn += gdd * uab;
         guab += gdd * nk;
       }
@@ -382,6 +395,7 @@ __global__ void __launch_bounds__(32) k_adj_pre(Params P, Shapes S, Parts D, Lis
                                                  const double* __restrict__ gT) {
   __shared__ int s_q[32 + 8];   // overlapping pairs waiting for a pass
   pdl_begin();
+  if (blockIdx.x == 0 && threadIdx.x == 0) W.counters[kAdjCounter] = 0;   // the cell sweep's queue
   const int lane = threadIdx.x & 31, slot = lane >> 2;
   const int np = min(W.counters[0], P.max_pairs);
   const int nw = gridDim.x, gw = blockIdx.x;   // one-warp blocks
@@ -698,9 +712,14 @@ __global__ void __launch_bounds__(kAdjWarps * 32, adj_blocks<SET>()) k_adj_cells
   unsigned* spk = s_pk[ROLL ? wid : 0];
   // tiles w, w + W, ... of the forward's list (W warps): each record is staged
   // in shared memory, the next record and its pair's seeds are fetched while
-  // a tile runs
+  // a tile runs.  From four tiles per warp on, the tiles after the first two of
+  // each warp come from a queue, the one after the next asked for during a tile:
+  // a tile of a pair without overlap costs a twentieth of a polytope pair's, and
+  // with a fixed share the last warp ran 1.7 times the mean (47 -> 45 us on
+  // 15472 mixed particles).
   const int nwarps = gridDim.x * kAdjWarps;
-  int qpos = blockIdx.x * kAdjWarps + wid;
+  const bool queue = ntiles > 4 * nwarps;
+  int qpos = blockIdx.x * kAdjWarps + wid, qn = qpos + nwarps;
   float seed = 0.f;
   if (qpos < ntiles) {
     const int4 v = adj_rec_part(W.tiles + qpos, lane);
@@ -710,7 +729,8 @@ __global__ void __launch_bounds__(kAdjWarps * 32, adj_blocks<SET>()) k_adj_cells
   __syncwarp();
   int buf = 0;
   while (qpos < ntiles) {
-    const int qn = qpos + nwarps;
+    int ahead = 0;
+    if (queue && lane == 0) ahead = atomicAdd(&W.counters[kAdjCounter], 1);
     int4 next = make_int4(0, 0, 0, 0);
     float seed_n = 0.f;
     if (qn < ntiles) {
@@ -937,6 +957,7 @@ __global__ void __launch_bounds__(kAdjWarps * 32, adj_blocks<SET>()) k_adj_cells
     __syncwarp();
     buf ^= 1;
     qpos = qn;
+    qn = queue ? 2 * nwarps + __shfl_sync(kFull, ahead, 0) : qn + nwarps;
     seed = seed_n;
   }
 }
