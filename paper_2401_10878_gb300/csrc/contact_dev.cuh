@@ -493,6 +493,32 @@ void launch_pose(const Params& P, const Shapes& S, const Parts& D, const Lists& 
 void launch_broad(const Params& P, const Parts& D, const Lists& W, cudaStream_t st);
 void launch_plan(const Params& P, const Parts& D, const Lists& W, int32_t* pair_ij, int32_t* n_pairs,
                  double* pair_out, cudaStream_t st);
+// Whether the FP64 kernels over the overlapping pairs gather them by blocks, so
+// that their passes of eight pairs are full: above 4096 particles.  Below, every
+// chunk of 16 pairs has a warp of its own and a pass of three pairs takes as
+// long as one of eight, while gathering would lengthen the step's chain.
+__host__ __device__ inline bool gather_overlaps(const Params& P) { return P.n > 4096; }
+constexpr int kGatherPairs = 1024;   // pairs gathered at a time
+
+// The overlapping pairs among [q0, q0 + cnt), cnt <= kGatherPairs, to s_q (in
+// any order: every pair is treated on its own), by the whole block; returns
+// their number.  s_n: a shared counter.
+__device__ __forceinline__ int gather_pairs(const int* oflag, int q0, int cnt, int* s_q, int* s_n) {
+  __syncthreads();   // (the entries of the round before)
+  if (threadIdx.x == 0) *s_n = 0;
+  __syncthreads();
+  const unsigned lane = threadIdx.x & 31;
+  for (int x = threadIdx.x; x < ((cnt + 31) & ~31); x += blockDim.x) {
+    const bool flag = x < cnt && oflag[q0 + x] != 0;
+    const unsigned m = __ballot_sync(0xffffffffu, flag);
+    int at = 0;
+    if (lane == 0 && m != 0u) at = atomicAdd_block(s_n, __popc(m));
+    at = __shfl_sync(0xffffffffu, at, 0);
+    if (flag) s_q[at + __popc(m & ((1u << lane) - 1u))] = q0 + x;
+  }
+  __syncthreads();
+  return *s_n;
+}
 constexpr int kRowGroup = 256;   // particles per group sum of the pair-row offsets
 // the row length of bin_cap entries, and whether BinRec's lengths suffice for particles of circumradius rmax
 inline int bin_row(int bin_cap) { return (bin_cap + 3) & ~3; }

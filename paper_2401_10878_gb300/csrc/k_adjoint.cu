@@ -384,53 +384,48 @@ __device__ __forceinline__ void adj_pre_pass(const Params& P, const Shapes& S, c
   }
 }
 
-// Eight pairs per pass.  Up to one pass per warp every warp takes eight
-// consecutive pairs, whether they overlap or not (gathering the overlapping
-// ones first cost a longer chain: the 1934 cubes' backward 41.2 -> 45.1 us).
-// Larger steps give each warp a contiguous range, zero its pairs' seeds and
-// gradients with consecutive lanes, and pass the overlapping pairs on eight at
-// a time: 84.8 -> 39.8 us on 15472 mixed particles (7304 of 38585 pairs overlap).
-__global__ void __launch_bounds__(32) k_adj_pre(Params P, Shapes S, Parts D, Lists W, AdjBufs B,
-                                                 const double* __restrict__ vel, const double* __restrict__ gF,
-                                                 const double* __restrict__ gT) {
-  __shared__ int s_q[32 + 8];   // overlapping pairs waiting for a pass
+// Eight pairs per pass.  GATHER = false (up to 4096 particles): one-warp blocks,
+// every warp takes eight consecutive pairs at a time, whether they overlap or
+// not (gathering the overlapping ones first cost a longer chain: the 1934
+// cubes' backward 41.2 -> 45.1 us).  GATHER = true: each block collects the
+// overlapping pairs of its range, zeroes the seeds and gradients of the others
+// with consecutive lanes, and its warps take passes of eight: 84.8 us over all
+// pairs, 36.0 us gathered by single warps, 23.5 us by blocks on 15472 mixed
+// particles (7304 of 38585 pairs overlap).
+constexpr int kPreWarps = 8;
+template <bool GATHER>
+__global__ void __launch_bounds__(GATHER ? kPreWarps * 32 : 32, GATHER ? 2 : 1) k_adj_pre(
+    Params P, Shapes S, Parts D, Lists W, AdjBufs B, const double* __restrict__ vel, const double* __restrict__ gF,
+    const double* __restrict__ gT) {
+  __shared__ int s_q[GATHER ? kGatherPairs : 1], s_n;
   pdl_begin();
   if (blockIdx.x == 0 && threadIdx.x == 0) W.counters[kAdjCounter] = 0;   // the cell sweep's queue
-  const int lane = threadIdx.x & 31, slot = lane >> 2;
+  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5, slot = lane >> 2;
   const int np = min(W.counters[0], P.max_pairs);
-  const int nw = gridDim.x, gw = blockIdx.x;   // one-warp blocks
-  const bool direct = np <= 8 * nw;
-  const int per = direct ? 8 : (((np + nw - 1) / nw) + 31) & ~31;
-  int qb = per * gw, n = 0;   // next pair of the warp's range, pairs waiting
-  const int q1 = min(qb + per, np);
-  if (qb >= q1) return;
-  for (;;) {
-    int p = qb + slot;
-    bool inr = p < q1;
-    if (!direct) {
-      while (n < 8 && qb < q1) {
-        const int q = qb + lane, cnt = min(32, q1 - qb);
-        const bool flag = lane < cnt && W.oflag[q] != 0;
-        const unsigned mask = __ballot_sync(kFull, flag);
-        float4* zs = reinterpret_cast<float4*>(B.seeds + static_cast<size_t>(qb) * kSeedFloats);
-        for (int x = lane; x < cnt * (kSeedFloats / 4); x += 32) zs[x] = make_float4(0.f, 0.f, 0.f, 0.f);
-        double2* zp = reinterpret_cast<double2*>(B.pgrad + static_cast<size_t>(qb) * kPairGrad);
-        for (int x = lane; x < cnt * (kPairGrad / 2); x += 32) zp[x] = make_double2(0.0, 0.0);
-        if (lane < cnt) B.done[q] = 0;
-        if (flag) s_q[n + __popc(mask & ((1u << lane) - 1u))] = q;
-        n += __popc(mask);
-        qb += 32;
-        __syncwarp();   // (the zeros of a pair come before its pass's values)
+  if constexpr (GATHER) {
+    const int per = (np + gridDim.x - 1) / gridDim.x;
+    const int q1 = min(per * static_cast<int>(blockIdx.x + 1), np);
+    // (two blocks per SM, the second one's passes two sub-partitions on)
+    const int w = (wid + (blockIdx.x >= gridDim.x / 2 ? 2 : 0)) % kPreWarps;
+    for (int q0 = per * static_cast<int>(blockIdx.x); q0 < q1; q0 += kGatherPairs) {
+      const int all = min(kGatherPairs, q1 - q0);
+      const int cnt = gather_pairs(W.oflag, q0, all, s_q, &s_n);
+      for (int e0 = 8 * w; e0 < cnt; e0 += 8 * kPreWarps) {
+        const bool inr = e0 + slot < cnt;
+        adj_pre_pass(P, S, D, W, B, vel, gF, gT, inr ? s_q[e0 + slot] : 0, inr, true);
       }
-      if (n == 0) return;
-      const int m = min(n, 8);
-      n -= m;
-      inr = slot < m;
-      p = inr ? s_q[n + slot] : 0;
+      float4* zs = reinterpret_cast<float4*>(B.seeds + static_cast<size_t>(q0) * kSeedFloats);
+      for (int x = threadIdx.x; x < all * (kSeedFloats / 4); x += blockDim.x)
+        if (W.oflag[q0 + x / (kSeedFloats / 4)] == 0) zs[x] = make_float4(0.f, 0.f, 0.f, 0.f);
+      double2* zp = reinterpret_cast<double2*>(B.pgrad + static_cast<size_t>(q0) * kPairGrad);
+      for (int x = threadIdx.x; x < all * (kPairGrad / 2); x += blockDim.x)
+        if (W.oflag[q0 + x / (kPairGrad / 2)] == 0) zp[x] = make_double2(0.0, 0.0);
+      for (int x = threadIdx.x; x < all; x += blockDim.x)
+        if (W.oflag[q0 + x] == 0) B.done[q0 + x] = 0;
     }
-    adj_pre_pass(P, S, D, W, B, vel, gF, gT, p, inr, !direct);
-    if (direct) return;
-    __syncwarp();
+  } else {
+    for (int e0 = 8 * blockIdx.x; e0 < np; e0 += 8 * gridDim.x)
+      adj_pre_pass(P, S, D, W, B, vel, gF, gT, e0 + slot, e0 + slot < np, false);
   }
 }
 
@@ -1042,7 +1037,10 @@ void launch_adjoint(const Params& P, const Shapes& S, const Parts& D, const List
   B.done = reinterpret_cast<int*>(B.pgrad + static_cast<size_t>(P.max_pairs) * kPairGrad);
   const int wneed0 = (P.max_pairs + 7) / 8;   // pre: eight pairs per warp pass
   const int wgrid0 = wneed0 < 8 * kSms ? (wneed0 > 0 ? wneed0 : 1) : 8 * kSms;
-  launch_pdl(k_adj_pre, dim3(wgrid0), dim3(32), 0, st, P, S, D, W, B, vel, gF, gT);
+  if (gather_overlaps(P))
+    launch_pdl(k_adj_pre<true>, dim3(2 * kSms), dim3(kPreWarps * 32), 0, st, P, S, D, W, B, vel, gF, gT);
+  else
+    launch_pdl(k_adj_pre<false>, dim3(wgrid0), dim3(32), 0, st, P, S, D, W, B, vel, gF, gT);
   // compiled per kind set, as the node sweep (2 cubes only, 1 spheres / cuboids / walls, 0 every kind)
   auto cells = P.kind_set == 2 ? k_adj_cells<2> : (P.kind_set == 1 ? k_adj_cells<1> : k_adj_cells<0>);
   if (ev0 != nullptr) cudaEventRecord(ev0, st);

@@ -978,85 +978,35 @@ __global__ void __launch_bounds__(narrow_warps<SET>() * 32, narrow_blocks<SET>()
 // The force law of the step's overlapping pairs, up to eight per warp pass
 // (four lanes each).  Bound: the FP64 pipe (one warp instruction per ~64 cycles
 // and sub-partition) and, with one pass per warp, the latency of its chain.
-//   * Up to one chunk of 16 consecutive pairs per warp (1216 warps): chunk c =
-//     b + grid * w for warp w of block b; the pairs' overlap flags and, in the
-//     same round of loads, all 16 entries of the overlap list (the flagged ones
-//     are kept, in pair order), so one memory round trip precedes the pass.
-//     With one block per SM the chunks land on different sub-partitions, so
-//     the passes run side by side.
-//   * Larger steps: a contiguous range of pairs per warp, its flagged pairs
-//     collected first and passed on eight at a time.  Chunks of 16 filled 2.7
-//     of the eight slots of a pass (one pair in six overlaps): 44.5 -> 31.8 us
-//     on 52218 cubes (29242 overlapping pairs of 175090), 22.8 -> 20.7 us with
-//     the whole contact law on 15472 spheres and cuboids.
-// Each warp adds its count of overlapping pairs to counters[5] (reported by
+//   * GATHER = false (up to 4096 particles): chunks of 16 consecutive pairs,
+//     chunk c = b + grid * w (then c + grid * 8, ...) for warp w of block b; the
+//     pairs' overlap flags and, in the same round of loads, all 16 entries of
+//     the overlap list (the flagged ones are kept, in pair order), so one memory
+//     round trip precedes the pass.  With one block per SM the chunks land on
+//     different sub-partitions, so the passes run side by side.
+//   * GATHER = true: each block collects the flagged pairs of its range, and its
+//     warps take passes of eight.  Chunks of 16 filled 2.7 of the eight slots of
+//     a pass (one pair in six overlaps), the ranges of single warps 4.7: 44.5 ->
+//     31.0 -> 19.9 us on 52218 cubes (29242 overlapping pairs of 175090), 22.8 ->
+//     20.1 -> 13.9 us with the whole contact law on 15472 spheres and cuboids.  (A
+//     list written by the node sweep gave 17.5 and 12.2 us but cost the sweep
+//     4.5 us, one atomic per pair or per 32.)
+// The count of overlapping pairs goes to counters[5] (reported by
 // contact_stats).
 constexpr int kForceChunk = 16;
 
-template <int SET, bool LAW>
-__global__ void __launch_bounds__(kWarps * 32, 1) k_force(Params P, Shapes S, Parts D, Lists W, const double* vel,
-                                                       double* pair_out) {
-  __shared__ __align__(16) OvlRec s_ovl[kWarps][kForceChunk];
-  __shared__ int s_q[kWarps][32 + kForcePairsPerPass];   // flagged pairs waiting for a pass (larger steps)
+template <int SET, bool LAW, bool GATHER>
+__global__ void __launch_bounds__(kWarps * 32, GATHER ? 2 : 1) k_force(Params P, Shapes S, Parts D, Lists W,
+                                                                       const double* vel, double* pair_out) {
+  __shared__ __align__(16) OvlRec s_ovl[kWarps][GATHER ? kForcePairsPerPass : kForceChunk];
+  __shared__ int s_q[GATHER ? kGatherPairs : 1], s_n;
   pdl_begin();
   if (W.counters[1] > P.max_tiles) return;   // the node sweep did not run (ECAPACITY)
   const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
   const int np = min(W.counters[0], P.max_pairs);
-  const int nwarps = gridDim.x * kWarps, c = blockIdx.x + gridDim.x * wid;
   constexpr int kPieces = static_cast<int>(sizeof(OvlRec) / 16);          // 16-byte pieces per entry
-  constexpr int kPerLane = kForceChunk * kPieces / 32;                    // pieces of a chunk per lane
   int4* dst = reinterpret_cast<int4*>(s_ovl[wid]);
-  const bool direct = np <= kForceChunk * nwarps;
-  const int per = direct ? kForceChunk : (((np + nwarps - 1) / nwarps) + 31) & ~31;
-  int qb = per * c;   // next pair of the warp's range
-  const int q1 = min(qb + per, np);
-  if (qb >= q1) return;
-  int nov = 0, nwait = 0;   // overlapping pairs, pairs waiting in s_q
-  unsigned mask = 0;        // direct: the chunk's flagged pairs
-  int4 piece[kPerLane];
-  if (direct) {
-    const bool flag = lane < kForceChunk && qb + lane < q1 && W.oflag[qb + lane] != 0;
-#pragma unroll
-    for (int u = 0; u < kPerLane; ++u) {   // entry e / kPieces, part e % kPieces of the chunk
-      const int e = lane + 32 * u;
-      const int qe = qb + e / kPieces;
-      piece[u] = qe < q1 ? reinterpret_cast<const int4*>(W.olist + qe)[e % kPieces] : make_int4(0, 0, 0, 0);
-    }
-    mask = __ballot_sync(kFull, flag);
-    nov = __popc(mask);
-  }
-  for (;;) {
-    int n;   // pairs of this pass, staged in pair order
-    if (direct) {
-      if (mask == 0u) break;
-      n = min(__popc(mask), kForcePairsPerPass);
-      unsigned take = mask;   // the lowest n flagged entries (all of them but in a rare 9th+)
-      if (n < __popc(mask)) take = mask & ((1u << __fns(mask, 0, n + 1)) - 1u);   // below the (n+1)-th
-#pragma unroll
-      for (int u = 0; u < kPerLane; ++u) {
-        const int e = lane + 32 * u, r = e / kPieces;
-        if ((take >> r) & 1u) dst[__popc(take & ((1u << r) - 1u)) * kPieces + e % kPieces] = piece[u];
-      }
-      mask &= ~take;
-    } else {
-      while (nwait < kForcePairsPerPass && qb < q1) {
-        const bool flag = qb + lane < q1 && W.oflag[qb + lane] != 0;
-        const unsigned m = __ballot_sync(kFull, flag);
-        if (flag) s_q[wid][nwait + __popc(m & ((1u << lane) - 1u))] = qb + lane;
-        nwait += __popc(m);
-        nov += __popc(m);
-        qb += 32;
-        __syncwarp();
-      }
-      if (nwait == 0) break;
-      n = min(nwait, kForcePairsPerPass);
-      nwait -= n;
-#pragma unroll
-      for (int u = 0; u < kForcePairsPerPass * kPieces / 32; ++u) {
-        const int e = lane + 32 * u, r = e / kPieces;
-        if (r < n) dst[e] = reinterpret_cast<const int4*>(W.olist + s_q[wid][nwait + r])[e % kPieces];
-      }
-    }
+  auto pass = [&](int n) {   // the n staged entries
     __syncwarp();
 #ifdef CONTACT_CHECKS
     if (lane < n) {   // the staged entries' pair and particles
@@ -1068,6 +1018,56 @@ __global__ void __launch_bounds__(kWarps * 32, 1) k_force(Params P, Shapes S, Pa
     __syncwarp();
 #endif
     flush_overlaps<SET, LAW>(P, S, D, W, vel, pair_out, s_ovl[wid], n);
+  };
+  int nov = 0;
+  if constexpr (GATHER) {
+    const int per = (np + gridDim.x - 1) / gridDim.x;
+    const int q1 = min(per * static_cast<int>(blockIdx.x + 1), np);
+    // (two blocks per SM, the second one's passes two sub-partitions on)
+    const int w = (wid + (blockIdx.x >= gridDim.x / 2 ? 2 : 0)) % kWarps;
+    for (int q0 = per * static_cast<int>(blockIdx.x); q0 < q1; q0 += kGatherPairs) {
+      const int cnt = gather_pairs(W.oflag, q0, min(kGatherPairs, q1 - q0), s_q, &s_n);
+      if (threadIdx.x == 0) nov += cnt;
+      for (int e0 = kForcePairsPerPass * w; e0 < cnt; e0 += kForcePairsPerPass * kWarps) {
+        const int n = min(kForcePairsPerPass, cnt - e0);
+#pragma unroll
+        for (int u = 0; u < kForcePairsPerPass * kPieces / 32; ++u) {   // entry e / kPieces, part e % kPieces
+          const int e = lane + 32 * u, r = e / kPieces;
+          if (r < n) dst[e] = reinterpret_cast<const int4*>(W.olist + s_q[e0 + r])[e % kPieces];
+        }
+        pass(n);
+      }
+    }
+  } else {
+    const int nchunk = (np + kForceChunk - 1) / kForceChunk;
+    constexpr int kPerLane = kForceChunk * kPieces / 32;                    // pieces per lane
+    for (int c = blockIdx.x + gridDim.x * wid; c < nchunk; c += gridDim.x * kWarps) {
+      const int q0 = kForceChunk * c;
+      const int q = q0 + lane;
+      const bool flag = lane < kForceChunk && q < np && W.oflag[q] != 0;
+      int4 piece[kPerLane];
+#pragma unroll
+      for (int u = 0; u < kPerLane; ++u) {   // entry e / kPieces, part e % kPieces of the chunk
+        const int e = lane + 32 * u;
+        const int qe = q0 + e / kPieces;
+        piece[u] = qe < np ? reinterpret_cast<const int4*>(W.olist + qe)[e % kPieces] : make_int4(0, 0, 0, 0);
+      }
+      unsigned mask = __ballot_sync(kFull, flag);
+      nov += __popc(mask);
+      while (mask != 0u) {
+        const int n = min(__popc(mask), kForcePairsPerPass);
+        // keep the next n flagged entries, packed in pair order
+        unsigned take = mask;   // the lowest n flagged entries (all of them but in a rare 9th+)
+        if (n < __popc(mask)) take = mask & ((1u << __fns(mask, 0, n + 1)) - 1u);   // below the (n+1)-th
+#pragma unroll
+        for (int u = 0; u < kPerLane; ++u) {
+          const int e = lane + 32 * u, r = e / kPieces;
+          if ((take >> r) & 1u) dst[__popc(take & ((1u << r) - 1u)) * kPieces + e % kPieces] = piece[u];
+        }
+        mask &= ~take;
+        pass(n);
+      }
+    }
   }
   if (lane == 0 && nov > 0) atomicAdd(&W.counters[5], nov);
 }
@@ -1324,9 +1324,12 @@ void launch_force(const Params& P, const Shapes& S, const Parts& D, const Lists&
   // compiled per kind set (cubes only, or any) and with or without the
   // velocity-dependent law (damping from velocities, contact history, friction)
   const bool law = P.history || P.friction || (vel != nullptr && P.damping_c != 0.0);
-  auto kern = P.kind_set == 2 ? (law ? k_force<2, true> : k_force<2, false>)
-                              : (law ? k_force<0, true> : k_force<0, false>);
-  launch_pdl(kern, dim3(sms > 0 ? sms : 1), dim3(kWarps * 32), 0, st, P, S, D, W, vel, pair_out);
+  const bool gather = gather_overlaps(P);
+  auto kern = P.kind_set == 2 ? (law ? (gather ? k_force<2, true, true> : k_force<2, true, false>)
+                                     : (gather ? k_force<2, false, true> : k_force<2, false, false>))
+                              : (law ? (gather ? k_force<0, true, true> : k_force<0, true, false>)
+                                     : (gather ? k_force<0, false, true> : k_force<0, false, false>));
+  launch_pdl(kern, dim3((gather ? 2 : 1) * (sms > 0 ? sms : 1)), dim3(kWarps * 32), 0, st, P, S, D, W, vel, pair_out);
 }
 
 void launch_narrow(const Params& P, const Shapes& S, const Parts& D, const Lists& W, const double* vel,

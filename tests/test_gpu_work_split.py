@@ -130,3 +130,50 @@ def test_pair_count_of_the_last_step(max_pairs):
         assert e.value.code == ECAPACITY
     assert m.lib.contact_pair_count(m.ctx, ctypes.byref(n)) == 0 and n.value == int(m.n_pairs.item()) > 8
     m.close()
+
+
+def _lattice_state(n, indicator=0):
+    """n small spheres, cubes and tetrahedra-like polytopes on a jittered grid, most touching a neighbour."""
+    rng = np.random.default_rng(n)
+    k = int(np.ceil(n ** (1.0 / 3.0)))
+    g = np.stack(np.meshgrid(*[np.arange(k)] * 3, indexing="ij"), -1).reshape(-1, 3)[:n]
+    step = 6.0
+    pos = (g + 0.5) * step + rng.uniform(-0.6, 0.6, size=(n, 3))
+    pl = W.random_polytope(rng, 12, 4.0)[0]
+    t = np.array([W.SPHERE, W.CUBOID, W.POLYTOPE])[np.arange(n) % 3]
+    params = np.where(t[:, None] == W.SPHERE, [[3.0, 0.0, 0.0]], [[2.5, 2.5, 2.5]])
+    return state(t, params, pos, quat=W.random_quaternions(rng, n), n=int(k * step),
+                 planes=[pl if x == W.POLYTOPE else None for x in t], indicator=indicator)
+
+
+# around the sizes where the pair kernels gather by blocks (4096) and a pose warp takes 32 particles (6080)
+@pytest.mark.parametrize("n", [4095, 4096, 4097, 6080, 6081, 6097])
+@pytest.mark.parametrize("precision", [0, 1])
+def test_larger_steps(n, precision):
+    rep, ref = _parity(_lattice_state(n), precision)
+    assert np.count_nonzero(ref.pair_out[:, 0]) > n // 4
+
+
+@pytest.mark.parametrize("law", [False, True])
+def test_larger_step_and_adjoint_equal_the_smaller(law):
+    """One more particle, alone in the box, takes the step from single chunks to
+    gathered blocks: the other 4096 keep their outputs and gradients bit for bit."""
+    from paper_2401_10878_gb300.contact import Contact
+    st = _lattice_state(4097, indicator=1)
+    st.pos[4096] = np.array([15.5, 8.5, 8.5]) * 6.0
+    rng = np.random.default_rng(1)
+    vel = torch.tensor(rng.normal(size=(4097, 6)) * 0.02, device="cuda") if law else None
+    kw = dict(friction=True, mu_s=0.3, mu_k=0.2, u_k=0.01, damping_c=0.4) if law else {}
+    gf, gt = (torch.tensor(w, device="cuda") for w in W.loss_weights(4097))
+    outs = []
+    for n in (4097, 4096):
+        s = st.subset(np.arange(n))
+        m = Contact.from_state(s, **kw)
+        o = m.step(torch.tensor(s.pos, device="cuda"), torch.tensor(s.quat, device="cuda"), None if vel is None else vel[:n].contiguous())
+        gp, gq = m.backward(gf[:n].contiguous(), gt[:n].contiguous())
+        outs.append([o["pair_ij"].clone(), o["pair_out"].clone(), o["force"][:4096].clone(), o["torque"][:4096].clone(),
+                     gp[:4096], gq[:4096]])
+        assert m.stats()["overlapping"] > 1000
+        m.close()
+    for a, b in zip(*outs):
+        assert torch.equal(a, b)
