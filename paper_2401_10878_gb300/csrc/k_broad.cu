@@ -328,19 +328,35 @@ __global__ void k_pose_poly(Params P, Shapes S, Parts D, Lists W) {
 // 4 R_max + 2 dx every range is shorter than n/2, so no other image can meet it.
 __device__ __forceinline__ int image_shift(int d, int n) { return d > (n >> 1) ? 1 : (d < -(n >> 1) ? -1 : 0); }
 
-// K3: one warp per particle p.  Lane b < 27 owns neighbour bin b of the
-// fixed-capacity cell list (only its own one along an axis of one bin); the
-// bin's entries (node range and particle, one 16-byte and one 4-byte word each)
-// are read four at a time and tested against p's node range, moved by the
-// bin's periodic image; the hits are collected with warp ballots and each goes
-// to its rank among the partners above (j > p) or below (j < p).  Bound:
-// instruction issue, and on small boxes load latency.  With the ranges in the
-// bins a candidate costs one load wavefront and no dependent load (nine
-// scattered words of its particle before): 84.1 -> 61.6 us on 52218 cubes (58
-// candidates each); with bin coordinates kept per particle (no divisions), the
-// image of a bin instead of a candidate's, one unsigned comparison per axis and
-// one list for both sides and four blocks per SM, 50.0 us.
-__global__ void __launch_bounds__(256, 4) k_broad(Params P, Parts D, Lists W) {
+// K3: LP lanes per particle p (a warp, or half of one).  The lanes share out
+// the 27 neighbour bins of the fixed-capacity cell list (only its own one along
+// an axis of one bin), number the bins' entries by a scan of the counts and
+// write the entries' places to a list in shared memory; then LP entries at a
+// time (node range and particle, one 16-byte and one 4-byte word) are tested
+// against p's node range.  The hits are collected with warp ballots and each
+// goes to its rank among the partners above (j > p) or below (j < p).  Bound:
+// instruction issue on large boxes, load latency on small ones.  A lane that
+// walks its own bin makes as many rounds as the fullest of the 27 has entries,
+// with 58 candidates in 160 lanes, each in a line of its own, and the set-up and
+// the ranks of one particle's 7 hits leave most of a warp idle: on 52218 cubes
+// 48 us with a bin per lane, 37 with four lanes per bin and two particles a warp,
+// 38 with the list, 29.4 with the list and two particles a warp (32 with four);
+// 15472 mixed particles 20.0 -> 13.4 us, 1934 cubes 6.05 -> 5.4 us (a warp each).
+constexpr int kBroadWarps = 4;   // warps of a block
+constexpr int kBroadList = 96;   // candidates of one particle listed at a time
+static_assert(kRowGroup % (2 * kBroadWarps) == 0, "the particles of a block share one row group");
+static_assert(kBroadList % 32 == 0, "the list is read by whole warps");
+// Two particles per warp from where warps of one particle each fill every SM
+// sub-partition with eight: fewer leave latency and not issue as the bound (a
+// warp each against half a warp: 5.4 and 6.0 us at 1934 cubes, 13.9 and 11.7 us
+// at 15472 spheres and cuboids).
+inline bool broad_halves(const Params& P) { return P.n > 8 * 4 * kSms; }
+
+template <int LP>
+__global__ void __launch_bounds__(kBroadWarps * 32, 8) k_broad(Params P, Parts D, Lists W) {
+  constexpr int PW = 32 / LP;                // particles of a warp
+  constexpr int BPL = (27 + LP - 1) / LP;    // bins of a lane
+  constexpr unsigned kGroup = LP == 32 ? kFull : (1u << (LP & 31)) - 1u;
   extern __shared__ int s_buf[];
   // the block's partner count (its particles share one row group), added
   // to the group sum by the block's last warp to finish: one global atomic per block
@@ -352,109 +368,135 @@ __global__ void __launch_bounds__(256, 4) k_broad(Params P, Parts D, Lists W) {
   __syncthreads();
   pdl_begin();
   const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-  const int p = blockIdx.x * (blockDim.x >> 5) + wid;
-  const int nw = static_cast<int>(blockDim.x >> 5);
+  const int grp = lane / LP, hl = lane % LP, g0 = lane - hl;
+  const int slot = PW * wid + grp;   // the particle's place in the block
+  const int p = blockIdx.x * PW * kBroadWarps + slot;
   auto group_sum = [&](int nup) {
     if (lane == 0) {
       if (nup > 0) atomicAdd_block(&s_gsum, nup);
       __threadfence_block();
-      if (atomicAdd_block(&s_gdone, 1) == nw - 1) {   // every warp's count is in
+      if (atomicAdd_block(&s_gdone, 1) == kBroadWarps - 1) {   // every warp's count is in
         __threadfence_block();
         const int tot = atomicAdd_block(&s_gsum, 0);
-        if (tot > 0) atomicAdd(&W.grp_sum[(blockIdx.x * nw) / kRowGroup], tot);
+        if (tot > 0) atomicAdd(&W.grp_sum[(blockIdx.x * PW * kBroadWarps) / kRowGroup], tot);
       }
     }
   };
-  if (p >= P.n) {
+  if (p - grp >= P.n) {   // (uniform) none of the warp's particles
     group_sum(0);
     return;
   }
   const int cap = P.max_nbr;
-  int* hits = s_buf + wid * 2 * cap;   // at most cap partners on either side, else ECAPACITY
-  const int4 own_lo = reinterpret_cast<const int4*>(D.rec + p)[0], own_hi = reinterpret_cast<const int4*>(D.rec + p)[1];
+  unsigned* list = reinterpret_cast<unsigned*>(s_buf) + slot * kBroadList;   // bin entries to test
+  int* hits = s_buf + PW * kBroadWarps * kBroadList + slot * 2 * cap;   // at most cap partners on either side, else ECAPACITY
+  const bool own = p < P.n;
+  const int4* own_rec = reinterpret_cast<const int4*>(D.rec + (own ? p : P.n - 1));
+  const int4 own_lo = own_rec[0], own_hi = own_rec[1];
   const int bin = own_hi.w;
   const int plo[3] = {own_lo.x, own_lo.y, own_lo.z}, phi[3] = {own_hi.x, own_hi.y, own_hi.z};
-  const bool nodes = plo[0] <= phi[0] && plo[1] <= phi[1] && plo[2] <= phi[2];
-  // the lane's bin, and p's corner (plus one) in its image: the particles of a
-  // bin beyond the boundary lie one period away.  (Bins are at least 2 R_max +
-  // 2 dx wide, so a partner in any other image is out of reach.)
-  const int off[3] = {lane % 3, (lane / 3) % 3, lane / 9};
-  int c[3], corner[3];
-  bool use = lane < 27 && nodes;
+  const bool nodes = own && plo[0] <= phi[0] && plo[1] <= phi[1] && plo[2] <= phi[2];
+  // the lane's bins: first entry and count
+  unsigned row[BPL];
+  int num[BPL];
+  bool wrapped = false;   // a bin beyond the boundary: its particles lie one period away
 #pragma unroll
-  for (int k = 0; k < 3; ++k) {
-    const int nb = P.nbin[k];
-    c[k] = ((bin >> (8 * k)) & 0xff) + off[k] - 1;
-    corner[k] = plo[k] + 1;
-    if (c[k] < 0) {
-      c[k] += nb;
-      corner[k] += P.ncell[k];
-    } else if (c[k] >= nb) {
-      c[k] -= nb;
-      corner[k] -= P.ncell[k];
+  for (int s = 0; s < BPL; ++s) {
+    const int b = hl + LP * s;
+    const int off[3] = {b % 3, (b / 3) % 3, b / 9};
+    int c[3];
+    bool use = b < 27 && nodes;
+#pragma unroll
+    for (int k = 0; k < 3; ++k) {
+      const int nb = P.nbin[k];
+      c[k] = ((bin >> (8 * k)) & 0xff) + off[k] - 1;
+      use = use && (nb >= 3 || off[k] == 1);
+      if (c[k] < 0 || c[k] >= nb) {
+        c[k] += c[k] < 0 ? nb : -nb;
+        wrapped = true;
+      }
     }
-    use = use && (nb >= 3 || off[k] == 1);
+    row[s] = 0;
+    num[s] = 0;
+    if (use) {
+      const int q = checked_index(W.err, c[0] + P.nbin[0] * (c[1] + P.nbin[1] * c[2]),
+                                  static_cast<long long>(P.nbin[0]) * P.nbin[1] * P.nbin[2], 0);
+      row[s] = static_cast<unsigned>(q) * static_cast<unsigned>(P.bin_stride);
+      num[s] = min(W.bin_count[q], P.bin_cap);
+    }
   }
-  int num = 0;
-  size_t row = 0;
-  int4 ids = make_int4(-1, -1, -1, -1), recs[4];   // the bin's next four entries (the first ones fetched with its count)
+  // their entries numbered lane by lane
+  int total = 0;
 #pragma unroll
-  for (int u = 0; u < 4; ++u) recs[u] = make_int4(0, 0, 0, 0);
-  const int4* bin_rec = reinterpret_cast<const int4*>(W.bin_rec);
-  if (use) {
-    const int q = checked_index(W.err, c[0] + P.nbin[0] * (c[1] + P.nbin[1] * c[2]),
-                                static_cast<long long>(P.nbin[0]) * P.nbin[1] * P.nbin[2], 0);
-    row = static_cast<size_t>(q) * P.bin_stride;   // (a multiple of four; entries past the count are stale and unused)
-    ids = *reinterpret_cast<const int4*>(W.bin_items + row);
+  for (int s = 0; s < BPL; ++s) total += num[s];
+  int start = total;
 #pragma unroll
-    for (int u = 0; u < 4; ++u) recs[u] = bin_rec[row + u];
-    num = min(W.bin_count[q], P.bin_cap);
+  for (int d = 1; d < LP; d <<= 1) {
+    const int up = __shfl_up_sync(kFull, start, d, LP);
+    if (hl >= d) start += up;
   }
-  const int maxn = __reduce_max_sync(kFull, num);
-  const bool one_bin = P.nbin[0] < 3 || P.nbin[1] < 3 || P.nbin[2] < 3;
+  start -= total;
+  total = __shfl_sync(kFull, start + total, LP - 1, LP);
+  const int most = PW == 1 ? total : __reduce_max_sync(kFull, total);
+  const bool image = __any_sync(kFull, wrapped) || P.nbin[0] < 3 || P.nbin[1] < 3 || P.nbin[2] < 3;
   const int reach[3] = {phi[0] - plo[0], phi[1] - plo[1], phi[2] - plo[2]};
-  const unsigned below = (1u << lane) - 1u;
+  const unsigned mine = kGroup << g0, below = ((1u << lane) - 1u) & mine;
+  const int4* bin_rec = reinterpret_cast<const int4*>(W.bin_rec);
   int nhit = 0;
-  for (int t0 = 0; t0 < maxn; t0 += 4) {
-    const int jj[4] = {ids.x, ids.y, ids.z, ids.w};
-    const bool more = t0 + 4 < num;
-    if (more) ids = *reinterpret_cast<const int4*>(W.bin_items + row + t0 + 4);
+  for (int w0 = 0; w0 < most; w0 += kBroadList) {   // (one window but for crowded bins)
+    int at = start - w0;
 #pragma unroll
-    for (int u = 0; u < 4; ++u) {
-      if (t0 + u >= maxn) break;   // warp-uniform
-      const int j = t0 + u < num ? checked_index(W.err, jj[u], P.n, p) : p;
-      int d[3] = {recs[u].x - corner[0], recs[u].y - corner[1], recs[u].z - corner[2]};
-      int len[3] = {recs[u].w & kMaxLen, (recs[u].w >> 10) & kMaxLen, recs[u].w >> 20};
-      if (more) recs[u] = bin_rec[row + t0 + 4 + u];   // (the next round's entry, under way during this one)
-      if (one_bin) {   // (uniform) the candidate's own image along an axis of one bin
+    for (int s = 0; s < BPL; ++s) {
+      const int e1 = min(num[s], kBroadList - at);
+#pragma unroll 1
+      for (int e = max(0, -at); e < e1; ++e) list[at + e] = row[s] + static_cast<unsigned>(e);
+      at += num[s];
+    }
+    __syncwarp();
+    const int end = min(total - w0, kBroadList), last = min(most - w0, kBroadList);
+    int4 rec = make_int4(0, 0, 0, 0);
+    int id = -1;
+    auto fetch = [&](int c) {
+      if (c < end) {
+        const unsigned e = list[c];
+        rec = bin_rec[e];
+        id = W.bin_items[e];
+      }
+    };
+    fetch(hl);
+    for (int c = hl; c - hl < last; c += LP) {
+      const int j = c < end ? checked_index(W.err, id, P.n, p) : p;
+      int d[3] = {rec.x - plo[0], rec.y - plo[1], rec.z - plo[2]};
+      int len[3] = {rec.w & kMaxLen, (rec.w >> 10) & kMaxLen, rec.w >> 20};
+      fetch(c + LP);   // (the next round's entry, under way during this one)
+      if (image) {   // (uniform) the candidate's nearest image
 #pragma unroll
-        for (int k = 0; k < 3; ++k)
-          if (P.nbin[k] < 3) d[k] -= image_shift(d[k] + 1, P.ncell[k]) * P.ncell[k];
+        for (int k = 0; k < 3; ++k) d[k] -= image_shift(d[k], P.ncell[k]) * P.ncell[k];
       }
       if (P.wide && j != p) {   // (uniform) ranges beyond kMaxLen nodes
 #pragma unroll
         for (int k = 0; k < 3; ++k) len[k] = D.rec[j].hi[k] - D.rec[j].lo[k] + 1;
       }
       // the ranges share a node: the partner's corner lies above p's by at most
-      // p's reach and below it by less than its own length, -len < d + 1 <= reach
+      // p's reach and below it by less than its own length, -len < d <= reach
       bool hit = j != p;
 #pragma unroll
       for (int k = 0; k < 3; ++k)
-        hit = hit && static_cast<unsigned>(d[k] + len[k]) < static_cast<unsigned>(reach[k] + len[k]);
+        hit = hit && static_cast<unsigned>(d[k] + len[k] - 1) < static_cast<unsigned>(reach[k] + len[k]);
       const unsigned bh = __ballot_sync(kFull, hit);
       if (hit) {
-        const int at = nhit + __popc(bh & below);
-        if (at < 2 * cap) hits[at] = j;
+        const int to = nhit + __popc(bh & below);
+        if (to < 2 * cap) hits[to] = j;
       }
-      nhit += __popc(bh);
+      nhit += __popc(bh & mine);
     }
+    __syncwarp();
   }
   // walls (partners n + w, after every particle): lane w tests wall w with an
   // FP32 prefilter, then exactly in FP64 (the node box must be non-empty)
-  for (int w0 = 0; w0 < P.nwall; w0 += 32) {
-    const int w = w0 + lane;
+  for (int w0 = 0; w0 < P.nwall; w0 += LP) {
+    const int w = w0 + hl;
     bool hit = false;
-    if (w < P.nwall) {
+    if (own && w < P.nwall) {
       const double* e = P.wall + 4 * w;
       const float m0 = static_cast<float>(e[0]), m1 = static_cast<float>(e[1]), m2 = static_cast<float>(e[2]);
       const float dxf = static_cast<float>(P.dx);
@@ -476,16 +518,17 @@ __global__ void __launch_bounds__(256, 4) k_broad(Params P, Parts D, Lists W) {
       const int at = nhit + __popc(bw & below);
       if (at < 2 * cap) hits[at] = P.n + w;
     }
-    nhit += __popc(bw);
+    nhit += __popc(bw & mine);
   }
   const bool over = nhit > 2 * cap;   // (then one side has more than cap)
   nhit = min(nhit, 2 * cap);
   __syncwarp();
   // each hit to its rank on its side (unique keys): above, the hits in (p, v);
   // below, those in [0, v)
+  const int longest = PW == 1 ? nhit : __reduce_max_sync(kFull, nhit);
   int nup = 0;
-  for (int e0 = 0; e0 < nhit; e0 += 32) {
-    const int e = e0 + lane;
+  for (int e0 = 0; e0 < longest; e0 += LP) {
+    const int e = e0 + hl;
     const int v = e < nhit ? hits[e] : -1;
     const bool up = v > p;
     const int from = up ? p + 1 : 0;
@@ -493,19 +536,20 @@ __global__ void __launch_bounds__(256, 4) k_broad(Params P, Parts D, Lists W) {
     int r = 0;
     for (int x = 0; x < nhit; ++x) r += static_cast<unsigned>(hits[x] - from) < key ? 1 : 0;
     if (e < nhit && r < cap) (up ? W.up_list : W.dn_list)[static_cast<size_t>(p) * cap + r] = v;
-    nup += __popc(__ballot_sync(kFull, e < nhit && up));
+    __syncwarp();
+    nup += __popc(__ballot_sync(kFull, e < nhit && up) & mine);
   }
   int ndn = nhit - nup;
   if (over || nup > cap || ndn > cap) {
-    if (lane == 0) set_error(W.err, kErrCapacity);
+    if (hl == 0) set_error(W.err, kErrCapacity);
     nup = min(nup, cap);
     ndn = min(ndn, cap);
   }
-  if (lane == 0) {
+  if (hl == 0 && own) {
     W.up_count[p] = nup;
     W.dn_count[p] = ndn;
   }
-  group_sum(nup);
+  group_sum(PW == 1 ? nup : nup + __shfl_xor_sync(kFull, nup, 16));
 }
 
 
@@ -1030,10 +1074,13 @@ void launch_pose(const Params& P, const Shapes& S, const Parts& D, const Lists& 
 
 
 void launch_broad(const Params& P, const Parts& D, const Lists& W, cudaStream_t st) {
-  const int warps = 8;
-  const int nb = (P.n + warps - 1) / warps;
-  const size_t smem = static_cast<size_t>(warps) * 2 * P.max_nbr * sizeof(int);
-  if (nb > 0) launch_pdl(k_broad, dim3(nb), dim3(warps * 32), smem, st, P, D, W);
+  const bool halves = broad_halves(P);
+  const int pw = halves ? 2 : 1;   // particles of a warp
+  const size_t each = (kBroadList + 2 * static_cast<size_t>(P.max_nbr)) * sizeof(int);
+  const int per = kBroadWarps * pw;   // particles of a block (at most 512 partners each: 36 KB)
+  const int nb = (P.n + per - 1) / per;
+  if (nb > 0)
+    launch_pdl(halves ? k_broad<16> : k_broad<32>, dim3(nb), dim3(kBroadWarps * 32), per * each, st, P, D, W);
 }
 
 void launch_plan(const Params& P, const Parts& D, const Lists& W, int32_t* pair_ij, int32_t* n_pairs,

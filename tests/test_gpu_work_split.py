@@ -73,6 +73,31 @@ def test_broad_phase_long_ranges(half, gap):
     assert ref.n_pairs == (1 if gap < 8.0 else 0) and np.all(ref.pair_out[:, 0] > 0)
 
 
+# candidates of one particle: at and around the 96 listed at a time, then the
+# most particles of one warp each and the fewest of half a warp each (odd and even)
+@pytest.mark.parametrize("n", [94, 95, 96, 97, 191, 192, 193, 215, 4864, 4865, 4866])
+@pytest.mark.parametrize("corner", [30.3, -9.6])
+def test_broad_phase_crowded_bins(n, corner):
+    """Small spheres on a jittered lattice around a larger one that sets the
+    bins' width, inside the box and across its corner; more of them spread over
+    the box for the larger counts."""
+    rng = np.random.default_rng(n)
+    box = 160 if n > 215 else 64
+    a = np.stack(np.meshgrid(*[np.arange(6)] * 3, indexing="ij"), -1).reshape(-1, 3)
+    x = corner + 3.4 * a + rng.uniform(-0.4, 0.4, (216, 3))
+    if n > 215:
+        g = np.stack(np.meshgrid(*[np.arange(18)] * 3, indexing="ij"), -1).reshape(-1, 3)
+        f = 8.8 * g + 4.0 + rng.uniform(-0.4, 0.4, g.shape)
+        near = np.all(np.abs(f - (corner + 8.5) - box * np.round((f - (corner + 8.5)) / box)) < 14.0, axis=1)
+        x = np.concatenate([x, f[~near]])
+    order = rng.permutation(n)
+    x = np.mod(x[:n][order], box)
+    r = np.where(order == 61, 4.4, 2.1)
+    st = state([W.SPHERE] * n, np.stack([r, 0 * r, 0 * r], 1), x, n=box)
+    rep, ref = _parity(st, 0)
+    assert ref.n_pairs > 60
+
+
 # one line and sample per direction up to the most, around the 32 lanes of a warp
 @pytest.mark.parametrize("nc", [1, 2, 5, 6, 7, 33])
 @pytest.mark.parametrize("kinds", ["grid", "cubes_walls", "polytopes"])
