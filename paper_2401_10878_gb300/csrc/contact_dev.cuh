@@ -308,7 +308,7 @@ struct Lists {
   double* partial64;   // [max_tiles, kPartialDoubles] (the all-FP64 form only, else null)
   int* pdone;       // [max_pairs] tiles of the pair swept so far (pairs of several tiles)
   double* tape;     // [max_pairs, kTapeDoubles]
-  double* ft;       // [max_pairs, kFtDoubles]
+  double* ft;       // [max_pairs, kFtDoubles] (node sweep: of the overlapping pairs alone)
   const int* kind;  // [N] sweep kind of each particle (Kind, polytopes by face bucket)
   BoxWork* box_work;   // [max_pairs] box pipeline: the pairs with a rough contact
   int* counters;    // [16]: 0 pairs, 1 tiles, 2 box pipeline rough contacts, 5 overlapping pairs, kStepCounter

@@ -1021,9 +1021,11 @@ __global__ void __launch_bounds__(32) k_build_pairs(Params P, Parts D, Lists W, 
       const size_t q0 = static_cast<size_t>(row_base) + base;
       const int np = max(0, min(min(32, total - base), P.max_pairs - (row_base + base)));
       double* po = pair_out + q0 * 11;
-      double* pf = W.ft + q0 * kFtDoubles;
       for (int x = lane; x < 11 * np; x += 32) po[x] = 0.0;
-      for (int x = lane; x < kFtDoubles * np; x += 32) pf[x] = 0.0;
+      if constexpr (BOXM) {   // (the node sweep's pairs are read by their flag)
+        double* pf = W.ft + q0 * kFtDoubles;
+        for (int x = lane; x < kFtDoubles * np; x += 32) pf[x] = 0.0;
+      }
       if (lane < np) {
         W.oflag[q0 + lane] = 0;
         W.pdone[q0 + lane] = 0;

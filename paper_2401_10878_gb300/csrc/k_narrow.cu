@@ -934,7 +934,7 @@ __global__ void __launch_bounds__(narrow_warps<SET>() * 32, narrow_blocks<SET>()
   if (ntiles > P.max_tiles) return;   // capacity exceeded: the step reports ECAPACITY
   // with at most one tile per warp a tile of many node passes would be the
   // kernel's tail: it is left for the whole block, whose other warps are done
-  // (400 cubes, one in seven pressed into a neighbour: 16.0 -> @COOP@ us)
+  // (400 cubes, one in seven pressed into a neighbour: 16.0 -> 11.9 us)
   const bool share = kShare && ntiles <= nwarps;
   if (share) {
     if (threadIdx.x == 0) s_ndeferred = 0;

@@ -61,6 +61,34 @@ def test_pair_builder_rows(n_small):
     assert np.sum(ref.pair_ij[:, 0] == 0) == n_small
 
 
+# partners of one particle around the eight read at a time, overlapping ones among them around the two
+@pytest.mark.parametrize("n_small", [1, 2, 3, 7, 8, 9, 16, 17, 60])
+@pytest.mark.parametrize("every", [1, 2, 5])
+@pytest.mark.parametrize("last", [False, True])
+def test_particle_sums_of_overlapping_pairs(n_small, every, last):
+    """The forces are the pairs' forces added in FP64 in partner order, bit for
+    bit: the ball first (partners above it) or last (below it), one partner in
+    `every` pressed into it and the others near."""
+    from paper_2401_10878_gb300.contact import Contact
+    st = _crowd(n_small)
+    st.shape_param[1:, 0] = np.where(np.arange(n_small) % every == 0, 1.6, 0.4)
+    if last:
+        st.shape_param[:] = st.shape_param[::-1].copy()
+        st.pos[:] = st.pos[::-1].copy()
+    m = Contact.from_state(st)
+    g = gpu_step(m, st)
+    m.close()
+    want = np.zeros((n_small + 1, 3))
+    for lower in (True, False):   # as j, by i; then as i, by j
+        for (i, j), row in zip(g["pair_ij"], g["pair_out"]):
+            if lower:
+                want[j] = want[j] + row[8:11]
+            else:
+                want[i] = want[i] - row[8:11]
+    assert np.array_equal(g["force"], want)
+    assert np.count_nonzero(g["pair_out"][:, 0]) >= (n_small + every - 1) // every
+
+
 # node ranges whose length the ten bits of a bin entry hold, and ones they do not
 @pytest.mark.parametrize("half", [505.3, 511.3, 530.3])
 @pytest.mark.parametrize("gap", [7.1, 8.1])
