@@ -500,6 +500,50 @@ void launch_plan(const Params& P, const Parts& D, const Lists& W, int32_t* pair_
 __host__ __device__ inline bool gather_overlaps(const Params& P) { return P.n > 4096; }
 constexpr int kGatherPairs = 1024;   // pairs gathered at a time
 
+// Component c (eight lanes per particle, six used) of particle p's sum over its
+// overlapping pairs, in FP64 in a fixed order: the pairs where it is j (by i;
+// entry offj of the pair's `width` values at src), then the pairs where it is i
+// (by j; entry offi, negated when neg_i).  Lane c reads the flag of partner
+// base + c; a pair without overlap would add zeros.  Called by the whole warp
+// (p >= n: zero).
+__device__ __forceinline__ double flagged_sum(const Params& P, const Lists& W, int p, int c, const double* src,
+                                              int width, int offi, int offj, bool neg_i) {
+  const unsigned full = 0xffffffffu;
+  const int g0 = (threadIdx.x & 31) & ~7;
+  const bool own = p < P.n;
+  const int* dp = W.dn_pair + static_cast<size_t>(own ? p : 0) * P.max_nbr;
+  const int pre = c < P.max_nbr ? dp[c] : 0;   // (fetched with the counts)
+  const int np = min(W.counters[0], P.max_pairs);
+  const int nd = own ? W.dn_count[p] : 0, nu = own ? W.up_count[p] : 0, r0 = own ? W.row_off[p] : 0;
+  const long long flip_i = neg_i ? static_cast<long long>(0x8000000000000000ULL) : 0LL;
+  const int total = nd + nu;
+  const int most = __reduce_max_sync(full, total);
+  double acc = 0.0;
+  for (int base = 0; base < most; base += 8) {
+    const int e = base + c;
+    int q = e < nd ? (base == 0 ? pre : dp[e]) : (e < total ? r0 + (e - nd) : np);
+    if (e < total) q = checked_index(W.err, q, np, -1);
+    const bool flag = q >= 0 && q < np && W.oflag[q] != 0;
+    unsigned m = (__ballot_sync(full, flag) >> g0) & 0xffu;
+    while (__any_sync(full, m != 0u)) {   // two at a time
+      const int u0 = m != 0u ? __ffs(m) - 1 : 0;
+      const unsigned m1 = m & (m - 1u);
+      const int u1 = m1 != 0u ? __ffs(m1) - 1 : 0;
+      const int q0 = __shfl_sync(full, q, g0 + u0), q1 = __shfl_sync(full, q, g0 + u1);
+      const bool j0 = base + u0 < nd, j1 = base + u1 < nd;
+      double v0 = 0.0, v1 = 0.0;
+      if (m != 0u && c < 6) v0 = src[static_cast<size_t>(q0) * width + (j0 ? offj : offi)];
+      if (m1 != 0u && c < 6) v1 = src[static_cast<size_t>(q1) * width + (j1 ? offj : offi)];
+      if (!j0) v0 = __longlong_as_double(__double_as_longlong(v0) ^ flip_i);
+      if (!j1) v1 = __longlong_as_double(__double_as_longlong(v1) ^ flip_i);
+      if (m != 0u) acc += v0;
+      if (m1 != 0u) acc += v1;
+      m = m1 & (m1 - 1u);
+    }
+  }
+  return acc;
+}
+
 // The overlapping pairs among [q0, q0 + cnt), cnt <= kGatherPairs, to s_q (in
 // any order: every pair is treated on its own), by the whole block; returns
 // their number.  s_n: a shared counter.

@@ -56,12 +56,6 @@ struct AdjBufs {
 };
 
 
-__device__ __forceinline__ void cross3(const double a[3], const double b[3], double c[3]) {
-  c[0] = a[1] * b[2] - a[2] * b[1];
-  c[1] = a[2] * b[0] - a[0] * b[2];
-  c[2] = a[0] * b[1] - a[1] * b[0];
-}
-
 // ---------------------------------------------------------------- pair level
 // The depth term of d = -phiA(x*) - phiB(x*) at the pair's deepest node x*
 // (the tape's node index), seeded with gd = dL/dd: d(-phi)/dX = grad phi and
@@ -367,17 +361,15 @@ __device__ __forceinline__ void adj_pre_pass(const Params& P, const Shapes& S, c
       if (k < 3) {
         sd[1 + k] = act ? static_cast<float>(s1) : 0.f;
         sd[4 + k] = act ? static_cast<float>(sg) : 0.f;
-        pg[k] = act ? gXA : 0.0;
-        pg[3 + k] = act ? dcA : 0.0;
-        pg[6 + k] = act ? gXB : 0.0;
-        pg[9 + k] = act ? dcB : 0.0;
+        if (act) {   // (read for the overlapping pairs alone)
+          pg[k] = gXA;
+          pg[3 + k] = dcA;
+          pg[6 + k] = gXB;
+          pg[9 + k] = dcB;
+        }
       } else {
         sd[0] = act ? static_cast<float>(s0) : 0.f;
         sd[7] = 0.f;
-        pg[12] = act ? gd : 0.0;
-        pg[13] = 0.0;
-        pg[14] = 0.0;
-        pg[15] = 0.0;
         B.done[p] = 0;
       }
     }
@@ -388,7 +380,7 @@ __device__ __forceinline__ void adj_pre_pass(const Params& P, const Shapes& S, c
 // every warp takes eight consecutive pairs at a time, whether they overlap or
 // not (gathering the overlapping ones first cost a longer chain: the 1934
 // cubes' backward 41.2 -> 45.1 us).  GATHER = true: each block collects the
-// overlapping pairs of its range, zeroes the seeds and gradients of the others
+// overlapping pairs of its range, zeroes the seeds of the others
 // with consecutive lanes, and its warps take passes of eight: 84.8 us over all
 // pairs, 36.0 us gathered by single warps, 23.5 us by blocks on 15472 mixed
 // particles (7304 of 38585 pairs overlap).
@@ -417,9 +409,6 @@ __global__ void __launch_bounds__(GATHER ? kPreWarps * 32 : 32, GATHER ? 2 : 1) 
       float4* zs = reinterpret_cast<float4*>(B.seeds + static_cast<size_t>(q0) * kSeedFloats);
       for (int x = threadIdx.x; x < all * (kSeedFloats / 4); x += blockDim.x)
         if (W.oflag[q0 + x / (kSeedFloats / 4)] == 0) zs[x] = make_float4(0.f, 0.f, 0.f, 0.f);
-      double2* zp = reinterpret_cast<double2*>(B.pgrad + static_cast<size_t>(q0) * kPairGrad);
-      for (int x = threadIdx.x; x < all * (kPairGrad / 2); x += blockDim.x)
-        if (W.oflag[q0 + x / (kPairGrad / 2)] == 0) zp[x] = make_double2(0.0, 0.0);
       for (int x = threadIdx.x; x < all; x += blockDim.x)
         if (W.oflag[q0 + x] == 0) B.done[q0 + x] = 0;
     }
@@ -958,53 +947,41 @@ __global__ void __launch_bounds__(kAdjWarps * 32, adj_blocks<SET>()) k_adj_cells
 }
 
 // Per particle and component (eight lanes per particle, six used), FP64 adds
-// in the forward order: the pairs where the particle is j (by i), then the
-// pairs where it is i (by j); lane 0 of each group then maps the rotation
-// gradient to the raw quaternion.
-__global__ void __launch_bounds__(32) k_adj_scatter(Params P, Parts D, Lists W, AdjBufs B,
-                                                    double* __restrict__ gpos, double* __restrict__ gquat) {
+// of the overlapping pairs' gradients in the forward order: the pairs where the
+// particle is j (by i), then the pairs where it is i (by j); four lanes of each
+// group then map the rotation gradient to the raw quaternion.  Bound: the FP64
+// pipe.  Every candidate's gradient read and added in one-warp blocks took
+// 14.4 us on 15472 mixed particles, the flagged ones alone in blocks of four
+// warps 12.2 us, with one lane per quaternion component 9.5 us.
+constexpr int kScatterThreads = 128;
+__global__ void __launch_bounds__(kScatterThreads) k_adj_scatter(Params P, Parts D, Lists W, AdjBufs B,
+                                                                 double* __restrict__ gpos,
+                                                                 double* __restrict__ gquat) {
   pdl_begin();
   const int t = blockIdx.x * blockDim.x + threadIdx.x;
   const int lane = threadIdx.x & 31, g0 = lane & ~7;
-  const int p0 = t >> 3, c = t & 7;
-  const bool ok = p0 < P.n;
-  const int p = ok ? p0 : P.n - 1;
-  const int np = min(W.counters[0], P.max_pairs);
-  double acc = 0.0;
-  if (ok && c < 6) {
-    // contributions in order (j side, then i side), eight loads in flight at a time
-    const int* dp = W.dn_pair + static_cast<size_t>(p) * P.max_nbr;
-    const int nd = W.dn_count[p], r0 = W.row_off[p], nu = W.up_count[p];
-    const int total = nd + nu;
-    for (int base = 0; base < total; base += 8) {
-      double v[8];
-#pragma unroll
-      for (int u = 0; u < 8; ++u) {
-        const int e = base + u;
-        const bool isj = e < nd;   // p is the pair's j: columns 6..11; else its i: columns 0..5
-        int q = isj ? dp[e] : (e < total ? r0 + (e - nd) : np);
-        if (e < total) q = checked_index(W.err, q, np, -1);
-        v[u] = (q >= 0 && q < np) ? B.pgrad[static_cast<size_t>(q) * kPairGrad + (isj ? 6 + c : c)] : 0.0;
-      }
-#pragma unroll
-      for (int u = 0; u < 8; ++u)
-        if (base + u < total) acc += v[u];
-    }
-  }
+  const int p = t >> 3, c = t & 7;
+  const bool ok = p < P.n;
+  // (columns 0..5 of a pair: its i, 6..11: its j)
+  const double acc = flagged_sum(P, W, p, c, B.pgrad, kPairGrad, c, 6 + c, false);
   double tau[3];
 #pragma unroll
   for (int k = 0; k < 3; ++k) tau[k] = __shfl_sync(kFull, acc, g0 + 3 + k);
   if (!ok) return;
   if (c < 3) gpos[3 * p + c] = acc;
-  if (c == 0) {
+  if (c < 4) {
+    // dL/dq = (2/|q|^2) (-v.tau, w tau + tau x v) of the raw q = (w, v): lane c
+    // forms component c, x0 y0 + x1 y1 - x2 y2
     const double* qr = D.qhat + 4 * p;
-    const double iq = fl::nr_rsqrt(qr[0] * qr[0] + qr[1] * qr[1] + qr[2] * qr[2] + qr[3] * qr[3]);
-    const double w = qr[0] * iq, v[3] = {qr[1] * iq, qr[2] * iq, qr[3] * iq};
-    const double s2 = 2.0 * iq;
-    double tv[3];
-    cross3(tau, v, tv);
-    gquat[4 * p] = -s2 * (v[0] * tau[0] + v[1] * tau[1] + v[2] * tau[2]);
-    for (int k = 0; k < 3; ++k) gquat[4 * p + 1 + k] = s2 * (w * tau[k] + tv[k]);
+    const double q0 = qr[0], q1 = qr[1], q2 = qr[2], q3 = qr[3];
+    const double iq = fl::nr_rsqrt(fma(q0, q0, fma(q1, q1, fma(q2, q2, q3 * q3))));
+    const double x0 = c == 0 ? -q1 : q0;
+    const double x1 = c == 0 ? -q2 : (c == 1 ? q3 : (c == 2 ? q1 : q2));
+    const double x2 = c == 0 ? q3 : (c == 1 ? q2 : (c == 2 ? q3 : q1));
+    const double y0 = c < 2 ? tau[0] : (c == 2 ? tau[1] : tau[2]);
+    const double y1 = c < 2 ? tau[1] : (c == 2 ? tau[2] : tau[0]);
+    const double y2 = c < 2 ? tau[2] : (c == 2 ? tau[0] : tau[1]);
+    gquat[4 * p + c] = (2.0 * iq * iq) * fma(x0, y0, fma(x1, y1, -(x2 * y2)));
   }
 }
 
@@ -1046,7 +1023,7 @@ void launch_adjoint(const Params& P, const Shapes& S, const Parts& D, const List
   if (ev0 != nullptr) cudaEventRecord(ev0, st);
   launch_pdl(cells, dim3(grid), dim3(kAdjWarps * 32), 0, st, P, S, D, W, B);
   if (ev1 != nullptr) cudaEventRecord(ev1, st);
-  launch_pdl(k_adj_scatter, dim3((8 * P.n + 31) / 32), dim3(32), 0, st, P, D, W, B, gpos, gquat);
+  launch_pdl(k_adj_scatter, dim3((8 * P.n + kScatterThreads - 1) / kScatterThreads), dim3(kScatterThreads), 0, st, P, D, W, B, gpos, gquat);
 }
 
 }  // namespace gbc

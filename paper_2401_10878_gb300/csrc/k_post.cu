@@ -46,48 +46,6 @@ __device__ __forceinline__ void particle_sum(const Params& P, const Lists& W, in
   else torque[3 * p + c - 3] = acc;
 }
 
-// The same sum from the overlapping pairs alone (whole warp, eight lanes per
-// particle): lane c reads the flag of partner base + c, and the flagged pairs'
-// forces follow in partner order.
-__device__ __forceinline__ void particle_sum_flagged(const Params& P, const Lists& W, int p, int c,
-                                                     double* __restrict__ force, double* __restrict__ torque) {
-  const int lane = threadIdx.x & 31, g0 = lane & ~7;
-  const bool own = p < P.n;
-  const int* dp = W.dn_pair + static_cast<size_t>(own ? p : 0) * P.max_nbr;
-  const int pre = c < P.max_nbr ? dp[c] : 0;
-  const int np = min(W.counters[0], P.max_pairs);
-  const int nd = own ? W.dn_count[p] : 0, nu = own ? W.up_count[p] : 0, r0 = own ? W.row_off[p] : 0;
-  const int offj = c < 3 ? c : c + 3, offi = c;
-  const long long flip_i = c < 3 ? static_cast<long long>(0x8000000000000000ULL) : 0LL;
-  const int total = nd + nu;
-  const int most = __reduce_max_sync(kFull, total);
-  double acc = 0.0;
-  for (int base = 0; base < most; base += 8) {
-    const int e = base + c;
-    int q = e < nd ? (base == 0 ? pre : dp[e]) : (e < total ? r0 + (e - nd) : np);
-    if (e < total) q = checked_index(W.err, q, np, -1);
-    const bool flag = q >= 0 && q < np && W.oflag[q] != 0;
-    unsigned m = (__ballot_sync(kFull, flag) >> g0) & 0xffu;
-    while (__any_sync(kFull, m != 0u)) {   // two at a time
-      const int u0 = m != 0u ? __ffs(m) - 1 : 0;
-      const unsigned m1 = m & (m - 1u);
-      const int u1 = m1 != 0u ? __ffs(m1) - 1 : 0;
-      const int q0 = __shfl_sync(kFull, q, g0 + u0), q1 = __shfl_sync(kFull, q, g0 + u1);
-      const bool j0 = base + u0 < nd, j1 = base + u1 < nd;
-      double v0 = 0.0, v1 = 0.0;
-      if (m != 0u && c < 6) v0 = W.ft[static_cast<size_t>(q0) * kFtDoubles + (j0 ? offj : offi)];
-      if (m1 != 0u && c < 6) v1 = W.ft[static_cast<size_t>(q1) * kFtDoubles + (j1 ? offj : offi)];
-      if (!j0) v0 = __longlong_as_double(__double_as_longlong(v0) ^ flip_i);
-      if (!j1) v1 = __longlong_as_double(__double_as_longlong(v1) ^ flip_i);
-      if (m != 0u) acc += v0;
-      if (m1 != 0u) acc += v1;
-      m = m1 & (m1 - 1u);
-    }
-  }
-  if (own && c < 3) force[3 * p + c] = acc;
-  else if (own && c < 6) torque[3 * p + c - 3] = acc;
-}
-
 // K6: per particle and component (eight lanes per particle, six used), FP64
 // adds in a fixed order: the pairs where the particle is j (by i), then the
 // pairs where it is i (by j).  j receives +F and T_B, i receives -F and T_A.
@@ -114,8 +72,11 @@ __global__ void __launch_bounds__(kSumThreads) k_particle_sum(Params P, Parts D,
   const int nbins = P.nbin[0] * P.nbin[1] * P.nbin[2];
   for (int b = t; b < nbins; b += gridDim.x * blockDim.x) W.bin_count[b] = 0;
   const int p = t >> 3, c = t & 7;
-  if constexpr (FLAGGED) particle_sum_flagged(P, W, p, c, force, torque);
-  else if (p < P.n && c < 6) particle_sum(P, W, p, c, force, torque);
+  if constexpr (FLAGGED) {
+    const double acc = flagged_sum(P, W, p, c, W.ft, kFtDoubles, c, c < 3 ? c : c + 3, c < 3);
+    if (p < P.n && c < 3) force[3 * p + c] = acc;
+    else if (p < P.n && c < 6) torque[3 * p + c - 3] = acc;
+  } else if (p < P.n && c < 6) particle_sum(P, W, p, c, force, torque);
   // a host-buffer step that returns on its token: the step is complete when
   // every warp's sums are stored, and the last warp to finish mirrors the
   // error word and then publishes the host's token of this step (mapped host
