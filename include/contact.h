@@ -89,7 +89,7 @@ typedef struct {
   int32_t precision;        /* CONTACT_PRECISION_FP32_TILE: FP32 node tests, FP32
                                tile partials, FP64 per-pair reduction;
                                CONTACT_PRECISION_FP64_PAIR: everything in FP64,
-                               one thread block per pair                           */
+                               over the same clipped node lines                    */
   int32_t max_pairs;        /* capacity of the pair list (> 0)                       */
   int32_t max_neighbors;    /* capacity of one particle's candidate list (0: 64)    */
   int32_t max_tiles;        /* capacity of the node-tile list (0: 8 * max_pairs)    */

@@ -254,7 +254,7 @@ __device__ __forceinline__ bool record_in_bounds(const Params& P, int* err, cons
 }
 
 // Work lists shared by the step's kernels.
-// One overlapping pair for the force law (appended to the step's overlap list
+// One overlapping pair for the force law (written to its entry of the overlap list
 // by the warp that completes it): its FP64 sums (count, first moments, band
 // terms of G), its deepest node, and the pair record's geometry.
 struct OvlRec {

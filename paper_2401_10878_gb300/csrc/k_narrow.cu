@@ -7,9 +7,9 @@
 //
 // k_narrow32 (FP32 node tests, FP32 tile partials):
 //   * persistent grid, one warp per tile; warp w takes tiles w, w + W, ...
-//     of the cost-ordered tile list (W warps; no queue atomics), the next
-//     tile's record fetched while the current one runs; pairs whose distance
-//     regions are apart never reach the list (the pair builder's test);
+//     of the tile list (W warps, numbered across the blocks; no queue atomics),
+//     the next tile's record fetched while the current one runs; pairs whose
+//     distance regions are apart never reach the list (the pair builder's test);
 //   * a pair's box is cut into node lines along its longest axis; a tile is
 //     32 lanes x 4 lines of one pair;
 //   * each lane clips its line to the interval where both signed distances
@@ -17,15 +17,12 @@
 //     quadratic) and evaluates only the nodes inside it: every node outside
 //     adds exact zeros to every sum, and ~99 % of a settling box's pair-box
 //     nodes lie outside;
-//   * along a line only the sweep coordinate changes, so the per-line part of
-//     each face value is computed once and a node costs one FMA per face;
+//   * the clipped nodes are spread one per lane (sweep_tile);
 //   * node coordinates relative to each particle are exact integers minus an
 //     FP32 remainder in [-1/2, 1/2] (no large-offset cancellation);
 //   * polytope faces (and their inverse slopes along the line) are staged
 //     in shared memory;
-//   * the volume/moment/depth update and the normal-band update run only when
-//     some lane of the warp needs them (warp-uniform branches);
-//   * warp-shuffle reduction per tile (skipped when no lane met a node to
+//   * warp reduction per tile (skipped when no lane met a node to
 //     evaluate); a pair of one tile is finished from the warp's registers,
 //     otherwise the partials go to HBM and the warp that completes the pair's
 //     last tile sums them in FP64 in tile order (deterministic).
@@ -225,7 +222,7 @@ struct CubeEval {
 // memory, and each face's inverse slope along u (the line clip) after them;
 // faces beyond nf are padded so that they never win the maximum (and are
 // constant along the line, below any threshold).
-__device__ __forceinline__ int stage_planes(const Shapes& S, const Parts& D, int pid, const Local& L,
+__device__ __forceinline__ void stage_planes(const Shapes& S, const Parts& D, int pid, const Local& L,
                                             float4* sm, int npad) {
   const int lane = threadIdx.x & 31;
   const int f0 = S.face_off[pid];
@@ -240,7 +237,6 @@ __device__ __forceinline__ int stage_planes(const Shapes& S, const Parts& D, int
     sm[lane] = e;
   }
   __syncwarp();
-  return nf;
 }
 
 // Any kind, chosen at run time (the variant with every kind): what the other
@@ -268,23 +264,31 @@ struct AnyEval {
   float fu, fv, fw;
   const float4* cs;
   float g0, g1, g2;   // band sum: local axes (sphere, polytope), body axes (cuboid), along the normal (wall)
-  __device__ void load(const PairRec& r, bool second, const Shapes& S, const Parts& D, const Local& L, float T,
-                       float4* sm) {
-    const int lane = threadIdx.x & 31;
+  // the registers, with the constants staged in sm (a shared tile: by the warp that clipped it)
+  __device__ void attach(const PairRec& r, bool second, const Shapes& S, const Local& L, float4* sm) {
     kind = second ? r.kinds >> 8 : r.kinds & 0xff;
     const int* ci = second ? r.bi : r.ai;
     const float* cf = second ? r.bf : r.af;
-    const float* rt = second ? r.rtb : r.rta;
-    const float* sz = second ? r.szb : r.sza;
     iu = ci[L.u]; iv = ci[L.v]; iw = ci[L.w];
     fu = cf[L.u]; fv = cf[L.v]; fw = cf[L.w];
     cs = sm;
     nf = nup = ndn = 0;
+    if (POLY && kind == KIND_POLY) {
+      const int pid = second ? r.j : r.i;
+      nf = S.face_off[pid + 1] - S.face_off[pid];
+    }
     g0 = g1 = g2 = 0.f;
+  }
+  __device__ void load(const PairRec& r, bool second, const Shapes& S, const Parts& D, const Local& L, float T,
+                       float4* sm) {
+    const int lane = threadIdx.x & 31;
+    attach(r, second, S, L, sm);
+    const float* rt = second ? r.rtb : r.rta;
+    const float* sz = second ? r.szb : r.sza;
     if (CUBE && kind == KIND_CUBE) {
       CubeEval::prep_lanes(r, second, L, T, sm, lane);
     } else if (POLY && kind == KIND_POLY) {
-      nf = stage_planes(S, D, second ? r.j : r.i, L, sm, kMaxFaces);
+      stage_planes(S, D, second ? r.j : r.i, L, sm, kMaxFaces);
       const bool act = lane < nf;
       const float4 e = sm[act ? lane : 0];
       const bool up = act && e.x > kClipFlat, dn = act && e.x < -kClipFlat, par = act && !up && !dn;
@@ -415,10 +419,16 @@ struct AnyEval {
     return fmaxf(a[0], fmaxf(a[1], a[2]));
   }
   __device__ __forceinline__ void add(float m, const float4& d) {
-    const float mi = m * d.w;
-    g0 = fmaf(mi, d.x, g0);
-    g1 = fmaf(mi, d.y, g1);
-    g2 = fmaf(mi, d.z, g2);
+    replay(record(m, d));
+  }
+  // what add(m, d) adds, and the same additions later (shared tiles)
+  static __device__ __forceinline__ float4 record(float m, const float4& d) {
+    return make_float4(m * d.w, d.x, d.y, d.z);
+  }
+  __device__ __forceinline__ void replay(const float4& e) {
+    g0 = fmaf(e.x, e.y, g0);
+    g1 = fmaf(e.x, e.z, g1);
+    g2 = fmaf(e.x, e.w, g2);
   }
   // component c of the band sum in the world frame
   __device__ float world(int c, const Local& L, const PairRec& r, bool second) const {
@@ -469,7 +479,7 @@ __device__ __forceinline__ float key_float(int k) { return __int_as_float(k >= 0
 // of the lanes with nodes, the slot by the owner's counts, and the evaluators
 // start that node's line at the node itself, so the node gets exactly the
 // arithmetic of a node walk (the same FP32 distances, bit for bit).
-// E: the evaluator of both particles.  With AnyEval the slot loops stay rolled,
+// E: the evaluator of both particles.  With AnyEval the slot loop stays rolled,
 // with the slots' clipped ranges in shared memory, to keep the kernel's code
 // small (unrolled: 38.8 -> 61.8 us on 15472 mixed particles); for two cubes they
 // are unrolled over registers.
@@ -484,7 +494,10 @@ __device__ __forceinline__ Partial sweep_tile(const Params& P, const Shapes& S, 
   const int du = r.dim[L.u], dv = r.dim[L.v];
   const float inv_dv = __fdividef(1.f, static_cast<float>(dv));
   const float inv_w = P.inv_w, hw = 0.5f * P.wdx_l, T = hw + kClipMargin;
-  if constexpr (ROLL) {
+  if constexpr (ROLL && COOP) {
+    A.attach(r, swap, S, L, smA);
+    B.attach(r, !swap, S, L, smB);
+  } else if constexpr (ROLL) {
     A.load(r, swap, S, D, L, T, smA);
     B.load(r, !swap, S, D, L, T, smB);
     __syncwarp();
@@ -567,16 +580,16 @@ __device__ __forceinline__ Partial sweep_tile(const Params& P, const Shapes& S, 
     if (total > 0) {
       const int rank = __popc(__ballot_sync(kFull, has) & ((1u << lane) - 1u));
       if (has) {
+        static_assert(kTileItemsPerLane == 4, "own holds four clipped ranges per lane");
         if constexpr (ROLL) {
-          own[rank] = make_int4(lane, excl, 0, 0);
-        } else {
-          static_assert(kTileItemsPerLane == 4, "own holds four clipped ranges per lane");
-          // and the lane's node counts before slots 2 and 3
-          const int c2 = static_cast<int>(pk[0] >> 16) + static_cast<int>(pk[1] >> 16);
-          own[rank] = make_int4(lane, excl, static_cast<int>(pk[0]), static_cast<int>(pk[1]));
-          own[32 + rank] = make_int4(static_cast<int>(pk[2]), static_cast<int>(pk[3]), c2,
-                                     c2 + static_cast<int>(pk[2] >> 16));
+#pragma unroll
+          for (int s = 0; s < kTileItemsPerLane; ++s) pk[s] = s < ns ? spk[s * 32 + lane] : 0u;
         }
+        // and the lane's node counts before slots 2 and 3
+        const int c2 = static_cast<int>(pk[0] >> 16) + static_cast<int>(pk[1] >> 16);
+        own[rank] = make_int4(lane, excl, static_cast<int>(pk[0]), static_cast<int>(pk[1]));
+        own[32 + rank] = make_int4(static_cast<int>(pk[2]), static_cast<int>(pk[3]), c2,
+                                   c2 + static_cast<int>(pk[2] >> 16));
       }
       __syncwarp();
     }
@@ -602,31 +615,14 @@ __device__ __forceinline__ Partial sweep_tile(const Params& P, const Shapes& S, 
     const int cnt_le = __popc(before) + __popc(inside & (lane == 31 ? 0xffffffffu : (2u << lane) - 1u));
     const int4 e = own[min(max(cnt_le - 1, 0), 31)];
     const int o = e.x;
-    int k = g - e.y;   // the node's rank among the owner's
-    int4 e2 = make_int4(0, 0, 0, 0);
-    if (!ROLL) e2 = own[32 + min(max(cnt_le - 1, 0), 31)];
-    int os = 0, u = 0;
-    if constexpr (ROLL) {
-#pragma unroll 1
-      for (int s = 0; s < kTileItemsPerLane; ++s) {
-        if (s < ns) {
-          const unsigned q = spk[s * 32 + o];
-          const int n = static_cast<int>(q >> 16);
-          if (k >= 0 && k < n) {
-            os = s;
-            u = static_cast<int>(q & 0xffffu) + k;
-          }
-          k -= n;
-        }
-      }
-    } else {
-      // the slot: how many of the owner's slot boundaries (node counts before
-      // slots 1, 2, 3; empty slots repeat a boundary) lie at or below k
-      const int c1 = static_cast<int>(static_cast<unsigned>(e.z) >> 16), c2 = e2.z, c3 = e2.w;
-      os = (k >= c1 ? 1 : 0) + (k >= c2 ? 1 : 0) + (k >= c3 ? 1 : 0);
-      const unsigned q = static_cast<unsigned>(os == 0 ? e.z : (os == 1 ? e.w : (os == 2 ? e2.x : e2.y)));
-      u = static_cast<int>(q & 0xffffu) + k - (os == 0 ? 0 : (os == 1 ? c1 : (os == 2 ? c2 : c3)));
-    }
+    const int k = g - e.y;   // the node's rank among the owner's
+    const int4 e2 = own[32 + min(max(cnt_le - 1, 0), 31)];
+    // the slot: how many of the owner's slot boundaries (node counts before
+    // slots 1, 2, 3; empty slots repeat a boundary) lie at or below k
+    const int c1 = static_cast<int>(static_cast<unsigned>(e.z) >> 16), c2 = e2.z, c3 = e2.w;
+    const int os = (k >= c1 ? 1 : 0) + (k >= c2 ? 1 : 0) + (k >= c3 ? 1 : 0);
+    const unsigned q = static_cast<unsigned>(os == 0 ? e.z : (os == 1 ? e.w : (os == 2 ? e2.x : e2.y)));
+    const int u = static_cast<int>(q & 0xffffu) + k - (os == 0 ? 0 : (os == 1 ? c1 : (os == 2 ? c2 : c3)));
     int ocv;
     const int ocw = div_small(it0 + os * 32 + o, dv, inv_dv, &ocv);
     float fa, fb;
@@ -661,8 +657,13 @@ __device__ __forceinline__ Partial sweep_tile(const Params& P, const Shapes& S, 
     if constexpr (COOP) {
       if (base < total) {   // warp-uniform
         CoopNode& c = coop[32 * wid + lane];
-        c.ga = A.record(ma);
-        c.gb = B.record(mb);
+        if constexpr (ROLL) {
+          c.ga = E::record(ma, da);
+          c.gb = E::record(mb, db);
+        } else {
+          c.ga = A.record(ma);
+          c.gb = B.record(mb);
+        }
         c.mom = make_float4(w, static_cast<float>(u), static_cast<float>(ocv), static_cast<float>(ocw));
         c.f = f;
         c.idx = idx;
@@ -915,11 +916,7 @@ __global__ void __launch_bounds__(narrow_warps<SET>() * 32, narrow_blocks<SET>()
   __shared__ float4 s_planes[NW][2][SET == SET_ALL ? 2 * kMaxFaces : 8];
   __shared__ unsigned s_pk[SET == SET_CUBE ? 1 : NW][kTileItemsPerLane * 32];   // clipped ranges (rolled sweep)
   __shared__ int4 s_own[NW][64];   // the lanes with clipped nodes (sweep_tile)
-  // tiles shared by the block: in the cubes-only variant (the others hold nine
-  // kind pairs, and the second sweep of each would cost their instruction
-  // fetches more than it gives: 10.8 -> 11.1 us on 1934 mixed particles)
-  constexpr bool kShare = SET == SET_CUBE;
-  __shared__ CoopNode s_coop[kShare ? NW * 32 : 1];   // a shared tile's nodes
+  __shared__ CoopNode s_coop[NW * 32];   // a shared tile's nodes
   __shared__ int3 s_deferred[NW];   // warp that clipped it, lanes with nodes, clipped nodes
   __shared__ int s_ndeferred;
   pdl_begin();
@@ -934,8 +931,12 @@ __global__ void __launch_bounds__(narrow_warps<SET>() * 32, narrow_blocks<SET>()
   if (ntiles > P.max_tiles) return;   // capacity exceeded: the step reports ECAPACITY
   // with at most one tile per warp a tile of many node passes would be the
   // kernel's tail: it is left for the whole block, whose other warps are done
-  // (400 cubes, one in seven pressed into a neighbour: 16.0 -> 11.9 us)
-  const bool share = kShare && ntiles <= nwarps;
+  // (400 cubes, one in seven pressed into a neighbour: 16.0 -> 11.9 us; 135 larger
+  // cubes between walls, hundreds of nodes per wall contact: 28.3 -> 15.4 us; 123
+  // mixed particles with walls: 24.7 -> 14.3 us; 2568 spheres and cuboids, one in
+  // ten pressed: 25.0 -> 14.0 us.  The run-time evaluator alone was slower there
+  // than a sweep per kind pair, 22.1, 25.3 and 20.1 us.)
+  const bool share = ntiles <= nwarps;
   if (share) {
     if (threadIdx.x == 0) s_ndeferred = 0;
     __syncthreads();
@@ -961,17 +962,15 @@ __global__ void __launch_bounds__(narrow_warps<SET>() * 32, narrow_blocks<SET>()
     buf ^= 1;
     t = tn;
   }
-  if constexpr (kShare) {
-    if (!share) return;
-    __syncthreads();
-    const int nd = s_ndeferred;
-    for (int d = 0; d < nd; ++d) {
-      const int3 e = s_deferred[d];
-      const PairRec& r = s_rec[e.x][0];
-      const Partial o = dispatch<SMOOTH, SET, true>(P, S, D, r, r.tile, s_planes[e.x][0], s_planes[e.x][1], s_pk[0],
-                                                    s_own[e.x], 0, s_coop, e.y, e.z);
-      if (wid == 0) tile_done(W, r, reduce_tile<SMOOTH>(o));
-    }
+  if (!share) return;
+  __syncthreads();
+  const int nd = s_ndeferred;
+  for (int d = 0; d < nd; ++d) {
+    const int3 e = s_deferred[d];
+    const PairRec& r = s_rec[e.x][0];
+    const Partial o = dispatch<SMOOTH, SET, true>(P, S, D, r, r.tile, s_planes[e.x][0], s_planes[e.x][1], nullptr,
+                                                  s_own[e.x], 0, s_coop, e.y, e.z);
+    if (wid == 0) tile_done(W, r, reduce_tile<SMOOTH>(o));
   }
 }
 

@@ -163,6 +163,29 @@ def test_shared_tiles_of_cubes(pen, indicator, half):
     assert ref.pair_out[0, 0] > 0.0
 
 
+# the same for the other kinds: tiles of about 128 clipped nodes (the limit of sharing) and of many node passes
+@pytest.mark.parametrize("pen", [0.6, 1.1, 2.2, 7.0])
+@pytest.mark.parametrize("indicator", [0, 1])
+@pytest.mark.parametrize("kinds", ["sphere-sphere", "cuboid-sphere", "cuboid-cuboid", "cube-cuboid", "polytope-polytope",
+                                   "polytope-sphere", "cuboid-polytope", "cube-wall", "polytope-wall"])
+def test_shared_tiles_of_other_kinds(pen, indicator, kinds):
+    """Two particles pressed together along x (a face on a face where they have
+    one), or one pressed on a wall."""
+    h = {"sphere": (14.0, 0, 0), "cuboid": (5.0, 9.0, 7.3), "cube": (6.0,) * 3, "polytope": (5.2, 8.1, 7.7)}
+    code = {"sphere": W.SPHERE, "cuboid": W.CUBOID, "cube": W.CUBOID, "polytope": W.POLYTOPE}
+    a, b = kinds.split("-")
+    ks = [a] if b == "wall" else [a, b]
+    c = np.array([40.23, 41.31, 42.17])
+    pos = [c] if b == "wall" else [c, c + [h[a][0] + h[b][0] - pen, 0.21, -0.17]]
+    q = [quat_axis_angle([0.3, 1.0, 0.2], 0.004), quat_axis_angle([1.0, 0.1, 0.4], 0.006)][:len(ks)]
+    st = state([code[k] for k in ks], [h[k] for k in ks], pos, quat=q, n=128, indicator=indicator,
+               planes=[cube_planes(h[k]) if k == "polytope" else None for k in ks])
+    if b == "wall":
+        st = W.with_walls(st, [[1.0, 0.0, 0.0, c[0] + h[a][0] - pen]])
+    rep, ref = _parity(st, 0)
+    assert ref.pair_out[0, 0] > 0.0
+
+
 @pytest.mark.parametrize("max_pairs", [None, 8])
 def test_pair_count_of_the_last_step(max_pairs):
     """contact_pair_count is the step's n_pairs, also beyond the capacity (0 before the first step)."""
