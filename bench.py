@@ -10,7 +10,7 @@ rotations ~ N(0, 0.01 rad)).  A "step" is one contact_step: pose -> AABB,
 broad phase, work partition, node sweep, pair reduction, force law,
 per-particle sums.  Secondary lines in the same JSON: the 1934-particle mixed
 spheres/cubes/polytopes box, the smoothed-indicator forward + adjoint pass on
-the cuboid box, and the all-FP64 one-pair-per-block form.
+the cuboid box, and the all-FP64 form.
 
   python bench.py [--gpus N] [--steps K] [--warmup W] [--impl ours|reference]
 
@@ -559,7 +559,7 @@ def extras(args, dev, flush, peak):
     out["mixed1934_223"]["fp64_form"] = {"cell_evals_per_s": r["cells"] / (r["ms"] * 1e-3),
                                          "ms_per_step": r["ms"] / steps, "narrow_ms": r["narrow_ms"] / steps}
     m.close()
-    # all-FP64 one-pair-per-block form on the headline workload
+    # all-FP64 form on the headline workload
     st = headline_state(0)
     pos, quat = W.pose_sequence(st, steps + 3)
     m = Contact.from_state(st, precision=FP64_PAIR, narrow_events=True)
@@ -567,17 +567,13 @@ def extras(args, dev, flush, peak):
     out["cubes1934_fp64_form"] = {"cell_evals_per_s": r["cells"] / (r["ms"] * 1e-3),
                                   "ms_per_step": r["ms"] / steps, "narrow_ms": r["narrow_ms"] / steps}
     m.close()
-    # its node sweep against the FP64 pipe: the same nominal lane-ops, in FP64, over the
-    # measured DFMA rate of this GPU
+    # (bound by the FP64 pipe; the nominal lane-ops count every node of every pair box, of which
+    # the clipped sweep evaluates about one in a hundred, so they give no fraction of its peak)
     try:
         from paper_2401_10878_gb300.contact import fp64_dfma_rate
-        dfma = fp64_dfma_rate() / 1e12
-        a64 = r["ops"] / (r["narrow_ms"] * 1e-3) / 1e12
-        out["cubes1934_fp64_form"]["roofline"] = {"bound": "fp64", "achieved": a64, "peak": dfma,
-                                                  "unit": "T FP64 lane-ops/s", "frac": a64 / dfma,
-                                                  "peak_basis": "measured DFMA rate (contact_fp64_dfma_rate)"}
+        out["cubes1934_fp64_form"]["dfma_rate_t"] = fp64_dfma_rate() / 1e12
     except Exception as e:   # a measurement aid only
-        out["cubes1934_fp64_form"]["roofline_error"] = str(e)[:200]
+        out["cubes1934_fp64_form"]["dfma_rate_error"] = str(e)[:200]
     # the headline workload with velocities: shared damping, then contact history + friction
     # (timed like the other extras, with the library's events around the node sweep; the
     # first entry, without velocities, is the same timing of the headline step)
@@ -611,7 +607,7 @@ def extras(args, dev, flush, peak):
         # roofline of the box kernel: the nominal FP32 lane-ops of its sample
         # tests (the overlapping pairs' N_c^3 samples, the same ops per test as
         # the node sweep's) against the FP32 peak; its FP64 pipe is the busier
-        # unit (ncu: 55 % of active cycles at N_c = 8)
+        # unit
         kern_s = r["narrow_ms"] / steps * 1e-3
         ops_per_test = s_["nominal_ops"] / max(s_["cells"], 1)
         sample_ops = s_["overlapping"] * nc ** 3 * ops_per_test
