@@ -284,13 +284,39 @@ struct Frac {
   }
 };
 
+// The world plane n . x <= e[3] of a body plane e = (n, d), of a particle at X.
+__device__ __forceinline__ void world_plane_d(const Params& P, const double* e, const double* R, const double X[3],
+                                              double o[4]) {
+  const double n0 = (R[0] * e[0] + R[1] * e[1]) + R[2] * e[2];
+  const double n1 = (R[3] * e[0] + R[4] * e[1]) + R[5] * e[2];
+  const double n2 = (R[6] * e[0] + R[7] * e[1]) + R[8] * e[2];
+  o[0] = n0;
+  o[1] = n1;
+  o[2] = n2;
+  o[3] = ((n0 * X[0] + n1 * X[1]) + n2 * X[2]) + e[3] + P.inflate;
+}
+
+// The same of every face of polytope (or wall) `pid`, a face per lane (the
+// caller syncs the warp).  Formed by the lane of each line and particle, one face
+// after the other, they were ~22 of ~36 FP64 instructions per face of a pair's
+// chain: 81 -> 72 us on 86 mixed particles between walls at N_c = 6 (the time
+// of one pair), 250 -> 239 us on 241 mixed at N_c = 16.
+__device__ __forceinline__ void stage_planes_d(const Params& P, const Shapes& S, const Parts& D, int pid,
+                                               const double X[3], double (*pl)[4]) {
+  const int lane = threadIdx.x & 31, type = S.type[pid];
+  if (type == 0 || type == 1) return;
+  const int f0 = S.face_off[pid], nf = S.face_off[pid + 1] - f0;
+  if (lane < nf) world_plane_d(P, S.planes + 4 * (f0 + lane), D.R + 9 * static_cast<size_t>(pid), X, pl[lane]);
+}
+
 // FP64 bounds of the line p + t e (e = sgn axis k, physical units) inside
 // particle / wall `pid`, the same clipping as the FP32 form; used for each
 // face's nearest line.  Returns false when the line misses the shape.  SET as
-// for phi_f.
+// for phi_f; pl: a polytope's (or wall's) world planes (SET 0, stage_planes_d).
 template <int SET>
 __device__ __forceinline__ bool clip_d(const Params& P, const Shapes& S, const Parts& D, int pid, const double X[3],
-                                       const double p[3], int k, double sgn, Frac& lo, Frac& hi) {
+                                       const double p[3], int k, double sgn, const double (*pl)[4], Frac& lo,
+                                       Frac& hi) {
   const int type = SET == 2 ? 1 : S.type[pid];
   const double* R = D.R + 9 * static_cast<size_t>(pid);
   const double q0 = p[0] - X[0], q1 = p[1] - X[1], q2 = p[2] - X[2];
@@ -330,12 +356,14 @@ __device__ __forceinline__ bool clip_d(const Params& P, const Shapes& S, const P
   } else {   // polytope, or a wall's single plane
     const int f0 = S.face_off[pid], nf = S.face_off[pid + 1] - f0;
     for (int f = 0; f < nf; ++f) {
-      const double* e = S.planes + 4 * (f0 + f);
-      const double n0 = (R[0] * e[0] + R[1] * e[1]) + R[2] * e[2];
-      const double n1 = (R[3] * e[0] + R[4] * e[1]) + R[5] * e[2];
-      const double n2 = (R[6] * e[0] + R[7] * e[1]) + R[8] * e[2];
-      const double off = ((n0 * X[0] + n1 * X[1]) + n2 * X[2]) + e[3] + P.inflate;
-      bound(((n0 * p[0] + n1 * p[1]) + n2 * p[2]) - off, sgn * (k == 0 ? n0 : (k == 1 ? n1 : n2)));
+      double e[4];
+      if constexpr (SET == 0) {
+#pragma unroll
+        for (int x = 0; x < 4; ++x) e[x] = pl[f][x];
+      } else {
+        world_plane_d(P, S.planes + 4 * (f0 + f), R, X, e);
+      }
+      bound(((e[0] * p[0] + e[1] * p[1]) + e[2] * p[2]) - e[3], sgn * (k == 0 ? e[0] : (k == 1 ? e[1] : e[2])));
     }
   }
   return !empty;
@@ -659,6 +687,7 @@ __global__ void __launch_bounds__(kBoxWarps * 32, 2) k_box_pairs(Params P, Shape
   __shared__ __align__(16) PairRec s_rec[kBoxWarps];
   __shared__ double s_b0[kBoxWarps][6];   // B0: lower, upper
   __shared__ double s_x[kBoxWarps][6];    // both centres
+  __shared__ double s_pd[SET == 0 ? kBoxWarps : 1][2][kMaxFaces][4];   // polytopes' world planes (re-clip)
   pdl_begin();
   if (W.counters[1] > P.max_tiles) return;   // capacity exceeded: the step reports ECAPACITY
   const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
@@ -714,6 +743,11 @@ __global__ void __launch_bounds__(kBoxWarps * 32, 2) k_box_pairs(Params P, Shape
     __syncwarp();
     // (two boxes, the usual pair, without the other kinds' branches)
     const bool boxes = SET == 2 || ((A.kind == KIND_CUBE || A.kind == KIND_CUBOID) && (B.kind == KIND_CUBE || B.kind == KIND_CUBOID));
+    if constexpr (SET == 0) {
+#pragma unroll
+      for (int x = 0; x < 2; ++x) stage_planes_d(P, S, D, x == 0 ? i : j, s_x[wid] + 3 * x, s_pd[wid][x]);
+      __syncwarp();
+    }
     unsigned my_key = 0xffffffffu;
     int my_line = 0;
     if (boxes) nearest_lines<2>(A, B, off, spl, lnl, Nc, rcp_nc, ff, my_key, my_line);
@@ -738,7 +772,8 @@ __global__ void __launch_bounds__(kBoxWarps * 32, 2) k_box_pairs(Params P, Shape
           p[x] = x == fk ? (fside == 0 ? l : h) : l + ic * (h - l) * inv_nc;
           X[x] = s_x[wid][3 * second + x];
         }
-        empty = !clip_d<SET>(P, S, D, second ? j : i, X, p, fk, fside == 0 ? 1.0 : -1.0, lo, hi);
+        empty = !clip_d<SET>(P, S, D, second ? j : i, X, p, fk, fside == 0 ? 1.0 : -1.0,
+                                 s_pd[SET == 0 ? wid : 0][second], lo, hi);
       }
       // (lanes l and l + 6: the two particles of a face)
       const int o = lane < 6 ? lane + 6 : (lane < 12 ? lane - 6 : lane);

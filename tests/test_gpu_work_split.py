@@ -148,6 +148,26 @@ def test_box_pipeline_line_grids(nc, kinds):
     assert ref.n_pairs > 0
 
 
+# faces of a polytope, one per lane in the box correction: few, and up to a lane each
+@pytest.mark.parametrize("faces", [5, 12, 31, 32])
+@pytest.mark.parametrize("other", ["sphere", "polytope", "wall"])
+def test_box_pipeline_polytope_faces(faces, other):
+    k = np.arange(faces) + 0.5
+    th, ph = np.arccos(1.0 - 2.0 * k / faces), np.pi * (1.0 + 5.0 ** 0.5) * k
+    n = np.stack([np.sin(th) * np.cos(ph), np.sin(th) * np.sin(ph), np.cos(th)], 1)
+    pl = np.concatenate([n, np.full((faces, 1), 5.0)], 1)
+    c = np.array([25.2, 26.1, 25.7])
+    q = [quat_axis_angle([0.3, 1.0, 0.2], 0.4), quat_axis_angle([1.0, 0.1, 0.4], 0.9)]
+    if other == "wall":
+        st = W.with_walls(state([W.POLYTOPE], [[0, 0, 0]], [c], quat=q[:1], n=96, planes=[pl]), [[1.0, 0, 0, c[0] + 3.3]])
+    else:
+        kinds = [W.POLYTOPE, W.POLYTOPE if other == "polytope" else W.SPHERE]
+        st = state(kinds, [[0, 0, 0], [5.0 * (other == "sphere"), 0, 0]], [c, c + [6.3, 1.2, -0.9]], quat=q, n=96,
+                   planes=[pl, pl if other == "polytope" else None])
+    rep, ref = run_box(boxed(st, 8))
+    assert ref.pair_out[0, 0] > 0.0
+
+
 # clipped nodes per tile: about one per line (at the limit above which a block shares a tile), several, many
 @pytest.mark.parametrize("pen", [0.6, 1.1, 1.6, 3.2, 9.0])
 @pytest.mark.parametrize("indicator", [0, 1])
