@@ -115,6 +115,7 @@ struct Params {
   int max_pairs, max_nbr, max_tiles;
   // FP32 copies for the node sweep (lattice units)
   float inflate_l, inv_w, neg6_over_w, wdx_l;   // wdx_l: smoothing width in cells
+  float clip_margin;   // of the FP32 clips and of the pair builder's separation test (line_clip.cuh)
 };
 
 // Shape tables (read-only after contact_init); rows N .. N + nwall - 1 are

@@ -433,17 +433,6 @@ contact_status contact_init(const contact_config* cfg, const int32_t* shape_type
       if (v.size() < 12) return CONTACT_EINVAL;
       for (size_t t = 0; t < v.size(); t += 3)
         circ = std::max(circ, std::sqrt(v[t] * v[t] + v[t + 1] * v[t + 1] + v[t + 2] * v[t + 2]));
-      // the node sweep's pair test bounds a polytope by balls (lattice units,
-      // rounded up): its region {phi <= 0} (offset inflate) in size slot 0, its
-      // region {phi < w/2 + the clip margin} in slot 1
-      const double tcut = (0.5 * C.smooth_width + static_cast<double>(kClipMargin)) * C.dx;
-      for (int s = 0; s < 2; ++s) {
-        const std::vector<double> vs = offset_vertices(pl, F, C.inflate + (s == 0 ? 0.0 : tcut));
-        double r = 0.0;
-        for (size_t t = 0; t < vs.size(); t += 3)
-          r = std::max(r, std::sqrt(vs[t] * vs[t] + vs[t + 1] * vs[t + 1] + vs[t + 2] * vs[t + 2]));
-        size_l[3 * p + s] = std::nextafter(static_cast<float>(r / C.dx), 3.0e38f);
-      }
       verts.insert(verts.end(), v.begin(), v.end());
       kind[p] = KIND_POLY;
       nomops[p] = 4 * F;
@@ -452,6 +441,23 @@ contact_status contact_init(const contact_config* cfg, const int32_t* shape_type
     }
     vert_off[p + 1] = static_cast<int>(verts.size() / 3);
     rmax = std::max(rmax, circ);
+  }
+  const float margin = clip_margin(rmax / C.dx, C.smooth_width);
+  // the node sweep's pair test bounds a polytope by balls (lattice units,
+  // rounded up): its region {phi <= 0} (offset inflate) in size slot 0, its
+  // region {phi < w/2 + the clip margin} in slot 1
+  const double tcut = (0.5 * C.smooth_width + static_cast<double>(margin)) * C.dx;
+  for (int p = 0; p < n; ++p) {
+    if (kind[p] != KIND_POLY) continue;
+    for (int s = 0; s < 2; ++s) {
+      const std::vector<double> vs =
+          offset_vertices(pl_in.data() + 4 * face_offset[p], face_offset[p + 1] - face_offset[p],
+                          C.inflate + (s == 0 ? 0.0 : tcut));
+      double r = 0.0;
+      for (size_t t = 0; t < vs.size(); t += 3)
+        r = std::max(r, std::sqrt(vs[t] * vs[t] + vs[t + 1] * vs[t + 1] + vs[t + 2] * vs[t + 2]));
+      size_l[3 * p + s] = std::nextafter(static_cast<float>(r / C.dx), 3.0e38f);
+    }
   }
   // walls: rows n .. n + nw - 1 of the shape tables, one world-frame plane each
   for (int w = 0; w < nw; ++w) {
@@ -531,6 +537,7 @@ contact_status contact_init(const contact_config* cfg, const int32_t* shape_type
   P.inv_w = static_cast<float>(1.0 / C.smooth_width);
   P.neg6_over_w = static_cast<float>(-6.0 / C.smooth_width);
   P.wdx_l = static_cast<float>(C.smooth_width);
+  P.clip_margin = margin;
 
   cudaError_t e = cudaSuccess;
   std::vector<double> pl_vec(std::move(pl_in));

@@ -692,7 +692,7 @@ __global__ void __launch_bounds__(kAdjWarps * 32, adj_blocks<SET>()) k_adj_cells
   pdl_begin();
   const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
   const int ntiles = min(W.counters[1], P.max_tiles);
-  const float inv_w = P.inv_w, hw = 0.5f * P.wdx_l, T = hw + kClipMargin;
+  const float inv_w = P.inv_w, hw = 0.5f * P.wdx_l, T = hw + P.clip_margin;
   unsigned* spk = s_pk[ROLL ? wid : 0];
   // tiles w, w + W, ... of the forward's list (W warps): each record is staged
   // in shared memory, the next record and its pair's seeds are fetched while
@@ -747,7 +747,7 @@ __global__ void __launch_bounds__(kAdjWarps * 32, adj_blocks<SET>()) k_adj_cells
       AdjGeom A, Bg;
       adj_load_rec(r, false, S, D, s_pl[wid][0], A, ax0);
       adj_load_rec(r, true, S, D, s_pl[wid][1], Bg, ax0);
-      const float Tc = hw + kClipMargin;
+      const float Tc = hw + P.clip_margin;
       if (SET == 2 || A.type == 1) adj_prep_clip(A, ax0, ax1, ax2, Tc);
       if (SET == 2 || Bg.type == 1) adj_prep_clip(Bg, ax0, ax1, ax2, Tc);
       const int dm0 = r.dim[0], dm1 = r.dim[1], dm2 = r.dim[2];

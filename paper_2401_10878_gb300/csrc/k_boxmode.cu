@@ -413,7 +413,7 @@ __global__ void __launch_bounds__(kBoxWarps * 32, 2) k_box_rough(Params P, Shape
   const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
   const int ntl = W.counters[1];
   if (ntl > P.max_tiles) return;   // capacity exceeded: the step reports ECAPACITY
-  const float T = kRoughT + kClipMargin;
+  const float T = kRoughT + P.clip_margin;
   for (int t = blockIdx.x + gridDim.x * wid; t < ntl; t += gridDim.x * kBoxWarps) {
     stage_rec(W, P, t, &s_rec[wid]);
     const PairRec& r = s_rec[wid];

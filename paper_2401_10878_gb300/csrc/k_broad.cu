@@ -601,7 +601,7 @@ static_assert(offsetof(PairRec, rta) == 30 * 4 && offsetof(PairRec, szb) == 51 *
               "store_pair_rec follows the PairRec layout");
 
 // Whether the regions {phi_A < Ta} and {phi_B < Tb} of the pair are
-// disjoint (by more than kCullMargin cells).  A node adds to the node sweep's
+// disjoint (by more than `margin` cells, the clip margin).  A node adds to the node sweep's
 // sums only when both distances lie below w/2 and, with the sharp indicator,
 // one of them is <= 0; so with T = w/2 (+ the clip margin) a pair apart for
 // (T, T) (smoothed), or for both (0, T) and (T, 0) (sharp), has zero
@@ -613,7 +613,6 @@ static_assert(offsetof(PairRec, rta) == 30 * 4 && offsetof(PairRec, szb) == 51 *
 // distance; walls are never skipped.  FP32 in lattice units: the centres
 // differ by an exact integer plus the FP32 difference of two remainders, and
 // every rounding is far below the margin.
-constexpr float kCullMargin = 1e-3f;
 
 __device__ __forceinline__ float dot3(const float* a, const float* b) { return fmaf(a[0], b[0], fmaf(a[1], b[1], a[2] * b[2])); }
 
@@ -622,14 +621,15 @@ __device__ __forceinline__ float dot3(const float* a, const float* b) { return f
 // axis the reach of a box's region is R0 + T S (R0 its reach at 0, S the sum
 // of its axes' projections), of a ball r + T or its tabulated radius.
 struct Apart {
+  float margin;
   unsigned bits = 0;
   __device__ __forceinline__ void axis(float proj, float ra0, float sa, float rb0, float sb, float T) {
-    const float base = proj - kCullMargin - ra0 - rb0;
+    const float base = proj - margin - ra0 - rb0;
     bits |= (base > T * (sa + sb) ? 1u : 0u) | (base > T * sb ? 2u : 0u) | (base > T * sa ? 4u : 0u);
   }
 };
 
-__device__ unsigned pair_apart(const PairRec& r, float T) {
+__device__ unsigned pair_apart(const PairRec& r, float T, float margin) {
   const int ka = r.kinds & 0xff, kb = r.kinds >> 8;
   const bool pa = ka == KIND_POLY, pb = kb == KIND_POLY;
   const bool sa = ka == KIND_SPHERE || pa, sb = kb == KIND_SPHERE || pb;   // balls
@@ -638,7 +638,7 @@ __device__ unsigned pair_apart(const PairRec& r, float T) {
   float d[3];   // centre of B minus centre of A (lattice units)
 #pragma unroll
   for (int k = 0; k < 3; ++k) d[k] = static_cast<float>(r.bi[k] - r.ai[k]) + (r.bf[k] - r.af[k]);
-  Apart ap;
+  Apart ap{margin};
   if (sa && sb) {
     // ball radii at 0 and at T: a sphere's r and r + T, a polytope's two tabulated radii
     const float a0 = r.sza[0], aT = pa ? r.sza[1] : r.sza[0] + T;
@@ -670,7 +670,7 @@ __device__ unsigned pair_apart(const PairRec& r, float T) {
         const float o = fmaxf(y[k] - (sz[k] + (t ? T : 0.f)), 0.f);
         d2 = fmaf(o, o, d2);
       }
-      dist[t] = sqrtf(d2) - kCullMargin;
+      dist[t] = sqrtf(d2) - margin;
     }
     // (T, T): box T, ball T; (0, T) and (T, 0) with the ball on side A or B
     const bool tt = dist[1] > rT, box0_ballT = dist[0] > rT, boxT_ball0 = dist[1] > r0;
@@ -949,7 +949,7 @@ __global__ void __launch_bounds__(32) k_build_pairs(Params P, Parts D, Lists W, 
       const int ka = pr.kinds & 0xff, kb = pr.kinds >> 8;
       constexpr bool boxm = BOXM;
       const bool test = !boxm || (boxm && ka != KIND_POLY && kb != KIND_POLY);
-      const unsigned apart = test ? pair_apart(pr, boxm ? kRoughT : 0.5f * P.wdx_l + kClipMargin) : 0u;
+      const unsigned apart = test ? pair_apart(pr, boxm ? kRoughT : 0.5f * P.wdx_l + P.clip_margin, P.clip_margin) : 0u;
       skip = (P.smooth || boxm) ? (apart & 1u) != 0u : (apart & 6u) == 6u;
       cut = boxm && !skip && (ka == KIND_CUBE || ka == KIND_CUBOID) && (kb == KIND_CUBE || kb == KIND_CUBOID);
       pr.tile = 0;

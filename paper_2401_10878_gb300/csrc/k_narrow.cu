@@ -493,7 +493,7 @@ __device__ __forceinline__ Partial sweep_tile(const Params& P, const Shapes& S, 
   E A, B;
   const int du = r.dim[L.u], dv = r.dim[L.v];
   const float inv_dv = __fdividef(1.f, static_cast<float>(dv));
-  const float inv_w = P.inv_w, hw = 0.5f * P.wdx_l, T = hw + kClipMargin;
+  const float inv_w = P.inv_w, hw = 0.5f * P.wdx_l, T = hw + P.clip_margin;
   if constexpr (ROLL && COOP) {
     A.attach(r, swap, S, L, smA);
     B.attach(r, !swap, S, L, smB);
@@ -1074,9 +1074,9 @@ __global__ void __launch_bounds__(kWarps * 32, GATHER ? 2 : 1) k_force(Params P,
 // ---------------------------------------------------------------- FP64 form
 // The all-FP64 form takes the FP32 form's tiles: warp w sweeps tiles w, w + W,
 // ...; each lane clips its lines in FP32 to the nodes near both surfaces (the
-// margin kClipMargin is far above the FP32 rounding, so every node left out has
-// a distance of at least w/2 in FP64 too and would add exact zeros), and the
-// clipped nodes, one per lane, are evaluated in FP64.  Bound: the FP64 pipe,
+// margin is above the FP32 rounding at every size (line_clip.cuh), so every node
+// left out has a distance of at least w/2 in FP64 too and would add exact
+// zeros), and the clipped nodes, one per lane, are evaluated in FP64.  Bound: the FP64 pipe,
 // ~64 cycles a warp instruction on this GPU.  One block per pair walking every
 // node of the pair box in FP64 spent 1006 us on 1934 cubes at 30 % (2.64e6
 // nodes, 1 % of which add to the sums); the clipped sweep takes 31 us.
@@ -1161,7 +1161,7 @@ __global__ void __launch_bounds__(kWarps * 32, 2) k_narrow64(Params P, Shapes S,
   if (ntiles > P.max_tiles) return;   // capacity exceeded: the step reports ECAPACITY
   const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
   const int nwarps = gridDim.x * kWarps;
-  const float hw = 0.5f * P.wdx_l, T = hw + kClipMargin;
+  const float hw = 0.5f * P.wdx_l, T = hw + P.clip_margin;
   const double inv_wdx = 1.0 / P.wdx;
   for (int t = blockIdx.x * kWarps + wid; t < ntiles; t += nwarps) {
     __syncwarp();

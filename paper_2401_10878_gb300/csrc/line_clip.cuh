@@ -9,26 +9,38 @@
 // (volume, moments, the normal's band terms, the deepest node) has both
 // distances below w/2 (Sec. 3.3.1's sweep restricted to the nodes where the
 // indicator product or one indicator's derivative is non-zero), so a sweep
-// clips each line to the two intervals at T = w/2 + kClipMargin and evaluates
+// clips each line to the two intervals at T = w/2 + the clip margin and evaluates
 // the nodes in between exactly as before: the nodes it skips would have added
 // exact zeros.
 //
 // The bounds are computed in FP32 in the line's node-counter space (the node
-// offset along the line relative to the particle's nearest node).  Their
-// rounding error is far below the margin: a face value has an absolute error
-// below 1e-5 cells, and a bound's relative error of a few ulps moves it by
-// less than 1e-5 cells divided by the face's slope along the line, the scale
-// at which the margin of 1e-3 cells acts too.  So every node whose FP32
-// distances are both below w/2 lies inside the clipped interval.
+// offset along the line relative to the particle's nearest node).  With u =
+// 2^-24 and D the largest distance of a node from a particle's centre (the
+// largest circumradius plus the band, cells), a face value's terms are rounded
+// to a few u D each, and a bound's relative error of a few u moves it by a few
+// u D divided by the face's slope along the line, the scale at which the margin
+// acts too: ~32 u D in all, taken as cells of distance, for a box (rotation
+// entries 2, offsets 5, quotients 11, sums 14), 8 u D for a sphere, and ~60 u D
+// for the pair builder's test of two boxes.  The margin is 128 u D = 2^-17 D,
+// and at least 1e-3 cells (the larger up to D = 131).  So every
+// node whose distances are both below w/2, in FP32 or in FP64, lies inside the
+// clipped interval.
 #pragma once
 
+#include <algorithm>
 #include <cuda_runtime.h>
 
 namespace gbc {
 
-constexpr float kClipMargin = 1e-3f;     // cells, added to the threshold of the clip
+constexpr float kClipMargin = 1e-3f;     // cells: the least margin added to the threshold of the clip
 constexpr float kClipFlat = 1e-20f;      // a face this parallel to the line is constant along it
 constexpr float kClipEmpty = 3.0e38f;    // a lower bound that empties the interval
+
+// The margin for particles of circumradius rmax and a band w (cells; host code):
+// two cells more reach every node of their node ranges.
+inline float clip_margin(double rmax, double w) {
+  return std::max(kClipMargin, static_cast<float>((rmax + w + 2.0) / 131072.0));
+}
 
 // Three-operand maximum and minimum (one instruction each on this GPU; like
 // fmaxf / fminf, a NaN operand gives way to the others).

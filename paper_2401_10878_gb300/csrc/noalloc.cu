@@ -22,6 +22,7 @@
 
 #include "../../include/contact.h"
 #include "contact_dev.cuh"
+#include "line_clip.cuh"
 
 using namespace gbc;
 
@@ -206,6 +207,7 @@ extern "C" contact_status contact_step_noalloc(const contact_config* cfg, const 
   P.inv_w = static_cast<float>(1.0 / C.smooth_width);
   P.neg6_over_w = static_cast<float>(-6.0 / C.smooth_width);
   P.wdx_l = static_cast<float>(C.smooth_width);
+  P.clip_margin = clip_margin(rmax / C.dx, C.smooth_width);
 
   int dev = 0;
   if (cudaGetDevice(&dev) != cudaSuccess) return CONTACT_ECUDA;

@@ -273,3 +273,23 @@ def test_larger_step_and_adjoint_equal_the_smaller(law):
         m.close()
     for a, b in zip(*outs):
         assert torch.equal(a, b)
+
+
+# turned so that the far corner's coordinates (tens of thousands of cells) cancel in every face value
+@pytest.mark.parametrize("seed", [13, 16, 201, 229])
+@pytest.mark.parametrize("kind", ["cuboid", "polytope"])
+def test_fp64_form_far_from_the_centres(seed, kind):
+    """Two long rods end to end, smoothed over a fiftieth of a cell: FP32 rounds
+    the ends' distances by a thousandth of a cell, and the all-FP64 form still
+    takes every node of the band."""
+    rng = np.random.default_rng(seed)
+    axis, angle = rng.normal(size=3), rng.uniform(0.3, 1.2)
+    q = [quat_axis_angle(axis, angle), quat_axis_angle(axis, angle + 1e-5)]
+    h, n = (32000.0, 30.0, 30.0), 128200
+    along = oracle.rotation(q[0])[:, 0]
+    a = np.full(3, 40000.0) + rng.random(3)
+    b = a + along * (2 * h[0] - 2.0) + 0.3 * rng.random(3)
+    t, planes = (W.CUBOID, None) if kind == "cuboid" else (W.POLYTOPE, [cube_planes(h)] * 2)
+    st = state([t] * 2, [h, h], np.mod([a, b], n), quat=q, n=n, planes=planes, indicator=1, w=0.02)
+    rep, ref = _parity(st, 1)
+    assert ref.n_pairs == 1 and ref.pair_out[0, 0] > 6000.0
