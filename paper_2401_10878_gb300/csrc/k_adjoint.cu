@@ -264,8 +264,9 @@ __device__ __forceinline__ void adj_pre_pass(const Params& P, const Shapes& S, c
       fric = fmag > 0.0 && utn2 > 0.0;
       const bool slip = a2 < 1e30;   // (above, the coefficient is mu_k)
       const double den1 = fma(a2, a2, 1.0), den2 = a2 + 1.0;
+      // (any positive argument; the two denominators only where they are used: finite)
       const double arg = k == 0 ? utn2 : (k == 1 ? den1 : (k == 2 ? den2 : damp));
-      const double yr = fl::nr_rsqrt(arg > 0.0 && arg < 1e60 ? arg : 1.0);
+      const double yr = fl::nr_rsqrt(arg > 0.0 && (slip || k == 0 || k == 3) ? arg : 1.0);
       inv_utn = at(yr, 0);
       const double i1 = at(yr, 1) * at(yr, 1), i2 = at(yr, 2) * at(yr, 2);
       inv_damp = __shfl_sync(kFull, yr, b0 + 3);

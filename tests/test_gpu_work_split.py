@@ -293,3 +293,26 @@ def test_fp64_form_far_from_the_centres(seed, kind):
     st = state([t] * 2, [h, h], np.mod([a, b], n), quat=q, n=n, planes=planes, indicator=1, w=0.02)
     rep, ref = _parity(st, 1)
     assert ref.n_pairs == 1 and ref.pair_out[0, 0] > 6000.0
+
+
+# small steps and ones whose overlapping pairs are gathered
+@pytest.mark.parametrize("n", [27, 4097])
+def test_adjoint_of_friction_at_any_speed(n):
+    """Velocities and u_K scaled by the same power of two leave the friction law,
+    and so forces and gradients, unchanged, also where |u_t|^2 is beyond 1e60.
+    (The adjoint's node seeds are FP32: an ulp of theirs is 6e-8.)"""
+    from paper_2401_10878_gb300.contact import Contact
+    st = W.mixed_grid_27() if n == 27 else _lattice_state(n)
+    st.indicator = 1
+    vel = np.random.default_rng(3).normal(size=(n, 6)) * 0.02
+    gf, gt = (torch.tensor(w, device="cuda") for w in W.loss_weights(n))
+    outs = []
+    for scale in (1.0, 2.0 ** 110):
+        m = Contact.from_state(st, friction=True, mu_s=0.3, mu_k=0.2, u_k=0.01 * scale)
+        o = m.step(torch.tensor(st.pos, device="cuda"), torch.tensor(st.quat, device="cuda"),
+                   torch.tensor(vel * scale, device="cuda"))
+        gp, gq = m.backward(gf, gt)
+        outs.append([o["force"].clone(), o["torque"].clone(), gp, gq])
+        m.close()
+    for (a, b), tol in zip(zip(*outs), (1e-12, 1e-12, 1e-6, 1e-6)):
+        assert float((a - b).abs().max()) <= tol * float(a.abs().max())
