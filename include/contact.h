@@ -342,7 +342,7 @@ void contact_destroy(contact_ctx* ctx);
  * pair boxes of up to 256 lines on average), and the cell list's limits (at
  * most CONTACT_NOALLOC_MAX_BINS bins per axis, and bins x bin capacity at
  * most CONTACT_NOALLOC_MAX_BIN_ENTRIES).  contact_init allows 8 tiles per
- * pair, 256 bins per axis and 2^26 bin entries. */
+ * pair, 256 bins per axis and 2^26 bin entries (of 20 bytes: at most 1.25 GiB). */
 #define CONTACT_NOALLOC_SCRATCH_MIB 32
 #define CONTACT_NOALLOC_MAX_PARTICLES 2048
 #define CONTACT_NOALLOC_MAX_PAIRS 8192

@@ -107,8 +107,7 @@ struct Params {
   double damp_K;         // history: c = damp_K / u0 at a contact's first step (u0 > 0)
   double mu_s_star, mu_k, inv_u_k;   // friction law
   int nbin[3];           // bins per axis
-  int bin_cap;           // particles one bin can hold
-  int bin_stride;        // entries of a bin's rows (bin_cap rounded up to a multiple of four: 16-byte loads)
+  int bin_cap;           // particles one bin can hold (its row length)
   int wide;              // 1: a node range may span more than kMaxLen nodes (BinRec's lengths do not hold it)
   double binw[3];        // bin width (physical)
   float inv_binw_f[3];   // FP32 reciprocal of the bin width
@@ -164,6 +163,7 @@ struct __align__(16) BinRec {
   int lo[3];
   unsigned len;
 };
+constexpr int kBinEntryBytes = sizeof(BinRec) + sizeof(int);   // with the particle's number
 constexpr int kMaxLen = 1023;
 constexpr int kNoNodes = -0x40000000;
 
@@ -287,8 +287,8 @@ static_assert(sizeof(BoxWork) % 16 == 0, "consecutive records stay aligned");
 
 struct Lists {
   int* bin_count;   // [nbins]
-  int* bin_items;   // [nbins, bin_stride] particles of each bin, in arrival order
-  BinRec* bin_rec;  // [nbins, bin_stride] their node ranges
+  int* bin_items;   // [nbins, bin_cap] particles of each bin, in arrival order
+  BinRec* bin_rec;  // [nbins, bin_cap] their node ranges
   int* up_count;    // [N] partners j > p
   int* up_list;     // [N, max_nbr]
   int* dn_count;    // [N] partners i < p
@@ -565,8 +565,7 @@ __device__ __forceinline__ int gather_pairs(const int* oflag, int q0, int cnt, i
   return *s_n;
 }
 constexpr int kRowGroup = 256;   // particles per group sum of the pair-row offsets
-// the row length of bin_cap entries, and whether BinRec's lengths suffice for particles of circumradius rmax
-inline int bin_row(int bin_cap) { return (bin_cap + 3) & ~3; }
+// whether node ranges of particles of circumradius rmax may exceed BinRec's lengths
 inline int wide_ranges(double rmax, double dx) { return 2.0 * rmax / dx + 3.0 >= kMaxLen ? 1 : 0; }
 int bin_capacity(int n, const double binw[3], double rin_min, long long nbins, long long max_entries);
 void launch_narrow(const Params& P, const Shapes& S, const Parts& D, const Lists& W, const double* vel,

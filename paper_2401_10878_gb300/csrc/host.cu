@@ -79,7 +79,8 @@ namespace gbc {
 // Slots per cell-list bin: at most n, else twice the bin volume over the
 // smallest inscribed-ball volume plus 8 (particles overlap only by their
 // contact indentation, so far fewer centres fit in a bin), at least 16, and
-// at most max_entries / nbins.  A fuller bin is reported as ECAPACITY.
+// at most max_entries / nbins (nbins is at most max_entries).  An entry takes
+// kBinEntryBytes.  A fuller bin is reported as ECAPACITY.
 int bin_capacity(int n, const double binw[3], double rin_min, long long nbins, long long max_entries) {
   const double vmin = 4.0 / 3.0 * 3.14159265358979323846 * rin_min * rin_min * rin_min;
   const double bound = 2.0 * binw[0] * binw[1] * binw[2] / vmin + 8.0;
@@ -498,7 +499,6 @@ contact_status contact_init(const contact_config* cfg, const int32_t* shape_type
     P.inv_binw_f[k] = static_cast<float>(nb / L[k]);
   }
   P.bin_cap = bin_capacity(n, P.binw, rin_min, static_cast<long long>(P.nbin[0]) * P.nbin[1] * P.nbin[2], 1LL << 26);
-  P.bin_stride = bin_row(P.bin_cap);
   P.wide = wide_ranges(rmax, C.dx);
   P.dx = C.dx;
   P.inv_dx = 1.0 / C.dx;
@@ -633,8 +633,8 @@ contact_status contact_init(const contact_config* cfg, const int32_t* shape_type
   const size_t nbins = static_cast<size_t>(P.nbin[0]) * P.nbin[1] * P.nbin[2];
   const size_t mp = static_cast<size_t>(C.max_pairs), mt = static_cast<size_t>(P.max_tiles);
   GBC_TRY(dev_alloc(c, &W.bin_count, nbins));
-  GBC_TRY(dev_alloc(c, &W.bin_items, nbins * static_cast<size_t>(P.bin_stride)));
-  GBC_TRY(dev_alloc(c, &W.bin_rec, nbins * static_cast<size_t>(P.bin_stride)));
+  GBC_TRY(dev_alloc(c, &W.bin_items, nbins * static_cast<size_t>(P.bin_cap)));
+  GBC_TRY(dev_alloc(c, &W.bin_rec, nbins * static_cast<size_t>(P.bin_cap)));
   GBC_TRY(dev_alloc(c, &W.up_count, static_cast<size_t>(n)));
   GBC_TRY(dev_alloc(c, &W.up_list, static_cast<size_t>(n) * max_nbr));
   GBC_TRY(dev_alloc(c, &W.dn_count, static_cast<size_t>(n)));

@@ -26,7 +26,7 @@ __device__ __forceinline__ void bin_insert(const Params& P, const Lists& W, int 
     set_error(W.err, kErrCapacity);
     return;
   }
-  const size_t at = static_cast<size_t>(b) * P.bin_stride + slot;
+  const size_t at = static_cast<size_t>(b) * P.bin_cap + slot;
   const bool empty = hi[0] < lo[0] || hi[1] < lo[1] || hi[2] < lo[2];
   unsigned len = 0;
 #pragma unroll
@@ -420,7 +420,7 @@ __global__ void __launch_bounds__(kBroadWarps * 32, 8) k_broad(Params P, Parts D
     if (use) {
       const int q = checked_index(W.err, c[0] + P.nbin[0] * (c[1] + P.nbin[1] * c[2]),
                                   static_cast<long long>(P.nbin[0]) * P.nbin[1] * P.nbin[2], 0);
-      row[s] = static_cast<unsigned>(q) * static_cast<unsigned>(P.bin_stride);
+      row[s] = static_cast<unsigned>(q) * static_cast<unsigned>(P.bin_cap);
       num[s] = min(W.bin_count[q], P.bin_cap);
     }
   }

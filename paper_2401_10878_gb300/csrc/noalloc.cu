@@ -32,6 +32,20 @@ constexpr size_t kScratchBytes = static_cast<size_t>(CONTACT_NOALLOC_SCRATCH_MIB
 constexpr int kMaxNbr = 64;
 constexpr int kMaxTilesPerPair = CONTACT_NOALLOC_TILES_PER_PAIR;
 constexpr int kMaxBinsPerAxis = CONTACT_NOALLOC_MAX_BINS;
+constexpr size_t kMaxBins = static_cast<size_t>(kMaxBinsPerAxis) * kMaxBinsPerAxis * kMaxBinsPerAxis;
+
+// The largest call fits: per particle (shape tables, pose, line, neighbour
+// lists), per pair (overlap record and flag, tape, forces, tile counter), per
+// tile, the cell list, and 256 bytes for each region's alignment.
+constexpr size_t kMaxCarve =
+    CONTACT_NOALLOC_MAX_PARTICLES *
+        (8 * sizeof(int) + 3 * sizeof(float) + 25 * sizeof(double) + sizeof(PartRec) + 3 * kMaxNbr * sizeof(int)) +
+    CONTACT_NOALLOC_MAX_PAIRS *
+        (sizeof(OvlRec) + 2 * sizeof(int) + (kTapeDoubles + kFtDoubles) * sizeof(double)) +
+    static_cast<size_t>(kMaxTilesPerPair) * CONTACT_NOALLOC_MAX_PAIRS * (sizeof(PairRec) + kPartialFloats * sizeof(float)) +
+    kMaxBins * sizeof(int) + static_cast<size_t>(CONTACT_NOALLOC_MAX_BIN_ENTRIES) * kBinEntryBytes + 64 * 256;
+static_assert(kMaxBins <= CONTACT_NOALLOC_MAX_BIN_ENTRIES && kMaxCarve <= kScratchBytes,
+              "the scratch array holds the largest call");
 
 __device__ __align__(256) unsigned char g_scratch[kScratchBytes];
 
@@ -182,7 +196,6 @@ extern "C" contact_status contact_step_noalloc(const contact_config* cfg, const 
   }
   P.bin_cap = bin_capacity(n, P.binw, rin_min, static_cast<long long>(P.nbin[0]) * P.nbin[1] * P.nbin[2],
                            CONTACT_NOALLOC_MAX_BIN_ENTRIES);
-  P.bin_stride = bin_row(P.bin_cap);
   P.wide = wide_ranges(rmax, C.dx);
   P.dx = C.dx;
   P.inv_dx = 1.0 / C.dx;
@@ -245,8 +258,8 @@ extern "C" contact_status contact_step_noalloc(const contact_config* cfg, const 
   D.wplane = cv.take<float4>(1);
   Lists W{};
   W.bin_count = cv.take<int>(nbins);
-  W.bin_items = cv.take<int>(static_cast<size_t>(nbins) * P.bin_stride);
-  W.bin_rec = cv.take<BinRec>(static_cast<size_t>(nbins) * P.bin_stride);
+  W.bin_items = cv.take<int>(static_cast<size_t>(nbins) * P.bin_cap);
+  W.bin_rec = cv.take<BinRec>(static_cast<size_t>(nbins) * P.bin_cap);
   W.up_count = cv.take<int>(N);
   W.up_list = cv.take<int>(N * kMaxNbr);
   W.dn_count = cv.take<int>(N);

@@ -316,3 +316,19 @@ def test_adjoint_of_friction_at_any_speed(n):
         m.close()
     for (a, b), tol in zip(zip(*outs), (1e-12, 1e-12, 1e-6, 1e-6)):
         assert float((a - b).abs().max()) <= tol * float(a.abs().max())
+
+
+def test_cell_list_memory():
+    """The cell list keeps to its 2^26 entries of 20 bytes (five in each of 235^3 bins here)."""
+    from paper_2401_10878_gb300.contact import Contact
+    n, box = 16, 940
+    x = np.random.default_rng(0).random((n, 3)) * 900.0
+    st = state([W.SPHERE] * n, [[1.0, 0, 0]] * n, x, n=box)
+    torch.cuda.synchronize()
+    before = torch.cuda.mem_get_info()[0]
+    m = Contact.from_state(st)
+    used = before - torch.cuda.mem_get_info()[0]
+    assert m.stats()["bins_x"] == 235
+    m.close()
+    entries, counts, rest = 2 ** 26 * 20, 4 * 235 ** 3, 64 << 20
+    assert 235 ** 3 * 5 * 20 <= used <= entries + counts + rest
