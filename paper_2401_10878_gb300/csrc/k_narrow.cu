@@ -79,6 +79,7 @@ __device__ __forceinline__ float world_comp(int c, const Local& L, float au, flo
 // |y_k| < h + T is the node-counter interval centred at
 // c_k = fu - (tv_k rv + tw_k rw) / tu_k with half-width (h + T) / |tu_k|.
 struct CubeEval {
+  static constexpr bool kCube = true;
   int iu;
   float fu, tu0, tu1, tu2, h, itu0, itu1, itu2;
   bool flat;   // a slab parallel to the lines (|tu_k| <= kClipFlat): the general clip
@@ -258,8 +259,10 @@ __device__ __forceinline__ void stage_planes(const Shapes& S, const Parts& D, in
 // kClipFlat: the plane, which keeps or empties the whole line).  POLY: there
 // are polytopes; CUBE: cubes are swept as CubeEval does (its constants in cs),
 // else as cuboids.
+constexpr int kAnyKind = -1;   // as a kind known at compile time: none, the evaluator's own
 template <bool POLY, bool CUBE>
 struct AnyEval {
+  static constexpr bool kCube = CUBE;
   int kind, iu, iv, iw, nf, nup, ndn;
   float fu, fv, fw;
   const float4* cs;
@@ -365,8 +368,10 @@ struct AnyEval {
     hi = h + o;
   }
   // phi at node (u, cv, cw), and d: the direction that add(m, d) adds m times
-  // (a sphere's d.w scales m)
+  // (a sphere's d.w scales m).  K: the kind, or kAnyKind
+  template <int K>
   __device__ __forceinline__ float phi(int u, int cv, int cw, float4& d) const {
+    const int kind = K == kAnyKind ? this->kind : K;
     if (CUBE && kind == KIND_CUBE) {
       CubeEval e;
       e.fetch(cs);
@@ -418,8 +423,10 @@ struct AnyEval {
                     (!s0 && !s1) ? copysignf(1.f, y[2]) : 0.f, 1.f);
     return fmaxf(a[0], fmaxf(a[1], a[2]));
   }
+  template <int K>
   __device__ __forceinline__ void add(float m, const float4& d) {
-    replay(record(m, d));
+    if (K == KIND_WALL) g0 += m;   // (all of its band sum)
+    else replay(record(m, d));
   }
   // what add(m, d) adds, and the same additions later (shared tiles)
   static __device__ __forceinline__ float4 record(float m, const float4& d) {
@@ -461,6 +468,37 @@ struct CoopNode {
   float f;              // depth and node index
   int idx;
 };
+template <int K>
+using KindC = std::integral_constant<int, K>;
+// f(kind of A, kind of B) as compile-time constants, for pairs without a polytope (A is the cheaper kind,
+// sweep_swap's order); CUBE: cubes are a kind of their own, else cuboids
+template <bool CUBE, class F>
+__device__ __forceinline__ void with_kinds(int a, int b, const F& f) {
+  if (a == KIND_WALL) {
+    if (b == KIND_SPHERE) f(KindC<KIND_WALL>{}, KindC<KIND_SPHERE>{});
+    else if (CUBE && b == KIND_CUBE) f(KindC<KIND_WALL>{}, KindC<KIND_CUBE>{});
+    else f(KindC<KIND_WALL>{}, KindC<KIND_CUBOID>{});
+  } else if (a == KIND_SPHERE) {
+    if (b == KIND_SPHERE) f(KindC<KIND_SPHERE>{}, KindC<KIND_SPHERE>{});
+    else if (CUBE && b == KIND_CUBE) f(KindC<KIND_SPHERE>{}, KindC<KIND_CUBE>{});
+    else f(KindC<KIND_SPHERE>{}, KindC<KIND_CUBOID>{});
+  } else if (CUBE && a == KIND_CUBE) {
+    if (b == KIND_CUBE) f(KindC<KIND_CUBE>{}, KindC<KIND_CUBE>{});
+    else f(KindC<KIND_CUBE>{}, KindC<KIND_CUBOID>{});
+  } else {
+    f(KindC<KIND_CUBOID>{}, KindC<KIND_CUBOID>{});
+  }
+}
+// The node passes of a tile of more clipped nodes than this, of two particles
+// that are no polytopes, run through a loop compiled for their kinds: it keeps
+// their constants in registers, a quarter of the run-time evaluator's
+// instructions fewer.  In shallow tiles the loops' code would be fetched for one
+// or two passes (32, 64 and 128 nodes differ by less than the runs).  Node sweep
+// with a sweep compiled per kind pair, with the run-time evaluator alone and
+// with these loops: 4000 cuboids of 26 cells pressed on a floor and a ceiling
+// 262, 322, 260 us; 2000 spheres and cuboids 137, 168, 134; 4000 mixed particles
+// 272, 262, 235; 4000 cuboids and one polytope 374, 378, 305.
+constexpr int kDeepNodes = 64;
 constexpr int kShareNodes = 128;   // a tile of more clipped nodes is shared when every warp has at most one tile
 
 // Order-preserving map of FP32 values to signed ints (for integer max).
@@ -606,105 +644,115 @@ __device__ __forceinline__ Partial sweep_tile(const Params& P, const Shapes& S, 
   // lanes) - 1 of own, counted from the lanes that start before the pass and
   // a mask of the first nodes inside it
   const int step = COOP ? 32 * nwarp : 32;
-  for (int base0 = 0; base0 < total; base0 += step) {
-    const int base = COOP ? base0 + 32 * wid : base0;
-    const int g = base + lane;
-    const unsigned before = __ballot_sync(kFull, has && excl < base);
-    const unsigned inside =
-        __reduce_or_sync(kFull, (has && excl >= base && excl - base < 32) ? 1u << (excl - base) : 0u);
-    const int cnt_le = __popc(before) + __popc(inside & (lane == 31 ? 0xffffffffu : (2u << lane) - 1u));
-    const int4 e = own[min(max(cnt_le - 1, 0), 31)];
-    const int o = e.x;
-    const int k = g - e.y;   // the node's rank among the owner's
-    const int4 e2 = own[32 + min(max(cnt_le - 1, 0), 31)];
-    // the slot: how many of the owner's slot boundaries (node counts before
-    // slots 1, 2, 3; empty slots repeat a boundary) lie at or below k
-    const int c1 = static_cast<int>(static_cast<unsigned>(e.z) >> 16), c2 = e2.z, c3 = e2.w;
-    const int os = (k >= c1 ? 1 : 0) + (k >= c2 ? 1 : 0) + (k >= c3 ? 1 : 0);
-    const unsigned q = static_cast<unsigned>(os == 0 ? e.z : (os == 1 ? e.w : (os == 2 ? e2.x : e2.y)));
-    const int u = static_cast<int>(q & 0xffffu) + k - (os == 0 ? 0 : (os == 1 ? c1 : (os == 2 ? c2 : c3)));
-    int ocv;
-    const int ocw = div_small(it0 + os * 32 + o, dv, inv_dv, &ocv);
-    float fa, fb;
-    float4 da, db;
-    if constexpr (ROLL) {
-      fa = A.phi(u, ocv, ocw, da);
-      fb = B.phi(u, ocv, ocw, db);
-    } else {
-      A.begin_node(csA, ocv, ocw, u);
-      B.begin_node(csB, ocv, ocw, u);
-      fa = A.phi();
-      fb = B.phi();
-    }
-    // W > 0, or a band term of the normal: max < w/2 and (sharp) min <= 0
-    const bool any = g < total && fmaxf(fa, fb) < hw && (SMOOTH || fminf(fa, fb) <= 0.f);
-    const float ta = __saturatef(fmaf(fa, -inv_w, 0.5f));
-    const float tb = __saturatef(fmaf(fb, -inv_w, 0.5f));
-    float w, ma, mb;
-    if (SMOOTH) {
-      const float ha = ta * ta * fmaf(-2.f, ta, 3.f);
-      const float hb = tb * tb * fmaf(-2.f, tb, 3.f);
-      w = any ? ha * hb : 0.f;
-      ma = any ? fmaf(-ta, ta, ta) * hb : 0.f;
-      mb = any ? ha * fmaf(-tb, tb, tb) : 0.f;
-    } else {
-      w = (any && fmaxf(fa, fb) <= 0.f) ? 1.f : 0.f;
-      ma = (any && fb <= 0.f) ? fmaf(-ta, ta, ta) : 0.f;
-      mb = (any && fa <= 0.f) ? fmaf(-tb, tb, tb) : 0.f;
-    }
-    float f = -(fa + fb);
-    int idx = u * L.su + ocv * L.sv + ocw * L.sw;
-    if constexpr (COOP) {
-      if (base < total) {   // warp-uniform
-        CoopNode& c = coop[32 * wid + lane];
-        if constexpr (ROLL) {
-          c.ga = E::record(ma, da);
-          c.gb = E::record(mb, db);
-        } else {
-          c.ga = A.record(ma);
-          c.gb = B.record(mb);
-        }
-        c.mom = make_float4(w, static_cast<float>(u), static_cast<float>(ocv), static_cast<float>(ocw));
-        c.f = f;
-        c.idx = idx;
-      }
-      __syncthreads();
-      if (wid == 0) {
-        for (int q = 0; q < nwarp && base0 + 32 * q < total; ++q) {
-          const CoopNode& c = coop[32 * q + lane];
-          const float4 m = c.mom;
-          cnt += m.x;
-          mu = fmaf(m.x, m.y, mu);
-          mv = fmaf(m.x, m.z, mv);
-          mw = fmaf(m.x, m.w, mw);
-          f = c.f;
-          idx = c.idx;
-          if (m.x > 0.f && (f > bestf || (f == bestf && idx < bestidx))) {
-            bestf = f;
-            bestidx = idx;
-          }
-          A.replay(c.ga);
-          B.replay(c.gb);
-        }
-      }
-      __syncthreads();
-    } else {
-      cnt += w;
-      mu = fmaf(w, static_cast<float>(u), mu);
-      mv = fmaf(w, static_cast<float>(ocv), mv);
-      mw = fmaf(w, static_cast<float>(ocw), mw);
-      if (w > 0.f && (f > bestf || (f == bestf && idx < bestidx))) {
-        bestf = f;
-        bestidx = idx;
-      }
+  // (KA, KB: the kinds of A and B where the caller knows them)
+  auto passes = [&](auto ka, auto kb) {
+    [[maybe_unused]] constexpr int KA = decltype(ka)::value, KB = decltype(kb)::value;
+    for (int base0 = 0; base0 < total; base0 += step) {
+      const int base = COOP ? base0 + 32 * wid : base0;
+      const int g = base + lane;
+      const unsigned before = __ballot_sync(kFull, has && excl < base);
+      const unsigned inside =
+          __reduce_or_sync(kFull, (has && excl >= base && excl - base < 32) ? 1u << (excl - base) : 0u);
+      const int cnt_le = __popc(before) + __popc(inside & (lane == 31 ? 0xffffffffu : (2u << lane) - 1u));
+      const int4 e = own[min(max(cnt_le - 1, 0), 31)];
+      const int o = e.x;
+      const int k = g - e.y;   // the node's rank among the owner's
+      const int4 e2 = own[32 + min(max(cnt_le - 1, 0), 31)];
+      // the slot: how many of the owner's slot boundaries (node counts before
+      // slots 1, 2, 3; empty slots repeat a boundary) lie at or below k
+      const int c1 = static_cast<int>(static_cast<unsigned>(e.z) >> 16), c2 = e2.z, c3 = e2.w;
+      const int os = (k >= c1 ? 1 : 0) + (k >= c2 ? 1 : 0) + (k >= c3 ? 1 : 0);
+      const unsigned q = static_cast<unsigned>(os == 0 ? e.z : (os == 1 ? e.w : (os == 2 ? e2.x : e2.y)));
+      const int u = static_cast<int>(q & 0xffffu) + k - (os == 0 ? 0 : (os == 1 ? c1 : (os == 2 ? c2 : c3)));
+      int ocv;
+      const int ocw = div_small(it0 + os * 32 + o, dv, inv_dv, &ocv);
+      float fa, fb;
+      float4 da, db;
       if constexpr (ROLL) {
-        A.add(ma, da);
-        B.add(mb, db);
+        fa = A.template phi<KA>(u, ocv, ocw, da);
+        fb = B.template phi<KB>(u, ocv, ocw, db);
       } else {
-        A.grad(ma);
-        B.grad(mb);
+        A.begin_node(csA, ocv, ocw, u);
+        B.begin_node(csB, ocv, ocw, u);
+        fa = A.phi();
+        fb = B.phi();
+      }
+      // W > 0, or a band term of the normal: max < w/2 and (sharp) min <= 0
+      const bool any = g < total && fmaxf(fa, fb) < hw && (SMOOTH || fminf(fa, fb) <= 0.f);
+      const float ta = __saturatef(fmaf(fa, -inv_w, 0.5f));
+      const float tb = __saturatef(fmaf(fb, -inv_w, 0.5f));
+      float w, ma, mb;
+      if (SMOOTH) {
+        const float ha = ta * ta * fmaf(-2.f, ta, 3.f);
+        const float hb = tb * tb * fmaf(-2.f, tb, 3.f);
+        w = any ? ha * hb : 0.f;
+        ma = any ? fmaf(-ta, ta, ta) * hb : 0.f;
+        mb = any ? ha * fmaf(-tb, tb, tb) : 0.f;
+      } else {
+        w = (any && fmaxf(fa, fb) <= 0.f) ? 1.f : 0.f;
+        ma = (any && fb <= 0.f) ? fmaf(-ta, ta, ta) : 0.f;
+        mb = (any && fa <= 0.f) ? fmaf(-tb, tb, tb) : 0.f;
+      }
+      float f = -(fa + fb);
+      int idx = u * L.su + ocv * L.sv + ocw * L.sw;
+      if constexpr (COOP) {
+        if (base < total) {   // warp-uniform
+          CoopNode& c = coop[32 * wid + lane];
+          if constexpr (ROLL) {
+            c.ga = E::record(ma, da);
+            c.gb = E::record(mb, db);
+          } else {
+            c.ga = A.record(ma);
+            c.gb = B.record(mb);
+          }
+          c.mom = make_float4(w, static_cast<float>(u), static_cast<float>(ocv), static_cast<float>(ocw));
+          c.f = f;
+          c.idx = idx;
+        }
+        __syncthreads();
+        if (wid == 0) {
+          for (int q = 0; q < nwarp && base0 + 32 * q < total; ++q) {
+            const CoopNode& c = coop[32 * q + lane];
+            const float4 m = c.mom;
+            cnt += m.x;
+            mu = fmaf(m.x, m.y, mu);
+            mv = fmaf(m.x, m.z, mv);
+            mw = fmaf(m.x, m.w, mw);
+            f = c.f;
+            idx = c.idx;
+            if (m.x > 0.f && (f > bestf || (f == bestf && idx < bestidx))) {
+              bestf = f;
+              bestidx = idx;
+            }
+            A.replay(c.ga);
+            B.replay(c.gb);
+          }
+        }
+        __syncthreads();
+      } else {
+        cnt += w;
+        mu = fmaf(w, static_cast<float>(u), mu);
+        mv = fmaf(w, static_cast<float>(ocv), mv);
+        mw = fmaf(w, static_cast<float>(ocw), mw);
+        if (w > 0.f && (f > bestf || (f == bestf && idx < bestidx))) {
+          bestf = f;
+          bestidx = idx;
+        }
+        if constexpr (ROLL) {
+          A.template add<KA>(ma, da);
+          B.template add<KB>(mb, db);
+        } else {
+          A.grad(ma);
+          B.grad(mb);
+        }
       }
     }
+  };
+  if constexpr (ROLL && !COOP) {
+    if (total > kDeepNodes && A.kind != KIND_POLY && B.kind != KIND_POLY) with_kinds<E::kCube>(A.kind, B.kind, passes);
+    else passes(KindC<kAnyKind>{}, KindC<kAnyKind>{});
+  } else {
+    passes(KindC<kAnyKind>{}, KindC<kAnyKind>{});
   }
   Partial o;
   o.cnt = cnt;
@@ -934,8 +982,7 @@ __global__ void __launch_bounds__(narrow_warps<SET>() * 32, narrow_blocks<SET>()
   // (400 cubes, one in seven pressed into a neighbour: 16.0 -> 11.9 us; 135 larger
   // cubes between walls, hundreds of nodes per wall contact: 28.3 -> 15.4 us; 123
   // mixed particles with walls: 24.7 -> 14.3 us; 2568 spheres and cuboids, one in
-  // ten pressed: 25.0 -> 14.0 us.  The run-time evaluator alone was slower there
-  // than a sweep per kind pair, 22.1, 25.3 and 20.1 us.)
+  // ten pressed: 25.0 -> 14.0 us)
   const bool share = ntiles <= nwarps;
   if (share) {
     if (threadIdx.x == 0) s_ndeferred = 0;
