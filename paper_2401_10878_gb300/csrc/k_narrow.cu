@@ -1119,8 +1119,8 @@ __global__ void __launch_bounds__(kWarps * 32, GATHER ? 2 : 1) k_force(Params P,
 }
 
 // ---------------------------------------------------------------- FP64 form
-// The all-FP64 form takes the FP32 form's tiles: warp w sweeps tiles w, w + W,
-// ...; each lane clips its lines in FP32 to the nodes near both surfaces (the
+// The all-FP64 form takes the FP32 form's tiles, one per warp or, when there are
+// few, one per two to eight warps of a block; each lane clips its lines in FP32 to the nodes near both surfaces (the
 // margin is above the FP32 rounding at every size (line_clip.cuh), so every node
 // left out has a distance of at least w/2 in FP64 too and would add exact
 // zeros), and the clipped nodes, one per lane, are evaluated in FP64.  Bound: the FP64 pipe,
@@ -1197,30 +1197,43 @@ __device__ __forceinline__ void tile_done64(const Lists& W, const PairRec& r, do
   pair_done(W, r, acc, __shfl_sync(kFull, bi, 7));
 }
 
-template <bool SMOOTH>
-__global__ void __launch_bounds__(kWarps * 32, 2) k_narrow64(Params P, Shapes S, Parts D, Lists W) {
-  __shared__ __align__(16) PairRec s_rec[kWarps];
-  __shared__ float4 s_planes[kWarps][2][2 * kMaxFaces];       // the clips' constants
-  __shared__ unsigned s_pk[kWarps][kTileItemsPerLane * 32];   // clipped ranges: first node | count << 16
-  __shared__ int s_excl[kWarps][32];                          // nodes before each lane's
-  pdl_begin();
-  const int ntiles = W.counters[1];
-  if (ntiles > P.max_tiles) return;   // capacity exceeded: the step reports ECAPACITY
+// What a node adds to the sums.
+struct Node64 {
+  double w, g[3];   // weight, band terms
+  long long key;    // depth (order_key)
+  int c[3], idx;    // node, linear index
+};
+
+// The sweep's shared memory, per warp of a block.
+struct Shared64 {
+  alignas(16) PairRec rec[kWarps];
+  float4 planes[kWarps][2][2 * kMaxFaces];       // the clips' constants
+  unsigned pk[kWarps][kTileItemsPerLane * 32];   // clipped ranges: first node | count << 16
+  int excl[kWarps][32];                          // nodes before each lane's
+  Node64 node[kWarps][32];                       // a shared tile's nodes
+};
+
+// The tiles of the calling warp.  SHARE: G = 2, 4 or 8 warps of a block have one
+// tile, warp gw of them its node passes gw, gw + G, ... (at most one tile a group).
+template <bool SMOOTH, bool SHARE>
+__device__ __forceinline__ void sweep64(const Params& P, const Shapes& S, const Parts& D, const Lists& W, Shared64& sm,
+                                        int ntiles, int G) {
   const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-  const int nwarps = gridDim.x * kWarps;
   const float hw = 0.5f * P.wdx_l, T = hw + P.clip_margin;
   const double inv_wdx = 1.0 / P.wdx;
-  for (int t = blockIdx.x * kWarps + wid; t < ntiles; t += nwarps) {
+  const int group = SHARE ? wid / G : wid, gw = SHARE ? wid % G : 0;
+  auto group_sync = [&]() { asm volatile("bar.sync %0, %1;" ::"r"(group + 1), "r"(32 * G) : "memory"); };
+  for (int t = blockIdx.x + gridDim.x * group; t < ntiles; t += SHARE ? ntiles : gridDim.x * kWarps) {
     __syncwarp();
-    store_rec_part(&s_rec[wid], lane, load_rec_part(W.tiles + t, lane));
+    store_rec_part(&sm.rec[wid], lane, load_rec_part(W.tiles + t, lane));
     __syncwarp();
-    const PairRec& r = s_rec[wid];
+    const PairRec& r = sm.rec[wid];
     if (!record_in_bounds(P, W.err, r, true)) continue;   // warp-uniform (checked build only)
     const Local L = make_local(r);
     const int i = r.i, j = r.j;
     AnyEval<true, false> A, B;
-    A.load(r, false, S, D, L, T, s_planes[wid][0]);
-    B.load(r, true, S, D, L, T, s_planes[wid][1]);
+    A.load(r, false, S, D, L, T, sm.planes[wid][0]);
+    B.load(r, true, S, D, L, T, sm.planes[wid][1]);
     __syncwarp();
     // both particles in FP64 (the same address on every lane)
     double XA[3], XB[3], RA[9], RB[9];
@@ -1254,7 +1267,7 @@ __global__ void __launch_bounds__(kWarps * 32, 2) k_narrow64(Params P, Shapes S,
       B.clip_line(r, true, L, nullptr, cv, cw, T, clo, chi);
       int ub;
       const int nk = clip_nodes(clo, chi, 0, len, &ub);
-      s_pk[wid][s * 32 + lane] = static_cast<unsigned>(ub) | (static_cast<unsigned>(nk) << 16);
+      sm.pk[wid][s * 32 + lane] = static_cast<unsigned>(ub) | (static_cast<unsigned>(nk) << 16);
       nl += nk;
     }
     int incl = nl;
@@ -1264,61 +1277,96 @@ __global__ void __launch_bounds__(kWarps * 32, 2) k_narrow64(Params P, Shapes S,
       if (lane >= d) incl += v;
     }
     const int total = __shfl_sync(kFull, incl, 31);
-    s_excl[wid][lane] = incl - nl;
+    sm.excl[wid][lane] = incl - nl;
     __syncwarp();
     // (B) node g of the clipped nodes on lane g mod 32
     double acc[8] = {0.0, 0.0, 0.0, 0.0, 0.0, 0.0, 0.0, 0.0};
     long long bk = LLONG_MIN;
     int bi = 0x7fffffff;
-    for (int base = 0; base < total; base += 32) {
-      const int g = base + lane;
-      if (g < total) {
-        int o = 0;   // the owner: the last lane whose first node is <= g (lanes without nodes repeat the next one's)
+    auto node = [&](int g, Node64& e) {
+      int o = 0;   // the owner: the last lane whose first node is <= g (lanes without nodes repeat the next one's)
 #pragma unroll
-        for (int d = 16; d > 0; d >>= 1)
-          if (s_excl[wid][o + d] <= g) o += d;
-        int k = g - s_excl[wid][o], s = 0, n;
-        unsigned q = s_pk[wid][o];
-        while (k >= (n = static_cast<int>(q >> 16)) && s < ns - 1) {
-          k -= n;
-          q = s_pk[wid][++s * 32 + o];
-        }
-        const int u = static_cast<int>(q & 0xffffu) + k;
-        int cv;
-        const int cw = div_small(it0 + s * 32 + o, dv, inv_dv, &cv);
-        const int c[3] = {L.u == 0 ? u : (L.u == 1 ? cw : cv), L.u == 1 ? u : (L.u == 2 ? cw : cv),
-                          L.u == 2 ? u : (L.u == 0 ? cw : cv)};
-        const double x[3] = {(r.lo[0] + c[0]) * P.dx, (r.lo[1] + c[1]) * P.dx, (r.lo[2] + c[2]) * P.dx};
-        double gA[3], gB[3];
-        const double pa = sdf64(ta, S.param + 3 * i, pla, nfa, XA, RA, x, P.inflate, gA);
-        const double pb = sdf64(tb, S.param + 3 * j, plb, nfb, XB, RB, x, P.inflate, gB);
-        const double tA = fmin(fmax(fma(-pa, inv_wdx, 0.5), 0.0), 1.0);
-        const double tB = fmin(fmax(fma(-pb, inv_wdx, 0.5), 0.0), 1.0);
-        double hA, hB;
-        if (SMOOTH) {
-          hA = tA * tA * (3.0 - 2.0 * tA);
-          hB = tB * tB * (3.0 - 2.0 * tB);
-        } else {
-          hA = pa <= 0.0 ? 1.0 : 0.0;
-          hB = pb <= 0.0 ? 1.0 : 0.0;
-        }
-        const double w = hA * hB;
-        const double ma = tA * (1.0 - tA) * hB, mb = hA * tB * (1.0 - tB);
-        acc[0] += w;
+      for (int d = 16; d > 0; d >>= 1)
+        if (sm.excl[wid][o + d] <= g) o += d;
+      int k = g - sm.excl[wid][o], s = 0, n;
+      unsigned q = sm.pk[wid][o];
+      while (k >= (n = static_cast<int>(q >> 16)) && s < ns - 1) {
+        k -= n;
+        q = sm.pk[wid][++s * 32 + o];
+      }
+      const int u = static_cast<int>(q & 0xffffu) + k;
+      int cv;
+      const int cw = div_small(it0 + s * 32 + o, dv, inv_dv, &cv);
+      e.c[0] = L.u == 0 ? u : (L.u == 1 ? cw : cv);
+      e.c[1] = L.u == 1 ? u : (L.u == 2 ? cw : cv);
+      e.c[2] = L.u == 2 ? u : (L.u == 0 ? cw : cv);
+      const double x[3] = {(r.lo[0] + e.c[0]) * P.dx, (r.lo[1] + e.c[1]) * P.dx, (r.lo[2] + e.c[2]) * P.dx};
+      double gA[3], gB[3];
+      const double pa = sdf64(ta, S.param + 3 * i, pla, nfa, XA, RA, x, P.inflate, gA);
+      const double pb = sdf64(tb, S.param + 3 * j, plb, nfb, XB, RB, x, P.inflate, gB);
+      const double tA = fmin(fmax(fma(-pa, inv_wdx, 0.5), 0.0), 1.0);
+      const double tB = fmin(fmax(fma(-pb, inv_wdx, 0.5), 0.0), 1.0);
+      double hA, hB;
+      if (SMOOTH) {
+        hA = tA * tA * (3.0 - 2.0 * tA);
+        hB = tB * tB * (3.0 - 2.0 * tB);
+      } else {
+        hA = pa <= 0.0 ? 1.0 : 0.0;
+        hB = pb <= 0.0 ? 1.0 : 0.0;
+      }
+      e.w = hA * hB;
+      const double ma = tA * (1.0 - tA) * hB, mb = hA * tB * (1.0 - tB);
 #pragma unroll
-        for (int a = 0; a < 3; ++a) {
-          acc[1 + a] = fma(w, fl::int_to_double(c[a]), acc[1 + a]);
-          acc[4 + a] += ma * gA[a] - mb * gB[a];
-        }
-        if (w > 0.0) {
-          const long long f = order_key(-(pa + pb));
-          const int ci = c[0] + r.dim[0] * (c[1] + r.dim[1] * c[2]);
-          if (f > bk || (f == bk && ci < bi)) {
-            bk = f;
-            bi = ci;
-          }
+      for (int a = 0; a < 3; ++a) e.g[a] = ma * gA[a] - mb * gB[a];
+      e.key = e.w > 0.0 ? order_key(-(pa + pb)) : LLONG_MIN;
+      e.idx = e.c[0] + r.dim[0] * (e.c[1] + r.dim[1] * e.c[2]);
+    };
+    // the warp's components of the sums, k mod G = gw (7: the deepest node)
+    auto mine = [&](int k) { return !SHARE || (k & (G - 1)) == gw; };
+    auto add = [&](const Node64& e) {
+      if (mine(0)) acc[0] += e.w;
+#pragma unroll
+      for (int a = 0; a < 3; ++a) {
+        if (mine(1 + a)) acc[1 + a] = fma(e.w, fl::int_to_double(e.c[a]), acc[1 + a]);
+        if (mine(4 + a)) acc[4 + a] += e.g[a];
+      }
+      if (mine(7) && e.w > 0.0 && (e.key > bk || (e.key == bk && e.idx < bi))) {
+        bk = e.key;
+        bi = e.idx;
+      }
+    };
+    if constexpr (!SHARE) {
+      for (int base = 0; base < total; base += 32) {
+        if (base + lane < total) {
+          Node64 e;
+          node(base + lane, e);
+          add(e);
         }
       }
+    } else {
+      Node64(*nodes)[32] = sm.node + group * G;
+      for (int base0 = 0; base0 < total; base0 += 32 * G) {   // (total: the same in every warp of the group)
+        const int g = base0 + 32 * gw + lane;
+        if (g < total) node(g, nodes[gw][lane]);
+        group_sync();
+        for (int q = 0; q < G && base0 + 32 * q + lane < total; ++q) add(nodes[q][lane]);
+        __syncwarp();
+        group_sync();
+      }
+      // the components to the group's first warp
+      double* red = reinterpret_cast<double*>(nodes);
+      int* red_idx = reinterpret_cast<int*>(red + 8 * 32);
+      static_assert(2 * 32 * sizeof(Node64) >= 8 * 32 * sizeof(double) + 32 * sizeof(int), "in the nodes' place");
+#pragma unroll
+      for (int k = 0; k < 8; ++k)
+        if (mine(k)) red[32 * k + lane] = k < 7 ? acc[k] : __longlong_as_double(bk);
+      if (mine(7)) red_idx[lane] = bi;
+      group_sync();
+      if (gw != 0) return;   // (one tile a group)
+#pragma unroll
+      for (int k = 0; k < 7; ++k) acc[k] = red[32 * k + lane];
+      bk = __double_as_longlong(red[32 * 7 + lane]);
+      bi = red_idx[lane];
     }
     double v = 0.0;
     if (total > 0) {   // warp-uniform
@@ -1335,6 +1383,26 @@ __global__ void __launch_bounds__(kWarps * 32, 2) k_narrow64(Params P, Shapes S,
     }
     tile_done64(W, r, v, bk, bi);
   }
+}
+
+// Fewer tiles than warps: several warps of a block share a tile.  Each of them
+// clips the lines; the sums' components are added by different warps, each in
+// pass order, so they are the same bit for bit however many share.  One warp a
+// tile left most sub-partitions' FP64 pipes idle: 4000 spheres, twelve pairs of
+// them deep in one another, step 81 -> 46 us (one block per pair box over every
+// node: 53); 100 spheres and cuboids of 26 cells between walls 495 -> 295 us,
+// 400 spheres and cuboids in four layers 218 -> 106 us.
+template <bool SMOOTH>
+__global__ void __launch_bounds__(kWarps * 32, 2) k_narrow64(Params P, Shapes S, Parts D, Lists W) {
+  __shared__ Shared64 sm;
+  pdl_begin();
+  const int ntiles = W.counters[1];
+  if (ntiles > P.max_tiles) return;   // capacity exceeded: the step reports ECAPACITY
+  const long long nwarps = static_cast<long long>(gridDim.x) * kWarps;
+  int G = 1;
+  while (G < kWarps && 2 * G * static_cast<long long>(ntiles) <= nwarps) G *= 2;
+  if (G == 1) sweep64<SMOOTH, false>(P, S, D, W, sm, ntiles, 1);
+  else sweep64<SMOOTH, true>(P, S, D, W, sm, ntiles, G);
 }
 
 }  // namespace

@@ -358,3 +358,31 @@ def test_deep_tiles_on_single_warps(kinds, indicator):
     s = m.stats()
     m.close()
     assert s["tiles"] > 8 * s["narrow_grid"] and s["overlapping"] > 3 * n
+
+
+# one tile a pair: around the counts up to which eight, four and two warps share one (on 304 blocks of eight)
+@pytest.mark.parametrize("pairs", [1, 303, 304, 305, 608, 609, 1216, 1217, 2500])
+@pytest.mark.parametrize("indicator", [0, 1])
+def test_fp64_form_shared_tiles(pairs, indicator):
+    """Pairs pressed together over a face, each alone, tiles of some twenty node
+    passes: the first ones' outputs are the same bit for bit whatever number of
+    warps shares a tile, and every pair agrees with the oracle."""
+    from paper_2401_10878_gb300.contact import Contact
+    rng = np.random.default_rng(2)
+    g = np.stack(np.meshgrid(np.arange(14), np.arange(14), np.arange(14), indexing="ij"), -1).reshape(-1, 3)[:2500]
+    at = g * [37.0, 27.0, 27.0] + 14.0 + rng.uniform(-1.0, 1.0, (2500, 3))
+    q = [quat_axis_angle(a, 0.03) for a in rng.normal(size=(5000, 3))]
+    h = np.array([6.5, 7.0, 7.0])
+    sub = np.arange(2500)[:pairs]
+    pos = np.stack([at[sub], at[sub] + [2 * h[0] - 2.6, 0.3, -0.2]], 1).reshape(-1, 3)
+    st = state([W.CUBOID] * (2 * pairs), [h] * (2 * pairs), pos, quat=q[:2 * pairs], n=(14 * 37, 14 * 27, 14 * 27),
+               indicator=indicator)
+    rep, ref = _parity(st, 1)
+    assert ref.n_pairs == pairs and ref.pair_out[:, 0].min() > 300.0
+    outs = []
+    for s in (st, st.subset(np.arange(2))):
+        m = Contact.from_state(s, precision=1)
+        outs.append(gpu_step(m, s)["pair_out"][0])
+        assert m.stats()["tiles"] == s.n // 2
+        m.close()
+    assert np.array_equal(outs[0], outs[1])
