@@ -200,7 +200,7 @@ struct CubeEval {
     gb1 += s1 ? copysignf(m, y1) : 0.f;
     gb2 += (!s0 && !s1) ? copysignf(m, y2) : 0.f;
   }
-  // what grad(m) adds for the current node, and the same additions later (shared tiles)
+  // what grad(m) adds for the current node (shared tiles): a factor and three components
   __device__ __forceinline__ float4 record(float m) const {
     const float a0 = fabsf(y0), a1 = fabsf(y1), a2 = fabsf(y2);
     const bool s0 = a0 >= a1 && a0 >= a2;
@@ -208,10 +208,10 @@ struct CubeEval {
     return make_float4(1.f, s0 ? copysignf(m, y0) : 0.f, s1 ? copysignf(m, y1) : 0.f,
                        (!s0 && !s1) ? copysignf(m, y2) : 0.f);
   }
-  __device__ __forceinline__ void replay(const float4& e) {
-    gb0 += e.y;
-    gb1 += e.z;
-    gb2 += e.w;
+  __device__ __forceinline__ void set_sums(float a, float b, float c) {
+    gb0 = a;
+    gb1 = b;
+    gb2 = c;
   }
   __device__ float world(int c, const Local&, const PairRec& r, bool second) const {
     const float* rt = second ? r.rtb : r.rta;
@@ -425,17 +425,23 @@ struct AnyEval {
   }
   template <int K>
   __device__ __forceinline__ void add(float m, const float4& d) {
-    if (K == KIND_WALL) g0 += m;   // (all of its band sum)
-    else replay(record(m, d));
-  }
-  // what add(m, d) adds, and the same additions later (shared tiles)
-  static __device__ __forceinline__ float4 record(float m, const float4& d) {
-    return make_float4(m * d.w, d.x, d.y, d.z);
-  }
-  __device__ __forceinline__ void replay(const float4& e) {
+    if (K == KIND_WALL) {
+      g0 += m;   // (all of its band sum)
+      return;
+    }
+    const float4 e = record(m, d);
     g0 = fmaf(e.x, e.y, g0);
     g1 = fmaf(e.x, e.z, g1);
     g2 = fmaf(e.x, e.w, g2);
+  }
+  // what add(m, d) adds: a factor and three components
+  static __device__ __forceinline__ float4 record(float m, const float4& d) {
+    return make_float4(m * d.w, d.x, d.y, d.z);
+  }
+  __device__ __forceinline__ void set_sums(float a, float b, float c) {
+    g0 = a;
+    g1 = b;
+    g2 = c;
   }
   // component c of the band sum in the world frame
   __device__ float world(int c, const Local& L, const PairRec& r, bool second) const {
@@ -453,20 +459,21 @@ struct Partial {
   float cnt, mx, my, mz, gx, gy, gz, bestf;
   int bestidx;
   bool touched;   // warp-uniform: some lane evaluated a node (else every sum is zero)
-  bool deferred;  // warp-uniform: more clipped nodes than the limit, nothing evaluated
-  int nown, total;   // deferred: lanes with nodes, clipped nodes
+  bool deferred;  // warp-uniform: left for the whole block, nothing evaluated
 };
 
 // A tile shared by the block's warps (COOP), clipped by one of them (its record,
 // staged constants and node table in shared memory; nown lanes with nodes,
 // total nodes): warp w evaluates node passes w, w + 8, ... and leaves what each
-// node adds in shared memory; warp 0 makes the additions pass by pass, in the
-// order of a tile swept by one warp, so the sums are the same bit for bit.
-struct CoopNode {
-  float4 ga, gb;        // both evaluators' band terms (record)
-  float4 mom;           // weight and node (u, v, w)
-  float f;              // depth and node index
-  int idx;
+// node adds in shared memory (term c of node l of the round at add[c][l]: both
+// evaluators' band terms as a factor and three components, the weight and node
+// (u, v, w), depth and node index).  Six warps make the additions, two sums or
+// the deepest node each, pass by pass in the order of a tile swept by one warp,
+// so the sums are the same bit for bit.
+enum CoopTerm : int { TERM_A = 0, TERM_B = 4, TERM_W = 8, TERM_F = 12, TERM_IDX = 13, kCoopTerms = 14 };
+struct Coop {
+  float add[kCoopTerms][kWarps * 32];
+  float sum[12][32];   // cnt, mu, mv, mw; A's three; B's three; depth, node index
 };
 template <int K>
 using KindC = std::integral_constant<int, K>;
@@ -499,7 +506,24 @@ __device__ __forceinline__ void with_kinds(int a, int b, const F& f) {
 // 262, 322, 260 us; 2000 spheres and cuboids 137, 168, 134; 4000 mixed particles
 // 272, 262, 235; 4000 cuboids and one polytope 374, 378, 305.
 constexpr int kDeepNodes = 64;
-constexpr int kShareNodes = 128;   // a tile of more clipped nodes is shared when every warp has at most one tile
+constexpr int kShareNodes = 128;   // a tile of more clipped nodes is deep (when every warp has at most one tile)
+struct DeepTiles {
+  int n;       // of the block
+  int3 tile;   // one: the warp that clipped it, lanes with nodes, clipped nodes
+};
+// Every warp of the block arrives here once, with its tile or without one.
+__device__ __forceinline__ void tiles_counted() {
+  asm volatile("bar.sync 1, %0;" ::"r"(blockDim.x) : "memory");
+}
+// Counts the warp's tile among the block's deep ones; true when it is the only one.
+__device__ __forceinline__ bool leave_to_block(DeepTiles* deep, int total, int nown) {
+  const bool mine = total > kShareNodes;
+  if (mine && (threadIdx.x & 31) == 0 && atomicAdd_block(&deep->n, 1) == 0)
+    deep->tile = make_int3(threadIdx.x >> 5, nown, total);
+  __syncwarp();
+  tiles_counted();
+  return mine && *reinterpret_cast<volatile int*>(&deep->n) == 1;
+}
 
 // Order-preserving map of FP32 values to signed ints (for integer max).
 __device__ __forceinline__ int float_key(float f) {
@@ -524,7 +548,7 @@ __device__ __forceinline__ float key_float(int k) { return __int_as_float(k >= 0
 template <bool SMOOTH, bool COOP, class E>
 __device__ __forceinline__ Partial sweep_tile(const Params& P, const Shapes& S, const Parts& D, const PairRec& r,
                                               bool swap, int tl, float4* smA, float4* smB, unsigned* spk,
-                                              int4* own, int limit, CoopNode* coop, int nown, int total_in) {
+                                              int4* own, DeepTiles* deep, Coop* coop, int nown, int total_in) {
   const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5, nwarp = blockDim.x >> 5;
   const Local L = make_local(r);
   constexpr bool ROLL = !std::is_same<E, CubeEval>::value;
@@ -554,6 +578,7 @@ __device__ __forceinline__ Partial sweep_tile(const Params& P, const Shapes& S, 
   const float4* csA = smA;
   const float4* csB = smB;
   float cnt = 0.f, mu = 0.f, mv = 0.f, mw = 0.f, bestf = -FLT_MAX;
+  [[maybe_unused]] float part0 = 0.f, part1 = 0.f;   // (COOP) the warp's two sums
   int bestidx = 0x7fffffff;
   const int it0 = tl * 32 * kTileItemsPerLane;
   const int ns = min(kTileItemsPerLane, (r.nitems - it0 + 31) >> 5);   // slots of this tile (warp-uniform)
@@ -631,11 +656,9 @@ __device__ __forceinline__ Partial sweep_tile(const Params& P, const Shapes& S, 
       }
       __syncwarp();
     }
-    if (total > limit) {
+    if (deep != nullptr && leave_to_block(deep, total, __popc(__ballot_sync(kFull, has)))) {
       Partial o{};
       o.deferred = true;
-      o.nown = __popc(__ballot_sync(kFull, has));
-      o.total = total;
       return o;
     }
   }
@@ -697,35 +720,47 @@ __device__ __forceinline__ Partial sweep_tile(const Params& P, const Shapes& S, 
       int idx = u * L.su + ocv * L.sv + ocw * L.sw;
       if constexpr (COOP) {
         if (base < total) {   // warp-uniform
-          CoopNode& c = coop[32 * wid + lane];
+          const int at = 32 * wid + lane;
+          float4 ga, gb;
           if constexpr (ROLL) {
-            c.ga = E::record(ma, da);
-            c.gb = E::record(mb, db);
+            ga = E::record(ma, da);
+            gb = E::record(mb, db);
           } else {
-            c.ga = A.record(ma);
-            c.gb = B.record(mb);
+            ga = A.record(ma);
+            gb = B.record(mb);
           }
-          c.mom = make_float4(w, static_cast<float>(u), static_cast<float>(ocv), static_cast<float>(ocw));
-          c.f = f;
-          c.idx = idx;
+          const float term[kCoopTerms] = {ga.x, ga.y, ga.z, ga.w, gb.x, gb.y, gb.z, gb.w,
+                                          w, static_cast<float>(u), static_cast<float>(ocv), static_cast<float>(ocw),
+                                          f, __int_as_float(idx)};
+#pragma unroll
+          for (int c = 0; c < kCoopTerms; ++c) coop->add[c][at] = term[c];
         }
         __syncthreads();
-        if (wid == 0) {
-          for (int q = 0; q < nwarp && base0 + 32 * q < total; ++q) {
-            const CoopNode& c = coop[32 * q + lane];
-            const float4 m = c.mom;
-            cnt += m.x;
-            mu = fmaf(m.x, m.y, mu);
-            mv = fmaf(m.x, m.z, mv);
-            mw = fmaf(m.x, m.w, mw);
-            f = c.f;
-            idx = c.idx;
-            if (m.x > 0.f && (f > bestf || (f == bestf && idx < bestidx))) {
+        const int nq = min(nwarp, (total - base0 + 31) / 32);
+        if (wid == 2) {
+          for (int q = 0; q < nq; ++q) {
+            const int at = 32 * q + lane;
+            f = coop->add[TERM_F][at];
+            idx = __float_as_int(coop->add[TERM_IDX][at]);
+            if (coop->add[TERM_W][at] > 0.f && (f > bestf || (f == bestf && idx < bestidx))) {
               bestf = f;
               bestidx = idx;
             }
-            A.replay(c.ga);
-            B.replay(c.gb);
+          }
+        } else if (wid < 6) {
+          // the warp's sums k: of (1, u, v, w) times the weight, of A's and of B's components times their factor
+          const int k0 = wid < 2 ? 2 * wid : 2 * wid - 2;
+#pragma unroll
+          for (int h = 0; h < 2; ++h) {
+            const int k = k0 + h;
+            const float* x = coop->add[k < 4 ? TERM_W : (k < 7 ? TERM_A : TERM_B)];
+            const float* y = k < 4 ? coop->add[TERM_W + k] : coop->add[k < 7 ? TERM_A + k - 3 : TERM_B + k - 6];
+            float acc = h == 0 ? part0 : part1;
+            for (int q = 0; q < nq; ++q) {
+              const int at = 32 * q + lane;
+              acc = fmaf(x[at], k == 0 ? 1.f : y[at], acc);
+            }
+            (h == 0 ? part0 : part1) = acc;
           }
         }
         __syncthreads();
@@ -753,6 +788,25 @@ __device__ __forceinline__ Partial sweep_tile(const Params& P, const Shapes& S, 
     else passes(KindC<kAnyKind>{}, KindC<kAnyKind>{});
   } else {
     passes(KindC<kAnyKind>{}, KindC<kAnyKind>{});
+  }
+  if constexpr (COOP) {   // the sums to the block's first warp
+    if (wid == 2) {
+      coop->sum[10][lane] = bestf;
+      coop->sum[11][lane] = __int_as_float(bestidx);
+    } else if (wid < 6) {
+      const int k0 = wid < 2 ? 2 * wid : 2 * wid - 2;
+      coop->sum[k0][lane] = part0;
+      coop->sum[k0 + 1][lane] = part1;
+    }
+    __syncthreads();
+    cnt = coop->sum[0][lane];
+    mu = coop->sum[1][lane];
+    mv = coop->sum[2][lane];
+    mw = coop->sum[3][lane];
+    A.set_sums(coop->sum[4][lane], coop->sum[5][lane], coop->sum[6][lane]);
+    B.set_sums(coop->sum[7][lane], coop->sum[8][lane], coop->sum[9][lane]);
+    bestf = coop->sum[10][lane];
+    bestidx = __float_as_int(coop->sum[11][lane]);
   }
   Partial o;
   o.cnt = cnt;
@@ -925,12 +979,12 @@ enum KindSet : int { SET_ALL = 0, SET_SC = 1, SET_CUBE = 2 };
 
 template <bool SMOOTH, int SET, bool COOP>
 __device__ __forceinline__ Partial dispatch(const Params& P, const Shapes& S, const Parts& D, const PairRec& r,
-                                            int tl, float4* smA, float4* smB, unsigned* spk, int4* own, int limit,
-                                            CoopNode* coop, int nown, int total) {
+                                            int tl, float4* smA, float4* smB, unsigned* spk, int4* own, DeepTiles* deep,
+                                            Coop* coop, int nown, int total) {
   // evaluate the cheaper kind as A (G's sign flips back below); two cubes keep the record's order
   const bool swap = SET == SET_CUBE ? false : sweep_swap(r.kinds & 0xff, r.kinds >> 8);
   using E = typename std::conditional<SET == SET_CUBE, CubeEval, AnyEval<SET == SET_ALL, SET == SET_SC>>::type;
-  Partial o = sweep_tile<SMOOTH, COOP, E>(P, S, D, r, swap, tl, smA, smB, spk, own, limit, coop, nown, total);
+  Partial o = sweep_tile<SMOOTH, COOP, E>(P, S, D, r, swap, tl, smA, smB, spk, own, deep, coop, nown, total);
   if (swap) {
     o.gx = -o.gx; o.gy = -o.gy; o.gz = -o.gz;
   }
@@ -964,9 +1018,8 @@ __global__ void __launch_bounds__(narrow_warps<SET>() * 32, narrow_blocks<SET>()
   __shared__ float4 s_planes[NW][2][SET == SET_ALL ? 2 * kMaxFaces : 8];
   __shared__ unsigned s_pk[SET == SET_CUBE ? 1 : NW][kTileItemsPerLane * 32];   // clipped ranges (rolled sweep)
   __shared__ int4 s_own[NW][64];   // the lanes with clipped nodes (sweep_tile)
-  __shared__ CoopNode s_coop[NW * 32];   // a shared tile's nodes
-  __shared__ int3 s_deferred[NW];   // warp that clipped it, lanes with nodes, clipped nodes
-  __shared__ int s_ndeferred;
+  __shared__ Coop s_coop;   // a shared tile's nodes
+  __shared__ DeepTiles s_deep;
   pdl_begin();
   const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
   const int ntiles = W.counters[1];
@@ -977,20 +1030,24 @@ __global__ void __launch_bounds__(narrow_warps<SET>() * 32, narrow_blocks<SET>()
   int t = blockIdx.x + gridDim.x * wid;
   const int4 first = t < P.max_tiles ? load_rec_part(W.tiles + t, lane) : make_int4(0, 0, 0, 0);
   if (ntiles > P.max_tiles) return;   // capacity exceeded: the step reports ECAPACITY
-  // with at most one tile per warp a tile of many node passes would be the
-  // kernel's tail: it is left for the whole block, whose other warps are done
-  // (400 cubes, one in seven pressed into a neighbour: 16.0 -> 11.9 us; 135 larger
-  // cubes between walls, hundreds of nodes per wall contact: 28.3 -> 15.4 us; 123
-  // mixed particles with walls: 24.7 -> 14.3 us; 2568 spheres and cuboids, one in
-  // ten pressed: 25.0 -> 14.0 us)
+  // with at most one tile per warp a block's only tile of many node passes would
+  // be its tail: it is left for all of its warps (by single warps, with one warp
+  // adding, with six: 400 cubes, one in seven pressed into a neighbour, with the
+  // contact law, step 37.0, 35.0, 32.9 us; 500 cubes of 24 cells 41.1, 37.2, 36.1; 49
+  // spheres and cuboids of 26 cells between walls, sweep 31.2, 24.0, 16.6).  Several
+  // deep tiles of a block keep its warps busy by themselves: sharing each of them
+  // took 38.6 us on 1000 smoothed cubes between walls and 29.6 on 1000 mixed
+  // particles (two of them, six warps adding: 16.2 and 13.5), one warp each 15.6
+  // and 12.5.
   const bool share = ntiles <= nwarps;
   if (share) {
-    if (threadIdx.x == 0) s_ndeferred = 0;
+    if (threadIdx.x == 0) s_deep.n = 0;
     __syncthreads();
   }
   if (t < ntiles) store_rec_part(&s_rec[wid][0], lane, first);
   __syncwarp();
   int buf = 0;
+  bool counted = false;   // the warp's tile among the block's deep ones
   while (t < ntiles) {
     const int tn = t + nwarps;
     const int4 next = tn < ntiles ? load_rec_part(W.tiles + tn, lane) : make_int4(0, 0, 0, 0);
@@ -998,9 +1055,9 @@ __global__ void __launch_bounds__(narrow_warps<SET>() * 32, narrow_blocks<SET>()
     if (record_in_bounds(P, W.err, r, true)) {
       const Partial o = dispatch<SMOOTH, SET, false>(P, S, D, r, r.tile, s_planes[wid][0], s_planes[wid][1],
                                                      s_pk[SET == SET_CUBE ? 0 : wid], s_own[wid],
-                                                     share ? kShareNodes : 0x7fffffff, nullptr, 0, 0);
+                                                     share ? &s_deep : nullptr, nullptr, 0, 0);
+      counted = true;
       if (!o.deferred) tile_done(W, r, o.touched ? reduce_tile<SMOOTH>(o) : empty_partial());
-      else if (lane == 0) s_deferred[atomicAdd_block(&s_ndeferred, 1)] = make_int3(wid, o.nown, o.total);
     }
     if (share) break;   // (one tile per warp at most: what it staged stays for the block)
     __syncwarp();
@@ -1010,13 +1067,12 @@ __global__ void __launch_bounds__(narrow_warps<SET>() * 32, narrow_blocks<SET>()
     t = tn;
   }
   if (!share) return;
-  __syncthreads();
-  const int nd = s_ndeferred;
-  for (int d = 0; d < nd; ++d) {
-    const int3 e = s_deferred[d];
+  if (!counted) tiles_counted();   // (a warp without a tile)
+  if (s_deep.n == 1) {
+    const int3 e = s_deep.tile;
     const PairRec& r = s_rec[e.x][0];
     const Partial o = dispatch<SMOOTH, SET, true>(P, S, D, r, r.tile, s_planes[e.x][0], s_planes[e.x][1], nullptr,
-                                                  s_own[e.x], 0, s_coop, e.y, e.z);
+                                                  s_own[e.x], nullptr, &s_coop, e.y, e.z);
     if (wid == 0) tile_done(W, r, reduce_tile<SMOOTH>(o));
   }
 }

@@ -334,22 +334,24 @@ def test_cell_list_memory():
     assert 235 ** 3 * 5 * 20 <= used <= entries + counts + rest
 
 
-# more tiles than warps, most of many node passes: every pair of kinds with the wall's, and polytopes among them
+# most tiles of many node passes, several in every block (400 particles) and more than there are warps (900):
+# every pair of kinds with the wall's, and polytopes among them
+@pytest.mark.parametrize("k", [20, 30])
 @pytest.mark.parametrize("kinds", [[0, 1, 3], [0, 1, 2]])
 @pytest.mark.parametrize("indicator", [0, 1])
-def test_deep_tiles_on_single_warps(kinds, indicator):
+def test_deep_tiles_on_single_warps(k, kinds, indicator):
     """A layer of spheres, cuboids and cubes (or polytopes) pressed into one
     another, a floor and a ceiling."""
     from paper_2401_10878_gb300.contact import Contact
     rng = np.random.default_rng(7)
-    k, edge = 30, 16.0
+    edge = 16.0
     n = k * k
     g = np.stack(np.meshgrid(np.arange(k), np.arange(k), indexing="ij"), -1).reshape(-1, 2)
     pos = np.concatenate([(g + 0.5) * edge, np.full((n, 1), 40.0)], 1) + rng.uniform(-0.4, 0.4, (n, 3))
     code = np.array(kinds)[rng.integers(0, 3, n)]
     half = np.where(code[:, None] == 0, [[9.6, 0, 0]], np.where(code[:, None] == 1, [[9.4, 8.1, 7.3]], [[7.9] * 3]))
     pl = W.random_polytope(rng, 14, 10.0)[0]
-    st = state(np.where(code == 3, W.CUBOID, code), half, pos, quat=W.random_quaternions(rng, n), n=(480, 480, 96),
+    st = state(np.where(code == 3, W.CUBOID, code), half, pos, quat=W.random_quaternions(rng, n), n=(16 * k, 16 * k, 96),
                planes=[pl if c == 2 else None for c in code], indicator=indicator)
     st = W.floor_and_ceiling(st, gap=5.0)
     rep, ref = _parity(st, 0)
@@ -357,7 +359,8 @@ def test_deep_tiles_on_single_warps(kinds, indicator):
     gpu_step(m, st)
     s = m.stats()
     m.close()
-    assert s["tiles"] > 8 * s["narrow_grid"] and s["overlapping"] > 3 * n
+    assert (s["tiles"] > 8 * s["narrow_grid"]) == (k == 30) and s["tiles"] > 2 * s["narrow_grid"]
+    assert s["overlapping"] > 3 * n
 
 
 # one tile a pair: around the counts up to which eight, four and two warps share one (on 304 blocks of eight)
