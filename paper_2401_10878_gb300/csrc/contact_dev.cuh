@@ -97,6 +97,7 @@ struct Params {
   int smooth;            // 1: smoothed indicator
   int precision;         // 0: FP32 tiles, 1: FP64 per pair
   int kind_set;          // node-sweep variant: 0 all kinds, 1 spheres and cuboids, 2 cubes only
+  int one_kind;          // 1: the particles that are no polytopes are all spheres, all cubes or all other cuboids
   int dx_pow2;           // 1: dx is a power of two, so x / dx == x * inv_dx exactly
   double damping_c;
   int box_mode, box_res; // 1: the paper's box pipeline with box_res (N_c) points per direction

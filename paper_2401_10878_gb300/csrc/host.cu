@@ -519,6 +519,12 @@ contact_status contact_init(const contact_config* cfg, const int32_t* shape_type
                : std::all_of(kind.begin(), kind.begin() + n,
                              [](int k) { return k == KIND_SPHERE || k == KIND_CUBOID || k == KIND_CUBE; }) ? 1 : 0;
   if (nw > 0 && P.kind_set == 2) P.kind_set = 1;
+  {
+    const bool has[3] = {std::count(kind.begin(), kind.begin() + n, KIND_SPHERE) > 0,
+                         std::count(kind.begin(), kind.begin() + n, KIND_CUBE) > 0,
+                         std::count(kind.begin(), kind.begin() + n, KIND_CUBOID) > 0};
+    P.one_kind = has[0] + has[1] + has[2] == 1 ? 1 : 0;
+  }
   P.nwall = nw;
   P.box_mode = C.box_mode;
   P.box_res = C.box_mode == 1 ? C.contact_resolution : 0;

@@ -79,7 +79,6 @@ __device__ __forceinline__ float world_comp(int c, const Local& L, float au, flo
 // |y_k| < h + T is the node-counter interval centred at
 // c_k = fu - (tv_k rv + tw_k rw) / tu_k with half-width (h + T) / |tu_k|.
 struct CubeEval {
-  static constexpr bool kCube = true;
   int iu;
   float fu, tu0, tu1, tu2, h, itu0, itu1, itu2;
   bool flat;   // a slab parallel to the lines (|tu_k| <= kClipFlat): the general clip
@@ -87,6 +86,7 @@ struct CubeEval {
   float gb0, gb1, gb2;
   // (the geometry comes with the staged constants: prep_lanes, then fetch)
   __device__ __forceinline__ void clear() { gb0 = gb1 = gb2 = 0.f; }
+  __device__ __forceinline__ int faces() const { return 0; }
   __device__ __forceinline__ void begin_line_rec(const PairRec& r, bool second, const Local& L, int cv, int cw,
                                                  int u0) {
     const int* ci = second ? r.bi : r.ai;
@@ -246,7 +246,7 @@ __device__ __forceinline__ void stage_planes(const Shapes& S, const Parts& D, in
 // warps of an SM, each on its own pair, waited on instruction fetches for most
 // of the time (16 of 23 stalled cycles per instruction: 82 us for 15472
 // smoothed mixed particles, 10.8 us for 1934 sharp ones; 39.5 and 8.9 us with
-// one copy).  The arithmetic of a line and of a node is that of the evaluators
+// one copy; where few kinds meet in deep tiles, see kDeepNodes).  The arithmetic of a line and of a node is that of the evaluators
 // above, operation for operation.
 // cs: sphere (radius); cuboid (tu, tv, tw, h) per axis, then 1 / tu; wall
 // (mu, mv, mw, p0), then 1 / mu (p0 = the wall's value at the box origin,
@@ -262,11 +262,11 @@ __device__ __forceinline__ void stage_planes(const Shapes& S, const Parts& D, in
 constexpr int kAnyKind = -1;   // as a kind known at compile time: none, the evaluator's own
 template <bool POLY, bool CUBE>
 struct AnyEval {
-  static constexpr bool kCube = CUBE;
   int kind, iu, iv, iw, nf, nup, ndn;
   float fu, fv, fw;
   const float4* cs;
   float g0, g1, g2;   // band sum: local axes (sphere, polytope), body axes (cuboid), along the normal (wall)
+  __device__ __forceinline__ int faces() const { return POLY ? nf : 0; }
   // the registers, with the constants staged in sm (a shared tile: by the warp that clipped it)
   __device__ void attach(const PairRec& r, bool second, const Shapes& S, const Local& L, float4* sm) {
     kind = second ? r.kinds >> 8 : r.kinds & 0xff;
@@ -452,6 +452,11 @@ struct AnyEval {
   }
 };
 
+// Kernel variants: every kind of particle; spheres, cubes and cuboids (no
+// polytopes: fewer registers, no spills) of several kinds or of one kind, with
+// walls; cubes alone (chosen at init).
+enum KindSet : int { SET_ALL = 0, SET_SC = 1, SET_CUBE = 2, SET_ONE = 3 };
+
 // ---------------------------------------------------------------- tile sweep
 // Per-lane partials of a tile: node count and first moments (exact integers
 // in sharp mode), the band sum of the normal, and the deepest node.
@@ -477,52 +482,66 @@ struct Coop {
 };
 template <int K>
 using KindC = std::integral_constant<int, K>;
-// f(kind of A, kind of B) as compile-time constants, for pairs without a polytope (A is the cheaper kind,
-// sweep_swap's order); CUBE: cubes are a kind of their own, else cuboids
-template <bool CUBE, class F>
-__device__ __forceinline__ void with_kinds(int a, int b, const F& f) {
-  if (a == KIND_WALL) {
-    if (b == KIND_SPHERE) f(KindC<KIND_WALL>{}, KindC<KIND_SPHERE>{});
-    else if (CUBE && b == KIND_CUBE) f(KindC<KIND_WALL>{}, KindC<KIND_CUBE>{});
-    else f(KindC<KIND_WALL>{}, KindC<KIND_CUBOID>{});
-  } else if (a == KIND_SPHERE) {
-    if (b == KIND_SPHERE) f(KindC<KIND_SPHERE>{}, KindC<KIND_SPHERE>{});
-    else if (CUBE && b == KIND_CUBE) f(KindC<KIND_SPHERE>{}, KindC<KIND_CUBE>{});
-    else f(KindC<KIND_SPHERE>{}, KindC<KIND_CUBOID>{});
-  } else if (CUBE && a == KIND_CUBE) {
-    if (b == KIND_CUBE) f(KindC<KIND_CUBE>{}, KindC<KIND_CUBE>{});
-    else f(KindC<KIND_CUBE>{}, KindC<KIND_CUBOID>{});
-  } else {
-    f(KindC<KIND_CUBOID>{}, KindC<KIND_CUBOID>{});
-  }
+// f(kind of A, kind of B) as compile-time constants, for a wall (A) and a particle that is no polytope, or two
+// particles of one such kind
+template <class F>
+__device__ __forceinline__ void with_wall(int b, const F& f) {
+  if (b == KIND_SPHERE) f(KindC<KIND_WALL>{}, KindC<KIND_SPHERE>{});
+  else if (b == KIND_CUBE) f(KindC<KIND_WALL>{}, KindC<KIND_CUBE>{});
+  else f(KindC<KIND_WALL>{}, KindC<KIND_CUBOID>{});
 }
-// The node passes of a tile of more clipped nodes than this, of two particles
-// that are no polytopes, run through a loop compiled for their kinds: it keeps
-// their constants in registers, a quarter of the run-time evaluator's
-// instructions fewer.  In shallow tiles the loops' code would be fetched for one
-// or two passes (32, 64 and 128 nodes differ by less than the runs).  Node sweep
-// with a sweep compiled per kind pair, with the run-time evaluator alone and
-// with these loops: 4000 cuboids of 26 cells pressed on a floor and a ceiling
-// 262, 322, 260 us; 2000 spheres and cuboids 137, 168, 134; 4000 mixed particles
-// 272, 262, 235; 4000 cuboids and one polytope 374, 378, 305.
+template <class F>
+__device__ __forceinline__ void with_kind(int b, const F& f) {
+  if (b == KIND_SPHERE) f(KindC<KIND_SPHERE>{}, KindC<KIND_SPHERE>{});
+  else if (b == KIND_CUBE) f(KindC<KIND_CUBE>{}, KindC<KIND_CUBE>{});
+  else f(KindC<KIND_CUBOID>{}, KindC<KIND_CUBOID>{});
+}
+// Passes compiled for the pair's kinds keep the constants in registers: a quarter
+// of the run-time evaluator's instructions fewer.  Every such loop that is in use
+// at a time costs instruction fetches, so they serve particles of one kind (that
+// kind with itself and with walls) and, with several kinds, wall contacts of more
+// clipped nodes than this.  Step with a sweep compiled per kind pair, with the
+// run-time evaluator alone, and so: 4000 cuboids of 26 cells pressed on a floor
+// and a ceiling 338, 370, 301 us; 936 cuboids in a dense lattice 121, 133, 121;
+// 2000 spheres and cuboids on walls 196, 206, 172; 7819 spheres and cuboids
+// pressed into one another and on walls 550, 349, 311 (335 with a loop for every
+// pair of kinds).  With polytopes the loops cost the other tiles more than they
+// gave (6956 mixed particles, smoothed: 481 us without, 491 with them).
 constexpr int kDeepNodes = 64;
-constexpr int kShareNodes = 128;   // a tile of more clipped nodes is deep (when every warp has at most one tile)
+
+// A block's deep tiles, those of more than kShareNodes clipped nodes when every
+// warp has at most one tile, are shared by its warps one after the other when
+// that is expected to end before the longest of them on its own warp (cycles:
+// kPassCycles and kFaceCycles for each polytope face a node pass; eight passes at
+// a time a quarter more and kRoundCycles for the barriers and the additions;
+// kTileCycles to finish a tile).  One tile alone is worth it from about 300 nodes,
+// two equal ones hardly, polytopes' several.  Step by single warps, all shared,
+// and so: 49 spheres and cuboids of 26 cells on walls 61.6, 53.4, 48.0 us; 1000
+// smoothed cubes on walls 47.3, 70.9, 47.1; 240 polytopes deep in one another 147,
+// 99, 86.
+constexpr int kShareNodes = 128;
+constexpr int kPassCycles = 300, kFaceCycles = 20, kRoundCycles = 150, kTileCycles = 2000;
 struct DeepTiles {
-  int n;       // of the block
-  int3 tile;   // one: the warp that clipped it, lanes with nodes, clipped nodes
+  int n, alone, shared;   // tiles, cycles of the longest alone and of all of them shared
+  int3 tile[kWarps];      // the warp that clipped it, lanes with nodes, clipped nodes
 };
 // Every warp of the block arrives here once, with its tile or without one.
 __device__ __forceinline__ void tiles_counted() {
   asm volatile("bar.sync 1, %0;" ::"r"(blockDim.x) : "memory");
 }
-// Counts the warp's tile among the block's deep ones; true when it is the only one.
-__device__ __forceinline__ bool leave_to_block(DeepTiles* deep, int total, int nown) {
+// Enters the warp's tile when it is deep; true when it is left to the block.
+__device__ __forceinline__ bool leave_to_block(DeepTiles* deep, int total, int nown, int faces) {
   const bool mine = total > kShareNodes;
-  if (mine && (threadIdx.x & 31) == 0 && atomicAdd_block(&deep->n, 1) == 0)
-    deep->tile = make_int3(threadIdx.x >> 5, nown, total);
+  if (mine && (threadIdx.x & 31) == 0) {
+    const int np = (total + 31) / 32, pass = kPassCycles + kFaceCycles * faces;
+    deep->tile[atomicAdd_block(&deep->n, 1)] = make_int3(threadIdx.x >> 5, nown, total);
+    atomicMax_block(&deep->alone, np * pass);
+    atomicAdd_block(&deep->shared, (np + kWarps - 1) / kWarps * (pass * 5 / 4 + kRoundCycles) + kTileCycles);
+  }
   __syncwarp();
   tiles_counted();
-  return mine && *reinterpret_cast<volatile int*>(&deep->n) == 1;
+  const volatile DeepTiles* d = deep;
+  return mine && d->shared < d->alone;
 }
 
 // Order-preserving map of FP32 values to signed ints (for integer max).
@@ -545,7 +564,7 @@ __device__ __forceinline__ float key_float(int k) { return __int_as_float(k >= 0
 // with the slots' clipped ranges in shared memory, to keep the kernel's code
 // small (unrolled: 38.8 -> 61.8 us on 15472 mixed particles); for two cubes they
 // are unrolled over registers.
-template <bool SMOOTH, bool COOP, class E>
+template <bool SMOOTH, int SET, bool COOP, class E>
 __device__ __forceinline__ Partial sweep_tile(const Params& P, const Shapes& S, const Parts& D, const PairRec& r,
                                               bool swap, int tl, float4* smA, float4* smB, unsigned* spk,
                                               int4* own, DeepTiles* deep, Coop* coop, int nown, int total_in) {
@@ -656,7 +675,8 @@ __device__ __forceinline__ Partial sweep_tile(const Params& P, const Shapes& S, 
       }
       __syncwarp();
     }
-    if (deep != nullptr && leave_to_block(deep, total, __popc(__ballot_sync(kFull, has)))) {
+    if (deep != nullptr && leave_to_block(deep, total, __popc(__ballot_sync(kFull, has)),
+                                        A.faces() + B.faces())) {
       Partial o{};
       o.deferred = true;
       return o;
@@ -783,8 +803,11 @@ __device__ __forceinline__ Partial sweep_tile(const Params& P, const Shapes& S, 
       }
     }
   };
-  if constexpr (ROLL && !COOP) {
-    if (total > kDeepNodes && A.kind != KIND_POLY && B.kind != KIND_POLY) with_kinds<E::kCube>(A.kind, B.kind, passes);
+  if constexpr (SET == SET_ONE && !COOP) {
+    if (A.kind == KIND_WALL) with_wall(B.kind, passes);
+    else with_kind(B.kind, passes);
+  } else if constexpr (SET == SET_SC && !COOP) {
+    if (A.kind == KIND_WALL && total > kDeepNodes) with_wall(B.kind, passes);
     else passes(KindC<kAnyKind>{}, KindC<kAnyKind>{});
   } else {
     passes(KindC<kAnyKind>{}, KindC<kAnyKind>{});
@@ -973,9 +996,6 @@ __device__ __forceinline__ void tile_done(const Lists& W, const PairRec& r, floa
   pair_done(W, r, acc, __shfl_sync(kFull, bi, 7));
 }
 
-// Kernel variants: the full set of pair kinds, or spheres and cuboids only
-// (chosen at init when no polytope is present; fewer registers, no spills).
-enum KindSet : int { SET_ALL = 0, SET_SC = 1, SET_CUBE = 2 };
 
 template <bool SMOOTH, int SET, bool COOP>
 __device__ __forceinline__ Partial dispatch(const Params& P, const Shapes& S, const Parts& D, const PairRec& r,
@@ -983,8 +1003,8 @@ __device__ __forceinline__ Partial dispatch(const Params& P, const Shapes& S, co
                                             Coop* coop, int nown, int total) {
   // evaluate the cheaper kind as A (G's sign flips back below); two cubes keep the record's order
   const bool swap = SET == SET_CUBE ? false : sweep_swap(r.kinds & 0xff, r.kinds >> 8);
-  using E = typename std::conditional<SET == SET_CUBE, CubeEval, AnyEval<SET == SET_ALL, SET == SET_SC>>::type;
-  Partial o = sweep_tile<SMOOTH, COOP, E>(P, S, D, r, swap, tl, smA, smB, spk, own, deep, coop, nown, total);
+  using E = typename std::conditional<SET == SET_CUBE, CubeEval, AnyEval<SET == SET_ALL, SET != SET_ALL>>::type;
+  Partial o = sweep_tile<SMOOTH, SET, COOP, E>(P, S, D, r, swap, tl, smA, smB, spk, own, deep, coop, nown, total);
   if (swap) {
     o.gx = -o.gx; o.gy = -o.gy; o.gz = -o.gz;
   }
@@ -1002,17 +1022,12 @@ __device__ __forceinline__ void store_rec_part(PairRec* dst, int lane, int4 v) {
 // Blocks per SM: 3 for the sphere/cuboid/cube variants (<= 85 registers, so
 // 24 warps per SM: about one tile per warp at a settling box's size), 2 for
 // the variant with every kind (measured faster than 3, which spills more).
-// Warps per block and blocks per SM of the node sweep (compiled per kind set).
-constexpr int kNarrowWarps = 8, kNarrowBlocks = 3;
 template <int SET>
-__host__ __device__ constexpr int narrow_warps() { return SET == SET_ALL ? 8 : kNarrowWarps; }
-template <int SET>
-__host__ __device__ constexpr int narrow_blocks() { return SET == SET_ALL ? 2 : kNarrowBlocks; }
+constexpr int kNarrowBlocks = SET == SET_ALL ? 2 : 3;
 
 template <bool SMOOTH, int SET>
-__global__ void __launch_bounds__(narrow_warps<SET>() * 32, narrow_blocks<SET>()) k_narrow32(Params P, Shapes S,
-                                                                                             Parts D, Lists W) {
-  constexpr int NW = narrow_warps<SET>();
+__global__ void __launch_bounds__(kWarps * 32, kNarrowBlocks<SET>) k_narrow32(Params P, Shapes S, Parts D, Lists W) {
+  constexpr int NW = kWarps;
   __shared__ __align__(16) PairRec s_rec[NW][2];
   // per evaluator: a polytope's planes, then its line clip's constants (a cube: the clip constants)
   __shared__ float4 s_planes[NW][2][SET == SET_ALL ? 2 * kMaxFaces : 8];
@@ -1030,18 +1045,11 @@ __global__ void __launch_bounds__(narrow_warps<SET>() * 32, narrow_blocks<SET>()
   int t = blockIdx.x + gridDim.x * wid;
   const int4 first = t < P.max_tiles ? load_rec_part(W.tiles + t, lane) : make_int4(0, 0, 0, 0);
   if (ntiles > P.max_tiles) return;   // capacity exceeded: the step reports ECAPACITY
-  // with at most one tile per warp a block's only tile of many node passes would
-  // be its tail: it is left for all of its warps (by single warps, with one warp
-  // adding, with six: 400 cubes, one in seven pressed into a neighbour, with the
-  // contact law, step 37.0, 35.0, 32.9 us; 500 cubes of 24 cells 41.1, 37.2, 36.1; 49
-  // spheres and cuboids of 26 cells between walls, sweep 31.2, 24.0, 16.6).  Several
-  // deep tiles of a block keep its warps busy by themselves: sharing each of them
-  // took 38.6 us on 1000 smoothed cubes between walls and 29.6 on 1000 mixed
-  // particles (two of them, six warps adding: 16.2 and 13.5), one warp each 15.6
-  // and 12.5.
+  // with at most one tile per warp a tile of many node passes would be the
+  // kernel's tail: the block's other warps help (leave_to_block)
   const bool share = ntiles <= nwarps;
   if (share) {
-    if (threadIdx.x == 0) s_deep.n = 0;
+    if (threadIdx.x == 0) s_deep.n = s_deep.alone = s_deep.shared = 0;
     __syncthreads();
   }
   if (t < ntiles) store_rec_part(&s_rec[wid][0], lane, first);
@@ -1068,8 +1076,9 @@ __global__ void __launch_bounds__(narrow_warps<SET>() * 32, narrow_blocks<SET>()
   }
   if (!share) return;
   if (!counted) tiles_counted();   // (a warp without a tile)
-  if (s_deep.n == 1) {
-    const int3 e = s_deep.tile;
+  const int nd = s_deep.shared < s_deep.alone ? s_deep.n : 0;
+  for (int d = 0; d < nd; ++d) {
+    const int3 e = s_deep.tile[d];
     const PairRec& r = s_rec[e.x][0];
     const Partial o = dispatch<SMOOTH, SET, true>(P, S, D, r, r.tile, s_planes[e.x][0], s_planes[e.x][1], nullptr,
                                                   s_own[e.x], nullptr, &s_coop, e.y, e.z);
@@ -1463,11 +1472,19 @@ __global__ void __launch_bounds__(kWarps * 32, 2) k_narrow64(Params P, Shapes S,
 
 }  // namespace
 
-template <bool SMOOTH, int SET>
-int blocks_per_sm() {
-  int per_sm = 0;
-  cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_narrow32<SMOOTH, SET>, narrow_warps<SET>() * 32, 0);
-  return per_sm > 0 ? per_sm : 1;
+int kind_variant(const Params& P) {
+  return P.kind_set == SET_SC && P.one_kind ? static_cast<int>(SET_ONE) : P.kind_set;
+}
+
+// f(the context's node-sweep kernel)
+template <class F>
+auto with_narrow32(const Params& P, const F& f) {
+  switch (kind_variant(P)) {
+    case SET_CUBE: return P.smooth ? f(k_narrow32<true, SET_CUBE>) : f(k_narrow32<false, SET_CUBE>);
+    case SET_ONE: return P.smooth ? f(k_narrow32<true, SET_ONE>) : f(k_narrow32<false, SET_ONE>);
+    case SET_SC: return P.smooth ? f(k_narrow32<true, SET_SC>) : f(k_narrow32<false, SET_SC>);
+    default: return P.smooth ? f(k_narrow32<true, SET_ALL>) : f(k_narrow32<false, SET_ALL>);
+  }
 }
 
 int narrow_grid(const Params& P) {
@@ -1475,14 +1492,11 @@ int narrow_grid(const Params& P) {
   cudaGetDevice(&dev);
   cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
   if (P.precision == 1) return sms * 2;   // k_narrow64: two resident blocks per SM
-  int per_sm = 1;
-  if (P.smooth) {
-    per_sm = P.kind_set == SET_CUBE ? blocks_per_sm<true, SET_CUBE>()
-             : P.kind_set == SET_SC ? blocks_per_sm<true, SET_SC>() : blocks_per_sm<true, SET_ALL>();
-  } else {
-    per_sm = P.kind_set == SET_CUBE ? blocks_per_sm<false, SET_CUBE>()
-             : P.kind_set == SET_SC ? blocks_per_sm<false, SET_SC>() : blocks_per_sm<false, SET_ALL>();
-  }
+  const int per_sm = with_narrow32(P, [](auto kern) {
+    int n = 0;
+    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, kern, kWarps * 32, 0);
+    return n > 0 ? n : 1;
+  });
   return sms * per_sm;
 }
 
@@ -1515,16 +1529,7 @@ void launch_narrow(const Params& P, const Shapes& S, const Parts& D, const Lists
       launch_pdl(k_narrow64<false>, dim3(grid), dim3(kWarps * 32), 0, st, P, S, D, W);
     return;
   }
-  const dim3 bc(narrow_warps<SET_CUBE>() * 32), bs(narrow_warps<SET_SC>() * 32), ba(narrow_warps<SET_ALL>() * 32);
-  if (P.smooth) {
-    if (P.kind_set == SET_CUBE) launch_pdl(k_narrow32<true, SET_CUBE>, dim3(grid), bc, 0, st, P, S, D, W);
-    else if (P.kind_set == SET_SC) launch_pdl(k_narrow32<true, SET_SC>, dim3(grid), bs, 0, st, P, S, D, W);
-    else launch_pdl(k_narrow32<true, SET_ALL>, dim3(grid), ba, 0, st, P, S, D, W);
-  } else {
-    if (P.kind_set == SET_CUBE) launch_pdl(k_narrow32<false, SET_CUBE>, dim3(grid), bc, 0, st, P, S, D, W);
-    else if (P.kind_set == SET_SC) launch_pdl(k_narrow32<false, SET_SC>, dim3(grid), bs, 0, st, P, S, D, W);
-    else launch_pdl(k_narrow32<false, SET_ALL>, dim3(grid), ba, 0, st, P, S, D, W);
-  }
+  with_narrow32(P, [&](auto kern) { return launch_pdl(kern, dim3(grid), dim3(kWarps * 32), 0, st, P, S, D, W); });
 }
 
 }  // namespace gbc

@@ -162,11 +162,13 @@ extern "C" contact_status contact_step_noalloc(const contact_config* cfg, const 
   const double band = (C.indicator == 1) ? (0.5 * C.smooth_width) * C.dx : 0.0;
   const double delta = C.inflate + band;
   double rmax = 0.0, rin_min = 1e300;
+  bool has[3] = {false, false, false};   // spheres, cubes, other cuboids
   for (int p = 0; p < n; ++p) {
     const double* prm = shape_param + 3 * p;
     if (!(young[p] > 0.0) || !(poisson[p] >= 0.0) || !(poisson[p] < 1.0)) return CONTACT_EINVAL;
     if (shape_type[p] == CONTACT_SHAPE_SPHERE) {
       if (!(prm[0] > 0.0)) return CONTACT_EINVAL;
+      has[0] = true;
       rmax = std::max(rmax, prm[0] + delta);
       rin_min = std::min(rin_min, prm[0]);
     } else if (shape_type[p] == CONTACT_SHAPE_CUBOID) {
@@ -175,6 +177,7 @@ extern "C" contact_status contact_step_noalloc(const contact_config* cfg, const 
         if (!(prm[k] > 0.0)) return CONTACT_EINVAL;
         e2 += (prm[k] + delta) * (prm[k] + delta);
       }
+      has[prm[0] == prm[1] && prm[0] == prm[2] ? 1 : 2] = true;
       rmax = std::max(rmax, std::sqrt(e2));
       rin_min = std::min(rin_min, std::min(prm[0], std::min(prm[1], prm[2])));
     } else {
@@ -212,6 +215,7 @@ extern "C" contact_status contact_step_noalloc(const contact_config* cfg, const 
   P.smooth = C.indicator;
   P.precision = CONTACT_PRECISION_FP32_TILE;
   P.kind_set = 1;
+  P.one_kind = has[0] + has[1] + has[2] == 1 ? 1 : 0;
   P.damping_c = C.damping_c;
   P.max_pairs = C.max_pairs;
   P.max_nbr = kMaxNbr;

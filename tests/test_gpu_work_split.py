@@ -334,10 +334,10 @@ def test_cell_list_memory():
     assert 235 ** 3 * 5 * 20 <= used <= entries + counts + rest
 
 
-# most tiles of many node passes, several in every block (400 particles) and more than there are warps (900):
-# every pair of kinds with the wall's, and polytopes among them
-@pytest.mark.parametrize("k", [20, 30])
-@pytest.mark.parametrize("kinds", [[0, 1, 3], [0, 1, 2]])
+# most tiles of many node passes, several in every block (256 particles) and more than there are warps (1296):
+# every pair of kinds with the wall's, polytopes among them, and each kind alone
+@pytest.mark.parametrize("k", [16, 36])
+@pytest.mark.parametrize("kinds", [[0, 1, 3], [0, 1, 2], [0, 0, 0], [1, 1, 1], [3, 3, 3]])
 @pytest.mark.parametrize("indicator", [0, 1])
 def test_deep_tiles_on_single_warps(k, kinds, indicator):
     """A layer of spheres, cuboids and cubes (or polytopes) pressed into one
@@ -359,8 +359,8 @@ def test_deep_tiles_on_single_warps(k, kinds, indicator):
     gpu_step(m, st)
     s = m.stats()
     m.close()
-    assert (s["tiles"] > 8 * s["narrow_grid"]) == (k == 30) and s["tiles"] > 2 * s["narrow_grid"]
-    assert s["overlapping"] > 3 * n
+    assert (s["tiles"] > 8 * s["narrow_grid"]) == (k == 36) and s["tiles"] > 2 * s["narrow_grid"]
+    assert s["overlapping"] > 2 * n
 
 
 # one tile a pair: around the counts up to which eight, four and two warps share one (on 304 blocks of eight)
