@@ -514,13 +514,14 @@ constexpr int kDeepNodes = 64;
 // that is expected to end before the longest of them on its own warp (cycles:
 // kPassCycles and kFaceCycles for each polytope face a node pass; eight passes at
 // a time a quarter more and kRoundCycles for the barriers and the additions;
-// kTileCycles to finish a tile).  One tile alone is worth it from about 300 nodes,
-// two equal ones hardly, polytopes' several.  Step by single warps, all shared,
+// kTileCycles more for a further tile, whose additions wait for the one before).
+// One tile alone is always worth it, two equal ones of boxes or spheres hardly,
+// polytopes' several.  Step by single warps, all shared,
 // and so: 49 spheres and cuboids of 26 cells on walls 61.6, 53.4, 48.0 us; 1000
 // smoothed cubes on walls 47.3, 70.9, 47.1; 240 polytopes deep in one another 147,
 // 99, 86.
 constexpr int kShareNodes = 128;
-constexpr int kPassCycles = 300, kFaceCycles = 20, kRoundCycles = 150, kTileCycles = 2000;
+constexpr int kPassCycles = 300, kFaceCycles = 20, kRoundCycles = 150, kTileCycles = 3200, kShareCycles = 300;
 struct DeepTiles {
   int n, alone, shared;   // tiles, cycles of the longest alone and of all of them shared
   int3 tile[kWarps];      // the warp that clipped it, lanes with nodes, clipped nodes
@@ -1049,7 +1050,10 @@ __global__ void __launch_bounds__(kWarps * 32, kNarrowBlocks<SET>) k_narrow32(Pa
   // kernel's tail: the block's other warps help (leave_to_block)
   const bool share = ntiles <= nwarps;
   if (share) {
-    if (threadIdx.x == 0) s_deep.n = s_deep.alone = s_deep.shared = 0;
+    if (threadIdx.x == 0) {
+      s_deep.n = s_deep.alone = 0;
+      s_deep.shared = kShareCycles - kTileCycles;
+    }
     __syncthreads();
   }
   if (t < ntiles) store_rec_part(&s_rec[wid][0], lane, first);
@@ -1386,8 +1390,10 @@ __device__ __forceinline__ void sweep64(const Params& P, const Shapes& S, const 
       e.key = e.w > 0.0 ? order_key(-(pa + pb)) : LLONG_MIN;
       e.idx = e.c[0] + r.dim[0] * (e.c[1] + r.dim[1] * e.c[2]);
     };
-    // the warp's components of the sums, k mod G = gw (7: the deepest node)
-    auto mine = [&](int k) { return !SHARE || (k & (G - 1)) == gw; };
+    const bool one = !SHARE || total <= 32;   // a single pass: no partners
+    if (one && gw != 0) return;
+    // the warp's components of the sums, k mod G = gw or all (7: the deepest node)
+    auto mine = [&](int k) { return !SHARE || one || (k & (G - 1)) == gw; };
     auto add = [&](const Node64& e) {
       if (mine(0)) acc[0] += e.w;
 #pragma unroll
@@ -1413,25 +1419,28 @@ __device__ __forceinline__ void sweep64(const Params& P, const Shapes& S, const 
       for (int base0 = 0; base0 < total; base0 += 32 * G) {   // (total: the same in every warp of the group)
         const int g = base0 + 32 * gw + lane;
         if (g < total) node(g, nodes[gw][lane]);
-        group_sync();
+        __syncwarp();
+        if (!one) group_sync();
         for (int q = 0; q < G && base0 + 32 * q + lane < total; ++q) add(nodes[q][lane]);
         __syncwarp();
-        group_sync();
+        if (!one) group_sync();
       }
       // the components to the group's first warp
-      double* red = reinterpret_cast<double*>(nodes);
-      int* red_idx = reinterpret_cast<int*>(red + 8 * 32);
       static_assert(2 * 32 * sizeof(Node64) >= 8 * 32 * sizeof(double) + 32 * sizeof(int), "in the nodes' place");
+      if (!one) {
+        double* red = reinterpret_cast<double*>(nodes);
+        int* red_idx = reinterpret_cast<int*>(red + 8 * 32);
 #pragma unroll
-      for (int k = 0; k < 8; ++k)
-        if (mine(k)) red[32 * k + lane] = k < 7 ? acc[k] : __longlong_as_double(bk);
-      if (mine(7)) red_idx[lane] = bi;
-      group_sync();
-      if (gw != 0) return;   // (one tile a group)
+        for (int k = 0; k < 8; ++k)
+          if (mine(k)) red[32 * k + lane] = k < 7 ? acc[k] : __longlong_as_double(bk);
+        if (mine(7)) red_idx[lane] = bi;
+        group_sync();
+        if (gw != 0) return;   // (one tile a group)
 #pragma unroll
-      for (int k = 0; k < 7; ++k) acc[k] = red[32 * k + lane];
-      bk = __double_as_longlong(red[32 * 7 + lane]);
-      bi = red_idx[lane];
+        for (int k = 0; k < 7; ++k) acc[k] = red[32 * k + lane];
+        bk = __double_as_longlong(red[32 * 7 + lane]);
+        bi = red_idx[lane];
+      }
     }
     double v = 0.0;
     if (total > 0) {   // warp-uniform
