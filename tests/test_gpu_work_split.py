@@ -389,3 +389,85 @@ def test_fp64_form_shared_tiles(pairs, indicator):
         assert m.stats()["tiles"] == s.n // 2
         m.close()
     assert np.array_equal(outs[0], outs[1])
+
+
+# rows of particles per block of the pair builder: up to four, then eight; in the box pipeline two, then four
+@pytest.mark.parametrize("n", [9727, 9728, 9735])
+def test_pair_builder_rows_of_larger_steps(n):
+    rep, ref = _parity(_lattice_state(n), 0)
+    assert np.count_nonzero(ref.pair_out[:, 0]) > n // 4
+
+
+@pytest.mark.parametrize("n", [4863, 4864, 4867])
+def test_pair_builder_rows_of_larger_box_steps(n):
+    rep, ref = run_box(boxed(_lattice_state(n), 3))
+    assert np.count_nonzero(ref.pair_out[:, 0]) > n // 4
+
+
+def _packed_block(kinds):
+    """1728 small particles in 55^3, about a dozen candidate partners each; positions are multiples of 2^-20."""
+    rng = np.random.default_rng(17)
+    g = np.stack(np.meshgrid(*[np.arange(12)] * 3, indexing="ij"), -1).reshape(-1, 3)
+    pos = (g + 0.5) * (55.0 / 12) + rng.uniform(-0.5, 0.5, g.shape)
+    pos = np.mod(np.round(pos * 2.0 ** 20) / 2.0 ** 20, 55.0)
+    pl = cube_planes([1.5, 1.3, 1.2])
+    t = np.array(kinds)[np.arange(len(g)) % len(kinds)]
+    params = np.where(t[:, None] == W.SPHERE, [[2.5, 0.0, 0.0]], [[2.0, 2.0, 2.0]])
+    return state(t, params, pos, quat=W.random_quaternions(rng, len(g)), n=55,
+                 planes=[pl if x == W.POLYTOPE else None for x in t], indicator=1)
+
+
+def _repeated(st, m):
+    """m^3 copies of the periodic state side by side (copy-major particle numbers)."""
+    off = np.stack(np.meshgrid(*[np.arange(m)] * 3, indexing="ij"), -1).reshape(-1, 3) * st.box
+    c = len(off)
+    big = st.subset(np.tile(np.arange(st.n), c))
+    big.pos = (st.pos[None] + off[:, None]).reshape(-1, 3)
+    big.n_cells = tuple(int(v) * m for v in st.n_cells)
+    return big
+
+
+def _copies_agree(small, big, tol):
+    """Every copy's rows equal the block's: the sums add in another order, and a pair across copies may name its
+    particles the other way round, so FP32 sums of some thirty nodes differ by a few ulps of their terms."""
+    for a, b in zip(small, big):
+        assert float((b.reshape(-1, *a.shape) - a).abs().max()) <= tol * float(a.abs().max())
+
+
+# more than 1024 candidate pairs for every block that gathers them, tiles enough for the adjoint's queue
+@pytest.mark.parametrize("kinds", [[W.SPHERE], [W.CUBOID], [W.SPHERE, W.CUBOID, W.POLYTOPE]])
+@pytest.mark.parametrize("law", [False, True])
+def test_many_pairs_step_and_adjoint(kinds, law):
+    from paper_2401_10878_gb300.contact import Contact
+    st = _packed_block(kinds)
+    vel = np.random.default_rng(2).normal(size=(st.n, 6)) * 0.02
+    kw = dict(friction=True, mu_s=0.3, mu_k=0.2, u_k=0.01, damping_c=0.4) if law else {}
+    gw = W.loss_weights(st.n)
+    outs = []
+    for m in (1, 3):
+        s = st if m == 1 else _repeated(st, m)
+        model = Contact.from_state(s, **kw)
+        rep = lambda x: torch.tensor(np.tile(x, (m ** 3, 1)), device="cuda")  # noqa: E731
+        o = model.step(torch.tensor(s.pos, device="cuda"), torch.tensor(s.quat, device="cuda"), rep(vel) if law else None)
+        gp, gq = model.backward(rep(gw[0]), rep(gw[1]))
+        outs.append([o["force"].clone(), o["torque"].clone(), gp, gq])
+        pairs, tiles = o["n_pairs"], model.stats()["tiles"]
+        model.close()
+        if m == 1:
+            block = pairs
+            assert tiles < 4 * 8 * (2 if W.POLYTOPE in kinds else 3) * 152
+    assert pairs == 27 * block > 2 * 152 * 1024 and tiles > 4 * 8 * 3 * 152
+    _copies_agree(outs[0], outs[1], 1e-5)
+
+
+def test_many_pairs_of_the_box_pipeline():
+    from paper_2401_10878_gb300.contact import Contact
+    st = _packed_block([W.SPHERE, W.CUBOID, W.POLYTOPE])
+    outs = []
+    for m in (1, 3):
+        s = st if m == 1 else _repeated(st, m)
+        model = Contact.from_state(s, box_mode=1, contact_resolution=3)
+        o = model.step(torch.tensor(s.pos, device="cuda"), torch.tensor(s.quat, device="cuda"))
+        outs.append([o["force"].clone(), o["torque"].clone()])
+        model.close()
+    _copies_agree(outs[0], outs[1], 1e-5)
