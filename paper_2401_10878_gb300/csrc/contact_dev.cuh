@@ -40,9 +40,12 @@ constexpr int kPartialFloats = 12;    // FP32 partial sums per tile
 constexpr int kPartialDoubles = 10;   // FP64 partial sums per tile (the all-FP64 form: 7 sums, deepest node's key and index)
 constexpr int kTapeDoubles = 16;      // FP64 per-pair values kept for the adjoint
 constexpr int kStepCounter = 12;      // counters[] slot of the completed-step count
-constexpr int kDoneCounter = 13;      // counters[] slot: particle-sum blocks finished (the last resets it)
+constexpr int kDoneCounter = 13;      // counters[] slot: particle-sum warps finished (the last resets it)
 constexpr int kTokenCounter = 14;     // counters[] slot: the host's token of this step
 constexpr int kAdjCounter = 15;       // counters[] slot: tiles the adjoint's cell sweep took from its queue
+constexpr int kCounters = 16;
+static_assert(kStepCounter < kCounters && kDoneCounter < kCounters && kTokenCounter < kCounters && kAdjCounter < kCounters,
+              "slots of counters[]");
 constexpr int kFtDoubles = 9;         // per-pair F, T_A, T_B
 
 // Error codes written by kernels (same numbering as contact_status).
@@ -114,7 +117,7 @@ struct Params {
   float inv_binw_f[3];   // FP32 reciprocal of the bin width
   int max_pairs, max_nbr, max_tiles;
   // FP32 copies for the node sweep (lattice units)
-  float inflate_l, inv_w, neg6_over_w, wdx_l;   // wdx_l: smoothing width in cells
+  float inv_w, wdx_l;   // 1 / wdx_l; smoothing width in cells
   float clip_margin;   // of the FP32 clips and of the pair builder's separation test (line_clip.cuh)
 };
 
@@ -186,9 +189,8 @@ struct __align__(16) PairRec {   // 16-byte aligned: records are copied with 16-
   int dim[3];      // nodes per axis
   int shift[3];    // image index s of j: X_j' = X_j - s L
   int axis;        // sweep axis (the box's longest)
-  int seglen;      // nodes per line segment (the whole line)
-  int nseg;        // segments per line (1)
-  int nitems;      // lines * nseg
+  int pad[2];
+  int nitems;      // node lines
   int tile0;       // first tile of the pair
   int ntiles;
   int kinds;       // kind of i | kind of j << 8 (set by the planner)
@@ -313,15 +315,16 @@ struct Lists {
   double* ft;       // [max_pairs, kFtDoubles] (node sweep: of the overlapping pairs alone)
   const int* kind;  // [N] sweep kind of each particle (Kind, polytopes by face bucket)
   BoxWork* box_work;   // [max_pairs] box pipeline: the pairs with a rough contact
-  int* counters;    // [16]: 0 pairs, 1 tiles, 2 box pipeline rough contacts, 5 overlapping pairs, kStepCounter
-                    // steps completed (its parity selects the contact-history buffer)
+  int* counters;    // [kCounters]: 0 pairs, 1 tiles, 2 box pipeline rough contacts, 5 overlapping pairs;
+                    // kStepCounter steps completed (its parity selects the contact-history buffer),
+                    // kDoneCounter, kTokenCounter, kAdjCounter
   unsigned long long* u64;  // [4]: 0 node evaluations, 1 nominal lane-ops of the node sweep
   int* err;         // [1] sticky device error
   int* err_host;    // [4] mapped host words: 0 mirrors err; 1 the token of the last completed step
-                    // (written by the step's last block); 2 the token the host gave the step being
+                    // (written by the step's last warp); 2 the token the host gave the step being
                     // launched (read by k_pose into counters[kTokenCounter]); 3 the last step's pairs
   int publish;      // 1 in a host-buffer step that returns on its token: k_pose reads the token, the
-                    // particle sums' last block mirrors err and publishes it (0: err mirrored at the
+                    // particle sums' last warp mirrors err and publishes it (0: err mirrored at the
                     // start of the particle sums, no token)
 };
 
@@ -331,44 +334,6 @@ struct Lists {
 __device__ __forceinline__ double dmul(double a, double b) { return __dmul_rn(a, b); }
 __device__ __forceinline__ double dadd(double a, double b) { return __dadd_rn(a, b); }
 __device__ __forceinline__ double dsub(double a, double b) { return __dsub_rn(a, b); }
-
-// Row k of the rotation of q / |q| (w, x, y, z), body -> world, in homogeneous
-// form with s = 2 / |q|^2 (2 RN(1/nn) == RN(2/nn): scaling by 2 is exact).
-__device__ inline void rotation_row_rn(const double q[4], double s, int k, double r[3]) {
-  const double w = q[0], x = q[1], y = q[2], z = q[3];
-  if (k == 0) {
-    r[0] = dsub(1.0, dmul(s, dadd(dmul(y, y), dmul(z, z))));
-    r[1] = dmul(s, dsub(dmul(x, y), dmul(w, z)));
-    r[2] = dmul(s, dadd(dmul(x, z), dmul(w, y)));
-  } else if (k == 1) {
-    r[0] = dmul(s, dadd(dmul(x, y), dmul(w, z)));
-    r[1] = dsub(1.0, dmul(s, dadd(dmul(x, x), dmul(z, z))));
-    r[2] = dmul(s, dsub(dmul(y, z), dmul(w, x)));
-  } else {
-    r[0] = dmul(s, dsub(dmul(x, z), dmul(w, y)));
-    r[1] = dmul(s, dadd(dmul(y, z), dmul(w, x)));
-    r[2] = dsub(1.0, dmul(s, dadd(dmul(x, x), dmul(y, y))));
-  }
-}
-
-// Rotation of the normalised quaternion (w, x, y, z), body -> world, row-major.
-__device__ inline void rotation_rn(const double q[4], double* qh, double* qn, double R[9]) {
-  const double nrm = __dsqrt_rn(dadd(dadd(dadd(dmul(q[0], q[0]), dmul(q[1], q[1])), dmul(q[2], q[2])),
-                                     dmul(q[3], q[3])));
-  const double w = __ddiv_rn(q[0], nrm), x = __ddiv_rn(q[1], nrm), y = __ddiv_rn(q[2], nrm),
-               z = __ddiv_rn(q[3], nrm);
-  qh[0] = w; qh[1] = x; qh[2] = y; qh[3] = z;
-  *qn = nrm;
-  R[0] = dsub(1.0, dmul(2.0, dadd(dmul(y, y), dmul(z, z))));
-  R[1] = dmul(2.0, dsub(dmul(x, y), dmul(w, z)));
-  R[2] = dmul(2.0, dadd(dmul(x, z), dmul(w, y)));
-  R[3] = dmul(2.0, dadd(dmul(x, y), dmul(w, z)));
-  R[4] = dsub(1.0, dmul(2.0, dadd(dmul(x, x), dmul(z, z))));
-  R[5] = dmul(2.0, dsub(dmul(y, z), dmul(w, x)));
-  R[6] = dmul(2.0, dsub(dmul(x, z), dmul(w, y)));
-  R[7] = dmul(2.0, dadd(dmul(y, z), dmul(w, x)));
-  R[8] = dsub(1.0, dmul(2.0, dadd(dmul(x, x), dmul(y, y))));
-}
 
 // Order-preserving integer key of an FP64 value (comparisons without FP64 instructions).
 __device__ __forceinline__ long long order_key(double x) {

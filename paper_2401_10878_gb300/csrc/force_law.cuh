@@ -1,6 +1,7 @@
 // FP64 force law of one overlapping pair (Sec. 2.3 Eq. (contact_force_normal),
-// Sec. 2.2 torques, Sec. 3.3.1 contact point, normal and indentation depth),
-// run by a node-sweep warp for up to eight overlapping pairs it has completed.
+// Sec. 2.2 torques, Sec. 3.3.1 contact point, normal and indentation depth): a
+// warp runs it for up to eight overlapping pairs of the step (k_force), or of the
+// box pipeline's contacts (k_box_law).
 //
 // Every FP64 warp instruction occupies a sub-partition's FP64 pipe for ~64
 // cycles however many lanes are active, so each pair's chain is split over

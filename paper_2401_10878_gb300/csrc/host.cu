@@ -539,9 +539,7 @@ contact_status contact_init(const contact_config* cfg, const int32_t* shape_type
   P.max_pairs = C.max_pairs;
   P.max_nbr = max_nbr;
   P.max_tiles = static_cast<int>(max_tiles_ll);
-  P.inflate_l = static_cast<float>(C.inflate / C.dx);
   P.inv_w = static_cast<float>(1.0 / C.smooth_width);
-  P.neg6_over_w = static_cast<float>(-6.0 / C.smooth_width);
   P.wdx_l = static_cast<float>(C.smooth_width);
   P.clip_margin = margin;
 
@@ -665,12 +663,12 @@ contact_status contact_init(const contact_config* cfg, const int32_t* shape_type
   GBC_TRY(dev_alloc(c, &W.pdone, mp));
   GBC_TRY(dev_alloc(c, &W.tape, mp * kTapeDoubles));
   GBC_TRY(dev_alloc(c, &W.ft, mp * kFtDoubles));
-  GBC_TRY(dev_alloc(c, &W.counters, 16));
+  GBC_TRY(dev_alloc(c, &W.counters, kCounters));
   GBC_TRY(dev_alloc(c, &W.u64, 4));
   GBC_TRY(dev_alloc(c, &W.err, 1));
   GBC_TRY(dev_alloc(c, &c->adj_scratch, adjoint_scratch_doubles(C.max_pairs, P.max_tiles)));
   W.kind = d_kind;
-  GBC_TRY(cudaMemset(W.counters, 0, 16 * sizeof(int)));
+  GBC_TRY(cudaMemset(W.counters, 0, kCounters * sizeof(int)));
   GBC_TRY(cudaMemset(W.u64, 0, 4 * sizeof(unsigned long long)));
   GBC_TRY(cudaMemset(W.err, 0, sizeof(int)));
   GBC_TRY(cudaMemset(W.up_count, 0, sizeof(int) * n));
@@ -812,7 +810,7 @@ contact_status contact_stats(contact_ctx* c, int64_t* stats) {
   if (c == nullptr || stats == nullptr) return CONTACT_EINVAL;
   cudaError_t e = cudaStreamSynchronize(c->stream);
   if (e != cudaSuccess) return cuda_fail(c, e, "cudaStreamSynchronize");
-  int h[16];
+  int h[kCounters];
   unsigned long long u[4];
   e = cudaMemcpy(h, c->W.counters, sizeof(h), cudaMemcpyDeviceToHost);
   if (e == cudaSuccess) e = cudaMemcpy(u, c->W.u64, sizeof(u), cudaMemcpyDeviceToHost);
@@ -1062,7 +1060,7 @@ contact_status contact_step_host(contact_ctx* c, const double* pos, const double
   };
   // When the kernels write the results in place (no copies after the last
   // kernel) and no step of contact_step may still be queued, the step gets a
-  // fresh token (read by its first kernel, published by its last block once
+  // fresh token (read by its first kernel, published by its last warp once
   // the results are stored) and the call waits for that token instead of
   // synchronising the stream; a queued step could carry the token, so after
   // contact_step, as with copies, it synchronises (and later calls use tokens

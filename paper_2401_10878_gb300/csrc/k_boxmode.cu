@@ -383,8 +383,6 @@ __device__ __forceinline__ float warp_sum_f(float v) {
   return v;
 }
 
-__device__ __forceinline__ int comp3i(int a, int b, int c, int k) { return k == 0 ? a : (k == 1 ? b : c); }
-
 // Component c of the partner's position in the pair's image.
 __device__ __forceinline__ double image_x(const Params& P, const Parts& D, const PairRec& r, int j, int c) {
   return D.X[3 * j + c] - (r.shift[c] == 0 ? 0.0 : (r.shift[c] > 0 ? P.L[c] : -P.L[c]));

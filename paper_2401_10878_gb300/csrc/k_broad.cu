@@ -108,7 +108,8 @@ __global__ void k_pose(Params P, Shapes S, Parts D, Lists W, const double* __res
     const int k = ROWS == 1 ? (k0 < 3 ? k0 : 0) : row;
     const int k1 = k == 2 ? 0 : k + 1;
     const double Xk = k == 0 ? X[0] : (k == 1 ? X[1] : X[2]);
-    // row k of the rotation (rotation_row_rn with the row's cyclic axes k, k1, k2):
+    // row k of the rotation of q / |q|, body -> world, in homogeneous form (s = 2 / |q|^2;
+    // 2 RN(1/nn) == RN(2/nn): scaling by 2 is exact), with the row's cyclic axes k, k1, k2:
     // 1 - s (q_k1^2 + q_k2^2), s (q_k q_k1 - w q_k2), s (q_k q_k2 + w q_k1)
     const double qk = k == 0 ? q[1] : (k == 1 ? q[2] : q[3]);
     const double qk1 = k == 0 ? q[2] : (k == 1 ? q[3] : q[1]);
@@ -584,7 +585,7 @@ __device__ __forceinline__ void store_pair_rec(PairRec* dst, const PairRec& r, i
   d[0] = make_int4(r.i, r.j, r.lo[0], r.lo[1]);
   d[1] = make_int4(r.lo[2], r.dim[0], r.dim[1], r.dim[2]);
   d[2] = make_int4(r.shift[0], r.shift[1], r.shift[2], r.axis);
-  d[3] = make_int4(r.seglen, r.nseg, r.nitems, r.tile0);
+  d[3] = make_int4(0, 0, r.nitems, r.tile0);
   d[4] = make_int4(r.ntiles, r.kinds, r.ai[0], r.ai[1]);
   d[5] = make_int4(r.ai[2], r.bi[0], r.bi[1], r.bi[2]);
   d[6] = make_int4(f(r.af[0]), f(r.af[1]), f(r.af[2]), f(r.bf[0]));
@@ -995,8 +996,6 @@ __global__ void __launch_bounds__(32) k_build_pairs(Params P, Parts D, Lists W, 
       {
         const int a = pr.dim[1] > pr.dim[0] ? (pr.dim[2] > pr.dim[1] ? 2 : 1) : (pr.dim[2] > pr.dim[0] ? 2 : 0);
         pr.axis = a;
-        pr.nseg = 1;
-        pr.seglen = a == 0 ? pr.dim[0] : (a == 1 ? pr.dim[1] : pr.dim[2]);
       }
       pr.nitems = pr.axis == 0 ? lines_of[0] : (pr.axis == 1 ? lines_of[1] : lines_of[2]);
       // the box pipeline takes each kept pair as one entry of the tile list

@@ -20,8 +20,8 @@
 //   * the clipped nodes are spread one per lane (sweep_tile);
 //   * node coordinates relative to each particle are exact integers minus an
 //     FP32 remainder in [-1/2, 1/2] (no large-offset cancellation);
-//   * polytope faces (and their inverse slopes along the line) are staged
-//     in shared memory;
+//   * polytope faces (and their bounds along the lines) are staged in shared
+//     memory;
 //   * warp reduction per tile (skipped when no lane met a node to
 //     evaluate); a pair of one tile is finished from the warp's registers,
 //     otherwise the partials go to HBM and the warp that completes the pair's
@@ -220,8 +220,7 @@ struct CubeEval {
 };
 
 // Stage a polytope's world planes in local axes (u, v, w, offset) into shared
-// memory, and each face's inverse slope along u (the line clip) after them;
-// faces beyond nf are padded so that they never win the maximum (and are
+// memory; faces beyond nf are padded so that they never win the maximum (and are
 // constant along the line, below any threshold).
 __device__ __forceinline__ void stage_planes(const Shapes& S, const Parts& D, int pid, const Local& L,
                                             float4* sm, int npad) {

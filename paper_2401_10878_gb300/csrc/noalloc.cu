@@ -128,7 +128,7 @@ __global__ void k_noalloc_prep(Params P, int* type, int* kind, double* param, fl
     vert_off[t] = 0;
   }
   for (int b = t; b < nbins; b += gridDim.x * blockDim.x) W.bin_count[b] = 0;
-  if (t < 16) W.counters[t] = 0;
+  if (t < kCounters) W.counters[t] = 0;
   if (t < 4) W.u64[t] = 0;
   if (t == 0) *W.err = 0;
   if (t < 4) W.err_host[t] = 0;
@@ -220,9 +220,7 @@ extern "C" contact_status contact_step_noalloc(const contact_config* cfg, const 
   P.max_pairs = C.max_pairs;
   P.max_nbr = kMaxNbr;
   P.max_tiles = C.max_tiles > 0 ? C.max_tiles : kMaxTilesPerPair * C.max_pairs;
-  P.inflate_l = static_cast<float>(C.inflate / C.dx);
   P.inv_w = static_cast<float>(1.0 / C.smooth_width);
-  P.neg6_over_w = static_cast<float>(-6.0 / C.smooth_width);
   P.wdx_l = static_cast<float>(C.smooth_width);
   P.clip_margin = clip_margin(rmax / C.dx, C.smooth_width);
 
@@ -279,7 +277,7 @@ extern "C" contact_status contact_step_noalloc(const contact_config* cfg, const 
   W.tape = cv.take<double>(MP * kTapeDoubles);
   W.ft = cv.take<double>(MP * kFtDoubles);
   W.kind = kind;
-  W.counters = cv.take<int>(16);
+  W.counters = cv.take<int>(kCounters);
   W.u64 = cv.take<unsigned long long>(4);
   W.err = cv.take<int>(1);
   W.err_host = cv.take<int>(4);   // the mapped-host words of the context path, here on the device
