@@ -1280,10 +1280,9 @@ struct Node64 {
 // The sweep's shared memory, per warp of a block.
 struct Shared64 {
   alignas(16) PairRec rec[kWarps];
-  float4 planes[kWarps][2][2 * kMaxFaces];       // the clips' constants
+  float4 planes[kWarps][2][2 * kMaxFaces];       // the clips' constants; then a shared tile's nodes (Node64)
   unsigned pk[kWarps][kTileItemsPerLane * 32];   // clipped ranges: first node | count << 16
   int excl[kWarps][32];                          // nodes before each lane's
-  Node64 node[kWarps][32];                       // a shared tile's nodes
 };
 
 // The tiles of the calling warp.  SHARE: G = 2, 4 or 8 warps of a block have one
@@ -1419,20 +1418,22 @@ __device__ __forceinline__ void sweep64(const Params& P, const Shapes& S, const 
         }
       }
     } else {
-      Node64(*nodes)[32] = sm.node + group * G;
+      // warp q's nodes, where its clips' constants were
+      auto nodes = [&](int q) { return reinterpret_cast<Node64*>(sm.planes[group * G + q]); };
+      static_assert(sizeof(sm.planes[0]) >= 32 * sizeof(Node64), "in the planes' place");
       for (int base0 = 0; base0 < total; base0 += 32 * G) {   // (total: the same in every warp of the group)
         const int g = base0 + 32 * gw + lane;
-        if (g < total) node(g, nodes[gw][lane]);
+        if (g < total) node(g, nodes(gw)[lane]);
         __syncwarp();
         if (!one) group_sync();
-        for (int q = 0; q < G && base0 + 32 * q + lane < total; ++q) add(nodes[q][lane]);
+        for (int q = 0; q < G && base0 + 32 * q + lane < total; ++q) add(nodes(q)[lane]);
         __syncwarp();
         if (!one) group_sync();
       }
       // the components to the group's first warp
-      static_assert(2 * 32 * sizeof(Node64) >= 8 * 32 * sizeof(double) + 32 * sizeof(int), "in the nodes' place");
+      static_assert(2 * sizeof(sm.planes[0]) >= 8 * 32 * sizeof(double) + 32 * sizeof(int), "in the nodes' place");
       if (!one) {
-        double* red = reinterpret_cast<double*>(nodes);
+        double* red = reinterpret_cast<double*>(nodes(0));
         int* red_idx = reinterpret_cast<int*>(red + 8 * 32);
 #pragma unroll
         for (int k = 0; k < 8; ++k)
